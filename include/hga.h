@@ -293,9 +293,8 @@ HGA_API int64_t hga_kernel_launch_count(void);
 #define HGA_KERNELS_ROUTE_GENERIC 2  /* hga_route / hga_route_static, CUDA-core router (three launches) */
 #define HGA_KERNELS_FWD_TENSOR 3     /* hga_attn_fwd, tensor-core kernel */
 #define HGA_KERNELS_FWD_GENERIC 4    /* hga_attn_fwd, one warp per query row */
-#define HGA_KERNELS_BWD_TENSOR 5     /* hga_attn_bwd, tensor-core kernels (local band + routed sweep, and
-                                        the delta pre-pass where one is launched) */
-#define HGA_KERNELS_BWD_GENERIC 6    /* hga_attn_bwd, CUDA-core kernels (delta, dQ, dK/dV) */
+#define HGA_KERNELS_BWD_TENSOR 5     /* hga_attn_bwd, tensor-core kernels (local band + routed sweep) */
+#define HGA_KERNELS_BWD_GENERIC 6    /* hga_attn_bwd, CUDA-core kernel */
 #define HGA_KERNELS_AUX 7            /* conversions (bf16 gradient outputs) and the self-test kernel */
 #define HGA_KERNELS_FAMILIES 8
 HGA_API int64_t hga_kernel_launch_count_by_family(int family);

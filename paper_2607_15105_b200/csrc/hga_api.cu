@@ -104,7 +104,8 @@ static size_t bwd_delta_bytes(const Dims& dm) {
 }
 
 size_t bwd_workspace_bytes(const Dims& dm) {
-  // delta = rowsum(dO * O), fp32 [B, Hq, S]; with bf16 gradient outputs also the fp32 dK and dV sums
+  // fp32 [B, Hq, S] (room for per-row sums; no kernel uses it at present, the size is part of the call's contract);
+  // with bf16 gradient outputs also the fp32 dK and dV sums
   size_t bytes = bwd_delta_bytes(dm) + 16;
   if (dm.flags & HGA_FLAG_BWD_BF16_GRADS) bytes += 2 * (size_t)dm.B * dm.Hkv * dm.S * dm.d * sizeof(float);
   return bytes;
@@ -258,7 +259,6 @@ int hga_attn_bwd(const hga_params* p, const void* Q, const void* K, const void* 
   if (!workspace || workspace_bytes < bwd_workspace_bytes(dm)) return HGA_ERR_WORKSPACE;
   if (!aligned16(workspace)) return HGA_ERR_ALIGN;
   cudaStream_t st = (cudaStream_t)stream;
-  const bool zero_grads = !(dm.flags & HGA_FLAG_BWD_ACCUMULATE);
   const size_t n_kv = (size_t)dm.B * dm.Hkv * dm.S * dm.d;
   if (bf16_grads) {
     // the sums over query blocks run in fp32 in the workspace and are rounded once at the end, by one
@@ -273,16 +273,8 @@ int hga_attn_bwd(const hga_params* p, const void* Q, const void* K, const void* 
     rc = launch_attn_bwd_sm100(dm, Q, K, V, O, LSE, dO, group_idx, n_groups, dQ, dK, dV, status_word, st);
     tensor_path = rc == HGA_OK;
   }
-  if (rc == HGA_ERR_UNSUPPORTED) {
-    if (zero_grads) {
-      rc = record_cuda(cudaMemsetAsync(dK, 0, n_kv * sizeof(float), st));
-      if (rc) return rc;
-      rc = record_cuda(cudaMemsetAsync(dV, 0, n_kv * sizeof(float), st));
-      if (rc) return rc;
-    }
-    rc = launch_attn_bwd_generic(dm, Q, K, V, O, LSE, dO, group_idx, n_groups, dQ, dK, dV,
-                                 (float*)workspace, status_word, st);
-  }
+  if (rc == HGA_ERR_UNSUPPORTED)
+    rc = launch_attn_bwd_generic(dm, Q, K, V, O, LSE, dO, group_idx, n_groups, dQ, dK, dV, status_word, st);
   if (rc || !bf16_grads) return rc;
   return launch_grads_to_bf16(dK, dK_out, dV_out, n_kv, tensor_path && !(dm.flags & kFlagNoPdl), st);
 }

@@ -1,6 +1,6 @@
 // Shape-generic CUDA-core kernels for routed exact-token attention (Section 2.1 item 3) and
-// its backward under segment-wise TBPTT (Section 2.2).  One warp owns one query row (or,
-// for dK/dV, one key row); a lane owns d/32 consecutive elements.  These kernels accept
+// its backward under segment-wise TBPTT (Section 2.2).  Forward: one warp owns one query row, a lane owns
+// d/32 consecutive elements.  Backward: one CTA owns 8 query rows of an item.  These kernels accept
 // every shape hga_params allows and serve as the cross-check of the tensor-core kernels.
 #include <cfloat>
 
@@ -60,37 +60,62 @@ __device__ inline float warp_sum(float x) {
   return x;
 }
 
-// Builds the item's routed token list in shared memory: sink, valid groups, local window.
-// Invalid group entries are skipped and reported.  Returns the number of tokens; s_meta[0]
-// receives the number of valid groups.
-__device__ int build_token_list(const Dims& dm, const Window& w, const int32_t* gi, int ng,
-                                int* toks, int* s_meta, int32_t* status_word) {
-  const int tid = threadIdx.x;
-  // thread 0 validates sequentially (ascending, inside [se, ls)) and compacts group ids
-  int* vg = toks + max_routed_tokens(dm);     // scratch for valid group ids, `width` entries
-  if (tid == 0) {
-    int n = 0, prev = -1, bad = 0;
-    if (ng > dm.width) { ng = dm.width; bad = 1; }
-    if (ng < 0) { ng = 0; bad = 1; }
-    for (int i = 0; i < ng; ++i) {
-      const int m = gi[i];
-      const bool ok = m > prev && (int64_t)m * dm.g >= w.se && ((int64_t)m + 1) * dm.g <= w.ls;
-      if (ok) { vg[n++] = m; prev = m; } else bad = 1;
+// The item's valid group ids in shared memory (vg, up to `width` entries); returns how many.  Invalid entries (not
+// ascending, or not wholly between sink and local window) are skipped and reported.
+__device__ int build_group_list(const Dims& dm, const Window& w, const int32_t* gi, int ng, int* vg, int* s_meta,
+                                int32_t* status_word) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  auto fits = [&](int m, int last) {
+    return m > last && (int64_t)m * dm.g >= w.se && ((int64_t)m + 1) * dm.g <= w.ls;
+  };
+  if (tid < 32) {
+    // a valid list (the common case) passes 32 entries per vote; only an invalid one is walked sequentially
+    bool bad = ng < 0 || ng > dm.width;
+    ng = ng < 0 ? 0 : ng > dm.width ? dm.width : ng;
+    bool clean = true;
+    int prev = -1;
+    for (int base = 0; base < ng; base += 32) {
+      const int i = base + lane;
+      const int m = i < ng ? gi[i] : 0x7fffffff;
+      int left = __shfl_up_sync(0xffffffffu, m, 1);
+      if (lane == 0) left = prev;
+      clean = clean && __all_sync(0xffffffffu, i >= ng || fits(m, left));
+      if (i < ng) vg[i] = m;
+      prev = __shfl_sync(0xffffffffu, m, 31);
     }
-    s_meta[0] = n;
-    if (bad && status_word) atomicOr(status_word, HGA_STATUS_BAD_INDEX);
+    __syncwarp();
+    int n = ng;
+    if (!clean && lane == 0) {
+      n = 0;
+      int last = -1;
+      for (int i = 0; i < ng; ++i) {
+        const int m = vg[i];
+        if (fits(m, last)) { vg[n++] = m; last = m; }
+      }
+    }
+    if (lane == 0) {
+      s_meta[0] = n;
+      if ((bad || !clean) && status_word) atomicOr(status_word, HGA_STATUS_BAD_INDEX);
+    }
   }
   __syncthreads();
-  const int nvg = s_meta[0];
-  const int n_far = w.se + nvg * dm.g;
+  return s_meta[0];
+}
+
+// Token i of the routed set (sink, valid groups, local window), n_far = sink and group tokens
+__device__ inline int routed_token(const Dims& dm, const Window& w, const int* vg, int n_far, int i) {
+  if (i < w.se) return i;
+  if (i < n_far) return vg[(i - w.se) / dm.g] * dm.g + (i - w.se) % dm.g;
+  return w.ls + (i - n_far);
+}
+
+// The item's whole token list in shared memory; returns its length, s_meta[0] receives the number of valid groups.
+__device__ int build_token_list(const Dims& dm, const Window& w, const int32_t* gi, int ng,
+                                int* toks, int* s_meta, int32_t* status_word) {
+  int* vg = toks + max_routed_tokens(dm);
+  const int n_far = w.se + build_group_list(dm, w, gi, ng, vg, s_meta, status_word) * dm.g;
   const int n_tok = n_far + (w.p0 + dm.Bq - w.ls);
-  for (int i = tid; i < n_tok; i += blockDim.x) {
-    int t;
-    if (i < w.se) t = i;
-    else if (i < n_far) t = vg[(i - w.se) / dm.g] * dm.g + (i - w.se) % dm.g;
-    else t = w.ls + (i - n_far);
-    toks[i] = t;
-  }
+  for (int i = threadIdx.x; i < n_tok; i += blockDim.x) toks[i] = routed_token(dm, w, vg, n_far, i);
   __syncthreads();
   return n_tok;
 }
@@ -162,136 +187,201 @@ k_attn_fwd_generic(const uint16_t* __restrict__ Q, const uint16_t* __restrict__ 
   }
 }
 
-// delta[row] = sum_e dO[row][e] * O[row][e]
-template <int D>
-__global__ void __launch_bounds__(kAttnThreads)
-k_bwd_delta(const uint16_t* __restrict__ O, const uint16_t* __restrict__ dO, Dims dm,
-            float* __restrict__ delta) {
-  constexpr int EPL = D / 32;
-  const int lane = threadIdx.x & 31;
-  const int64_t row = (int64_t)blockIdx.x * kAttnWarps + (threadIdx.x >> 5);
-  const int64_t n_rows = (int64_t)dm.B * dm.Hq * dm.S;
-  if (row >= n_rows) return;
-  const int s = row % dm.S, hq = (row / dm.S) % dm.Hq, b = row / ((int64_t)dm.S * dm.Hq);
-  const int64_t off = b * dm.os[0] + hq * dm.os[1] + s * dm.os[2] + lane * EPL;
-  const float x = warp_sum(dot_frag<EPL>(load_frag<EPL>(O + off), load_frag<EPL>(dO + off)));
-  if (lane == 0) delta[row] = x;
-}
+// Backward.  One CTA owns kBwdRows query rows of an item; its eight warps take the item's routed keys in turn, eight
+// at a time, each on its own (no block barrier in the loop; the next keys' loads are in flight during the work on
+// the current ones).  Per warp and eight keys:
+//   S = Q K^T, dP = dO V^T   lane = one row, two keys        -> P, dS in shared memory
+//   dQ += dS K               lane = one row, d/4 elements (registers; the warps' sums meet at the end)
+//   dV = P^T dO, dK = dS^T Q lane = one key, d/4 elements, added to global memory 16 bytes at a time (keys of the
+//                            active segment only: history keys are detached constants)
+// Everything is fp32.  Taken for shapes the tensor-core kernels do not cover and for problems too small to fill
+// them, so what counts is the length of one CTA's chain and how many CTAs there are; the work itself is bound by
+// shared-memory reads, 216 per 640 fused multiply-adds of a warp.
+constexpr int kBwdRows = 8, kBwdKeys = 8, kBwdWarps = 8;
 
 template <int D>
-__global__ void __launch_bounds__(kAttnThreads)
-k_bwd_dq_generic(const uint16_t* __restrict__ Q, const uint16_t* __restrict__ K,
-                 const uint16_t* __restrict__ V, const uint16_t* __restrict__ dO,
-                 const float* __restrict__ LSE, const float* __restrict__ delta,
-                 const int32_t* __restrict__ group_idx, const int32_t* __restrict__ n_groups,
-                 Dims dm, uint16_t* __restrict__ dQ, int32_t* status_word) {
-  constexpr int EPL = D / 32;
-  extern __shared__ int s_int[];
+struct BwdTile {
+  static constexpr int kPitch = D + 4;           // floats; 16-byte aligned rows that start 4 banks apart
+  float q[kBwdRows][kPitch], dO[kBwdRows][kPitch];
+  struct PerWarp {
+    float k[kBwdKeys][kPitch], v[kBwdKeys][kPitch];       // (at the end: the warp's dQ sums)
+    float p[kBwdRows][kBwdKeys], ds[kBwdRows][kBwdKeys];
+    int tok[kBwdKeys];                           // -1 past the end of the list
+  } w[kBwdWarps];
+  static_assert(kBwdRows <= kBwdKeys, "dQ sums fit the K tile");
+};
+
+__device__ inline void bf16x8_to_smem(float* dst, uint4 w) {
+  const uint32_t x[4] = {w.x, w.y, w.z, w.w};
+  float4* d4 = reinterpret_cast<float4*>(dst);
+  d4[0] = make_float4(__uint_as_float(x[0] << 16), __uint_as_float(x[0] & 0xffff0000u), __uint_as_float(x[1] << 16), __uint_as_float(x[1] & 0xffff0000u));
+  d4[1] = make_float4(__uint_as_float(x[2] << 16), __uint_as_float(x[2] & 0xffff0000u), __uint_as_float(x[3] << 16), __uint_as_float(x[3] & 0xffff0000u));
+}
+__device__ inline float dot4(float4 a, float4 b, float s) {
+  return fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, s))));
+}
+__device__ inline void fma4(float4& acc, float s, float4 x) {
+  acc.x = fmaf(s, x.x, acc.x); acc.y = fmaf(s, x.y, acc.y); acc.z = fmaf(s, x.z, acc.z); acc.w = fmaf(s, x.w, acc.w);
+}
+__device__ inline float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+
+template <int D>
+__global__ void __launch_bounds__(32 * kBwdWarps)
+k_attn_bwd_generic(const uint16_t* __restrict__ Q, const uint16_t* __restrict__ K, const uint16_t* __restrict__ V,
+                   const uint16_t* __restrict__ O, const float* __restrict__ LSE, const uint16_t* __restrict__ dO,
+                   const int32_t* __restrict__ group_idx, const int32_t* __restrict__ n_groups, Dims dm,
+                   uint16_t* __restrict__ dQ, float* __restrict__ dK, float* __restrict__ dV, int32_t* status_word) {
+  constexpr int kParts = D / 8, kLoads = kBwdKeys * kParts / 32;     // 16-byte pieces of a row; pieces per lane and tensor
+  extern __shared__ __align__(16) uint8_t s_raw[];
+  BwdTile<D>& sm = *reinterpret_cast<BwdTile<D>*>(s_raw);
+  int* vg = reinterpret_cast<int*>(s_raw + sizeof(BwdTile<D>));      // valid group ids
   __shared__ int s_meta[2];
-  const int item = blockIdx.x;
+  __shared__ float s_lse[kBwdRows], s_delta[kBwdRows];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int slices = (dm.rows + kBwdRows - 1) / kBwdRows;
+  const int item = blockIdx.x / slices, r0 = (blockIdx.x % slices) * kBwdRows;
   int b, h, qb;
   item_coords(dm, item, b, h, qb);
   const Window w = window_of(dm, qb);
-  build_token_list(dm, w, group_idx + (int64_t)item * dm.width, n_groups[item], s_int, s_meta, status_word);
-  const int n_far = w.se + s_meta[0] * dm.g;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint16_t* Kb = K + b * dm.ks[0] + h * dm.ks[1] + lane * EPL;
-  const uint16_t* Vb = V + b * dm.vs[0] + h * dm.vs[1] + lane * EPL;
-  for (int r = warp; r < dm.rows; r += kAttnWarps) {
-    const int a = r / dm.Bq, t = r % dm.Bq;
-    const int hq = h * dm.G + a, srow = qb * dm.Bq + t;
-    const int n_vis = n_far + (w.p0 + t - w.ls + 1);
-    const Frag<EPL> q = load_frag<EPL>(Q + b * dm.qs[0] + hq * dm.qs[1] + srow * dm.qs[2] + lane * EPL);
-    const Frag<EPL> go = load_frag<EPL>(dO + b * dm.os[0] + hq * dm.os[1] + srow * dm.os[2] + lane * EPL);
-    const int64_t row = ((int64_t)b * dm.Hq + hq) * dm.S + srow;
-    const float lse = LSE[row], dl = delta[row];
-    Frag<EPL> dq;
+
+  {
+    // warp = row: Q and dO to shared memory, delta = rowsum(dO o O)
+    const int r = r0 + warp;
+    const bool real = r < dm.rows;
+    const int hq = h * dm.G + (real ? r / dm.Bq : 0), sr = qb * dm.Bq + (real ? r % dm.Bq : 0);
+    const int64_t q_off = b * dm.qs[0] + hq * dm.qs[1] + sr * dm.qs[2], o_off = b * dm.os[0] + hq * dm.os[1] + sr * dm.os[2];
+    float acc = 0.f;
+    if (lane < kParts) {
+      const uint4 zero = make_uint4(0, 0, 0, 0);
+      const uint4 q8 = real ? *reinterpret_cast<const uint4*>(Q + q_off + 8 * lane) : zero;
+      const uint4 g8 = real ? *reinterpret_cast<const uint4*>(dO + o_off + 8 * lane) : zero;
+      bf16x8_to_smem(&sm.q[warp][8 * lane], q8);
+      bf16x8_to_smem(&sm.dO[warp][8 * lane], g8);
+      if (real)
+        acc = dot_frag<4>(load_frag<4>(O + o_off + 8 * lane), load_frag<4>(dO + o_off + 8 * lane)) +
+              dot_frag<4>(load_frag<4>(O + o_off + 8 * lane + 4), load_frag<4>(dO + o_off + 8 * lane + 4));
+    }
+    acc = warp_sum(acc);
+    if (lane == 0) {
+      s_delta[warp] = acc;
+      s_lse[warp] = real ? LSE[((int64_t)b * dm.Hq + hq) * dm.S + sr] : INFINITY;      // padding rows: P = 0
+    }
+  }
+  const int n_far = w.se + dm.g * build_group_list(dm, w, group_idx + (int64_t)item * dm.width, n_groups[item], vg, s_meta,
+                                                   r0 == 0 ? status_word : nullptr);   // (ends with a block barrier)
+  const int n_tok = n_far + (w.p0 + dm.Bq - w.ls);
+  const uint16_t* Kb = K + b * dm.ks[0] + h * dm.ks[1];
+  const uint16_t* Vb = V + b * dm.vs[0] + h * dm.vs[1];
+  auto& tile = sm.w[warp];
+  uint4 kk[kLoads], vv[kLoads];
+  int tok[kLoads];
+  auto fetch = [&](int t0) {                       // this lane's pieces of keys t0 .. t0+7 of the list
 #pragma unroll
-    for (int e = 0; e < EPL; ++e) dq.v[e] = 0.f;
-    for (int i = 0; i < n_vis; i += 2) {
-      float s[2], dp[2];
-      Frag<EPL> kk[2];
+    for (int i = 0; i < kLoads; ++i) {
+      const int key = (i * 32 + lane) / kParts, part = (i * 32 + lane) % kParts;
+      tok[i] = t0 + key < n_tok ? routed_token(dm, w, vg, n_far, t0 + key) : -1;
+      kk[i] = vv[i] = make_uint4(0, 0, 0, 0);
+      if (tok[i] >= 0) {
+        kk[i] = *reinterpret_cast<const uint4*>(Kb + (int64_t)tok[i] * dm.ks[2] + 8 * part);
+        vv[i] = *reinterpret_cast<const uint4*>(Vb + (int64_t)tok[i] * dm.vs[2] + 8 * part);
+      }
+    }
+  };
+  const int row = lane >> 2, quad = lane & 3;       // S, dP and dQ: row, keys 2*quad, 2*quad+1 / elements 16*c + 4*quad ..
+  const int pos = w.p0 + (r0 + row) % dm.Bq;
+  const float lse = s_lse[row], delta = s_delta[row];
+  float4 dq[D / 16];
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const int idx = i + u < n_vis ? i + u : n_vis - 1;
-        const int64_t tok = s_int[idx];
-        kk[u] = load_frag<EPL>(Kb + tok * dm.ks[2]);
-        s[u] = dot_frag<EPL>(q, kk[u]);
-        dp[u] = dot_frag<EPL>(go, load_frag<EPL>(Vb + tok * dm.vs[2]));
+  for (int c = 0; c < D / 16; ++c) dq[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+  bool waited = false;
+
+  fetch(kBwdKeys * warp);
+  for (int t0 = kBwdKeys * warp; t0 < n_tok; t0 += kBwdKeys * kBwdWarps) {
+#pragma unroll
+    for (int i = 0; i < kLoads; ++i) {
+      const int key = (i * 32 + lane) / kParts, part = (i * 32 + lane) % kParts;
+      bf16x8_to_smem(&tile.k[key][8 * part], kk[i]);
+      bf16x8_to_smem(&tile.v[key][8 * part], vv[i]);
+      if (part == 0) tile.tok[key] = tok[i];
+    }
+    __syncwarp();
+    fetch(t0 + kBwdKeys * kBwdWarps);
+    {
+      float s[2] = {0.f, 0.f}, dp[2] = {0.f, 0.f};
+#pragma unroll 8
+      for (int e = 0; e < D; e += 4) {
+        const float4 q4 = ld4(&sm.q[row][e]), g4 = ld4(&sm.dO[row][e]);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          s[u] = dot4(q4, ld4(&tile.k[2 * quad + u][e]), s[u]);
+          dp[u] = dot4(g4, ld4(&tile.v[2 * quad + u][e]), dp[u]);
+        }
       }
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
-        s[u] = warp_sum(s[u]);
-        dp[u] = warp_sum(dp[u]);
-        if (i + u < n_vis) {
-          const float p = __expf(s[u] * dm.scale - lse);
-          const float ds = p * (dp[u] - dl);
+        const int t = tile.tok[2 * quad + u];
+        const float p = t >= 0 && t <= pos ? __expf(s[u] * dm.scale - lse) : 0.f;
+        tile.p[row][2 * quad + u] = p;
+        tile.ds[row][2 * quad + u] = p * (dp[u] - delta) * dm.scale;
+      }
+    }
+    __syncwarp();
 #pragma unroll
-          for (int e = 0; e < EPL; ++e) dq.v[e] = fmaf(ds, kk[u].v[e], dq.v[e]);
+    for (int key = 0; key < kBwdKeys; ++key) {
+      const float ds = tile.ds[row][key];
+#pragma unroll
+      for (int c = 0; c < D / 16; ++c) fma4(dq[c], ds, ld4(&tile.k[key][16 * c + 4 * quad]));
+    }
+    const int mine = tile.tok[row];                 // dK, dV: key `row` of the eight
+    if (__any_sync(0xffffffffu, mine >= dm.H)) {
+      float4 gk[D / 16], gv[D / 16];
+#pragma unroll
+      for (int c = 0; c < D / 16; ++c) gk[c] = gv[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int r = 0; r < kBwdRows; ++r) {
+        const float ds = tile.ds[r][row], p = tile.p[r][row];
+#pragma unroll
+        for (int c = 0; c < D / 16; ++c) {
+          fma4(gk[c], ds, ld4(&sm.q[r][16 * c + 4 * quad]));
+          fma4(gv[c], p, ld4(&sm.dO[r][16 * c + 4 * quad]));
+        }
+      }
+      if (!waited) {
+        // dK and dV are zeroed by the launch before this one, which this one may overlap
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        waited = true;
+      }
+      if (mine >= dm.H) {
+        const int64_t off = (((int64_t)b * dm.Hkv + h) * dm.S + (mine - dm.H)) * D + 4 * quad;
+#pragma unroll
+        for (int c = 0; c < D / 16; ++c) {
+          atomicAdd(reinterpret_cast<float4*>(dK + off + 16 * c), gk[c]);
+          atomicAdd(reinterpret_cast<float4*>(dV + off + 16 * c), gv[c]);
         }
       }
     }
+    __syncwarp();
+  }
+  // the warps' dQ sums meet in the K tiles
 #pragma unroll
-    for (int e = 0; e < EPL; ++e) dq.v[e] *= dm.scale;
-    store_frag_bf16<EPL>(dQ + b * dm.qs[0] + hq * dm.qs[1] + srow * dm.qs[2] + lane * EPL, dq);
+  for (int c = 0; c < D / 16; ++c) *reinterpret_cast<float4*>(&tile.k[row][16 * c + 4 * quad]) = dq[c];
+  __syncthreads();
+  if (r0 + warp < dm.rows && lane < D / 4) {
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < kBwdWarps; ++u) fma4(a, 1.f, ld4(&sm.w[u].k[warp][4 * lane]));
+    const int r = r0 + warp, hq = h * dm.G + r / dm.Bq, sr = qb * dm.Bq + r % dm.Bq;
+    Frag<4> f;
+    f.v[0] = a.x; f.v[1] = a.y; f.v[2] = a.z; f.v[3] = a.w;
+    store_frag_bf16<4>(dQ + b * dm.qs[0] + hq * dm.qs[1] + sr * dm.qs[2] + 4 * lane, f);
   }
 }
 
-// dK/dV: one warp per routed ACTIVE key of the item (position >= H); history keys are
-// detached constants (Section 2.2) and are skipped.  Partial sums over the item's rows stay
-// in registers; one atomic add per element per (item, key) merges the query blocks.
-template <int D>
-__global__ void __launch_bounds__(kAttnThreads)
-k_bwd_dkv_generic(const uint16_t* __restrict__ Q, const uint16_t* __restrict__ K,
-                  const uint16_t* __restrict__ V, const uint16_t* __restrict__ dO,
-                  const float* __restrict__ LSE, const float* __restrict__ delta,
-                  const int32_t* __restrict__ group_idx, const int32_t* __restrict__ n_groups,
-                  Dims dm, float* __restrict__ dK, float* __restrict__ dV) {
-  constexpr int EPL = D / 32;
-  extern __shared__ int s_int[];
-  __shared__ int s_meta[2];
-  const int item = blockIdx.x;
-  int b, h, qb;
-  item_coords(dm, item, b, h, qb);
-  const Window w = window_of(dm, qb);
-  const int n_tok = build_token_list(dm, w, group_idx + (int64_t)item * dm.width, n_groups[item],
-                                     s_int, s_meta, nullptr);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint16_t* Qb = Q + b * dm.qs[0] + (int64_t)(h * dm.G) * dm.qs[1] + (int64_t)(qb * dm.Bq) * dm.qs[2] + lane * EPL;
-  const uint16_t* dOb = dO + b * dm.os[0] + (int64_t)(h * dm.G) * dm.os[1] + (int64_t)(qb * dm.Bq) * dm.os[2] + lane * EPL;
-  for (int i = warp; i < n_tok; i += kAttnWarps) {
-    const int tok = s_int[i];
-    if (tok < dm.H) continue;
-    const Frag<EPL> kk = load_frag<EPL>(K + b * dm.ks[0] + h * dm.ks[1] + (int64_t)tok * dm.ks[2] + lane * EPL);
-    const Frag<EPL> vv = load_frag<EPL>(V + b * dm.vs[0] + h * dm.vs[1] + (int64_t)tok * dm.vs[2] + lane * EPL);
-    Frag<EPL> dk, dv;
-#pragma unroll
-    for (int e = 0; e < EPL; ++e) dk.v[e] = dv.v[e] = 0.f;
-    const int t_first = tok > w.p0 ? tok - w.p0 : 0;    // causal: rows at or after the key
-    for (int a = 0; a < dm.G; ++a) {
-      const int64_t row0 = ((int64_t)b * dm.Hq + h * dm.G + a) * dm.S + qb * dm.Bq;
-      for (int t = t_first; t < dm.Bq; ++t) {
-        const Frag<EPL> q = load_frag<EPL>(Qb + a * dm.qs[1] + t * dm.qs[2]);
-        const Frag<EPL> go = load_frag<EPL>(dOb + a * dm.os[1] + t * dm.os[2]);
-        const float s = warp_sum(dot_frag<EPL>(q, kk));
-        const float dp = warp_sum(dot_frag<EPL>(go, vv));
-        const float p = __expf(s * dm.scale - LSE[row0 + t]);
-        const float ds = p * (dp - delta[row0 + t]);
-#pragma unroll
-        for (int e = 0; e < EPL; ++e) {
-          dk.v[e] = fmaf(ds, q.v[e], dk.v[e]);
-          dv.v[e] = fmaf(p, go.v[e], dv.v[e]);
-        }
-      }
-    }
-    float* dKr = dK + (((int64_t)b * dm.Hkv + h) * dm.S + (tok - dm.H)) * D + lane * EPL;
-    float* dVr = dV + (((int64_t)b * dm.Hkv + h) * dm.S + (tok - dm.H)) * D + lane * EPL;
-#pragma unroll
-    for (int e = 0; e < EPL; ++e) {
-      atomicAdd(dKr + e, dk.v[e] * dm.scale);
-      atomicAdd(dVr + e, dv.v[e]);
-    }
-  }
+// dK and dV to zero, one launch for both tensors (n elements each, a multiple of 8)
+__global__ void __launch_bounds__(256) k_zero_grads(float4* __restrict__ a, float4* __restrict__ b, size_t n4) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n4) a[i] = b[i] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 static size_t token_smem_bytes(const Dims& dm) {
@@ -357,38 +447,44 @@ template <int D>
 static int bwd_generic(const Dims& dm, const uint16_t* Q, const uint16_t* K, const uint16_t* V,
                        const uint16_t* O, const float* LSE, const uint16_t* dO,
                        const int32_t* group_idx, const int32_t* n_groups, uint16_t* dQ, float* dK,
-                       float* dV, float* delta, int32_t* status_word, cudaStream_t st) {
-  const int items = dm.B * dm.Hkv * dm.NQB;
-  const size_t smem = token_smem_bytes(dm);
-  if (smem > 200 * 1024) return HGA_ERR_UNSUPPORTED;
-  cudaError_t e = cudaFuncSetAttribute(k_bwd_dq_generic<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_bwd_dkv_generic<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return record_cuda(e);
-  const int64_t n_rows = (int64_t)dm.B * dm.Hq * dm.S;
-  k_bwd_delta<D><<<(unsigned)((n_rows + kAttnWarps - 1) / kAttnWarps), kAttnThreads, 0, st>>>(O, dO, dm, delta);
-  count_launch(HGA_KERNELS_BWD_GENERIC);
-  int rc = record_cuda(cudaGetLastError());
+                       float* dV, int32_t* status_word, cudaStream_t st) {
+  const size_t smem = sizeof(BwdTile<D>) + sizeof(int) * ((size_t)dm.width + 4);
+  if (smem > 227 * 1024) return HGA_ERR_UNSUPPORTED;
+  const int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(&k_attn_bwd_generic<D>), smem);
   if (rc) return rc;
-  k_bwd_dq_generic<D><<<items, kAttnThreads, smem, st>>>(Q, K, V, dO, LSE, delta, group_idx, n_groups, dm, dQ, status_word);
+  const bool zero = !(dm.flags & HGA_FLAG_BWD_ACCUMULATE);
+  if (zero) {
+    const size_t n4 = (size_t)dm.B * dm.Hkv * dm.S * D / 4;
+    k_zero_grads<<<(unsigned)((n4 + 255) / 256), 256, 0, st>>>((float4*)dK, (float4*)dV, n4);
+    count_launch(HGA_KERNELS_BWD_GENERIC);
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((int64_t)dm.B * dm.Hkv * dm.NQB * ((dm.rows + kBwdRows - 1) / kBwdRows)));
+  cfg.blockDim = dim3(32 * kBwdWarps);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr;                 // may start under the zero fill; waits for it before its first add
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = zero ? 1 : 0;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_attn_bwd_generic<D>, Q, K, V, O, LSE, dO, group_idx, n_groups, dm, dQ, dK, dV,
+                                           status_word);
   count_launch(HGA_KERNELS_BWD_GENERIC);
-  rc = record_cuda(cudaGetLastError());
-  if (rc) return rc;
-  k_bwd_dkv_generic<D><<<items, kAttnThreads, smem, st>>>(Q, K, V, dO, LSE, delta, group_idx, n_groups, dm, dK, dV);
-  count_launch(HGA_KERNELS_BWD_GENERIC);
-  return record_cuda(cudaGetLastError());
+  return record_cuda(e);
 }
 
 int launch_attn_bwd_generic(const Dims& dm, const void* Q, const void* K, const void* V,
                             const void* O, const float* LSE, const void* dO,
                             const int32_t* group_idx, const int32_t* n_groups, void* dQ, float* dK,
-                            float* dV, float* delta_ws, int32_t* status_word, cudaStream_t st) {
+                            float* dV, int32_t* status_word, cudaStream_t st) {
   if (dm.d == 128)
     return bwd_generic<128>(dm, (const uint16_t*)Q, (const uint16_t*)K, (const uint16_t*)V,
                             (const uint16_t*)O, LSE, (const uint16_t*)dO, group_idx, n_groups,
-                            (uint16_t*)dQ, dK, dV, delta_ws, status_word, st);
+                            (uint16_t*)dQ, dK, dV, status_word, st);
   return bwd_generic<64>(dm, (const uint16_t*)Q, (const uint16_t*)K, (const uint16_t*)V,
                          (const uint16_t*)O, LSE, (const uint16_t*)dO, group_idx, n_groups,
-                         (uint16_t*)dQ, dK, dV, delta_ws, status_word, st);
+                         (uint16_t*)dQ, dK, dV, status_word, st);
 }
 
 }  // namespace hga

@@ -89,7 +89,7 @@ int launch_attn_fwd_generic(const Dims& dm, const void* Q, const void* K, const 
 int launch_attn_bwd_generic(const Dims& dm, const void* Q, const void* K, const void* V,
                             const void* O, const float* LSE, const void* dO,
                             const int32_t* group_idx, const int32_t* n_groups, void* dQ, float* dK,
-                            float* dV, float* delta_ws, int32_t* status_word, cudaStream_t st);
+                            float* dV, int32_t* status_word, cudaStream_t st);
 
 // tensor-core (tcgen05 / TMEM / TMA) kernels; *_supported says whether the shape qualifies
 bool attn_fwd_sm100_supported(const Dims& dm);
@@ -106,6 +106,10 @@ int launch_attn_bwd_sm100(const Dims& dm, const void* Q, const void* K, const vo
                           const float* LSE, const void* dO, const int32_t* group_idx,
                           const int32_t* n_groups, void* dQ, float* dK, float* dV, int32_t* status_word,
                           cudaStream_t st);
+int launch_attn_bwd_d64_sm100(const Dims& dm, const void* Q, const void* K, const void* V, const void* O,   // head_dim 64, called by the above
+                              const float* LSE, const void* dO, const int32_t* group_idx,
+                              const int32_t* n_groups, void* dQ, float* dK, float* dV, int32_t* status_word,
+                              cudaStream_t st);
 // Key-major dK/dV of the local band (plain stores covering every active-segment row); launched by the above.
 bool attn_bwd_band_sm100_supported(const Dims& dm);
 int launch_attn_bwd_band_sm100(const Dims& dm, const void* Q, const void* K, const void* V, const void* O,
