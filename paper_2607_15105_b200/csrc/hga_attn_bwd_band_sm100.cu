@@ -1,11 +1,11 @@
-// Key-major backward of the local band for sm_100a (head_dim 128): dK and dV of the keys that query
+// Key-major backward of the local band for sm_100a: dK and dV of the keys that query
 // blocks see through their local window or their own causal block (Section 2.1: the dense part of
 // the routed set; Section 2.2: only keys of the active segment receive gradients).
 //
 // Every key of the active segment lies in the band of a few consecutive query blocks (its own
 // block and the ones whose local window still reaches it).  Summing those contributions with
 // atomics from the query-major sweep costs one red.add per element per contributing M-tile; here
-// one CTA owns a 128-key tile instead, loops over every 128-row M-tile of every query block whose
+// one CTA owns a 128-key tile instead, loops over the query rows of every query block whose
 // band touches the tile, accumulates dK and dV in tensor memory and writes the tile once with plain
 // stores.  The query-major sweep (k_attn_bwd_sm100) then adds only the contributions of keys
 // selected through routing (and of sink keys inside the active segment), and computes dQ.
@@ -15,9 +15,11 @@
 //   P^T  = 2^(S^T*c - LSE*log2e),  dS^T = scale * P^T o (dP^T - delta)    one thread per KEY (TMEM lane),
 //          written back as bf16 over the columns just read
 //   dV  += P^T dO,  dK += dS^T Q         (M = 128 keys, N = head_dim, K = 64 query rows)   A from TMEM
-// An M-tile (128 query rows) is taken in two HALF-STEPS of 64 rows that alternate between two 128-column
-// regions of tensor memory, so that the GEMMs of one half-step run while the key threads work on the other
-// (with one 256-column region per M-tile the tensor pipe idled through the key threads' work and vice versa).
+// The query rows of those blocks, block after block, are taken in HALF-STEPS of 64 rows (64 consecutive positions
+// of one query head) that alternate between two 128-column regions of tensor memory, so that the GEMMs of one
+// half-step run while the key threads work on the other (with one 256-column region per 128 rows the tensor pipe
+// idled through the key threads' work and vice versa).  Two half-steps share a ring stage and are called an M-tile; an
+// odd number of half-steps is padded with one whose rows arrive as zeros and are wholly masked.
 // delta = rowsum(dO o O) of the M-tile's rows is computed here, by four otherwise idle warps (one
 // thread per query row, from the O and dO tiles in shared memory; the O tile arrives by TMA one step
 // ahead), so the backward needs no separate pass over O and dO.
@@ -39,11 +41,11 @@ using namespace sm100;
 namespace {
 
 constexpr int kBandThreads = 448;
-constexpr int kD = 128;
 constexpr int kKeys = 128;                       // keys per CTA
-constexpr int kTile = 128 * kD * 2;              // bytes of one K, V, Q or dO tile: [panel][128 rows][128 B]
 
+template <int D>
 struct BandSmem {
+  static constexpr int kTile = 128 * D * 2;      // bytes of one K, V, Q or dO tile: [panel][128 rows][128 B]
   alignas(1024) uint8_t k[kTile];
   alignas(1024) uint8_t v[kTile];
   alignas(1024) uint8_t q[2][kTile];
@@ -59,24 +61,35 @@ struct BandSmem {
   volatile int abort;
 };
 
-// query block of step m, and the first query row (inside the item) of its M-tile
-struct Step {
-  int qb, r0;
+// Where a half-step's 64 rows are: query block, first row inside the item, query head of the group and position
+// inside the block.  Every role walks along by additions: the divisions of a direct look-up, repeated per half-step in
+// each role, cost the kernel 2 us of 32.
+struct HalfStep {
+  int qb, r0, head, t;
+  __device__ void next(const Dims& dm, int qb_last) {
+    r0 += 64;
+    t += 64;
+    if (t == dm.Bq) { t = 0; ++head; }
+    if (r0 == dm.rows && qb < qb_last) { ++qb; r0 = 0; head = 0; }      // (behind the last block: r0 == rows, padding)
+  }
 };
 
 }  // namespace
 
+template <int D>
 __global__ void __launch_bounds__(kBandThreads, 1)
 k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_do,
                       const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                       const __grid_constant__ CUtensorMap map_o, const float* __restrict__ LSE, Dims dm,
                       float* __restrict__ dK, float* __restrict__ dV, int32_t* status_word) {
   constexpr uint32_t kColS = 0, kColDP = 64, kRegion = 128, kColDV = 256, kColDK = 384;   // (S^T, dP^T: inside a region)
+  constexpr int kD = D, kPanels = D / 64, kTile = BandSmem<D>::kTile;
+  constexpr int kHalfBoxes = 2 * kPanels;          // boxes (64 rows x 64 elements) of one half-step's Q and dO, or of one 128-row tile
   extern __shared__ uint8_t smem_raw[];
-  BandSmem& sm = *reinterpret_cast<BandSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  BandSmem<D>& sm = *reinterpret_cast<BandSmem<D>*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  HGA_TRACE_DECL;
+  HGA_TRACE_DECL(448);
   const int tiles_per_seq = (dm.S + kKeys - 1) / kKeys;
   const int kt = blockIdx.x % tiles_per_seq;
   const int bh = blockIdx.x / tiles_per_seq;
@@ -88,9 +101,9 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
   const int qb_first = (kt * kKeys) / dm.Bq;
   int n_qb = 1;
   while (qb_first + n_qb < dm.NQB && window_of(dm, qb_first + n_qb).ls < k_end) ++n_qb;
-  const int n_mt = dm.rows / 128;
-  const int n_steps = n_qb * n_mt;
-  auto step_of = [&](int m) { return Step{qb_first + m / n_mt, (m % n_mt) * 128}; };
+  const int n_hq = dm.rows / 64;                  // half-steps of a query block
+  const int n_steps = (n_qb * n_hq + 1) / 2;
+  const int qb_last = qb_first + n_qb - 1;
 
   if (tid == 0) {
     mbar_init(&sm.kv_full, 1);
@@ -127,41 +140,47 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
   HGA_TRACE_POINT(1);
 
   // A copy is latency-bound per box and costs its issuing warp a few hundred cycles, so every tile travels as
-  // four boxes of 64 rows x one 64-element panel (8 KB each); the 28 boxes a CTA starts with go out from
+  // boxes of 64 rows x one 64-element panel (8 KB each); the 28 boxes a CTA starts with (head_dim 128) go out from
   // twelve warps in parallel, in the order they are needed: K, V, the first half-step's Q and dO rows, the
   // second half-step's, the first O tile, then the second step's Q and dO.
-  auto qdo_coords = [&](int m, int half, int& row, int& head) {
-    const Step sp = step_of(m);
-    const int r = sp.r0 + 64 * half;
-    row = sp.qb * dm.Bq + r % dm.Bq;
-    head = h * dm.G + r / dm.Bq;
+  auto coords = [&](const HalfStep& hs, int& row, int& head) {
+    const bool real = hs.r0 < dm.rows;
+    row = real ? hs.qb * dm.Bq + hs.t : dm.S;                // (padding: out of range, zeros)
+    head = h * dm.G + (real ? hs.head : 0);
   };
+  // box i of a tile of 128 rows: (half, panel); box i of a half-step's Q and dO: (panel, Q or dO)
+  auto copy_kv = [&](uint8_t* dst, const CUtensorMap* map, int i) {
+    const int half = i & 1, panel = i >> 1;
+    tma_load_5d(dst + panel * 16384 + half * 8192, map, &sm.kv_full, 0, k0 + 64 * half, panel, h, b);
+  };
+  auto copy_qdo = [&](const HalfStep& hs, int st, int half, int i) {
+    const int panel = i % kPanels, is_do = i / kPanels;
+    int row, head;
+    coords(hs, row, head);
+    tma_load_5d((is_do ? sm.dO[st] : sm.q[st]) + panel * 16384 + half * 8192, is_do ? &map_do : &map_q, &sm.qdo_full[st][half],
+                0, row, panel, head, b);
+  };
+  auto copy_o = [&](const HalfStep& h0, const HalfStep& h1, int i) {
+    const int half = i & 1, panel = i >> 1;
+    int row, head;
+    coords(half ? h1 : h0, row, head);
+    tma_load_5d(sm.o + panel * 16384 + half * 8192, &map_o, &sm.o_full, 0, row, panel, head, b);
+  };
+  HalfStep first[4];                               // the half-steps of the first two M-tiles
+  first[0] = HalfStep{qb_first, 0, 0, 0};
+#pragma unroll
+  for (int i = 1; i < 4; ++i) { first[i] = first[i - 1]; first[i].next(dm, qb_last); }
   if (warp >= 2 && lane == 0) {
-    for (int i = warp - 2; i < (n_steps > 1 ? 28 : 20); i += 12) {
-      int row, head;
+    constexpr int n = kHalfBoxes;
+    for (int i = warp - 2; i < (n_steps > 1 ? 7 * n : 5 * n); i += 12) {
       // All CTAs start at once and HBM is the bottleneck of these first microseconds: what the first
-      // half-step needs (the first twelve boxes) goes out alone, the rest once that has arrived
-      if (i >= 12 && !(bwd_wait(&sm.kv_full, 0, abort) && bwd_wait(&sm.qdo_full[0][0], 0, abort))) break;
-      if (i < 8) {                                   // K, V: (half, panel) = (i & 1, (i >> 1) & 1)
-        const int half = i & 1, panel = (i >> 1) & 1;
-        const uint32_t off = (uint32_t)panel * 16384 + (uint32_t)half * 8192;
-        tma_load_5d((i < 4 ? sm.k : sm.v) + off, i < 4 ? &map_k : &map_v, &sm.kv_full, 0, k0 + 64 * half, panel, h, b);
-      } else if (i < 16) {                           // step 0: half (i - 8) / 4, then Q panel 0, 1, dO panel 0, 1
-        const int half = (i - 8) >> 2, panel = i & 1, is_do = (i >> 1) & 1;
-        const uint32_t off = (uint32_t)panel * 16384 + (uint32_t)half * 8192;
-        qdo_coords(0, half, row, head);
-        tma_load_5d((is_do ? sm.dO[0] : sm.q[0]) + off, is_do ? &map_do : &map_q, &sm.qdo_full[0][half], 0, row, panel, head, b);
-      } else if (i < 20) {                           // O tile of step 0
-        const int half = i & 1, panel = (i >> 1) & 1;
-        const uint32_t off = (uint32_t)panel * 16384 + (uint32_t)half * 8192;
-        qdo_coords(0, half, row, head);
-        tma_load_5d(sm.o + off, &map_o, &sm.o_full, 0, row, panel, head, b);
-      } else {                                       // step 1, as step 0
-        const int half = (i - 20) >> 2, panel = i & 1, is_do = (i >> 1) & 1;
-        const uint32_t off = (uint32_t)panel * 16384 + (uint32_t)half * 8192;
-        qdo_coords(1, half, row, head);
-        tma_load_5d((is_do ? sm.dO[1] : sm.q[1]) + off, is_do ? &map_do : &map_q, &sm.qdo_full[1][half], 0, row, panel, head, b);
-      }
+      // half-step needs (the first three groups of boxes) goes out alone, the rest once that has arrived
+      if (i >= 3 * n && !(bwd_wait(&sm.kv_full, 0, abort) && bwd_wait(&sm.qdo_full[0][0], 0, abort))) break;
+      const int grp = i / n, k = i % n;
+      if (grp < 2) copy_kv(grp == 0 ? sm.k : sm.v, grp == 0 ? &map_k : &map_v, k);
+      else if (grp < 4) copy_qdo(grp == 2 ? first[0] : first[1], 0, grp - 2, k);
+      else if (grp == 4) copy_o(first[0], first[1], k);
+      else copy_qdo(grp == 5 ? first[2] : first[3], 1, grp - 5, k);
     }
   }
   __syncwarp();
@@ -173,9 +192,10 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
     }
     bool ok = true;
     int issued = n_steps > 1 ? 4 : 2;                // half-steps whose copies have been issued
+    HalfStep next = first[3];
     for (int m = 2; m < n_steps && ok; ++m) {
       const int st = m & 1;
-      // one half of the rows (Q panel 0, 1, dO panel 0, 1: lanes 0-3) at a time: a half is free again as soon
+      // one half of the rows (one box per lane) at a time: a half is free again as soon
       // as the GEMMs of its half-step two steps ago are done
       for (int hf = 0; hf < 2 && ok; ++hf) {
         if (lane == 0) ok = bwd_wait(&sm.qdo_empty[st][hf], ((m >> 1) - 1) & 1, abort);
@@ -183,13 +203,8 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
         if (!ok) break;
         if (lane == 0) mbar_arrive_expect_tx(&sm.qdo_full[st][hf], kTile);
         __syncwarp();
-        if (lane < 4) {
-          const int panel = lane & 1, is_do = lane >> 1;
-          const uint32_t off = (uint32_t)panel * 16384 + (uint32_t)hf * 8192;
-          int row, head;
-          qdo_coords(m, hf, row, head);
-          tma_load_5d((is_do ? sm.dO[st] : sm.q[st]) + off, is_do ? &map_do : &map_q, &sm.qdo_full[st][hf], 0, row, panel, head, b);
-        }
+        next.next(dm, qb_last);
+        if (lane < kHalfBoxes) copy_qdo(next, st, hf, lane);
         issued = 2 * m + hf + 1;
         HGA_TRACE_POINT(2);
       }
@@ -284,15 +299,15 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
     const float sl2 = dm.scale * 1.4426950408889634f;
     const uint64_t sl2_2 = pack_f32x2(sl2, sl2), scale_2 = pack_f32x2(dm.scale, dm.scale);
     bool ok = true;
+    HalfStep sp = first[0];
     for (int hs = 0; hs < 2 * n_steps; ++hs) {
       const int m = hs >> 1, hf = hs & 1;
-      const Step sp = step_of(m);
       const Window w = window_of(dm, sp.qb);
       // the warpgroup's 32 columns are 32 consecutive positions of one query head (Bq is a multiple of 64);
       // column i is visible to this key iff the key is inside the block's band and not after the query
       const int r_first = 64 * hf + 32 * wg;         // first of those rows inside the M-tile
-      const int qp0 = w.p0 + (sp.r0 + r_first) % dm.Bq;
-      const int imin = (kp < w.ls || kp >= k_end) ? 32 : kp - qp0;       // first visible column (may be <= 0)
+      const int qp0 = w.p0 + sp.t + 32 * wg;
+      const int imin = (kp < w.ls || kp >= k_end || sp.r0 >= dm.rows) ? 32 : kp - qp0;       // first visible column (may be <= 0)
       const bool none = __all_sync(0xffffffffu, imin >= 32);
       const bool masked = __any_sync(0xffffffffu, imin > 0);
       const uint32_t nlse_a = smem_u32(&sm.nlse[r_first]), nds_a = smem_u32(&sm.nds[r_first]);
@@ -366,6 +381,7 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
       tc_fence_before_sync();
       mbar_arrive(&sm.pds_full[hf]);
       HGA_TRACE_POINT(14);
+      sp.next(dm, qb_last);
     }
     if (ok) ok = __all_sync(0xffffffffu, bwd_wait(&sm.acc_done, 0, abort));
     HGA_TRACE_POINT(20);
@@ -401,18 +417,24 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
     // ------------------------------------------------------------------ row statistics, one thread per query row
     const int j = (warp - 10) * 32 + lane;           // row of the M-tile
     const uint32_t key7 = (uint32_t)(j & 7);
-    auto lse_of = [&](int m) {
-      const Step sp = step_of(m);
-      const int r = sp.r0 + j;
-      return LSE[((int64_t)b * dm.Hq + h * dm.G + r / dm.Bq) * dm.S + sp.qb * dm.Bq + r % dm.Bq];
+    HalfStep h0 = first[0], h1 = first[1];           // the two half-steps of the M-tile whose LSE (and O tile) comes next
+    auto next_lse = [&]() {
+      const HalfStep& hs = j < 64 ? h0 : h1;
+      return hs.r0 < dm.rows ? LSE[((int64_t)b * dm.Hq + h * dm.G + hs.head) * dm.S + hs.qb * dm.Bq + hs.t + (j & 63)] : 0.f;
     };
-    float lse_next = lse_of(0);
+    float lse_next = next_lse();
     bool ok = true;
     int o_issued = 1;                                // O tiles whose copies have been issued
     for (int m = 0; m < n_steps; ++m) {
       const int st = m & 1;
       const float lse = lse_next;
-      if (m + 1 < n_steps) lse_next = lse_of(m + 1);
+      if (m + 1 < n_steps) {
+        h0 = h1;
+        h0.next(dm, qb_last);
+        h1 = h0;
+        h1.next(dm, qb_last);
+        lse_next = next_lse();
+      }
       ok = __all_sync(0xffffffffu, bwd_wait(&sm.qdo_full[st][j >> 6], (m >> 1) & 1, abort));   // (this row's half of dO)
       HGA_TRACE_POINT(11);
       if (ok) ok = __all_sync(0xffffffffu, bwd_wait(&sm.o_full, m & 1, abort));
@@ -421,7 +443,7 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
       float acc[4] = {0.f, 0.f, 0.f, 0.f};
       const uint32_t do_line = smem_u32(sm.dO[st]) + (uint32_t)j * 128, o_line = smem_u32(sm.o) + (uint32_t)j * 128;
 #pragma unroll
-      for (int i = 0; i < 16; ++i) {                 // 16-byte chunk i of the row: panel i / 8, chunk i % 8 (XOR-swizzled)
+      for (int i = 0; i < D / 8; ++i) {              // 16-byte chunk i of the row: panel i / 8, chunk i % 8 (XOR-swizzled)
         const uint32_t off = (uint32_t)(i >> 3) * 16384 + (((uint32_t)(i & 7) ^ key7) * 16);
         uint32_t xs[4], ys[4];
         ld_shared_v4(o_line + off, xs[0], xs[1], xs[2], xs[3]);
@@ -441,12 +463,7 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
         if (!ok) break;
         if (lane == 0) mbar_arrive_expect_tx(&sm.o_full, kTile);
         __syncwarp();
-        if (lane < 4) {
-          const int half = lane & 1, panel = lane >> 1;
-          int row, head;
-          qdo_coords(m + 1, half, row, head);
-          tma_load_5d(sm.o + (uint32_t)panel * 16384 + (uint32_t)half * 8192, &map_o, &sm.o_full, 0, row, panel, head, b);
-        }
+        if (lane < kHalfBoxes) copy_o(h0, h1, lane);
         o_issued = m + 2;
       }
       const float delta = (acc[0] + acc[1]) + (acc[2] + acc[3]);
@@ -483,16 +500,17 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
 
 bool attn_bwd_band_sm100_supported(const Dims& dm) {
   if (dm.flags & HGA_FLAG_GENERIC_KERNELS) return false;
-  return dm.d == 128 && dm.rows % 128 == 0 && dm.Bq % 64 == 0;
+  if (dm.Bq % 64 != 0) return false;
+  return dm.d == 128 || dm.d == 64;
 }
 
-int launch_attn_bwd_band_sm100(const Dims& dm, const void* Q, const void* K, const void* V, const void* O,
-                               const float* LSE, const void* dO, float* dK, float* dV, int32_t* status_word,
-                               cudaStream_t st) {
+template <int D>
+static int launch_band(const Dims& dm, const void* Q, const void* K, const void* V, const void* O,
+                       const float* LSE, const void* dO, float* dK, float* dV, int32_t* status_word, cudaStream_t st) {
   CUtensorMap mq, mdo, mk, mv, mo;
   const uint32_t box[5] = {64, 64, 1, 1, 1};
-  const uint64_t dq[5] = {64, (uint64_t)dm.S, 2, (uint64_t)dm.Hq, (uint64_t)dm.B};
-  const uint64_t dk[5] = {64, (uint64_t)dm.L, 2, (uint64_t)dm.Hkv, (uint64_t)dm.B};
+  const uint64_t dq[5] = {64, (uint64_t)dm.S, (uint64_t)(D / 64), (uint64_t)dm.Hq, (uint64_t)dm.B};
+  const uint64_t dk[5] = {64, (uint64_t)dm.L, (uint64_t)(D / 64), (uint64_t)dm.Hkv, (uint64_t)dm.B};
   const uint64_t sq[4] = {(uint64_t)dm.qs[2] * 2, 128, (uint64_t)dm.qs[1] * 2, (uint64_t)dm.qs[0] * 2};
   const uint64_t so[4] = {(uint64_t)dm.os[2] * 2, 128, (uint64_t)dm.os[1] * 2, (uint64_t)dm.os[0] * 2};
   const uint64_t sk[4] = {(uint64_t)dm.ks[2] * 2, 128, (uint64_t)dm.ks[1] * 2, (uint64_t)dm.ks[0] * 2};
@@ -503,13 +521,20 @@ int launch_attn_bwd_band_sm100(const Dims& dm, const void* Q, const void* K, con
       encode_tensor_map_bf16(&mk, K, 5, dk, sk, box, true) ||
       encode_tensor_map_bf16(&mv, V, 5, dk, sv, box, true))
     return HGA_ERR_UNSUPPORTED;
-  const size_t smem = sizeof(BandSmem) + 1024;
-  const int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(&k_attn_bwd_band_sm100), smem);
+  const size_t smem = sizeof(BandSmem<D>) + 1024;
+  const int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(&k_attn_bwd_band_sm100<D>), smem);
   if (rc) return rc;
   const int units = dm.B * dm.Hkv * ((dm.S + kKeys - 1) / kKeys);
-  k_attn_bwd_band_sm100<<<units, kBandThreads, smem, st>>>(mq, mdo, mk, mv, mo, LSE, dm, dK, dV, status_word);
+  k_attn_bwd_band_sm100<D><<<units, kBandThreads, smem, st>>>(mq, mdo, mk, mv, mo, LSE, dm, dK, dV, status_word);
   count_launch(HGA_KERNELS_BWD_TENSOR);
   return record_cuda(cudaGetLastError());
+}
+
+int launch_attn_bwd_band_sm100(const Dims& dm, const void* Q, const void* K, const void* V, const void* O,
+                               const float* LSE, const void* dO, float* dK, float* dV, int32_t* status_word,
+                               cudaStream_t st) {
+  return dm.d == 128 ? launch_band<128>(dm, Q, K, V, O, LSE, dO, dK, dV, status_word, st)
+                     : launch_band<64>(dm, Q, K, V, O, LSE, dO, dK, dV, status_word, st);
 }
 
 }  // namespace hga

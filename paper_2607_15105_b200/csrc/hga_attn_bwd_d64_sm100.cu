@@ -1,0 +1,690 @@
+// hga_attn_bwd for sm_100a, head_dim 64: the query-major sweep (routing frozen, Section 2.1 last paragraph; history K/V
+// detached, Section 2.2).
+//
+// Work unit (one CTA): one 128-row M-tile of one item (b, kv head, query block), swept over the item's routed
+// keys in 64-key tiles (eight octets of 8 consecutive tokens, one TMA box each).  At head_dim 64 a CTA takes less than
+// half of an SM (88 KB of shared memory, 256 TMEM columns, 256 threads), so two CTAs run on an SM: a tile is
+// a chain of hand-offs (copy -> S -> P -> dS -> dQ), and while one CTA is in its exponentials, its set-up, its
+// dK/dV reduction or its epilogue, the other one has the tensor pipe.  (At head_dim 128 the same layout was slower than
+// the pairs of tiles of k_attn_bwd_sm100, 3.3k against 3.0k cycles per 128 keys and SM: its GEMMs have twice the K
+// steps and an N = 64 instruction costs nearly as much as one with N = 128, so the pipe itself was the bound.)
+//
+// Order of the tiles of an item:
+//   1. the local window and the causal block, [ls, p0 + Bq): known without the routing list, so their copies
+//      start at once and the list is fetched and checked behind them;
+//   2. "far" keys (sink, then the selected groups, ascending) of the detached history: dQ only;
+//   3. far keys of the active segment, which also get dK/dV from this kernel (the local band's dK/dV are written by
+//      the key-major kernel k_attn_bwd_band_sm100, which precedes this one and stores every row).
+// Per tile: S = Q K^T, dP = dO V^T (smem x smem -> TMEM); one thread per query row turns them into
+// P = 2^(S*c - LSE*log2e) (packed bf16 in registers) and dS = scale * P o (dP - delta);
+//   kinds 1, 2:  dS (bf16) goes over the dP columns just read; dQ += dS K with A from TMEM
+//   kind 3:      P and dS go to shared memory; dQ += dS K; dV^T = dO^T P over S's columns, dK^T = Q^T dS over dP's, both
+//                with M = 128: A = [dO^T ; Q^T] (the two tiles are neighbours), of whose products with P and dS one half
+//                each is wanted; the row threads stage the transposed tiles in shared memory as key rows (dV | dK) and
+//                add them to global memory with bulk reductions, one 256-byte row per instruction.
+// S(j+1) is issued as soon as the rows have read S(j), dP(j+1) behind dQ(j): the in-order tensor pipe makes every
+// reuse of a region safe.  A wait on S(j+1)'s K tile never holds up dQ(j), which frees the stage of K(j+2).
+//
+// Warp roles (256 threads):
+//   warps 0, 7   producers: octets 0-3 / 4-7 of every K and V tile (a box costs its issuing warp ~100 cycles)
+//   warp 6       Q and dO tiles, then the check of the routing list       warp 1   MMA issuer
+//   warps 2-5    one thread per query row (TMEM lane = row); delta = rowsum(dO o O) of its own row
+// TMEM (256 columns): S 64 | dP / dS 64 | dQ 64.
+#include "hga_bwd_sm100.cuh"
+#include "hga_common.cuh"
+#include "hga_octets.cuh"
+#include "hga_sm100.cuh"
+
+namespace hga {
+
+using namespace sm100;
+
+namespace {
+
+constexpr int kThreads = 256;
+constexpr int D = 64;
+constexpr int kKT = 64;                         // keys per tile
+constexpr int kPdsTile = 128 * kKT * 2;         // bytes of one P or dS tile: [16 row octets][8 rows][128 B], 128-byte swizzle
+
+constexpr int kQBytes = 128 * D * 2;            // the Q or dO tile: [128 rows][128 B]
+constexpr int kKv = kKT * D * 2;                // one K or V tile: [octet][8 rows][128 B]
+constexpr int kOct = 8 * D * 2;
+
+struct SweepSmem {
+  alignas(1024) uint8_t dO[kQBytes];            // (dO and Q adjacent: one MN-major operand of 128 rows, see above)
+  alignas(1024) uint8_t q[kQBytes];
+  alignas(1024) uint8_t k[2][kKv];
+  alignas(1024) uint8_t v[kKv];
+  alignas(1024) uint8_t p[kPdsTile];            // dK/dV tiles: P and dS, then the staged dV | dK rows of 32 keys each
+  alignas(1024) uint8_t ds[kPdsTile];
+  uint64_t q_full, k_full[2], k_empty[2], v_full;
+  uint64_t s_full, s_read, dp_full, ds_full;            // per tile
+  uint64_t dkv_full, staged, dk_read;                   // per dK/dV tile
+  uint64_t info_full, dq_done, dq_staged, drain;
+  uint32_t tmem_base;
+  int n_far, first_active, n_listed;                    // far octets; the first of them that belongs to the active segment; list entries (see FarList)
+  bool clean;
+  volatile int abort;
+  int rows[4][8];                                       // token rows of the last four tiles' octets (dK/dV tiles read them back)
+};
+static_assert(sizeof(SweepSmem) + 1024 <= 113 * 1024, "two CTAs per SM");
+
+// The "far" part of an item's routed set (sink, then selected groups) as octets, looked up in the group list
+// itself: no table in shared memory.  A list is checked once, 32 entries per vote; a valid list (every entry
+// ascending and wholly between sink and local window) is then read directly, an invalid one is walked, skipping the
+// entries build_octet_table would skip.
+struct FarList {
+  const int32_t* gi;
+  int ng, opg, n_sink, n_far, first_active, se, ls, g;
+  bool clean;
+  __device__ bool fits(int m, int last) const {
+    return m > last && (int64_t)m * g >= se && ((int64_t)m + 1) * g <= ls;
+  }
+  __device__ FarList(const Dims& dm, const Window& w, const int32_t* list)
+      : gi(list), ng(0), opg(dm.g / 8), n_sink(w.se / 8), n_far(0), first_active(0), se(w.se), ls(w.ls), g(dm.g), clean(true) {}
+  // checks the list and counts its octets; all 32 lanes of a warp
+  __device__ void check(const Dims& dm, const int32_t* ng_ptr) {
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int pre0 = lane < dm.width ? gi[lane] : 0x7fffffff;      // (overlaps the load of the count)
+    const int pre1 = lane + 32 < dm.width ? gi[lane + 32] : 0x7fffffff;
+    ng = *ng_ptr;
+    ng = ng < 0 ? 0 : ng > dm.width ? dm.width : ng;               // (the forward call reports such a count)
+    int prev = -1, below = 0;
+    for (int base = 0; base < ng; base += 32) {
+      const int i = base + lane;
+      const int m = i >= ng ? 0x7fffffff : base == 0 ? pre0 : base == 32 ? pre1 : gi[i];
+      int left = __shfl_up_sync(full, m, 1);
+      if (lane == 0) left = prev;
+      clean = clean && __all_sync(full, i >= ng || fits(m, left));
+      below += __popc(__ballot_sync(full, i < ng && (int64_t)m * g < dm.H));
+      prev = __shfl_sync(full, m, 31);
+    }
+    int n = ng;
+    if (!clean) {
+      n = below = 0;
+      if (lane == 0) {
+        int last = -1;
+        for (int i = 0; i < ng; ++i) {
+          const int m = gi[i];
+          if (fits(m, last)) { ++n; below += (int64_t)m * g < dm.H; last = m; }
+        }
+      }
+      n = __shfl_sync(full, n, 0);
+      below = __shfl_sync(full, below, 0);
+    }
+    n_far = n_sink + n * opg;
+    first_active = dm.H / 8 < n_sink ? dm.H / 8 : n_sink + below * opg;      // H is a multiple of g
+  }
+  // first token of far octet o (o < n_far)
+  __device__ int row(int o) const {
+    if (o < n_sink) return 8 * o;
+    const int k = o - n_sink, u = opg == 1 ? k : k / opg, sub = k - u * opg;
+    if (clean) return __ldg(gi + u) * g + 8 * sub;
+    int last = -1, n = -1;
+    for (int i = 0; i < ng; ++i) {
+      const int m = gi[i];
+      if (fits(m, last)) { last = m; if (++n == u) break; }
+    }
+    return last * g + 8 * sub;
+  }
+};
+
+}  // namespace
+
+__global__ void __launch_bounds__(kThreads, 2)
+k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_do,
+                 const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
+                 const __grid_constant__ CUtensorMap map_dq, const uint16_t* __restrict__ O,
+                 const float* __restrict__ LSE, const int32_t* __restrict__ group_idx,
+                 const int32_t* __restrict__ n_groups, Dims dm,
+                 float* __restrict__ dK, float* __restrict__ dV, int32_t* status_word) {
+  constexpr uint32_t kColS = 0, kColDP = 64, kColDQ = 128;
+  extern __shared__ uint8_t smem_raw[];
+  SweepSmem& sm = *reinterpret_cast<SweepSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  HGA_TRACE_DECL(64);
+  const int n_mt_item = (dm.rows + 127) / 128;
+  // Launch order: late query blocks first.  They have the most routed keys inside the active segment (the
+  // expensive dK/dV tiles), early ones none, so the cheapest CTAs are the ones that fill the last wave.
+  const int unit = blockIdx.x / n_mt_item, n_bh = dm.B * dm.Hkv;
+  const int item = (unit % n_bh) * dm.NQB + (dm.NQB - 1 - unit / n_bh);
+  const int mt = blockIdx.x % n_mt_item;
+  int b, h, qb;
+  item_coords(dm, item, b, h, qb);
+  const Window w = window_of(dm, qb);
+  const int n_local = w.p0 + dm.Bq - w.ls;              // tokens of the local window and the block (a multiple of 8)
+  const int n_lt = (n_local + kKT - 1) / kKT;           // its tiles
+  volatile int* abort = &sm.abort;
+
+  // Row threads: LSE and the O row of the thread's own query row (rows past the item's last one: zeros), requested
+  // before anything else so that the latency hides behind the set-up.
+  float row_lse = 0.f;
+  uint4 o_row[D / 8];
+  if (warp >= 2 && warp < 6) {
+    const int r = mt * 128 + (warp & 3) * 32 + lane;
+#pragma unroll
+    for (int i = 0; i < D / 8; ++i) o_row[i] = make_uint4(0, 0, 0, 0);
+    if (r < dm.rows) {
+      const int hq = h * dm.G + r / dm.Bq, srow = qb * dm.Bq + r % dm.Bq;
+      row_lse = LSE[((int64_t)b * dm.Hq + hq) * dm.S + srow];
+      const uint4* op = reinterpret_cast<const uint4*>(O + b * dm.os[0] + hq * dm.os[1] + (int64_t)srow * dm.os[2]);
+#pragma unroll
+      for (int i = 0; i < D / 8; ++i) o_row[i] = __ldg(op + i);
+    }
+  }
+  // Octet rows of local tile j for the producers (lane < 4: octet 4 * half + lane); past the window: out of range, zeros
+  const int half = warp == 7 ? 1 : 0;
+  auto local_row = [&](int j) {
+    const int off = kKT * j + 8 * (4 * half + lane);
+    return off < n_local ? w.ls + off : dm.L;
+  };
+  auto copy_tile = [&](uint8_t* dst, const CUtensorMap* map, uint64_t* full, int row) {
+    if (lane == 0) mbar_arrive_expect_tx(full, 4 * kOct);
+    __syncwarp();
+    if (lane < 4) tma_load_5d(dst + (4 * half + lane) * kOct, map, full, 0, row, 0, h, b);
+  };
+  auto note_rows = [&](int j, int row) {
+    if (lane < 4) sm.rows[j & 3][4 * half + lane] = row;
+  };
+  if (warp == 0 && lane == 0) {
+    mbar_init(&sm.q_full, 1);
+    for (int s = 0; s < 2; ++s) { mbar_init(&sm.k_full[s], 2); mbar_init(&sm.k_empty[s], 1); }
+    mbar_init(&sm.v_full, 2);
+    mbar_init(&sm.s_full, 1); mbar_init(&sm.s_read, 128);
+    mbar_init(&sm.dp_full, 1); mbar_init(&sm.ds_full, 128);
+    mbar_init(&sm.dkv_full, 1); mbar_init(&sm.staged, 128); mbar_init(&sm.dk_read, 128);
+    mbar_init(&sm.info_full, 1); mbar_init(&sm.dq_done, 1); mbar_init(&sm.dq_staged, 128); mbar_init(&sm.drain, 1);
+    sm.abort = 0;
+    fence_barrier_init();
+  }
+  if (warp == 0 || warp >= 6) {
+    // Q, dO and the first local tile depend on nothing: their copies start before the CTA meets.  Barrier 2 makes
+    // the mbarrier initialisation above visible to the three issuing warps.
+    asm volatile("bar.sync 2, 96;" ::: "memory");
+    if (warp == 6) {
+      if (lane == 0) mbar_arrive_expect_tx(&sm.q_full, 2 * kQBytes);
+      __syncwarp();
+      if (lane < 4) {
+        // boxes of 64 rows, Q first, then dO; rows past the item's last one (an M-tile may hold 64 rows only) arrive as zeros
+        const int is_do = lane >> 1, hf = lane & 1;
+        const int r = mt * 128 + 64 * hf;
+        const bool real = r < dm.rows;
+        tma_load_5d((is_do ? sm.dO : sm.q) + hf * 8192, is_do ? &map_do : &map_q, &sm.q_full, 0,
+                    real ? qb * dm.Bq + r % dm.Bq : dm.S, 0, h * dm.G + (real ? r / dm.Bq : 0), b);
+      }
+    } else {
+      const int row = local_row(0);
+      copy_tile(sm.k[0], &map_k, &sm.k_full[0], row);
+      copy_tile(sm.v, &map_v, &sm.v_full, row);
+    }
+    __syncwarp();
+  }
+  if (warp == 1) {
+    tmem_alloc(&sm.tmem_base, 256);
+    tmem_relinquish();
+    // with bf16 outputs the conversion kernel follows this grid: let its launch overlap this grid's tail
+    if (lane == 0 && (dm.flags & HGA_FLAG_BWD_BF16_GRADS)) pdl_launch_dependents();
+  }
+  __syncwarp();
+  tc_fence_before_sync();
+  __syncthreads();
+  tc_fence_after_sync();
+
+  const uint32_t tmem = sm.tmem_base;
+  HGA_TRACE_POINT(1);
+  // Tile counts, once the list is known: tiles [0, n_a) are of kinds 1 and 2, tiles [n_a, n) of kind 3.
+  auto counts = [&](int n_far, int first_active, int& n, int& n_a) {
+    n = n_lt + (n_far + 7) / 8;
+    n_a = first_active < n_far ? n_lt + first_active / 8 : n;
+  };
+
+  if (warp == 0 || warp == 7) {
+    // ------------------------------------------------------------------ producers
+    bool ok = true;
+    FarList far(dm, w, group_idx + (int64_t)item * dm.width);
+    int n = 0, n_a = 0;
+    bool known = false;                                   // the list has been checked (warp 6) and its counts read
+    auto learn = [&]() {
+      if (lane == 0) ok = bwd_wait(&sm.info_full, 0, abort);
+      ok = __shfl_sync(0xffffffffu, ok, 0);
+      far.ng = sm.n_listed; far.n_far = sm.n_far; far.first_active = sm.first_active; far.clean = sm.clean;
+      counts(far.n_far, far.first_active, n, n_a);
+      known = true;
+      return ok;
+    };
+    // row of this lane's octet of tile j (any kind; rows past the item's keys are out of range)
+    auto row_of = [&](int j) {
+      if (j < n_lt) return local_row(j);
+      const int o = 8 * (j - n_lt) + 4 * half + (lane & 3);
+      return o < far.n_far ? far.row(o) : dm.L;
+    };
+    auto wait_for = [&](uint64_t* bar, uint32_t parity) {
+      if (lane == 0) ok = bwd_wait(bar, parity, abort);
+      ok = __shfl_sync(0xffffffffu, ok, 0);
+      return ok;
+    };
+    auto copy_k = [&](int j, int row) {
+      note_rows(j, row);
+      copy_tile(sm.k[j & 1], &map_k, &sm.k_full[j & 1], row);
+    };
+    // Rows of the next two tiles, looked up ahead of their use.  Tile j + 1's K has been issued when tile j is
+    // handled, except behind a dK/dV tile.
+    if (n_lt < 3) learn();
+    int next_row = ok ? row_of(1) : dm.L, after_row = ok ? row_of(2) : dm.L;
+    if (ok && (n_lt > 1 || n > 1)) copy_k(1, next_row);
+    // The events this loop waits for come in this order: dP(j) done, dQ(j) done, dP(j+1) done, ...
+    for (int j = 0; ok; ++j) {
+      if (!known && j + 3 >= n_lt && !learn()) break;
+      if (known && j + 1 >= n) break;
+      if (!known || j < n_a) {
+        if (!wait_for(&sm.dp_full, j & 1)) break;                           // V(j) has been read
+        copy_tile(sm.v, &map_v, &sm.v_full, next_row);                       // V(j+1)
+        next_row = after_row;
+        after_row = row_of(j + 3);
+        if (!known || (j + 2 < n && j + 2 <= n_a)) {
+          if (!wait_for(&sm.k_empty[j & 1], (j >> 1) & 1)) break;           // dQ(j) is done
+          copy_k(j + 2, next_row);
+        }
+      } else {
+        // behind a dK/dV tile both stages are free
+        if (!wait_for(&sm.dkv_full, (j - n_a) & 1)) break;
+        copy_k(j + 1, next_row);
+        copy_tile(sm.v, &map_v, &sm.v_full, next_row);
+        next_row = after_row;
+        after_row = row_of(j + 3);
+      }
+      HGA_TRACE_POINT(2);
+    }
+    if (*abort && lane == 0) {
+      // giving up: give the copies still in flight time to land before shared memory is released
+      // (the full barriers may never complete once another role has stopped, hence a bounded sleep)
+      for (int it = 0; it < 64; ++it) __nanosleep(1000);
+    }
+  } else if (warp == 1) {
+    // ------------------------------------------------------------------ MMA issuer
+    // The whole warp runs this branch converged (waits included) and one elected lane issues: see mma_ss_w.
+    auto mma_wait = [&](uint64_t* bar, uint32_t parity) {
+      return __all_sync(0xffffffffu, bwd_wait(bar, parity, abort));
+    };
+    constexpr uint32_t idesc_sdp = idesc_bf16_f32(128, kKT, 0, 0);       // rows x 64 keys, both K-major
+    constexpr uint32_t idesc_dq = idesc_bf16_f32(128, D, 0, 1);          // dS K-major, K tile MN-major
+    constexpr uint32_t idesc_dkv = idesc_bf16_f32(128, kKT, 1, 1);       // both MN-major
+    // Descriptors are built once; inside the loops an MMA costs two integer adds.
+    // Q, dO: [128 rows][128 B] (8-row groups 1024 B apart)
+    const uint64_t q_k = smem_desc_sw128(smem_u32(sm.q), 16, 1024);         // Q  as K-major A   (S)
+    const uint64_t do_k = smem_desc_sw128(smem_u32(sm.dO), 16, 1024);       // dO as K-major A   (dP)
+    // MN-major A of dV^T and dK^T: dO, and Q 16 KB on, as the two 64-element atoms
+    const uint64_t doq_mn = smem_desc_sw128(smem_u32(sm.dO), 16384, 1024);
+    const uint64_t k_k0 = smem_desc_sw128(smem_u32(sm.k[0]), 16, kOct);     // K tile, K-major B  (S)
+    const uint64_t v_k = smem_desc_sw128(smem_u32(sm.v), 16, kOct);         // V tile, K-major B  (dP)
+    const uint64_t k_mn0 = smem_desc_sw128(smem_u32(sm.k[0]), 1024, kOct);  // K tile, MN-major B (dQ)
+    const uint64_t dsd = smem_desc_sw128(smem_u32(sm.ds), 16, 1024);       // dS: K-major A (dQ) and MN-major B (dK^T)
+    const uint64_t pd = smem_desc_sw128(smem_u32(sm.p), 16, 1024);          // P : MN-major B (dV^T)
+    auto issue_qk = [&](uint32_t acc, uint64_t a, uint64_t bd) {
+#pragma unroll
+      for (int kk = 0; kk < D / 16; ++kk) {
+        mma_ss_w(acc, desc_advance(a, kk * 32), desc_advance(bd, kk * 32), idesc_sdp, kk > 0);
+      }
+    };
+    auto issue_s = [&](int j) {
+      issue_qk(tmem + kColS, q_k, desc_advance(k_k0, (uint32_t)(j & 1) * kKv));
+      mma_commit_w(&sm.s_full);
+    };
+    auto issue_dp = [&]() {
+      issue_qk(tmem + kColDP, do_k, v_k);
+      mma_commit_w(&sm.dp_full);           // also tells the producers that the V tile is free
+    };
+    bool ok = mma_wait(&sm.q_full, 0) && mma_wait(&sm.k_full[0], 0);
+    HGA_TRACE_POINT(40);
+    if (ok) { tc_fence_after_sync(); issue_s(0); ok = mma_wait(&sm.v_full, 0); }
+    if (ok) { tc_fence_after_sync(); issue_dp(); }
+    HGA_TRACE_POINT(3);
+    int n = n_lt + 1, n_a = n_lt;                 // (bounds that do until the list is known)
+    auto k_parity = [](int j) { return (uint32_t)(j >> 1) & 1; };
+    for (int j = 0; j < n && ok; ++j) {
+      if (j + 1 == n_lt) {
+        ok = mma_wait(&sm.info_full, 0);
+        if (!ok) break;
+        counts(sm.n_far, sm.first_active, n, n_a);
+      }
+      const uint64_t kmn = desc_advance(k_mn0, (uint32_t)(j & 1) * kKv);
+      if (j < n_a) {
+        // S(j+1) goes ahead of dQ(j) if its K tile is already there; waiting for it first would hold up dQ(j), and with
+        // it the copy of K(j+2) into the stage that dQ(j) reads
+        bool s_ahead = false;
+        if (j + 1 < n) {
+          ok = mma_wait(&sm.s_read, j & 1);
+          if (!ok) break;
+          s_ahead = __all_sync(0xffffffffu, mbar_test_wait(&sm.k_full[(j + 1) & 1], k_parity(j + 1)));
+          if (s_ahead) {
+            tc_fence_after_sync();
+            issue_s(j + 1);
+            HGA_TRACE_POINT(6);
+          }
+        }
+        ok = mma_wait(&sm.ds_full, j & 1);
+        if (!ok) break;
+        tc_fence_after_sync();
+        HGA_TRACE_POINT(5);
+#pragma unroll
+        for (int kk = 0; kk < kKT / 16; ++kk)     // 16 keys per MMA: 8 TMEM columns of dS, two octets of the K tile
+          mma_ts_w(tmem + kColDQ, tmem + kColDP + 8 * kk, desc_advance(kmn, kk * 2 * kOct), idesc_dq, (j > 0 || kk > 0));
+        mma_commit_w(&sm.k_empty[j & 1]);
+        HGA_TRACE_POINT(7);
+        if (j + 1 < n) {
+          if (!s_ahead) {
+            ok = mma_wait(&sm.k_full[(j + 1) & 1], k_parity(j + 1));
+            if (!ok) break;
+            tc_fence_after_sync();
+            issue_s(j + 1);
+          }
+          ok = mma_wait(&sm.v_full, (j + 1) & 1);
+          if (!ok) break;
+          tc_fence_after_sync();
+          issue_dp();
+          HGA_TRACE_POINT(8);
+        }
+      } else {
+        ok = mma_wait(&sm.ds_full, j & 1);        // P and dS are in shared memory, S and dP have been read
+        if (!ok) break;
+        tc_fence_after_sync();
+        HGA_TRACE_POINT(45);
+#pragma unroll
+        for (int kk = 0; kk < kKT / 16; ++kk)
+          mma_ss_w(tmem + kColDQ, desc_advance(dsd, kk * 32), desc_advance(kmn, kk * 2 * kOct), idesc_dq, (j > 0 || kk > 0));
+#pragma unroll
+        for (int kk = 0; kk < 128 / 16; ++kk)     // 16 query rows per MMA (2 row octets)
+          mma_ss_w(tmem + kColS, desc_advance(doq_mn, kk * 2048), desc_advance(pd, kk * 2048), idesc_dkv, kk > 0);
+#pragma unroll
+        for (int kk = 0; kk < 128 / 16; ++kk)
+          mma_ss_w(tmem + kColDP, desc_advance(doq_mn, kk * 2048), desc_advance(dsd, kk * 2048), idesc_dkv, kk > 0);
+        mma_commit_w(&sm.dkv_full);
+        HGA_TRACE_POINT(4);
+        if (j + 1 < n) {
+          // the row threads have read dV^T: S(j+1) may take its place; then dK^T: dP(j+1)
+          ok = mma_wait(&sm.s_read, j & 1) && mma_wait(&sm.k_full[(j + 1) & 1], k_parity(j + 1));
+          if (!ok) break;
+          tc_fence_after_sync();
+          issue_s(j + 1);
+          ok = mma_wait(&sm.dk_read, (j - n_a) & 1) && mma_wait(&sm.v_full, (j + 1) & 1);
+          if (!ok) break;
+          tc_fence_after_sync();
+          issue_dp();
+        }
+      }
+    }
+    if (ok) mma_commit_w(&sm.dq_done);
+  } else if (warp == 6) {
+    // ------------------------------------------------------------------ routing list
+    FarList far(dm, w, group_idx + (int64_t)item * dm.width);
+    far.check(dm, n_groups + item);
+    if (lane == 0) {
+      sm.n_listed = far.ng; sm.n_far = far.n_far; sm.first_active = far.first_active; sm.clean = far.clean;
+      mbar_arrive(&sm.info_full);
+    }
+  } else if (warp < 6) {
+    // ------------------------------------------------------------------ one thread per query row
+    const int quarter = warp & 3;
+    const int row_in_tile = quarter * 32 + lane;
+    const int r = mt * 128 + row_in_tile;
+    const int limit = w.p0 - w.ls + r % dm.Bq + 1;          // visible keys of the local tiles (causal inside the block)
+    const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
+    const float sl2 = dm.scale * 1.4426950408889634f;
+    const float neg_lse2 = -row_lse * 1.4426950408889634f;
+    const uint32_t key7 = (uint32_t)(row_in_tile & 7);
+    bool ok = __all_sync(0xffffffffu, bwd_wait(&sm.q_full, 0, abort));
+    // delta (dO from the tile in shared memory: 128-byte lines of 16-byte chunks, XOR-swizzled)
+    float neg_delta_s = 0.f;
+    if (ok) {
+      float acc[4] = {0.f, 0.f, 0.f, 0.f};
+      const uint32_t line = smem_u32(sm.dO) + (uint32_t)row_in_tile * 128;
+#pragma unroll
+      for (int i = 0; i < D / 8; ++i) {
+        uint32_t ys[4];
+        ld_shared_v4(line + (((uint32_t)i ^ key7) * 16), ys[0], ys[1], ys[2], ys[3]);
+        const uint32_t xs[4] = {o_row[i].x, o_row[i].y, o_row[i].z, o_row[i].w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          acc[e] = fmaf(__uint_as_float(xs[e] << 16), __uint_as_float(ys[e] << 16), acc[e]);
+          acc[e] = fmaf(__uint_as_float(xs[e] & 0xffff0000u), __uint_as_float(ys[e] & 0xffff0000u), acc[e]);
+        }
+      }
+      neg_delta_s = -((acc[0] + acc[1]) + (acc[2] + acc[3])) * dm.scale;
+    }
+    HGA_TRACE_POINT(10);
+    int n = n_lt + 1, n_a = n_lt, n_far_keys = 0;      // (bounds that do until the list is known)
+    const uint64_t sl2_2 = pack_f32x2(sl2, sl2), neg_lse2_2 = pack_f32x2(neg_lse2, neg_lse2);
+    const uint64_t scale_2 = pack_f32x2(dm.scale, dm.scale), neg_delta_s_2 = pack_f32x2(neg_delta_s, neg_delta_s);
+    const uint32_t s_addr = lane_base + kColS, dp_addr = lane_base + kColDP;
+    uint32_t staged_phase = 0;
+    for (int j = 0; j < n && ok; ++j) {
+      if (j == n_lt) {
+        ok = __all_sync(0xffffffffu, bwd_wait(&sm.info_full, 0, abort));
+        if (!ok) break;
+        counts(sm.n_far, sm.first_active, n, n_a);
+        n_far_keys = sm.n_far * 8;
+        if (j >= n) break;
+      }
+      const int vis = j < n_lt ? limit - kKT * j : n_far_keys - kKT * (j - n_lt);
+      uint32_t pk[32];                                // P of this row, 64 keys, packed bf16
+      ok = __all_sync(0xffffffffu, bwd_wait(&sm.s_full, j & 1, abort));
+      if (!ok) break;
+      tc_fence_after_sync();
+      HGA_TRACE_POINT(11);
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        uint32_t sv[32];
+        tmem_ld32(s_addr + 32 * c, sv);
+        tmem_wait_ld();
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          float a0, a1;            // packed fp32 pairs: one FMA for the two exponent arguments
+          unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(sv[2 * i]), __uint_as_float(sv[2 * i + 1])), sl2_2, neg_lse2_2), a0, a1);
+          float p0 = fast_exp2(a0), p1 = fast_exp2(a1);
+          if (vis < kKT) {         // diagonal / ragged tile only
+            if (32 * c + 2 * i >= vis) p0 = 0.f;
+            if (32 * c + 2 * i + 1 >= vis) p1 = 0.f;
+          }
+          pk[16 * c + i] = pack_bf16(p0, p1);
+        }
+      }
+      const bool kind3 = j >= n_lt && j >= n_a;
+      if (!kind3) {
+        tc_fence_before_sync();
+        mbar_arrive(&sm.s_read);                      // S(j) has been read: S(j+1) may take its place
+      }
+      ok = __all_sync(0xffffffffu, bwd_wait(&sm.dp_full, j & 1, abort));
+      if (!ok) break;
+      tc_fence_after_sync();
+      HGA_TRACE_POINT(13);
+      const uint32_t p_line = smem_u32(sm.p) + (uint32_t)row_in_tile * 128, ds_line = smem_u32(sm.ds) + (uint32_t)row_in_tile * 128;
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        uint32_t dp[32], dk[16];
+        tmem_ld32(dp_addr + 32 * c, dp);
+        tmem_wait_ld();
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          const uint32_t pp = pk[16 * c + i];
+          const uint64_t p2 = pack_f32x2(__uint_as_float(pp << 16), __uint_as_float(pp & 0xffff0000u));
+          const uint64_t g2 = fma_f32x2(pack_f32x2(__uint_as_float(dp[2 * i]), __uint_as_float(dp[2 * i + 1])), scale_2, neg_delta_s_2);
+          float d0, d1;
+          unpack_f32x2(mul_f32x2(p2, g2), d0, d1);
+          dk[i] = pack_bf16(d0, d1);
+        }
+        if (!kind3) {
+          // bf16 dS over the dP columns already read (8 columns per 16 keys): the A operand of dQ
+          tmem_st16(dp_addr + 16 * c, dk);
+        } else {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {               // 16-byte chunks (8 keys each), XOR-swizzled
+            const uint32_t off = ((uint32_t)(4 * c + q) ^ key7) * 16;
+            st_shared_v4(p_line + off, pk[16 * c + 4 * q], pk[16 * c + 4 * q + 1], pk[16 * c + 4 * q + 2], pk[16 * c + 4 * q + 3]);
+            st_shared_v4(ds_line + off, dk[4 * q], dk[4 * q + 1], dk[4 * q + 2], dk[4 * q + 3]);
+          }
+        }
+      }
+      if (!kind3) {
+        tmem_wait_st();
+        tc_fence_before_sync();
+        mbar_arrive(&sm.ds_full);
+        HGA_TRACE_POINT(14);
+        continue;
+      }
+      // ---- dK/dV tile
+      tc_fence_before_sync();
+      fence_proxy_async_smem();
+      mbar_arrive(&sm.ds_full);
+      HGA_TRACE_POINT(17);
+      ok = __all_sync(0xffffffffu, bwd_wait(&sm.dkv_full, (j - n_a) & 1, abort));
+      if (!ok) break;
+      tc_fence_after_sync();
+      HGA_TRACE_POINT(16);
+      // (the band kernel, which precedes this one in the stream, stores its dK/dV rows plainly: the adds below must
+      // come after it; a no-op unless the launch carried the programmatic-serialization attribute)
+      if (j == n_a) pdl_wait();
+      // All GEMMs are done, the P and dS tiles are free: each takes 32 keys x (64 floats of dV | 64 of dK); thread =
+      // element of that row, so a warp writes 128 consecutive bytes per key.
+      auto wait_staged = [&]() {           // all 128 row threads have arrived
+        ok = __all_sync(0xffffffffu, bwd_wait(&sm.staged, staged_phase, abort));
+        staged_phase ^= 1u;
+        return ok;
+      };
+      auto stage = [&](uint8_t* buf, uint32_t col) {
+        uint32_t x[32];
+        tmem_ld32(lane_base + col, x);
+        tmem_wait_ld();
+        const uint32_t base = smem_u32(buf) + (uint32_t)row_in_tile * 4;
+#pragma unroll
+        for (int i = 0; i < 32; ++i) st_shared_b32(base + (uint32_t)i * 512, x[i]);
+      };
+      // adds the rows of one chunk (lane = key) to dst; `off` = byte offset inside the chunk's rows
+      auto reduce_rows = [&](float* dst, uint8_t* buf, int hf, uint32_t off) {
+        const int o = 8 * (j - n_lt) + 4 * hf + (lane >> 3);
+        if (o >= sm.first_active && o < sm.n_far) {
+          const int pos = sm.rows[j & 3][4 * hf + (lane >> 3)] + (lane & 7);
+          bulk_reduce_add_f32(dst + ((int64_t)(b * dm.Hkv + h) * dm.S + (pos - dm.H)) * D, smem_u32(buf) + (uint32_t)lane * 512 + off, D * 4);
+        }
+        tma_store_commit();
+      };
+      auto hand_over = [&]() {             // what this thread has written is complete and visible to bulk copies
+        fence_proxy_async_smem();
+        mbar_arrive(&sm.staged);
+        return wait_staged();
+      };
+      auto have_read = [&](uint64_t* bar) {
+        tc_fence_before_sync();
+        mbar_arrive(bar);
+      };
+      const uint32_t col = quarter < 2 ? kColS : kColDP;      // lanes 0-63: dV^T, lanes 64-127: dK^T
+      stage(sm.p, col);
+      stage(sm.ds, col + 32);
+      have_read(&sm.s_read);
+      have_read(&sm.dk_read);
+      if (!hand_over()) break;
+      reduce_rows((quarter & 1) ? dK : dV, quarter < 2 ? sm.p : sm.ds, quarter >> 1, (quarter & 1) * 256u);
+      tma_store_wait_read();
+      __syncwarp();
+      mbar_arrive(&sm.staged);
+      if (!wait_staged()) break;                      // P and dS may be written again
+      HGA_TRACE_POINT(18);
+    }
+    if (ok) ok = __all_sync(0xffffffffu, bwd_wait(&sm.dq_done, 0, abort));
+    HGA_TRACE_POINT(20);
+    if (ok) {
+      // dQ epilogue through shared memory and TMA: a thread's own row is 2 D bytes away from its neighbour's, so direct
+      // 16-byte stores would touch 32 different sectors per instruction.  The rows go into Q's shared memory (all
+      // GEMMs that read it are complete) in the swizzled [panel][128 rows][128 B] layout and leave as boxes.
+      tc_fence_after_sync();
+      uint32_t x[2][32];
+      tmem_ld32(lane_base + kColDQ, x[0]);
+      tmem_ld32(lane_base + kColDQ + 32, x[1]);
+      tmem_wait_ld();
+      const uint32_t line = smem_u32(sm.q) + (uint32_t)row_in_tile * 128;
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          st_shared_v4(line + (((uint32_t)(4 * c + i) ^ key7) * 16),
+                       pack_bf16(__uint_as_float(x[c][8 * i]), __uint_as_float(x[c][8 * i + 1])),
+                       pack_bf16(__uint_as_float(x[c][8 * i + 2]), __uint_as_float(x[c][8 * i + 3])),
+                       pack_bf16(__uint_as_float(x[c][8 * i + 4]), __uint_as_float(x[c][8 * i + 5])),
+                       pack_bf16(__uint_as_float(x[c][8 * i + 6]), __uint_as_float(x[c][8 * i + 7])));
+      fence_proxy_async_smem();
+      mbar_arrive(&sm.dq_staged);
+      if (warp == 2 && lane < 2 && bwd_wait(&sm.dq_staged, 0, abort)) {      // all 128 rows are in shared memory
+        const int r0 = mt * 128 + 64 * lane;
+        if (r0 < dm.rows) {
+          tma_store_5d(&map_dq, sm.q + lane * 8192, 0, qb * dm.Bq + r0 % dm.Bq, 0, h * dm.G + r0 / dm.Bq, b);
+          tma_store_commit();
+          tma_store_wait_read();      // (the source tile has been read; the writes complete before the grid does)
+        }
+      }
+    }
+  }
+  HGA_TRACE_POINT(30);
+
+  // Common exit.  Roles leave their warps diverged, so every warp reconverges first: a block barrier reached by
+  // part of a warp would count that warp as arrived.
+  __syncwarp();
+  if (warp == 1 && sm.abort) {
+    // giving up: GEMMs already issued may still be writing tensor memory; wait (bounded) until the tensor pipe has run
+    // dry before the columns are given back
+    mma_commit_w(&sm.drain);
+    mbar_wait(&sm.drain, 0);
+  }
+  __syncwarp();
+  tc_fence_before_sync();
+  __syncthreads();
+  HGA_TRACE_POINT(31);
+  HGA_TRACE_DUMP;
+  if (tid == 0 && sm.abort && status_word) atomicOr(status_word, HGA_ABORT_CODE(3, sm.abort));
+  if (warp == 1) tmem_dealloc(tmem, 256);
+}
+
+int launch_attn_bwd_d64_sm100(const Dims& dm, const void* Q, const void* K, const void* V, const void* O, const float* LSE,
+                              const void* dO, const int32_t* group_idx, const int32_t* n_groups, void* dQ, float* dK,
+                              float* dV, int32_t* status_word, cudaStream_t st) {
+  CUtensorMap mq, mdo, mk, mv, mdq;
+  const uint32_t box[5] = {64, 8, 1, 1, 1};
+  const uint32_t box_q[5] = {64, 64, 1, 1, 1};
+  const uint64_t dq[5] = {64, (uint64_t)dm.S, 1, (uint64_t)dm.Hq, (uint64_t)dm.B};
+  const uint64_t dk[5] = {64, (uint64_t)dm.L, 1, (uint64_t)dm.Hkv, (uint64_t)dm.B};
+  const uint64_t sq[4] = {(uint64_t)dm.qs[2] * 2, 128, (uint64_t)dm.qs[1] * 2, (uint64_t)dm.qs[0] * 2};
+  const uint64_t so[4] = {(uint64_t)dm.os[2] * 2, 128, (uint64_t)dm.os[1] * 2, (uint64_t)dm.os[0] * 2};
+  const uint64_t sk[4] = {(uint64_t)dm.ks[2] * 2, 128, (uint64_t)dm.ks[1] * 2, (uint64_t)dm.ks[0] * 2};
+  const uint64_t sv[4] = {(uint64_t)dm.vs[2] * 2, 128, (uint64_t)dm.vs[1] * 2, (uint64_t)dm.vs[0] * 2};
+  if (encode_tensor_map_bf16(&mq, Q, 5, dq, sq, box_q, true) ||
+      encode_tensor_map_bf16(&mdo, dO, 5, dq, so, box_q, true) ||
+      encode_tensor_map_bf16(&mdq, dQ, 5, dq, sq, box_q, true) ||
+      encode_tensor_map_bf16(&mk, K, 5, dk, sk, box, true) ||
+      encode_tensor_map_bf16(&mv, V, 5, dk, sv, box, true))
+    return HGA_ERR_UNSUPPORTED;
+  const size_t smem = sizeof(SweepSmem) + 1024;
+  // two CTAs per SM need the largest shared-memory carve-out
+  int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(&k_attn_bwd_d64_sm100), smem, true);
+  if (rc) return rc;
+  // dK/dV of the local band first: plain stores that cover every row of the active segment; this kernel then adds
+  // the contributions of the keys before the band.  Launched with programmatic serialization behind the band kernel: it
+  // waits for it only before the first add.
+  rc = launch_attn_bwd_band_sm100(dm, Q, K, V, O, LSE, dO, dK, dV, status_word, st);
+  if (rc != HGA_OK) return rc;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(dm.B * dm.Hkv * dm.NQB * ((dm.rows + 127) / 128)));
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = (dm.flags & kFlagNoPdl) ? 0 : 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_attn_bwd_d64_sm100, mq, mdo, mk, mv, mdq, (const uint16_t*)O, LSE,
+                                           group_idx, n_groups, dm, dK, dV, status_word);
+  count_launch(HGA_KERNELS_BWD_TENSOR);
+  return record_cuda(e);
+}
+
+}  // namespace hga

@@ -103,8 +103,8 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   BwdSmem& sm = *reinterpret_cast<BwdSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  HGA_TRACE_DECL;
-  const int n_mt_item = dm.rows / 128;
+  HGA_TRACE_DECL(512);
+  const int n_mt_item = (dm.rows + 127) / 128;           // (the last M-tile may hold 64 rows only)
   // Launch order: late query blocks first.  They have the most routed keys inside the active segment (the
   // expensive dK/dV steps), early ones none, so the cheapest CTAs are the ones that fill the last wave.
   const int unit = blockIdx.x / n_mt_item, n_bh = dm.B * dm.Hkv;
@@ -143,10 +143,12 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       // four boxes of 64 rows x one 64-element panel per tensor, laid out [panel][128 rows][128 B]
       const int half = warp & 1, panel = (warp >> 1) & 1;
       const int r = mt * 128 + 64 * half;
-      const int a = r / dm.Bq, t = r % dm.Bq;
+      const bool real = r < dm.rows;                     // (rows past the item's last one arrive as zeros)
+      const int a = real ? r / dm.Bq : 0, t = r % dm.Bq;
       const uint32_t off = (uint32_t)panel * 16384 + (uint32_t)half * 8192;
-      if (warp < 4) tma_load_5d(sm.q + off, &map_q, &sm.q_full, 0, qb * dm.Bq + t, panel, h * dm.G + a, b);
-      else tma_load_5d(sm.dO + off, &map_do, &sm.q_full, 0, qb * dm.Bq + t, panel, h * dm.G + a, b);
+      const int row = real ? qb * dm.Bq + t : dm.S;
+      if (warp < 4) tma_load_5d(sm.q + off, &map_q, &sm.q_full, 0, row, panel, h * dm.G + a, b);
+      else tma_load_5d(sm.dO + off, &map_do, &sm.q_full, 0, row, panel, h * dm.G + a, b);
     }
     __syncwarp();
   }
@@ -188,9 +190,9 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   float row_lse = 0.f;
   uint4 o_half[8];
   if (warp >= 2 && warp < 10) {
-    const int r = mt * 128 + (warp & 3) * 32 + lane;
+    const int r_own = mt * 128 + (warp & 3) * 32 + lane, r = min(r_own, dm.rows - 1);
     const int hq = h * dm.G + r / dm.Bq, srow = qb * dm.Bq + r % dm.Bq;
-    row_lse = LSE[((int64_t)b * dm.Hq + hq) * dm.S + srow];
+    row_lse = r_own < dm.rows ? LSE[((int64_t)b * dm.Hq + hq) * dm.S + srow] : INFINITY;   // (padding rows: P = 0)
     const uint4* op = reinterpret_cast<const uint4*>(O + b * dm.os[0] + hq * dm.os[1] + (int64_t)srow * dm.os[2]) +
                       8 * ((warp - 2) >> 2);
 #pragma unroll
@@ -627,10 +629,12 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       if (warp == 2 && lane < 4 && bwd_wait(&sm.dq_staged, 0, abort)) {      // all 256 rows are in shared memory
         const int half = lane & 1, panel = lane >> 1;
         const int r0 = mt * 128 + 64 * half;
-        tma_store_5d(&map_dq, sm.q + panel * 16384 + half * 8192, 0, qb * dm.Bq + r0 % dm.Bq, panel,
-                     h * dm.G + r0 / dm.Bq, b);
-        tma_store_commit();
-        tma_store_wait_read();      // (the source tile has been read; the writes complete before the grid does)
+        if (r0 < dm.rows) {
+          tma_store_5d(&map_dq, sm.q + panel * 16384 + half * 8192, 0, qb * dm.Bq + r0 % dm.Bq, panel,
+                       h * dm.G + r0 / dm.Bq, b);
+          tma_store_commit();
+          tma_store_wait_read();    // (the source tile has been read; the writes complete before the grid does)
+        }
       }
     }
   } else {
@@ -691,14 +695,19 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 
 bool attn_bwd_sm100_supported(const Dims& dm) {
   if (dm.flags & HGA_FLAG_GENERIC_KERNELS) return false;
-  return dm.d == 128 && dm.rows % 128 == 0 && dm.g % 8 == 0 && dm.Bq % 64 == 0;
+  if (dm.g % 8 != 0 || !attn_bwd_band_sm100_supported(dm)) return false;
+  // head_dim 64 with fewer than eight M-tiles: the two kernels' chains (17-22 us at 8 tiles, whatever the budget) and the
+  // CUDA-core kernel (25 us for 4 tiles x 320 keys, 41 us for 8 tiles x 768 keys, and exact fp32 probabilities) take about the same
+  if (dm.d == 64 && dm.B * dm.Hkv * dm.NQB * ((dm.rows + 127) / 128) < 8) return false;
+  return true;
 }
 
 int launch_attn_bwd_sm100(const Dims& dm, const void* Q, const void* K, const void* V, const void* O,
                           const float* LSE, const void* dO, const int32_t* group_idx,
                           const int32_t* n_groups, void* dQ, float* dK, float* dV, int32_t* status_word,
                           cudaStream_t st) {
-  if (!attn_bwd_band_sm100_supported(dm)) return HGA_ERR_UNSUPPORTED;
+  if (dm.d == 64)
+    return launch_attn_bwd_d64_sm100(dm, Q, K, V, O, LSE, dO, group_idx, n_groups, dQ, dK, dV, status_word, st);
   CUtensorMap mq, mdo, mk, mv, mdq;
   const uint32_t box[5] = {64, 8, 2, 1, 1};
   const uint32_t box_q[5] = {64, 64, 1, 1, 1};
@@ -725,7 +734,7 @@ int launch_attn_bwd_sm100(const Dims& dm, const void* Q, const void* K, const vo
   // contributions of the keys before the band atomically.
   rc = launch_attn_bwd_band_sm100(dm, Q, K, V, O, LSE, dO, dK, dV, status_word, st);
   if (rc != HGA_OK) return rc;
-  const int units = dm.B * dm.Hkv * dm.NQB * (dm.rows / 128);
+  const int units = dm.B * dm.Hkv * dm.NQB * ((dm.rows + 127) / 128);
   // The sweep is launched with programmatic serialization behind the band kernel: its CTAs may start on
   // SMs the band kernel leaves idle (they wait for it only before adding to dK/dV).
   cudaLaunchConfig_t cfg = {};

@@ -80,7 +80,7 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   FwdSmem<D>& sm = *reinterpret_cast<FwdSmem<D>*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  HGA_TRACE_DECL;
+  HGA_TRACE_DECL(256);
   // rows of the item: every head's Bq rows padded to whole octets (padding rows compute garbage
   // in their own TMEM lanes and are never stored)
   const int bq_pad = bq_padded(dm), rows_pad = rows_padded(dm);
@@ -448,11 +448,10 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 
 bool attn_fwd_sm100_supported(const Dims& dm) {
   if (dm.flags & HGA_FLAG_GENERIC_KERNELS) return false;
-  const int rows_pad = rows_padded(dm);
-  if (rows_pad > 128 && (rows_pad % 128 != 0 || rows_pad != dm.rows)) return false;
-  if (rows_pad < 128 && !(dm.flags & HGA_FLAG_DECODE)) return false;   // small training shapes stay on the generic kernel
-  if (dm.g % 8 != 0) return false;
-  return true;
+  // any number of rows: the last M-tile of an item may be partly filled (its other TMEM lanes compute garbage that is
+  // never stored), which still beats the one-warp-per-row kernel by far: 16 heads of 64 rows, head_dim 64, 512 items
+  // of 768 keys take 1.9 ms there
+  return dm.g % 8 == 0;
 }
 
 template <int D>

@@ -1,8 +1,8 @@
 // Optional in-kernel timelines for the tensor-core kernels (off unless HGA_TRACE is defined).
 //
 // HGA_TRACE_POINT(tag) records (SM cycle counter, tag) for lane 0 of every warp of ONE chosen CTA of ONE
-// chosen kernel (picked at run time through g_trace_threads = the kernel's block size and g_trace_blk = the
-// block index); HGA_TRACE_DECL / HGA_TRACE_DUMP additionally record every CTA's SM id, start and end on
+// chosen kernel (picked at run time through g_trace_threads = the kernel's number, the argument of its
+// HGA_TRACE_DECL, and g_trace_blk = the block index); HGA_TRACE_DECL / HGA_TRACE_DUMP additionally record every CTA's SM id, start and end on
 // the global timer.  The records go straight to global memory (the kernels have no shared memory to
 // spare).  A point costs on the order of a hundred cycles, so a traced kernel is slower than the real
 // one: read intervals, not totals.  The harness that sets the two selectors, runs the kernels on a
@@ -27,9 +27,9 @@ __device__ __forceinline__ unsigned hga_trace_smid() {
   asm volatile("mov.u32 %0, %smid;" : "=r"(s));
   return s;
 }
-#define HGA_TRACE_DECL                                                                                  \
+#define HGA_TRACE_DECL(id)                                                                               \
   int tr_n_ = 0;                                                                                        \
-  const bool tr_on_ = (int)blockDim.x == g_trace_threads;                                               \
+  const bool tr_on_ = (id) == g_trace_threads;                                               \
   if (tr_on_ && threadIdx.x == 0 && blockIdx.x < 2048) {                                                \
     g_trace_cta[blockIdx.x][0] = hga_trace_smid();                                                      \
     g_trace_cta[blockIdx.x][1] = hga_trace_gtimer();                                                    \
@@ -47,7 +47,7 @@ __device__ __forceinline__ unsigned hga_trace_smid() {
     if (tr_on_ && threadIdx.x == 0 && blockIdx.x < 2048) g_trace_cta[blockIdx.x][2] = hga_trace_gtimer(); \
   } while (0)
 #else
-#define HGA_TRACE_DECL
+#define HGA_TRACE_DECL(id)
 #define HGA_TRACE_POINT(tag)
 #define HGA_TRACE_DUMP
 #endif

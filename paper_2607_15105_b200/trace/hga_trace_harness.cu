@@ -5,7 +5,7 @@
 // each warp, cycles counted from the CTA's earliest record.
 //
 //   python -m paper_2607_15105_b200.build --trace          builds paper_2607_15105_b200/hga_trace
-//   ./paper_2607_15105_b200/hga_trace <block size of the kernel: 256 forward, 448 band, 512 sweep> [block index]
+//   ./paper_2607_15105_b200/hga_trace <kernel number: 256 forward, 448 band, 512 sweep> [block index]
 //
 // Tags (see the kernels): 1 set-up done; 2 a producer issued a tile; 3 first GEMMs issued; 5/6/7/8 the
 // issuing warp (barrier observed / S issued / dQ or PV issued / dP issued); 11/13/14/15 a row or key
