@@ -53,6 +53,14 @@ __device__ __forceinline__ uint32_t rt_orderable(float f) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
+// Query rows of an item on the MMA N dimension: equal parts of at most 256 columns, each a multiple of 32
+__host__ __device__ inline int route_parts(const Dims& dm) { return (rows_padded(dm) + 255) / 256; }
+__host__ __device__ inline int route_part_cols(const Dims& dm) {
+  const int n = route_parts(dm);
+  return ((rows_padded(dm) + n - 1) / n + 31) & ~31;
+}
+__host__ __device__ inline int route_cols(const Dims& dm) { return route_parts(dm) * route_part_cols(dm); }
+
 template <int D, int STAGES, int ACCS>
 __global__ void __launch_bounds__(kRtThreads, 2)
 k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_ct,
@@ -76,13 +84,11 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
   item_coords(dm, item, b, h, qb);
   const Window w = window_of(dm, qb);
   const int j0 = w.se / dm.c, n_cand = (w.ls - w.se) / dm.c;
-  // query rows on N: every head's Bq rows padded to whole octets, the total padded to a multiple of 32
-  // (padding columns hold whatever shared memory held and are masked when the columns are reduced)
+  // query rows on N: every head's Bq rows padded to whole octets, the total padded to one or more parts of at most
+  // 256 columns (padding columns hold whatever shared memory held and are masked when the columns are reduced)
   const int bq_pad = bq_padded(dm), rows_pad = rows_padded(dm);
-  const int n_cols = (rows_pad + 31) & ~31;
-  const bool all_rows_real = n_cols == dm.rows;
-  const int n_halves = n_cols > 256 ? n_cols / 256 : 1;
-  const int rows_half = n_cols / n_halves;                   // N of one MMA: <= 256, multiple of 32
+  const int n_halves = route_parts(dm), rows_half = route_part_cols(dm);
+  const bool all_rows_real = n_halves * rows_half == dm.rows;
   const int k_sel = dm.kc < n_cand ? dm.kc : n_cand;
   const int opc = dm.per / 8;                                // octets per opened chunk
   const int n_ct = (n_cand + 127) / 128;                     // chunk tiles
@@ -466,10 +472,10 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
 }
 
 // Generation shapes (few query rows) take the pipelined instantiation.
-static bool route_pipelined(const Dims& dm) { return ((rows_padded(dm) + 31) & ~31) <= 128; }
+static bool route_pipelined(const Dims& dm) { return route_cols(dm) <= 128; }
 
 static size_t route_sm100_smem(const Dims& dm, int max_cand) {
-  const size_t q_bytes = (size_t)((rows_padded(dm) + 31) & ~31) * dm.d * 2;
+  const size_t q_bytes = (size_t)route_cols(dm) * dm.d * 2;
   const size_t base = route_pipelined(dm) ? (dm.d == 128 ? sizeof(RouteSmem<128, 2, 2>) : sizeof(RouteSmem<64, 2, 2>))
                                           : (dm.d == 128 ? sizeof(RouteSmem<128, 1, 1>) : sizeof(RouteSmem<64, 1, 1>));
   return base + 1024 + q_bytes + 1024 + sizeof(unsigned long long) * (max_cand + 2) +
@@ -483,9 +489,7 @@ static int route_max_cand(const Dims& dm) {
 
 bool route_sm100_supported(const Dims& dm) {
   if (dm.flags & HGA_FLAG_GENERIC_KERNELS) return false;
-  const int n_cols = (rows_padded(dm) + 31) & ~31;
-  if (n_cols > 256 && (n_cols % 256 != 0 || n_cols != dm.rows)) return false;
-  if (n_cols != dm.rows && 32 % bq_padded(dm) != 0) return false;   // the padding mask repeats every 32 columns
+  if (bq_padded(dm) != dm.Bq && 32 % bq_padded(dm) != 0) return false;   // the padding mask repeats every 32 columns
   if (dm.per != 8 && dm.per != 16) return false;            // opened chunk = 1 or 2 octets of summaries
   if (dm.kc > 1024) return false;
   if ((dm.flags & HGA_FLAG_GLOBAL_GROUP_BUDGET) && dm.kc * dm.per > 4096) return false;   // bitmap in sel[]
@@ -516,7 +520,7 @@ static int launch_route(const Dims& dm, const void* Q, const void* chunk_sum, co
   if (rc) return rc;
   const int items = dm.B * dm.Hkv * dm.NQB;
   k_route_sm100<D, STAGES, ACCS><<<items, kRtThreads, smem, st>>>(mq, mc, mg, dm, chunk_idx, group_idx, n_groups, chunk_scores,
-                                                   group_scores, ((rows_padded(dm) + 31) & ~31) * D * 2, max_cand);
+                                                   group_scores, route_cols(dm) * D * 2, max_cand);
   count_launch(HGA_KERNELS_ROUTE_TENSOR);
   return record_cuda(cudaGetLastError());
 }
