@@ -107,17 +107,25 @@ def make_params(cfg, softmax_scale: float = 0.0, flags: int = 0, q_stride=None, 
     return p
 
 
+# The marshalling of a call is on the critical path of the smallest problems (a generation step for one sequence is two
+# calls of about 10 us of GPU time each), so addresses go to ctypes as plain integers, which the declared argument types
+# convert, and the current stream is asked for by its handle: torch.cuda.current_stream() builds a Stream object, 3.4 us.
+
+
 def _ptr(t):
-    if t is None:
-        return None
-    if isinstance(t, int):
-        return C.c_void_p(t)
-    return C.c_void_p(t.data_ptr())
+    if t is None or isinstance(t, int):
+        return t
+    return t.data_ptr()
 
 
 def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())      # (initialises CUDA on first use)
+
+
+def _nbytes(t):
+    return 0 if t is None else t.numel() * t.element_size()
 
 
 def _check(call, rc):
@@ -176,7 +184,7 @@ def hga_build_summaries(p, K, tok_begin, tok_end, chunk_sum, group_sum, stream=N
 
 def hga_route(p, Q, chunk_sum, group_sum, chunk_idx, group_idx, n_groups, workspace,
               chunk_scores=None, group_scores=None, stream=None):
-    nbytes = workspace.numel() * workspace.element_size() if workspace is not None else 0
+    nbytes = _nbytes(workspace)
     _check("hga_route", lib().hga_route(
         C.byref(p), _ptr(Q), _ptr(chunk_sum), _ptr(group_sum), _ptr(chunk_idx), _ptr(group_idx),
         _ptr(n_groups), _ptr(chunk_scores), _ptr(group_scores), _ptr(workspace), nbytes,
@@ -202,7 +210,7 @@ def hga_attn_fwd(p, Q, K, V, group_idx, n_groups, O, LSE, status_word=None, stre
 
 def hga_attn_bwd(p, Q, K, V, O, LSE, dO, group_idx, n_groups, dQ, dK, dV, workspace,
                  status_word=None, stream=None):
-    nbytes = workspace.numel() * workspace.element_size() if workspace is not None else 0
+    nbytes = _nbytes(workspace)
     _check("hga_attn_bwd", lib().hga_attn_bwd(
         C.byref(p), _ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(LSE), _ptr(dO), _ptr(group_idx),
         _ptr(n_groups), _ptr(dQ), _ptr(dK), _ptr(dV), _ptr(workspace), nbytes, _ptr(status_word),
