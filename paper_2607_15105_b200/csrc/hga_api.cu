@@ -56,7 +56,7 @@ static int resolve(const hga_params* p, Dims& dm) {
   if (p->chunk / p->group > 64) return HGA_ERR_UNSUPPORTED;
   if (p->topk_chunks > 1024) return HGA_ERR_UNSUPPORTED;
   if ((p->flags & HGA_FLAG_SCORE_MEAN) && (p->flags & HGA_FLAG_SCORE_LSE)) return HGA_ERR_UNSUPPORTED;
-  if (p->flags & ~0x7f & ~(t_internal_flags ? kFlagNoPdl : 0)) return HGA_ERR_UNSUPPORTED;   // unknown flag bits
+  if (p->flags & ~0x7f & ~(t_internal_flags ? kFlagNoPdl | kFlagChained : 0)) return HGA_ERR_UNSUPPORTED;   // unknown flag bits
   if ((p->flags & HGA_FLAG_GLOBAL_GROUP_BUDGET) && (int64_t)p->topk_chunks * (p->chunk / p->group) > 4096)
     return HGA_ERR_UNSUPPORTED;
   dm.B = p->batch; dm.Hq = p->n_q_heads; dm.Hkv = p->n_kv_heads; dm.G = dm.Hq / dm.Hkv;
@@ -69,6 +69,7 @@ static int resolve(const hga_params* p, Dims& dm) {
   if (p->summary_len != 0 && (p->summary_len < p->total_len || p->summary_len % p->chunk)) return HGA_ERR_SHAPE;
   dm.NcS = (p->summary_len ? p->summary_len : dm.L) / dm.c;
   dm.NgS = (p->summary_len ? p->summary_len : dm.L) / dm.g;
+  dm.rows_q = dm.S; dm.rows_k = dm.L;
   dm.width = dm.kc * dm.kge; dm.rows = dm.G * dm.Bq;
   dm.flags = p->flags;
   dm.scale = p->softmax_scale > 0.f ? p->softmax_scale : 1.0f / sqrtf((float)dm.d);
@@ -232,7 +233,7 @@ int hga_attn_fwd(const hga_params* p, const void* Q, const void* K, const void* 
   if (!Q || !K || !V || (!group_idx && dm.width > 0) || !n_groups || !O || !LSE) return HGA_ERR_NULL;
   if (!aligned16(Q) || !aligned16(K) || !aligned16(V) || !aligned16(O)) return HGA_ERR_ALIGN;
   if (attn_fwd_sm100_supported(dm)) {
-    rc = launch_attn_fwd_sm100(dm, Q, K, V, group_idx, n_groups, O, LSE, status_word, (cudaStream_t)stream);
+    rc = launch_attn_fwd_sm100(dm, nullptr, Q, K, V, group_idx, n_groups, O, LSE, status_word, (cudaStream_t)stream);
     if (rc != HGA_ERR_UNSUPPORTED) return rc;
   }
   return launch_attn_fwd_generic(dm, Q, K, V, group_idx, n_groups, O, LSE, status_word,

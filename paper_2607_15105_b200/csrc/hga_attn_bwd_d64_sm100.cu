@@ -69,67 +69,6 @@ struct SweepSmem {
 };
 static_assert(sizeof(SweepSmem) + 1024 <= 113 * 1024, "two CTAs per SM");
 
-// The "far" part of an item's routed set (sink, then selected groups) as octets, looked up in the group list
-// itself: no table in shared memory.  A list is checked once, 32 entries per vote; a valid list (every entry
-// ascending and wholly between sink and local window) is then read directly, an invalid one is walked, skipping the
-// entries build_octet_table would skip.
-struct FarList {
-  const int32_t* gi;
-  int ng, opg, n_sink, n_far, first_active, se, ls, g;
-  bool clean;
-  __device__ bool fits(int m, int last) const {
-    return m > last && (int64_t)m * g >= se && ((int64_t)m + 1) * g <= ls;
-  }
-  __device__ FarList(const Dims& dm, const Window& w, const int32_t* list)
-      : gi(list), ng(0), opg(dm.g / 8), n_sink(w.se / 8), n_far(0), first_active(0), se(w.se), ls(w.ls), g(dm.g), clean(true) {}
-  // checks the list and counts its octets; all 32 lanes of a warp
-  __device__ void check(const Dims& dm, const int32_t* ng_ptr) {
-    const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    const int pre0 = lane < dm.width ? gi[lane] : 0x7fffffff;      // (overlaps the load of the count)
-    const int pre1 = lane + 32 < dm.width ? gi[lane + 32] : 0x7fffffff;
-    ng = *ng_ptr;
-    ng = ng < 0 ? 0 : ng > dm.width ? dm.width : ng;               // (the forward call reports such a count)
-    int prev = -1, below = 0;
-    for (int base = 0; base < ng; base += 32) {
-      const int i = base + lane;
-      const int m = i >= ng ? 0x7fffffff : base == 0 ? pre0 : base == 32 ? pre1 : gi[i];
-      int left = __shfl_up_sync(full, m, 1);
-      if (lane == 0) left = prev;
-      clean = clean && __all_sync(full, i >= ng || fits(m, left));
-      below += __popc(__ballot_sync(full, i < ng && (int64_t)m * g < dm.H));
-      prev = __shfl_sync(full, m, 31);
-    }
-    int n = ng;
-    if (!clean) {
-      n = below = 0;
-      if (lane == 0) {
-        int last = -1;
-        for (int i = 0; i < ng; ++i) {
-          const int m = gi[i];
-          if (fits(m, last)) { ++n; below += (int64_t)m * g < dm.H; last = m; }
-        }
-      }
-      n = __shfl_sync(full, n, 0);
-      below = __shfl_sync(full, below, 0);
-    }
-    n_far = n_sink + n * opg;
-    first_active = dm.H / 8 < n_sink ? dm.H / 8 : n_sink + below * opg;      // H is a multiple of g
-  }
-  // first token of far octet o (o < n_far)
-  __device__ int row(int o) const {
-    if (o < n_sink) return 8 * o;
-    const int k = o - n_sink, u = opg == 1 ? k : k / opg, sub = k - u * opg;
-    if (clean) return __ldg(gi + u) * g + 8 * sub;
-    int last = -1, n = -1;
-    for (int i = 0; i < ng; ++i) {
-      const int m = gi[i];
-      if (fits(m, last)) { last = m; if (++n == u) break; }
-    }
-    return last * g + 8 * sub;
-  }
-};
-
 }  // namespace
 
 __global__ void __launch_bounds__(kThreads, 2)
@@ -419,7 +358,7 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
   } else if (warp == 6) {
     // ------------------------------------------------------------------ routing list
     FarList far(dm, w, group_idx + (int64_t)item * dm.width);
-    far.check(dm, n_groups + item);
+    far.check(dm, n_groups + item, dm.H);      // (the forward call reports invalid lists)
     if (lane == 0) {
       sm.n_listed = far.ng; sm.n_far = far.n_far; sm.first_active = far.first_active; sm.clean = far.clean;
       mbar_arrive(&sm.info_full);

@@ -20,6 +20,12 @@ __host__ __device__ inline int score_agg_of(int flags) {
 // kernels.
 constexpr int kFlagNoPdl = 1 << 30;
 
+// Kernels of the path are launched with programmatic serialization (they may start before their predecessor in the
+// stream has ended) and execute griddepcontrol.wait before they touch memory and before they end, so "the
+// predecessor has ended" includes all work before it.  Internal flag kFlagChained: the predecessor is the library's
+// own kernel of the step before, which writes neither Q, K, V nor dO; copies of those may start ahead of the wait.
+constexpr int kFlagChained = 1 << 29;
+
 // Resolved problem description handed to kernels by value.
 struct Dims {
   int B, Hq, Hkv, G, d;
@@ -29,6 +35,7 @@ struct Dims {
   int sink, local;
   int NQB, Nc, Ng;      // query blocks per sequence, chunks, groups
   int NcS, NgS;         // rows per (batch, kv head) in the chunk / group summary buffers (>= Nc, Ng)
+  int rows_q, rows_k;   // token rows of the Q / O and of the K / V tensors (S and L, unless a launch covers several segments)
   int width;            // group_idx entries per item = kc * kge
   int rows;             // G * Bq query rows per item
   int flags;
@@ -41,13 +48,60 @@ struct Window {
   int p0, ls, se;
 };
 
-__host__ __device__ inline Window window_of(const Dims& dm, int qb) {
+// Window of the query block that starts at position p0
+__host__ __device__ inline Window window_at(const Dims& dm, int p0) {
   Window w;
-  w.p0 = dm.H + qb * dm.Bq;
+  w.p0 = p0;
   int l = w.p0 - dm.local;
   w.ls = l <= 0 ? 0 : (l / dm.c) * dm.c;
   w.se = dm.sink < w.ls ? dm.sink : w.ls;
   return w;
+}
+__host__ __device__ inline Window window_of(const Dims& dm, int qb) { return window_at(dm, dm.H + qb * dm.Bq); }
+
+// One launch can cover several segments -- the sequences of a packed batch, or the segments of one long sequence, which
+// are independent problems once the summaries are built -- instead of one: a short segment's kernels are a partial wave
+// each, and twelve of them one after another are mostly tails.  Segment s has S active tokens behind H resident ones; its
+// query rows start at row q0 of the Q / O tensors, its position 0 is row k0 of the K / V tensors, and its summaries start
+// at rows k0 / c and k0 / g.  Its routing lists, LSE and dK / dV blocks follow those of the B * q0 query rows before it.
+struct Segment {
+  int first;                // its first CTA (the unit of the kernel that reads the table)
+  int H, S, q0, k0;
+};
+constexpr int kMaxSegments = 64;      // per launch: the table is a kernel parameter
+struct SegTable {
+  int n;
+  Segment seg[kMaxSegments];
+};
+struct OneSegment {};                 // the usual problem: the segment of Dims, no table
+
+// Segment of CTA `cta`, and the CTA's number inside it
+__device__ __forceinline__ Segment segment_of(const Dims& dm, const OneSegment&, int cta, int& local) {
+  local = cta;
+  return Segment{0, dm.H, dm.S, 0, 0};
+}
+__device__ __forceinline__ Segment segment_of(const Dims&, const SegTable& t, int cta, int& local) {
+  int lo = 0, hi = t.n;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (t.seg[mid].first <= cta) lo = mid; else hi = mid;
+  }
+  local = cta - t.seg[lo].first;
+  return t.seg[lo];
+}
+// Where a segment's routing lists (in items) and per-row outputs (in rows of one head) start for batch entry b
+__device__ __forceinline__ int64_t item_base(const Dims& dm, const Segment& sg, int b) {
+  return ((int64_t)dm.B * (sg.q0 / dm.Bq) + (int64_t)b * (sg.S / dm.Bq)) * dm.Hkv;
+}
+__device__ __forceinline__ int64_t row_base(const Dims& dm, const Segment& sg, int b) {
+  return (int64_t)dm.B * sg.q0 + (int64_t)b * sg.S;
+}
+// Fills in `first`, counting units_of(segment) CTAs each; returns their number (host)
+template <class F>
+inline int64_t number_units(SegTable& t, F units_of) {
+  int64_t n = 0;
+  for (int i = 0; i < t.n; ++i) { t.seg[i].first = (int)n; n += units_of(t.seg[i]); }
+  return n;
 }
 
 __host__ __device__ inline void item_coords(const Dims& dm, int item, int& b, int& h, int& qb) {
@@ -68,6 +122,23 @@ __host__ __device__ inline int rows_padded(const Dims& dm) { return dm.G * bq_pa
 __host__ __device__ inline int max_routed_tokens(const Dims& dm) {
   return dm.sink + dm.width * dm.g + dm.local + dm.Bq + dm.c;
 }
+
+// A launch with programmatic serialization (see kFlagChained), or a plain one with kFlagNoPdl.
+struct PdlLaunch {
+  cudaLaunchConfig_t c = {};
+  cudaLaunchAttribute attr;
+  PdlLaunch(dim3 grid, unsigned threads, size_t smem, cudaStream_t st, int flags) {
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    c.gridDim = grid;
+    c.blockDim = dim3(threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    c.attrs = &attr;
+    c.numAttrs = (flags & kFlagNoPdl) ? 0 : 1;
+  }
+  PdlLaunch(const PdlLaunch&) = delete;
+};
 
 // cudaFuncSetAttribute(max dynamic shared memory [, maximal carve-out]) for `func`, cached per device (hga_tma.cu)
 int ensure_dynamic_smem(const void* func, size_t bytes, bool max_carveout = false);
@@ -91,9 +162,10 @@ int launch_attn_bwd_generic(const Dims& dm, const void* Q, const void* K, const 
                             const int32_t* group_idx, const int32_t* n_groups, void* dQ, float* dK,
                             float* dV, int32_t* status_word, cudaStream_t st);
 
-// tensor-core (tcgen05 / TMEM / TMA) kernels; *_supported says whether the shape qualifies
+// tensor-core (tcgen05 / TMEM / TMA) kernels; *_supported says whether the shape qualifies; segs: the segments the launch
+// covers (renumbered by the call), or null for the one of dm
 bool attn_fwd_sm100_supported(const Dims& dm);
-int launch_attn_fwd_sm100(const Dims& dm, const void* Q, const void* K, const void* V,
+int launch_attn_fwd_sm100(const Dims& dm, SegTable* segs, const void* Q, const void* K, const void* V,
                           const int32_t* group_idx, const int32_t* n_groups, void* O, float* LSE,
                           int32_t* status_word, cudaStream_t st);
 

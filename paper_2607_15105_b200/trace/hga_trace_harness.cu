@@ -31,6 +31,8 @@
 
 namespace hga {
 void count_launch(int, int) {}
+int launch_attn_bwd_d64_sm100(const Dims&, const void*, const void*, const void*, const void*, const float*, const void*, const int32_t*,
+                              const int32_t*, void*, float*, float*, int32_t*, cudaStream_t) { return HGA_ERR_UNSUPPORTED; }   // (head_dim 128 only here)
 int record_cuda(cudaError_t e) { if (e != cudaSuccess) printf("cuda error %s\n", cudaGetErrorString(e)); return e == cudaSuccess ? 0 : -6; }
 }
 using namespace hga;
@@ -41,7 +43,7 @@ int main(int argc, char** argv) {
   Dims dm{};
   dm.B = 1; dm.Hq = 32; dm.Hkv = 8; dm.G = 4; dm.d = 128; dm.L = 16384; dm.S = 2048; dm.H = dm.L - dm.S;
   dm.c = 64; dm.g = 8; dm.Bq = 64; dm.kc = 16; dm.kg = 4; dm.kge = 4; dm.per = 8; dm.sink = 64; dm.local = 128;
-  dm.NQB = dm.S / dm.Bq; dm.Nc = dm.L / dm.c; dm.Ng = dm.L / dm.g; dm.NcS = dm.Nc; dm.NgS = dm.Ng; dm.width = 64; dm.rows = 256; dm.flags = 0;
+  dm.NQB = dm.S / dm.Bq; dm.Nc = dm.L / dm.c; dm.Ng = dm.L / dm.g; dm.NcS = dm.Nc; dm.NgS = dm.Ng; dm.width = 64; dm.rows = 256; dm.flags = 0; dm.rows_q = dm.S; dm.rows_k = dm.L;
   dm.scale = 1.f / sqrtf(128.f);
   auto dense = [&](int64_t* s, int heads, int toks) { s[2] = dm.d; s[1] = (int64_t)toks * dm.d; s[0] = (int64_t)heads * toks * dm.d; };
   dense(dm.qs, dm.Hq, dm.S); dense(dm.ks, dm.Hkv, dm.L); dense(dm.vs, dm.Hkv, dm.L); dense(dm.os, dm.Hq, dm.S);
@@ -75,13 +77,13 @@ int main(int argc, char** argv) {
   cudaMemcpyToSymbol(g_trace_threads, &trace_threads, 4); cudaMemcpyToSymbol(g_trace_blk, &trace_blk, 4);
   char* flush; cudaMalloc(&flush, 512u << 20);
   cudaEvent_t e0, e1; cudaEventCreate(&e0); cudaEventCreate(&e1);
-  launch_attn_fwd_sm100(dm, dq, dk, dv, dgi, dng, dO, dlse, dst, 0); cudaDeviceSynchronize();
+  launch_attn_fwd_sm100(dm, nullptr, dq, dk, dv, dgi, dng, dO, dlse, dst, 0); cudaDeviceSynchronize();
   const bool fwd_mode = trace_threads == 256 || trace_threads == 384;
   for (int rep = 0; rep < 4; ++rep) {
     cudaMemsetAsync(flush, rep, 512u << 20);
     { void* p_; cudaGetSymbolAddress(&p_, g_trace_log); cudaMemsetAsync(p_, 0, sizeof(unsigned) * HGA_TRACE_WARPS * HGA_TRACE_SLOTS); }
     cudaEventRecord(e0);
-    int rc = fwd_mode ? launch_attn_fwd_sm100(dm, dq, dk, dv, dgi, dng, dO, dlse, dst, 0)
+    int rc = fwd_mode ? launch_attn_fwd_sm100(dm, nullptr, dq, dk, dv, dgi, dng, dO, dlse, dst, 0)
                       : launch_attn_bwd_sm100(dm, dq, dk, dv, dO, dlse, ddO, dgi, dng, ddQ, ddK, ddV, dst, 0);
     cudaEventRecord(e1);
     cudaError_t ce = cudaDeviceSynchronize();
