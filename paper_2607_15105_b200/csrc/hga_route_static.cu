@@ -64,8 +64,8 @@ extern "C" int hga_route_static(const hga_params* p, const void* Q, const void* 
   if (rc) return rc;
   // Shapes the fused tensor-core router takes keep every score on chip: it runs first, as in
   // hga_route, and the array stays untouched.  Other shapes go to the CUDA-core router below.
-  if (route_sm100_supported(dm)) {
-    rc = launch_route_sm100(dm, Q, chunk_sum, group_sum, chunk_idx, group_idx, n_groups, nullptr, nullptr,
+  if (route_sm100_supported(dm, nullptr)) {
+    rc = launch_route_sm100(dm, nullptr, Q, chunk_sum, group_sum, chunk_idx, group_idx, n_groups, nullptr, nullptr,
                             (cudaStream_t)stream);
     if (rc != HGA_ERR_UNSUPPORTED) return rc;
   }
