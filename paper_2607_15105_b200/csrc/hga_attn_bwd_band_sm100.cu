@@ -143,7 +143,7 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
   // boxes of 64 rows x one 64-element panel (8 KB each); the 28 boxes a CTA starts with (head_dim 128) go out from
   // twelve warps in parallel, in the order they are needed: K, V, the first half-step's Q and dO rows, the
   // second half-step's, the first O tile, then the second step's Q and dO.
-  auto coords = [&](const HalfStep& hs, int& row, int& head) {
+  auto coords = [&](HalfStep hs, int& row, int& head) {
     const bool real = hs.r0 < dm.rows;
     row = real ? hs.qb * dm.Bq + hs.t : dm.S;                // (padding: out of range, zeros)
     head = h * dm.G + (real ? hs.head : 0);
@@ -153,14 +153,14 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
     const int half = i & 1, panel = i >> 1;
     tma_load_5d(dst + panel * 16384 + half * 8192, map, &sm.kv_full, 0, k0 + 64 * half, panel, h, b);
   };
-  auto copy_qdo = [&](const HalfStep& hs, int st, int half, int i) {
+  auto copy_qdo = [&](HalfStep hs, int st, int half, int i) {
     const int panel = i % kPanels, is_do = i / kPanels;
     int row, head;
     coords(hs, row, head);
     tma_load_5d((is_do ? sm.dO[st] : sm.q[st]) + panel * 16384 + half * 8192, is_do ? &map_do : &map_q, &sm.qdo_full[st][half],
                 0, row, panel, head, b);
   };
-  auto copy_o = [&](const HalfStep& h0, const HalfStep& h1, int i) {
+  auto copy_o = [&](HalfStep h0, HalfStep h1, int i) {
     const int half = i & 1, panel = i >> 1;
     int row, head;
     coords(half ? h1 : h0, row, head);

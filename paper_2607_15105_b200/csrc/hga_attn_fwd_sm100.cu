@@ -66,7 +66,7 @@ struct FwdSmem {
 // One row against its visible keys with a running maximum, by a whole warp (lane: D/32 elements): rows whose exponentials
 // left the range of the first tile's reference.  Returns log2 of the sum; o: the normalised output elements.
 template <int D>
-__device__ __noinline__ float row_with_running_maximum(const FarList& far, const uint16_t* q, const uint16_t* K, const uint16_t* V,
+__device__ __forceinline__ float row_with_running_maximum(const FarList& far, const uint16_t* q, const uint16_t* K, const uint16_t* V,
                                                        int64_t k_stride, int64_t v_stride, int pos, float sl2, float (&o)[D / 32]) {
   constexpr int E = D / 32;
   const int lane = threadIdx.x & 31;
@@ -356,6 +356,7 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         // the row's reference: its maximum over the first tile (ok or not, every softmax thread meets here once)
         float mx[2] = {-INFINITY, -INFINITY};
         if (ok && warp_real) {
+#pragma unroll 1
           for (int c = 0; c < (whole ? 2 : 1); ++c) {
             uint32_t x[32];
             tmem_ld32(lane_base + 64 * c + 32 * hw, x);
@@ -382,7 +383,8 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       // the MMA really applies: normalising O by THEIR sum makes the rounding of a dominant weight cancel.
       const uint64_t neg_m2 = pack_f32x2(neg_m, neg_m);
       uint64_t lsum = pack_f32x2(0.f, 0.f), rsum = pack_f32x2(0.f, 0.f);
-#pragma unroll
+      // (one copy of the code for both halves: a CTA of a few tiles pays for every line of it once in instruction-cache misses)
+#pragma unroll 1
       for (int c = 0; c < 2; ++c) {
         if (c == 1 && !whole) break;
         if (warp_real) {

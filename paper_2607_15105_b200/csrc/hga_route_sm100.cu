@@ -29,8 +29,8 @@ using namespace sm100;
 
 namespace {
 
-constexpr int kRtThreads = 320;     // warp 0 producer, warp 1 MMA, warps 2-5 readers, 6-9 help in select
-constexpr int kRtWarps = kRtThreads / 32;
+constexpr int kRtThreads = 256;     // warp 0 producer, warp 1 MMA, warps 2-5 readers, 6-7 help in select
+constexpr int kRtWarps = kRtThreads / 32, kRtCopyWarps = kRtWarps - 2;
 constexpr int kSlab = 128 * 128;    // bytes of 128 summaries x 64 elements
 constexpr int kRankMax = 640;       // up to here a candidate's rank is counted directly
 
@@ -176,168 +176,6 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
   // the forward kernel, the usual successor, may set itself up meanwhile
   if (tid == 0) pdl_launch_dependents();
 
-  // One GEMM phase: tiles [t_begin, t_begin + n_tiles) in the global tile numbering (which
-  // drives barrier parities); `phase2` selects the source of the summaries.
-  auto run_phase = [&](int t_begin, int n_tiles, bool phase2) {
-    if (!phase2 && warp >= 2) {
-      // The item's query rows.  Issuing a box costs its warp a few hundred
-      // cycles and warps issue in parallel, so the boxes are spread over the eight non-producer warps.
-      if (boxes) {
-        for (int i = (warp - 2) + 8 * lane; i < rows_pad / 64 * kPanels; i += 256) {
-          const int panel = i % kPanels, r = i / kPanels * 64;
-          tma_load_5d(q_smem + panel * q_panel + r * 128, &map_q, &sm.q_full, 0, sg.q0 + qb * dm.Bq + r % dm.Bq, panel, h * dm.G + r / dm.Bq, b);
-        }
-      } else {
-        for (int o = (warp - 2) + 8 * lane; o < rows_pad / 8; o += 256) {
-          const int r = 8 * o, a = r / bq_pad, t = r % bq_pad;    // rows past the segment arrive as zeros
-          tma_load_5d(q_smem + o * kOctBytes, &map_q, &sm.q_full, 0, sg.q0 + qb * dm.Bq + t, 0, h * dm.G + a, b);
-        }
-      }
-    }
-    // First tile of the opened chunks' group summaries, again spread over the eight warps (two octet boxes each).  Its
-    // stages are known to be free: every tile of the first phase has been read back, so no barrier needs to be
-    // observed; warp 0 announces the bytes.
-    if (phase2 && warp >= 2 && lane < 2) copy_group_octet(t_begin, 0, (warp - 2) * 2 + lane);
-    __syncwarp();
-    if (warp == 0) {
-      // ---------------------------------------------------------------- producer
-      bool ok = true;
-      auto wait_empty = [&](int g) {
-        if (lane == 0 && g >= NSTG) ok = rt_wait(&sm.a_empty[g % NSTG], (uint32_t)(g / NSTG - 1) & 1, abort);
-        ok = __shfl_sync(0xffffffffu, ok, 0);
-        return ok;
-      };
-      if (!phase2) {
-        for (int g = n_pre; g < n_slabs; ++g) {
-          if (!wait_empty(g)) break;
-          copy_slab(g, g / kPanels, g % kPanels);
-        }
-      } else {
-        announce_group_tile(t_begin);      // (its boxes come from the other warps, see above)
-        for (int t = 1; t < n_tiles && ok; ++t) {
-          const int tg = t_begin + t;
-          for (int p = 0; p < kPanels && ok; ++p) wait_empty(tg * kPanels + p);
-          if (!ok) break;
-          announce_group_tile(tg);
-          __syncwarp();
-          if (lane < 16) copy_group_octet(tg, t, lane);
-        }
-      }
-    } else if (warp == 1) {
-      // ---------------------------------------------------------------- MMA issuer
-      // The whole warp runs this branch converged (waits included) and one elected lane issues: see mma_ss_w.
-      auto mma_wait = [&](uint64_t* bar, uint32_t parity) {
-        return __all_sync(0xffffffffu, rt_wait(bar, parity, abort));
-      };
-      const uint32_t idesc = idesc_bf16_f32(128, lay.part_cols, 0, 0);
-      const uint64_t b_desc = smem_desc_sw128(smem_u32(q_smem), 16, boxes ? 1024 : kOctBytes);
-      const uint32_t part_bytes = (uint32_t)lay.part_cols * (boxes ? 128u : (uint32_t)D * 2);
-      bool ok = phase2 ? true : mma_wait(&sm.q_full, 0);
-      for (int t = 0; t < n_tiles && ok; ++t) {
-        const int tg = t_begin + t;
-        // parts that have accumulators at the same time; a slab is used by all of them before the next one
-        for (int p0 = 0; p0 < lay.parts && ok; p0 += ACCS) {
-          const int p1 = min(p0 + ACCS, lay.parts);
-#pragma unroll
-          for (int pn = 0; pn < kPanels; ++pn) {
-            const int g = tg * kPanels + pn, s = g % NSTG;
-            if (ok && p0 == 0) ok = mma_wait(&sm.a_full[s], (uint32_t)(g / NSTG) & 1);
-            // A: 8-row groups 1024 B apart inside a slab, or octets (8 rows x all panels) for the gathered group tiles
-            const uint64_t ad = phase2 ? desc_advance(smem_desc_sw128(smem_u32(sm.a[tg * kPanels % NSTG]), 16, kOctBytes), pn * 1024)
-                                       : smem_desc_sw128(smem_u32(sm.a[s]), 16, 1024);
-            for (int part = p0; part < p1 && ok; ++part) {
-              const int step = tg * lay.parts + part, acc = step % ACCS;
-              if (pn == 0 && step >= ACCS) ok = mma_wait(&sm.acc_free[acc], (uint32_t)(step / ACCS - 1) & 1);
-              if (!ok) break;
-              tc_fence_after_sync();
-              const uint64_t bd = desc_advance(b_desc, (uint32_t)part * part_bytes + pn * q_panel);
-#pragma unroll
-              for (int kk = 0; kk < 4; ++kk)
-                mma_ss_w(tmem + acc * 128, desc_advance(ad, kk * 32), desc_advance(bd, kk * 32), idesc, (pn > 0 || kk > 0));
-              if (pn == kPanels - 1) mma_commit_w(&sm.acc_full[acc]);
-            }
-            if (ok && p1 == lay.parts) mma_commit_w(&sm.a_empty[s]);
-          }
-        }
-      }
-    } else if (warp < 6) {
-      // ---------------------------------------------------------------- readers: thread = summary
-      const int quarter = warp & 3;
-      const int row = quarter * 32 + lane;
-      const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
-      bool ok = true;
-      for (int t = 0; t < n_tiles && ok; ++t) {
-        const int tg = t_begin + t;
-        float best = -FLT_MAX, sum = 0.f;    // log-sum-exp: (running maximum, sum of exp(dot - maximum))
-        for (int part = 0; part < lay.parts; ++part) {
-          const int step = tg * lay.parts + part, acc = step % ACCS;
-          ok = __all_sync(0xffffffffu, rt_wait(&sm.acc_full[acc], (uint32_t)(step / ACCS) & 1, abort));
-          if (!ok) break;
-          tc_fence_after_sync();
-          if (agg == 0 && all_rows_real) {
-            // the usual case: 64 columns per round trip to tensor memory
-            float m[4] = {best, -FLT_MAX, -FLT_MAX, -FLT_MAX};
-            for (int c = 0; c < lay.part_cols; c += 64) {
-              uint32_t x[32], y[32];
-              tmem_ld32(lane_base + acc * 128 + c, x);
-              if (c + 32 < lay.part_cols) tmem_ld32(lane_base + acc * 128 + c + 32, y);
-              else {
-#pragma unroll
-                for (int i = 0; i < 32; ++i) y[i] = 0xff7fffffu;      // -FLT_MAX
-              }
-              tmem_wait_ld();
-#pragma unroll
-              for (int i = 0; i < 32; ++i) m[i & 3] = fmaxf(fmaxf(m[i & 3], __uint_as_float(x[i])), __uint_as_float(y[i]));
-            }
-            best = fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
-          } else {
-            for (int c = 0; c < lay.part_cols; c += 32) {
-              uint32_t x[32];
-              tmem_ld32(lane_base + acc * 128 + c, x);
-              tmem_wait_ld();
-              if (!all_rows_real) {
-                // padding columns become the neutral element of the reduction (the pattern of real columns repeats in
-                // every block of 32; only the last block can be cut)
-                const float neutral = agg == 1 ? 0.f : -INFINITY;
-                const int left = rows_pad - (part * lay.part_cols + c);
-                const uint32_t m = left >= 32 ? col_mask : (col_mask & ((1u << (left > 0 ? left : 0)) - 1u));
-#pragma unroll
-                for (int i = 0; i < 32; ++i)
-                  if (!((m >> i) & 1u)) x[i] = __float_as_uint(neutral);
-              }
-              if (agg == 0) {
-#pragma unroll
-                for (int i = 0; i < 32; ++i) best = fmaxf(best, __uint_as_float(x[i]));
-              } else if (agg == 1) {
-#pragma unroll
-                for (int i = 0; i < 32; ++i) sum += __uint_as_float(x[i]);
-              } else {
-                float cm = -FLT_MAX;
-#pragma unroll
-                for (int i = 0; i < 32; ++i) cm = fmaxf(cm, __uint_as_float(x[i]));
-                if (cm > best) { sum *= exp2f((best - cm) * kLog2e); best = cm; }
-#pragma unroll
-                for (int i = 0; i < 32; ++i) sum += exp2f((__uint_as_float(x[i]) - best) * kLog2e);
-              }
-            }
-          }
-          tc_fence_before_sync();
-          mbar_arrive(&sm.acc_free[acc]);
-        }
-        if (!ok) break;
-        if (agg == 1) best = sum * (1.f / (float)dm.rows);
-        else if (agg == 2) best += logf(sum);
-        const int i = 128 * t + row;
-        if (!phase2) {
-          if (i < n_cand) okeys[i] = rt_orderable(best);
-          if (chunk_scores && i < n_cand) chunk_scores[item * dm.Nc + j0 + i] = best;
-        } else {
-          if (i < k_sel * dm.per) gscore[i] = best;
-        }
-      }
-    }
-  };
-
   // optional output: -inf outside the candidate range
   if (chunk_scores)
     for (int j = tid; j < dm.Nc; j += kRtThreads)
@@ -346,102 +184,268 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
     for (int i = tid; i < dm.kc * dm.per; i += kRtThreads)
       group_scores[item * dm.kc * dm.per + i] = -INFINITY;
 
-  if (k_sel > 0) run_phase(0, n_ct, false);
-  __syncwarp();          // the roles diverge inside a warp: reconverge before the block barrier
-  __syncthreads();
-
-  // ---------------------------------------------------------------------- chunk top-k
-  // Scores compare as 32-bit orderable integers; equal scores are told apart by their index (lowest first).
-  if (!sm.abort && k_sel > 0) {
-    if (n_cand <= kRankMax) {
-      // Few candidates: a candidate is selected when fewer than k_sel others beat it; counted for every one, four
-      // keys per 16-byte load.  Equal scores share a rank at first; that only matters when a tie straddles the k-th place,
-      // which shows as a selection of the wrong size and is redone with the index as the second criterion.
-      auto rank_select = [&](bool exact) {
-        for (int base = 0; base < n_cand; base += kRtThreads) {   // warp-uniform trip count (ballots below)
-          const int i = base + tid;
-          bool sel = false;
-          if (i < n_cand) {
-            int beat = 0, q = 0;
-            const uint32_t mine = okeys[i];
-            if (!exact) {
-              const uint4* k4 = reinterpret_cast<const uint4*>(okeys);
-#pragma unroll 4
-              for (; q + 4 <= n_cand; q += 4) {
-                const uint4 kk = k4[q >> 2];
-                beat += (int)(kk.x > mine) + (int)(kk.y > mine) + (int)(kk.z > mine) + (int)(kk.w > mine);
-              }
-              for (; q < n_cand; ++q) beat += okeys[q] > mine;
-            } else {
-              for (; q < n_cand; ++q) beat += okeys[q] > mine || (okeys[q] == mine && q < i);
-            }
-            sel = beat < k_sel;
+  // Two GEMM phases over the same code, one after the other: candidate chunks, then the groups of the opened chunks.
+  // Tiles are numbered through (t_begin + t), which drives barrier parities.  (One copy of the code: a CTA of a small
+  // problem runs it once or twice, and what it executes for the first time costs instruction-cache misses -- with a
+  // copy per phase the second phase's first tile was 2 us later.)
+#pragma unroll 1
+  for (int phase = 0; phase < 2; ++phase) {
+    const bool phase2 = phase == 1;
+    const int t_begin = phase2 ? n_ct : 0, n_tiles = phase2 ? n_gt : n_ct;
+    if (k_sel > 0 && !sm.abort) {
+      if (!phase2 && warp >= 2) {
+        // The item's query rows.  Issuing a box costs its warp a few hundred
+        // cycles and warps issue in parallel, so the boxes are spread over the non-producer warps.
+        if (boxes) {
+          for (int i = (warp - 2) + kRtCopyWarps * lane; i < rows_pad / 64 * kPanels; i += 32 * kRtCopyWarps) {
+            const int panel = i % kPanels, r = i / kPanels * 64;
+            tma_load_5d(q_smem + panel * q_panel + r * 128, &map_q, &sm.q_full, 0, sg.q0 + qb * dm.Bq + r % dm.Bq, panel, h * dm.G + r / dm.Bq, b);
           }
-          const uint32_t word = __ballot_sync(0xffffffffu, sel);
+        } else {
+          for (int o = (warp - 2) + kRtCopyWarps * lane; o < rows_pad / 8; o += 32 * kRtCopyWarps) {
+            const int r = 8 * o, a = r / bq_pad, t = r % bq_pad;    // rows past the segment arrive as zeros
+            tma_load_5d(q_smem + o * kOctBytes, &map_q, &sm.q_full, 0, sg.q0 + qb * dm.Bq + t, 0, h * dm.G + a, b);
+          }
+        }
+      }
+      // First tile of the opened chunks' group summaries, again spread over these warps (two or three octet boxes each).  Its
+      // stages are known to be free: every tile of the first phase has been read back, so no barrier needs to be
+      // observed; warp 0 announces the bytes.
+      if (phase2 && warp >= 2 && (warp - 2) + kRtCopyWarps * lane < 16) copy_group_octet(t_begin, 0, (warp - 2) + kRtCopyWarps * lane);
+      __syncwarp();
+      if (warp == 0) {
+        // ---------------------------------------------------------------- producer
+        bool ok = true;
+        auto wait_empty = [&](int g) {
+          if (lane == 0 && g >= NSTG) ok = rt_wait(&sm.a_empty[g % NSTG], (uint32_t)(g / NSTG - 1) & 1, abort);
+          ok = __shfl_sync(0xffffffffu, ok, 0);
+          return ok;
+        };
+        if (!phase2) {
+          for (int g = n_pre; g < n_slabs; ++g) {
+            if (!wait_empty(g)) break;
+            copy_slab(g, g / kPanels, g % kPanels);
+          }
+        } else {
+          announce_group_tile(t_begin);      // (its boxes come from the other warps, see above)
+          for (int t = 1; t < n_tiles && ok; ++t) {
+            const int tg = t_begin + t;
+            for (int p = 0; p < kPanels && ok; ++p) wait_empty(tg * kPanels + p);
+            if (!ok) break;
+            announce_group_tile(tg);
+            __syncwarp();
+            if (lane < 16) copy_group_octet(tg, t, lane);
+          }
+        }
+      } else if (warp == 1) {
+        // ---------------------------------------------------------------- MMA issuer
+        // The whole warp runs this branch converged (waits included) and one elected lane issues: see mma_ss_w.
+        auto mma_wait = [&](uint64_t* bar, uint32_t parity) {
+          return __all_sync(0xffffffffu, rt_wait(bar, parity, abort));
+        };
+        const uint32_t idesc = idesc_bf16_f32(128, lay.part_cols, 0, 0);
+        const uint64_t b_desc = smem_desc_sw128(smem_u32(q_smem), 16, boxes ? 1024 : kOctBytes);
+        // A: 8-row groups 1024 B apart inside a slab, or octets (8 rows x all panels) for the gathered group tiles
+        const uint64_t a_desc = smem_desc_sw128(smem_u32(sm.a[0]), 16, phase2 ? kOctBytes : 1024);
+        const uint32_t part_bytes = (uint32_t)lay.part_cols * (boxes ? 128u : (uint32_t)D * 2);
+        bool ok = phase2 ? true : mma_wait(&sm.q_full, 0);
+        for (int t = 0; t < n_tiles && ok; ++t) {
+          const int tg = t_begin + t;
+          // parts that have accumulators at the same time; a slab is used by all of them before the next one
+          for (int p0 = 0; p0 < lay.parts && ok; p0 += ACCS) {
+            const int p1 = min(p0 + ACCS, lay.parts);
+#pragma unroll
+            for (int pn = 0; pn < kPanels; ++pn) {
+              const int g = tg * kPanels + pn, s = g % NSTG;
+              if (ok && p0 == 0) ok = mma_wait(&sm.a_full[s], (uint32_t)(g / NSTG) & 1);
+              const uint64_t ad = desc_advance(a_desc, phase2 ? (uint32_t)(tg * kPanels % NSTG) * kSlab + pn * 1024 : (uint32_t)s * kSlab);
+            for (int part = p0; part < p1 && ok; ++part) {
+                const int step = tg * lay.parts + part, acc = step % ACCS;
+                if (pn == 0 && step >= ACCS) ok = mma_wait(&sm.acc_free[acc], (uint32_t)(step / ACCS - 1) & 1);
+                if (!ok) break;
+                tc_fence_after_sync();
+                const uint64_t bd = desc_advance(b_desc, (uint32_t)part * part_bytes + pn * q_panel);
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk)
+                  mma_ss_w(tmem + acc * 128, desc_advance(ad, kk * 32), desc_advance(bd, kk * 32), idesc, (pn > 0 || kk > 0));
+                if (pn == kPanels - 1) mma_commit_w(&sm.acc_full[acc]);
+              }
+              if (ok && p1 == lay.parts) mma_commit_w(&sm.a_empty[s]);
+            }
+          }
+        }
+      } else if (warp < 6) {
+        // ---------------------------------------------------------------- readers: thread = summary
+        const int quarter = warp & 3;
+        const int row = quarter * 32 + lane;
+        const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
+        bool ok = true;
+        for (int t = 0; t < n_tiles && ok; ++t) {
+          const int tg = t_begin + t;
+          float best = -FLT_MAX, sum = 0.f;    // log-sum-exp: (running maximum, sum of exp(dot - maximum))
+          for (int part = 0; part < lay.parts; ++part) {
+            const int step = tg * lay.parts + part, acc = step % ACCS;
+            ok = __all_sync(0xffffffffu, rt_wait(&sm.acc_full[acc], (uint32_t)(step / ACCS) & 1, abort));
+            if (!ok) break;
+            tc_fence_after_sync();
+            if (agg == 0 && all_rows_real) {
+              // the usual case: 64 columns per round trip to tensor memory
+              float m[4] = {best, -FLT_MAX, -FLT_MAX, -FLT_MAX};
+              for (int c = 0; c < lay.part_cols; c += 64) {
+                uint32_t x[32], y[32];
+                tmem_ld32(lane_base + acc * 128 + c, x);
+                if (c + 32 < lay.part_cols) tmem_ld32(lane_base + acc * 128 + c + 32, y);
+                else {
+#pragma unroll
+                  for (int i = 0; i < 32; ++i) y[i] = 0xff7fffffu;      // -FLT_MAX
+                }
+                tmem_wait_ld();
+#pragma unroll
+                for (int i = 0; i < 32; ++i) m[i & 3] = fmaxf(fmaxf(m[i & 3], __uint_as_float(x[i])), __uint_as_float(y[i]));
+              }
+              best = fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
+            } else {
+              for (int c = 0; c < lay.part_cols; c += 32) {
+                uint32_t x[32];
+                tmem_ld32(lane_base + acc * 128 + c, x);
+                tmem_wait_ld();
+                if (!all_rows_real) {
+                  // padding columns become the neutral element of the reduction (the pattern of real columns repeats in
+                  // every block of 32; only the last block can be cut)
+                  const float neutral = agg == 1 ? 0.f : -INFINITY;
+                  const int left = rows_pad - (part * lay.part_cols + c);
+                  const uint32_t m = left >= 32 ? col_mask : (col_mask & ((1u << (left > 0 ? left : 0)) - 1u));
+#pragma unroll
+                  for (int i = 0; i < 32; ++i)
+                    if (!((m >> i) & 1u)) x[i] = __float_as_uint(neutral);
+                }
+                if (agg == 0) {
+#pragma unroll
+                  for (int i = 0; i < 32; ++i) best = fmaxf(best, __uint_as_float(x[i]));
+                } else if (agg == 1) {
+#pragma unroll
+                  for (int i = 0; i < 32; ++i) sum += __uint_as_float(x[i]);
+                } else {
+                  float cm = -FLT_MAX;
+#pragma unroll
+                  for (int i = 0; i < 32; ++i) cm = fmaxf(cm, __uint_as_float(x[i]));
+                  if (cm > best) { sum *= exp2f((best - cm) * kLog2e); best = cm; }
+#pragma unroll
+                  for (int i = 0; i < 32; ++i) sum += exp2f((__uint_as_float(x[i]) - best) * kLog2e);
+                }
+              }
+            }
+            tc_fence_before_sync();
+            mbar_arrive(&sm.acc_free[acc]);
+          }
+          if (!ok) break;
+          if (agg == 1) best = sum * (1.f / (float)dm.rows);
+          else if (agg == 2) best += logf(sum);
+          const int i = 128 * t + row;
+          if (!phase2) {
+            if (i < n_cand) okeys[i] = rt_orderable(best);
+            if (chunk_scores && i < n_cand) chunk_scores[item * dm.Nc + j0 + i] = best;
+          } else {
+            if (i < k_sel * dm.per) gscore[i] = best;
+          }
+        }
+      }
+  
+    }
+    __syncwarp();          // the roles diverge inside a warp: reconverge before the block barrier
+    __syncthreads();
+    if (phase2) break;
+
+    // ---------------------------------------------------------------------- chunk top-k
+    // Scores compare as 32-bit orderable integers; equal scores are told apart by their index (lowest first).
+    if (!sm.abort && k_sel > 0) {
+      if (n_cand <= kRankMax) {
+        // Few candidates: a candidate is selected when fewer than k_sel others beat it; counted for every one, four
+        // keys per 16-byte load.  Equal scores share a rank at first; that only matters when a tie straddles the k-th place,
+        // which shows as a selection of the wrong size and is redone with the index as the second criterion.
+        auto rank_select = [&](bool exact) {
+          for (int base = 0; base < n_cand; base += kRtThreads) {   // warp-uniform trip count (ballots below)
+            const int i = base + tid;
+            bool sel = false;
+            if (i < n_cand) {
+              int beat = 0, q = 0;
+              const uint32_t mine = okeys[i];
+              if (!exact) {
+                const uint4* k4 = reinterpret_cast<const uint4*>(okeys);
+#pragma unroll 4
+                for (; q + 4 <= n_cand; q += 4) {
+                  const uint4 kk = k4[q >> 2];
+                  beat += (int)(kk.x > mine) + (int)(kk.y > mine) + (int)(kk.z > mine) + (int)(kk.w > mine);
+                }
+                for (; q < n_cand; ++q) beat += okeys[q] > mine;
+              } else {
+                for (; q < n_cand; ++q) beat += okeys[q] > mine || (okeys[q] == mine && q < i);
+              }
+              sel = beat < k_sel;
+            }
+            const uint32_t word = __ballot_sync(0xffffffffu, sel);
+            if (lane == 0 && base + warp * 32 < n_cand) flags[(base + warp * 32) >> 5] = word;
+          }
+        };
+        rank_select(false);
+        __syncthreads();
+        int n_picked = 0;
+        for (int q = 0; q < (n_cand + 31) / 32; ++q) n_picked += __popc(flags[q]);
+        if (n_picked != k_sel) {          // same value in every thread
+          __syncthreads();
+          rank_select(true);
+          __syncthreads();
+        }
+      } else {
+        // Many candidates: the k_sel-th largest key bit by bit from the top -- at most 32 rounds of one pass over a thread's
+        // few keys and one block-wide count, fewer when a prefix already splits off exactly k_sel.
+        uint32_t kth = 0;                 // largest value that at least k_sel keys reach, once the loop has ended
+        int reach = n_cand;               // how many keys reach it
+        int turn = 0;
+        for (uint32_t bit = 0x80000000u; bit != 0 && reach != k_sel; bit >>= 1, turn ^= 1) {
+          const uint32_t t = kth | bit;
+          int n = 0;
+          for (int i = tid; i < n_cand; i += kRtThreads) n += okeys[i] >= t ? 1 : 0;
+          n = __reduce_add_sync(0xffffffffu, n);
+          if (lane == 0) sm.count[turn][warp] = n;
+          __syncthreads();
+          n = 0;
+#pragma unroll
+          for (int q = 0; q < kRtWarps; ++q) n += sm.count[turn][q];
+          if (n >= k_sel) { kth = t; reach = n; }
+        }
+        for (int base = 0; base < n_cand; base += kRtThreads) {
+          const int i = base + tid;
+          const uint32_t word = __ballot_sync(0xffffffffu, i < n_cand && okeys[i] >= kth);
           if (lane == 0 && base + warp * 32 < n_cand) flags[(base + warp * 32) >> 5] = word;
         }
-      };
-      rank_select(false);
-      __syncthreads();
-      int n_picked = 0;
-      for (int q = 0; q < (n_cand + 31) / 32; ++q) n_picked += __popc(flags[q]);
-      if (n_picked != k_sel) {          // same value in every thread
         __syncthreads();
-        rank_select(true);
+        if (reach != k_sel && tid == 0) {
+          // ties at the k-th place: the last reach - k_sel of the keys equal to it, in index order, are not selected
+          int left = reach - k_sel;
+          for (int i = n_cand - 1; i >= 0 && left > 0; --i)
+            if (okeys[i] == kth) { flags[i >> 5] &= ~(1u << (i & 31)); --left; }
+        }
         __syncthreads();
       }
-    } else {
-      // Many candidates: the k_sel-th largest key bit by bit from the top -- at most 32 rounds of one pass over a thread's
-      // few keys and one block-wide count, fewer when a prefix already splits off exactly k_sel.
-      uint32_t kth = 0;                 // largest value that at least k_sel keys reach, once the loop has ended
-      int reach = n_cand;               // how many keys reach it
-      int turn = 0;
-      for (uint32_t bit = 0x80000000u; bit != 0 && reach != k_sel; bit >>= 1, turn ^= 1) {
-        const uint32_t t = kth | bit;
-        int n = 0;
-        for (int i = tid; i < n_cand; i += kRtThreads) n += okeys[i] >= t ? 1 : 0;
-        n = __reduce_add_sync(0xffffffffu, n);
-        if (lane == 0) sm.count[turn][warp] = n;
-        __syncthreads();
-        n = 0;
-#pragma unroll
-        for (int q = 0; q < kRtWarps; ++q) n += sm.count[turn][q];
-        if (n >= k_sel) { kth = t; reach = n; }
-      }
-      for (int base = 0; base < n_cand; base += kRtThreads) {
-        const int i = base + tid;
-        const uint32_t word = __ballot_sync(0xffffffffu, i < n_cand && okeys[i] >= kth);
-        if (lane == 0 && base + warp * 32 < n_cand) flags[(base + warp * 32) >> 5] = word;
-      }
-      __syncthreads();
-      if (reach != k_sel && tid == 0) {
-        // ties at the k-th place: the last reach - k_sel of the keys equal to it, in index order, are not selected
-        int left = reach - k_sel;
-        for (int i = n_cand - 1; i >= 0 && left > 0; --i)
-          if (okeys[i] == kth) { flags[i >> 5] &= ~(1u << (i & 31)); --left; }
+      for (int i = tid; i < n_cand; i += kRtThreads) {
+        const uint32_t word = flags[i >> 5];
+        if ((word >> (i & 31)) & 1u) {
+          int pos = __popc(word & ((1u << (i & 31)) - 1u));
+          for (int q = 0; q < (i >> 5); ++q) pos += __popc(flags[q]);
+          sorted[pos] = j0 + i;
+        }
       }
       __syncthreads();
     }
-    for (int i = tid; i < n_cand; i += kRtThreads) {
-      const uint32_t word = flags[i >> 5];
-      if ((word >> (i & 31)) & 1u) {
-        int pos = __popc(word & ((1u << (i & 31)) - 1u));
-        for (int q = 0; q < (i >> 5); ++q) pos += __popc(flags[q]);
-        sorted[pos] = j0 + i;
-      }
+    if (!sm.abort) {
+      for (int i = tid; i < dm.kc; i += kRtThreads)
+        chunk_idx[item * dm.kc + i] = i < k_sel ? sorted[i] : -1;
     }
     __syncthreads();
   }
-  if (!sm.abort) {
-    for (int i = tid; i < dm.kc; i += kRtThreads)
-      chunk_idx[item * dm.kc + i] = i < k_sel ? sorted[i] : -1;
-  }
-  __syncthreads();
 
   // ---------------------------------------------------------------------- groups of the opened chunks
-  if (k_sel > 0 && !sm.abort) run_phase(n_ct, n_gt, true);
-  __syncwarp();
-  __syncthreads();
   if (!sm.abort) {
     int32_t* gi = group_idx + item * dm.width;
     const bool global_budget = (dm.flags & HGA_FLAG_GLOBAL_GROUP_BUDGET) != 0;

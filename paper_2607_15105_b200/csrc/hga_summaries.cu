@@ -23,7 +23,7 @@ __device__ inline uint16_t f64_to_bf16_once(double x) {
 // lane, and request up to four such row sets before the first sum: the kernel is one round trip to memory
 // deep, which is what bounds a 4 MB stream spread over the whole GPU.
 template <int D>
-__global__ void __launch_bounds__(512)
+__global__ void __launch_bounds__(256, 3)
 k_build_summaries(const uint16_t* __restrict__ K, Dims dm, int chunk_begin,
                   uint16_t* __restrict__ chunk_sum, uint16_t* __restrict__ group_sum) {
   constexpr int VEC = D / 8;                  // lanes across one row
@@ -102,13 +102,17 @@ k_build_summaries(const uint16_t* __restrict__ K, Dims dm, int chunk_begin,
 
 int launch_build_summaries(const Dims& dm, const void* K, int tok_begin, int tok_end,
                            void* chunk_sum, void* group_sum, cudaStream_t st) {
-  const int n_warps = dm.per < 16 ? dm.per : 16;
+  const int n_warps = dm.per < 8 ? dm.per : 8;
   dim3 grid((tok_end - tok_begin) / dm.c, dm.B * dm.Hkv);
   dim3 block(n_warps * 32);
   size_t smem = (size_t)n_warps * dm.d * sizeof(double);
   auto Kp = (const uint16_t*)K;
   auto cs = (uint16_t*)chunk_sum;
   auto gs = (uint16_t*)group_sum;
+  // (the shared-memory carve-out of the other kernels of the path: an SM has to drain before it changes)
+  const int rc = ensure_dynamic_smem(dm.d == 128 ? reinterpret_cast<const void*>(&k_build_summaries<128>)
+                                                 : reinterpret_cast<const void*>(&k_build_summaries<64>), smem, true);
+  if (rc) return rc;
   if (dm.d == 128)
     k_build_summaries<128><<<grid, block, smem, st>>>(Kp, dm, tok_begin / dm.c, cs, gs);
   else
