@@ -232,6 +232,8 @@ int hga_attn_fwd(const hga_params* p, const void* Q, const void* K, const void* 
   if (rc) return rc;
   if (!Q || !K || !V || (!group_idx && dm.width > 0) || !n_groups || !O || !LSE) return HGA_ERR_NULL;
   if (!aligned16(Q) || !aligned16(K) || !aligned16(V) || !aligned16(O)) return HGA_ERR_ALIGN;
+  if (attn_decode_supported(dm))
+    return launch_attn_decode(dm, Q, K, V, group_idx, n_groups, O, LSE, status_word, (cudaStream_t)stream);
   if (attn_fwd_sm100_supported(dm)) {
     rc = launch_attn_fwd_sm100(dm, nullptr, Q, K, V, group_idx, n_groups, O, LSE, status_word, (cudaStream_t)stream);
     if (rc != HGA_ERR_UNSUPPORTED) return rc;

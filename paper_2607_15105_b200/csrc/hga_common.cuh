@@ -169,6 +169,11 @@ int launch_attn_fwd_sm100(const Dims& dm, SegTable* segs, const void* Q, const v
                           const int32_t* group_idx, const int32_t* n_groups, void* O, float* LSE,
                           int32_t* status_word, cudaStream_t st);
 
+// the smallest generation shapes (warp-level matrix instructions, no tiles)
+bool attn_decode_supported(const Dims& dm);
+int launch_attn_decode(const Dims& dm, const void* Q, const void* K, const void* V, const int32_t* group_idx,
+                       const int32_t* n_groups, void* O, float* LSE, int32_t* status_word, cudaStream_t st);
+
 bool route_sm100_supported(const Dims& dm, const SegTable* segs);
 int launch_route_sm100(const Dims& dm, SegTable* segs, const void* Q, const void* chunk_sum, const void* group_sum,
                        int32_t* chunk_idx, int32_t* group_idx, int32_t* n_groups, float* chunk_scores,
