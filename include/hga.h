@@ -236,9 +236,10 @@ HGA_API int hga_step_arena_bytes(const hga_params* p, size_t* bytes);
  *   LSE fp32 [L/S,B,Hq,S]    dK, dV fp32 [L/S,B,Hkv,S,d] (segment s holds the rows of its own tokens)
  * dO == NULL runs the forward half only (dQ, dK, dV may then be NULL).  p->summary_len is
  * ignored (the summary buffers are laid out for L).  workspace: device scratch of at least
- * route_bytes + bwd_bytes as hga_workspace_bytes(p) reports them.  The forward chain of every
- * segment is queued on `stream`; the backward calls (each depends only on its own segment's forward)
- * are queued on a second stream the library creates once per device, which starts after the work
+ * route_bytes + bwd_bytes as hga_workspace_bytes(p) reports them.  With the summaries of the whole sequence built
+ * first the segments are independent, so where the tensor-core kernels take the shape every step is one launch per 64
+ * segments on `stream`; otherwise (and with HGA_FLAG_BWD_BF16_GRADS) the segments follow one another, the
+ * backward calls on a second stream the library creates once per device, which starts after the work
  * already queued on `stream` and is joined back into `stream` before the call returns, so later work
  * on `stream` sees every result.  The call itself never synchronises. */
 HGA_API int hga_tbptt_walk(const hga_params* p, const void* Q, const void* K, const void* V, const void* dO,
@@ -264,7 +265,8 @@ HGA_API int hga_tbptt_walk(const hga_params* p, const void* Q, const void* K, co
  * p gives the head counts, head_dim, chunk/group/q_block, budgets, windows, scale and flags; its
  * batch, total_len, seg_len, summary_len and strides are ignored.  dO == NULL runs the forward half
  * only.  Every sequence runs build_summaries(active range) -> route -> attn_fwd -> attn_bwd as a
- * batch-1 problem (host logic only: the kernels are the ones above).  The sequences are independent, so
+ * batch-1 problem.  The sequences are independent: where the tensor-core kernels take the shape every step is one launch per
+ * 64 sequences on `stream`; otherwise (and with HGA_FLAG_BWD_BF16_GRADS)
  * they go alternately to two streams the library creates once per device, and the kernels of two
  * sequences run side by side; both streams start behind the work already queued on `stream` and are
  * joined back into it before the call returns.  workspace: device scratch of

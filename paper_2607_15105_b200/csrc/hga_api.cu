@@ -112,6 +112,45 @@ size_t bwd_workspace_bytes(const Dims& dm) {
   return bytes;
 }
 
+// ---- several segments per launch (hga_varlen_step, hga_tbptt_walk)
+// Whether the tensor-core kernels take every step of all segments; dm describes the whole tensors.
+static bool segments_supported(const Dims& dm, const std::vector<Segment>& segs, bool bwd) {
+  if (!attn_fwd_sm100_supported(dm) || (bwd && !attn_bwd_sm100_supported(dm))) return false;
+  // bf16 gradients are summed in a workspace that holds one segment's
+  if (bwd && (dm.flags & HGA_FLAG_BWD_BF16_GRADS)) return false;
+  SegTable t;
+  for (size_t i = 0; i < segs.size(); i += kMaxSegments) {
+    t.n = (int)std::min<size_t>(kMaxSegments, segs.size() - i);
+    std::copy_n(segs.begin() + i, t.n, t.seg);
+    if (!route_sm100_supported(dm, &t)) return false;
+  }
+  return true;
+}
+
+// Routing, forward and (dO given) backward of all segments, up to kMaxSegments per launch, longest first.  *bwd_done: the
+// backward was queued too (it is not where its kernels have no room for the widest item).
+static int run_segments(const Dims& dm, std::vector<Segment> segs, bool summaries, const void* Q, const void* K, const void* V,
+                        const void* dO, void* chunk_sum, void* group_sum, int32_t* chunk_idx, int32_t* group_idx, int32_t* n_groups,
+                        void* O, float* LSE, void* dQ, float* dK, float* dV, int32_t* status_word, cudaStream_t st, bool* bwd_done) {
+  std::stable_sort(segs.begin(), segs.end(), [](const Segment& a, const Segment& b) { return a.H + a.S > b.H + b.S; });
+  *bwd_done = dO != nullptr;
+  for (size_t i = 0; i < segs.size(); i += kMaxSegments) {
+    SegTable t;
+    t.n = (int)std::min<size_t>(kMaxSegments, segs.size() - i);
+    std::copy_n(segs.begin() + i, t.n, t.seg);
+    int rc = HGA_OK;
+    if (summaries) rc = launch_build_active_summaries(dm, t, K, chunk_sum, group_sum, st);
+    if (!rc) rc = launch_route_sm100(dm, &t, Q, chunk_sum, group_sum, chunk_idx, group_idx, n_groups, nullptr, nullptr, st);
+    if (!rc) rc = launch_attn_fwd_sm100(dm, &t, Q, K, V, group_idx, n_groups, O, LSE, status_word, st);
+    if (!rc && *bwd_done) {
+      rc = launch_attn_bwd_sm100(dm, &t, Q, K, V, O, LSE, dO, group_idx, n_groups, dQ, dK, dV, status_word, st);
+      if (rc == HGA_ERR_UNSUPPORTED) { *bwd_done = false; rc = HGA_OK; }      // (returned before any launch, for the first group already)
+    }
+    if (rc) return rc;
+  }
+  return HGA_OK;
+}
+
 // Copy streams and events of hga_step_host, created once per device and kept until exit.
 struct StepPipe {
   cudaStream_t in = nullptr, out = nullptr;
@@ -273,7 +312,7 @@ int hga_attn_bwd(const hga_params* p, const void* Q, const void* K, const void* 
   bool tensor_path = false;
   if (attn_bwd_sm100_supported(dm)) {
     // its band kernel stores every row of dK/dV (or adds to it); UNSUPPORTED is returned before any launch
-    rc = launch_attn_bwd_sm100(dm, Q, K, V, O, LSE, dO, group_idx, n_groups, dQ, dK, dV, status_word, st);
+    rc = launch_attn_bwd_sm100(dm, nullptr, Q, K, V, O, LSE, dO, group_idx, n_groups, dQ, dK, dV, status_word, st);
     tensor_path = rc == HGA_OK;
   }
   if (rc == HGA_ERR_UNSUPPORTED)
@@ -441,11 +480,38 @@ int hga_tbptt_walk(const hga_params* p, const void* Q, const void* K, const void
   const size_t items = (size_t)dmf.B * dmf.Hkv * dmf.NQB;
   const size_t lse_seg = (size_t)dmf.B * dmf.Hq * S, kv_seg = (size_t)dmf.B * dmf.Hkv * S * dmf.d;
   const size_t grad_bytes = (p->flags & HGA_FLAG_BWD_BF16_GRADS) ? 2 : 4;    // element size of dK/dV
-  // The backward of segment s depends on that segment's forward only, and the forward chain of segment
-  // s+1 (summaries -> route -> forward) on nothing the backward writes: the backward calls go to a
+  cudaStream_t st = (cudaStream_t)stream;
+  // All keys are there from the start, a segment's candidates are closed chunks before it, and gradients never cross a
+  // segment boundary: with the summaries of the whole sequence built first, the segments are independent problems, and
+  // every step runs once for all of them.  (Segment by segment, each kernel of the eight of a 16K sequence ended in a
+  // partial wave; the two chains of forward and backward calls on two streams filled some of that: 1.45 ms.)
+  bool fwd_done = false;
+  {
+    hga_params pa = ps;                        // the whole sequence as one problem
+    pa.total_len = pa.seg_len = p->total_len;
+    pa.summary_len = 0;
+    Dims dm;
+    rc = resolve(&pa, dm);
+    if (rc) return rc;
+    std::vector<Segment> segs;
+    for (int s = 0; s < n_seg; ++s) segs.push_back(Segment{0, s * S, S, s * S, 0});
+    if (segments_supported(dm, segs, bwd)) {
+      if (!aligned16(Q) || !aligned16(K) || !aligned16(V) || !aligned16(O) || !aligned16(chunk_sum) || !aligned16(group_sum) ||
+          (bwd && (!aligned16(dO) || !aligned16(dQ) || !aligned16(dK) || !aligned16(dV))))
+        return HGA_ERR_ALIGN;
+      rc = launch_build_summaries(dm, K, 0, dm.L, chunk_sum, group_sum, st);
+      if (rc) return rc;
+      bool bwd_done = false;
+      rc = run_segments(dm, segs, false, Q, K, V, dO, chunk_sum, group_sum, chunk_idx, group_idx, n_groups, O, LSE, dQ, (float*)dK,
+                        (float*)dV, status_word, st, &bwd_done);
+      if (rc || bwd_done || !bwd) return rc;
+      fwd_done = true;
+    }
+  }
+  // Otherwise segment by segment.  The backward of segment s depends on that segment's forward only, and the forward chain
+  // of segment s+1 (summaries -> route -> forward) on nothing the backward writes: the backward calls go to a
   // second, library-owned stream (the one hga_step_host copies in on), so the two chains fill each
   // other's idle SMs (kernel tails, the one-wave router).  The caller's stream is joined at the end.
-  cudaStream_t st = (cudaStream_t)stream;
   StepPipe* pipe = bwd ? step_pipe(n_seg) : nullptr;
   if (bwd && !pipe) return HGA_ERR_CUDA;
   if (bwd) {
@@ -463,12 +529,14 @@ int hga_tbptt_walk(const hga_params* p, const void* Q, const void* K, const void
     int32_t* gi = group_idx + s * items * dmf.width;
     int32_t* ng = n_groups + s * items;
     float* lse = LSE + s * lse_seg;
-    rc = hga_build_summaries(&ps, K, s * S, (s + 1) * S, chunk_sum, group_sum, stream);
-    if (rc) return rc;
-    rc = hga_route(&ps, Qs, chunk_sum, group_sum, ci, gi, ng, nullptr, nullptr, workspace, route_ws, stream);
-    if (rc) return rc;
-    rc = hga_attn_fwd(&ps, Qs, K, V, gi, ng, Os, lse, status_word, stream);
-    if (rc) return rc;
+    if (!fwd_done) {
+      rc = hga_build_summaries(&ps, K, s * S, (s + 1) * S, chunk_sum, group_sum, stream);
+      if (rc) return rc;
+      rc = hga_route(&ps, Qs, chunk_sum, group_sum, ci, gi, ng, nullptr, nullptr, workspace, route_ws, stream);
+      if (rc) return rc;
+      rc = hga_attn_fwd(&ps, Qs, K, V, gi, ng, Os, lse, status_word, stream);
+      if (rc) return rc;
+    }
     if (bwd) {
       rc = record_cuda(cudaEventRecord(pipe->in_done[s], st));          // forward of segment s queued
       if (rc) return rc;
@@ -547,12 +615,39 @@ int hga_varlen_step(const hga_params* p, int32_t n_seq, const int32_t* cu_q, con
   const int per = p->chunk / p->group;
   const int kge = p->topk_groups < per ? p->topk_groups : per;
   const size_t grad_bytes = (p->flags & HGA_FLAG_BWD_BF16_GRADS) ? 2 : 4;
-  // The sequences are independent problems.  A short sequence fills only part of the GPU (its kernels are
-  // one or two CTAs per SM wide and a few waves deep at most), so the sequences go alternately to two
-  // library-owned streams ("lanes"), each with its own half of the workspace: the kernels of two sequences
-  // run side by side.  Both lanes start behind the work already queued on `stream` and are joined back into
-  // it before the call returns.
   cudaStream_t st = (cudaStream_t)stream;
+  // The sequences are independent problems: where the tensor-core kernels take them, every step runs once for all of them.
+  // (A short sequence fills only part of the GPU, and one after another, even on two streams, is mostly kernel tails.)
+  bool fwd_done = false;
+  {
+    hga_params pa = *p;                        // the packed tensors as one problem
+    pa.batch = 1;
+    pa.total_len = pa.summary_len = cu_k[n_seq];
+    pa.seg_len = cu_q[n_seq];
+    const int64_t qs[3] = {(int64_t)cu_q[n_seq] * Hq * d, d, Hq * d}, ks[3] = {(int64_t)cu_k[n_seq] * Hkv * d, d, Hkv * d};
+    for (int a = 0; a < 3; ++a) { pa.q_stride[a] = pa.o_stride[a] = qs[a]; pa.k_stride[a] = pa.v_stride[a] = ks[a]; }
+    Dims dm;
+    rc = resolve(&pa, dm);
+    if (rc) return rc;
+    std::vector<Segment> segs;
+    for (int i = 0; i < n_seq; ++i) {
+      const int S = cu_q[i + 1] - cu_q[i], L = cu_k[i + 1] - cu_k[i];
+      segs.push_back(Segment{0, L - S, S, cu_q[i], cu_k[i]});
+    }
+    if (segments_supported(dm, segs, bwd)) {
+      if (!aligned16(Q) || !aligned16(K) || !aligned16(V) || !aligned16(O) || !aligned16(chunk_sum) || !aligned16(group_sum) ||
+          (bwd && (!aligned16(dO) || !aligned16(dQ) || !aligned16(dK) || !aligned16(dV))))
+        return HGA_ERR_ALIGN;
+      bool bwd_done = false;
+      rc = run_segments(dm, segs, true, Q, K, V, dO, chunk_sum, group_sum, chunk_idx, group_idx, n_groups, O, LSE, dQ, (float*)dK,
+                        (float*)dV, status_word, st, &bwd_done);
+      if (rc || bwd_done || !bwd) return rc;
+      fwd_done = true;
+    }
+  }
+  // Otherwise one sequence after another, alternately on two library-owned streams ("lanes"), each with its own half of the
+  // workspace, so that the kernels of two sequences run side by side.  Both lanes start behind the work already
+  // queued on `stream` and are joined back into it before the call returns.
   StepPipe* pipe = n_seq > 1 ? step_pipe(1) : nullptr;
   if (n_seq > 1 && !pipe) return HGA_ERR_CUDA;
   cudaStream_t lanes[2] = {pipe ? pipe->in : st, pipe ? pipe->out : st};
@@ -586,12 +681,14 @@ int hga_varlen_step(const hga_params* p, int32_t n_seq, const int32_t* cu_q, con
     int32_t* ng = n_groups + item0;
     float* lse = LSE + Hq * q0;
     const size_t route_ws = route_workspace_bytes(dm), bwd_ws = bwd_workspace_bytes(dm);
-    rc = hga_build_summaries(&ps, Ki, dm.H, dm.L, csi, gsi, lane_stream);
-    if (rc) return rc;
-    rc = hga_route(&ps, Qi, csi, gsi, ci, gi, ng, nullptr, nullptr, ws, route_ws, lane_stream);
-    if (rc) return rc;
-    rc = hga_attn_fwd(&ps, Qi, Ki, Vi, gi, ng, Oi, lse, status_word, lane_stream);
-    if (rc) return rc;
+    if (!fwd_done) {
+      rc = hga_build_summaries(&ps, Ki, dm.H, dm.L, csi, gsi, lane_stream);
+      if (rc) return rc;
+      rc = hga_route(&ps, Qi, csi, gsi, ci, gi, ng, nullptr, nullptr, ws, route_ws, lane_stream);
+      if (rc) return rc;
+      rc = hga_attn_fwd(&ps, Qi, Ki, Vi, gi, ng, Oi, lse, status_word, lane_stream);
+      if (rc) return rc;
+    }
     if (bwd) {
       rc = hga_attn_bwd(&ps, Qi, Ki, Vi, Oi, lse, (const char*)dO + q0 * Hq * d * 2, gi, ng,
                         (char*)dQ + q0 * Hq * d * 2, (char*)dK + Hkv * d * q0 * grad_bytes,

@@ -76,12 +76,12 @@ struct HalfStep {
 
 }  // namespace
 
-template <int D>
+template <int D, class Segs>
 __global__ void __launch_bounds__(kBandThreads, 1)
 k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_do,
                       const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
-                      const __grid_constant__ CUtensorMap map_o, const float* __restrict__ LSE, Dims dm,
-                      float* __restrict__ dK, float* __restrict__ dV, int32_t* status_word) {
+                      const __grid_constant__ CUtensorMap map_o, const float* __restrict__ LSE, const Dims dm,
+                      float* __restrict__ dK, float* __restrict__ dV, int32_t* status_word, const __grid_constant__ Segs segs) {
   constexpr uint32_t kColS = 0, kColDP = 64, kRegion = 128, kColDV = 256, kColDK = 384;   // (S^T, dP^T: inside a region)
   constexpr int kD = D, kPanels = D / 64, kTile = BandSmem<D>::kTile;
   constexpr int kHalfBoxes = 2 * kPanels;          // boxes (64 rows x 64 elements) of one half-step's Q and dO, or of one 128-row tile
@@ -90,17 +90,19 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   HGA_TRACE_DECL(448);
-  const int tiles_per_seq = (dm.S + kKeys - 1) / kKeys;
-  const int kt = blockIdx.x % tiles_per_seq;
-  const int bh = blockIdx.x / tiles_per_seq;
+  int cta;
+  const Segment sg = segment_of(dm, segs, blockIdx.x, cta);
+  const int tiles_per_seq = (sg.S + kKeys - 1) / kKeys;
+  const int kt = cta % tiles_per_seq;
+  const int bh = cta / tiles_per_seq;
   const int h = bh % dm.Hkv, b = bh / dm.Hkv;
-  const int k0 = dm.H + kt * kKeys;               // first key position of the tile
-  const int k_end = min(k0 + kKeys, dm.L);        // one past its last real key
+  const int k0 = sg.H + kt * kKeys;               // first key position of the tile
+  const int k_end = min(k0 + kKeys, sg.H + sg.S);        // one past its last real key
   // query blocks whose band [ls, p0 + Bq) touches the tile: from the block that holds the tile's first
   // key, while the local window still starts before the tile's end
   const int qb_first = (kt * kKeys) / dm.Bq;
   int n_qb = 1;
-  while (qb_first + n_qb < dm.NQB && window_of(dm, qb_first + n_qb).ls < k_end) ++n_qb;
+  while (qb_first + n_qb < sg.S / dm.Bq && window_at(dm, sg.H + (qb_first + n_qb) * dm.Bq).ls < k_end) ++n_qb;
   const int n_hq = dm.rows / 64;                  // half-steps of a query block
   const int n_steps = (n_qb * n_hq + 1) / 2;
   const int qb_last = qb_first + n_qb - 1;
@@ -131,8 +133,9 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
+  pdl_wait();
   // the sweep, next in the stream, may start on SMs this grid leaves idle (it waits for this grid only
-  // before it adds to dK/dV)
+  // before it adds to dK/dV; what it reads earlier was complete when this grid's wait returned)
   if (tid == 0) pdl_launch_dependents();
 
   const uint32_t tmem = sm.tmem_base;
@@ -145,13 +148,13 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
   // second half-step's, the first O tile, then the second step's Q and dO.
   auto coords = [&](HalfStep hs, int& row, int& head) {
     const bool real = hs.r0 < dm.rows;
-    row = real ? hs.qb * dm.Bq + hs.t : dm.S;                // (padding: out of range, zeros)
+    row = real ? sg.q0 + hs.qb * dm.Bq + hs.t : dm.rows_q;                // (padding: out of range, zeros)
     head = h * dm.G + (real ? hs.head : 0);
   };
   // box i of a tile of 128 rows: (half, panel); box i of a half-step's Q and dO: (panel, Q or dO)
   auto copy_kv = [&](uint8_t* dst, const CUtensorMap* map, int i) {
     const int half = i & 1, panel = i >> 1;
-    tma_load_5d(dst + panel * 16384 + half * 8192, map, &sm.kv_full, 0, k0 + 64 * half, panel, h, b);
+    tma_load_5d(dst + panel * 16384 + half * 8192, map, &sm.kv_full, 0, sg.k0 + k0 + 64 * half, panel, h, b);
   };
   auto copy_qdo = [&](HalfStep hs, int st, int half, int i) {
     const int panel = i % kPanels, is_do = i / kPanels;
@@ -302,7 +305,7 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
     HalfStep sp = first[0];
     for (int hs = 0; hs < 2 * n_steps; ++hs) {
       const int m = hs >> 1, hf = hs & 1;
-      const Window w = window_of(dm, sp.qb);
+      const Window w = window_at(dm, sg.H + sp.qb * dm.Bq);
       // the warpgroup's 32 columns are 32 consecutive positions of one query head (Bq is a multiple of 64);
       // column i is visible to this key iff the key is inside the block's band and not after the query
       const int r_first = 64 * hf + 32 * wg;         // first of those rows inside the M-tile
@@ -394,7 +397,7 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
       constexpr uint32_t kRowPitch = kD * 4 + 16;
       static_assert(2 * 128 * kRowPitch <= 5 * kTile, "staging area: q, dO and o tiles");
       const int srow = kt * kKeys + key;
-      float* dst = (wg == 0 ? dV : dK) + ((int64_t)(b * dm.Hkv + h) * dm.S + srow) * kD;
+      float* dst = (wg == 0 ? dV : dK) + (row_base(dm, sg, b) * dm.Hkv + (int64_t)h * sg.S + srow) * kD;
       const uint32_t col = wg == 0 ? kColDV : kColDK;
       const uint32_t stage = smem_u32(sm.q[0]) + (uint32_t)(wg * 128 + key) * kRowPitch;
 #pragma unroll
@@ -406,7 +409,7 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
         for (int i = 0; i < 8; ++i) st_shared_v4(stage + (uint32_t)(32 * c + 4 * i) * 4, x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3]);
       }
       fence_proxy_async_smem();
-      if (srow < dm.S) {
+      if (srow < sg.S) {
         if (dm.flags & HGA_FLAG_BWD_ACCUMULATE) bulk_reduce_add_f32(dst, stage, kD * 4);
         else bulk_store(dst, stage, kD * 4);
         tma_store_commit();
@@ -420,7 +423,7 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
     HalfStep h0 = first[0], h1 = first[1];           // the two half-steps of the M-tile whose LSE (and O tile) comes next
     auto next_lse = [&]() {
       const HalfStep& hs = j < 64 ? h0 : h1;
-      return hs.r0 < dm.rows ? LSE[((int64_t)b * dm.Hq + h * dm.G + hs.head) * dm.S + hs.qb * dm.Bq + hs.t + (j & 63)] : 0.f;
+      return hs.r0 < dm.rows ? LSE[row_base(dm, sg, b) * dm.Hq + (int64_t)(h * dm.G + hs.head) * sg.S + hs.qb * dm.Bq + hs.t + (j & 63)] : 0.f;
     };
     float lse_next = next_lse();
     bool ok = true;
@@ -504,13 +507,13 @@ bool attn_bwd_band_sm100_supported(const Dims& dm) {
   return dm.d == 128 || dm.d == 64;
 }
 
-template <int D>
-static int launch_band(const Dims& dm, const void* Q, const void* K, const void* V, const void* O,
+template <int D, class Segs>
+static int launch_band(const Dims& dm, const Segs& segs, int64_t units, const void* Q, const void* K, const void* V, const void* O,
                        const float* LSE, const void* dO, float* dK, float* dV, int32_t* status_word, cudaStream_t st) {
   CUtensorMap mq, mdo, mk, mv, mo;
   const uint32_t box[5] = {64, 64, 1, 1, 1};
-  const uint64_t dq[5] = {64, (uint64_t)dm.S, (uint64_t)(D / 64), (uint64_t)dm.Hq, (uint64_t)dm.B};
-  const uint64_t dk[5] = {64, (uint64_t)dm.L, (uint64_t)(D / 64), (uint64_t)dm.Hkv, (uint64_t)dm.B};
+  const uint64_t dq[5] = {64, (uint64_t)dm.rows_q, (uint64_t)(D / 64), (uint64_t)dm.Hq, (uint64_t)dm.B};
+  const uint64_t dk[5] = {64, (uint64_t)dm.rows_k, (uint64_t)(D / 64), (uint64_t)dm.Hkv, (uint64_t)dm.B};
   const uint64_t sq[4] = {(uint64_t)dm.qs[2] * 2, 128, (uint64_t)dm.qs[1] * 2, (uint64_t)dm.qs[0] * 2};
   const uint64_t so[4] = {(uint64_t)dm.os[2] * 2, 128, (uint64_t)dm.os[1] * 2, (uint64_t)dm.os[0] * 2};
   const uint64_t sk[4] = {(uint64_t)dm.ks[2] * 2, 128, (uint64_t)dm.ks[1] * 2, (uint64_t)dm.ks[0] * 2};
@@ -522,19 +525,24 @@ static int launch_band(const Dims& dm, const void* Q, const void* K, const void*
       encode_tensor_map_bf16(&mv, V, 5, dk, sv, box, true))
     return HGA_ERR_UNSUPPORTED;
   const size_t smem = sizeof(BandSmem<D>) + 1024;
-  const int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(&k_attn_bwd_band_sm100<D>), smem);
+  const int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(&k_attn_bwd_band_sm100<D, Segs>), smem);
   if (rc) return rc;
-  const int units = dm.B * dm.Hkv * ((dm.S + kKeys - 1) / kKeys);
-  k_attn_bwd_band_sm100<D><<<units, kBandThreads, smem, st>>>(mq, mdo, mk, mv, mo, LSE, dm, dK, dV, status_word);
+  PdlLaunch cfg((unsigned)units, kBandThreads, smem, st, dm.flags);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg.c, k_attn_bwd_band_sm100<D, Segs>, mq, mdo, mk, mv, mo, LSE, dm, dK, dV, status_word, segs);
   count_launch(HGA_KERNELS_BWD_TENSOR);
-  return record_cuda(cudaGetLastError());
+  return record_cuda(e);
 }
 
-int launch_attn_bwd_band_sm100(const Dims& dm, const void* Q, const void* K, const void* V, const void* O,
+int launch_attn_bwd_band_sm100(const Dims& dm, SegTable* segs, const void* Q, const void* K, const void* V, const void* O,
                                const float* LSE, const void* dO, float* dK, float* dV, int32_t* status_word,
                                cudaStream_t st) {
-  return dm.d == 128 ? launch_band<128>(dm, Q, K, V, O, LSE, dO, dK, dV, status_word, st)
-                     : launch_band<64>(dm, Q, K, V, O, LSE, dO, dK, dV, status_word, st);
+  auto tiles = [&](int S) { return (int64_t)dm.B * dm.Hkv * ((S + kKeys - 1) / kKeys); };
+  if (!segs)
+    return dm.d == 128 ? launch_band<128>(dm, OneSegment{}, tiles(dm.S), Q, K, V, O, LSE, dO, dK, dV, status_word, st)
+                       : launch_band<64>(dm, OneSegment{}, tiles(dm.S), Q, K, V, O, LSE, dO, dK, dV, status_word, st);
+  const int64_t units = number_units(*segs, [&](const Segment& g) { return tiles(g.S); });
+  return dm.d == 128 ? launch_band<128>(dm, *segs, units, Q, K, V, O, LSE, dO, dK, dV, status_word, st)
+                     : launch_band<64>(dm, *segs, units, Q, K, V, O, LSE, dO, dK, dV, status_word, st);
 }
 
 }  // namespace hga

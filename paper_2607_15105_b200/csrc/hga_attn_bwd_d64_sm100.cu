@@ -71,13 +71,14 @@ static_assert(sizeof(SweepSmem) + 1024 <= 113 * 1024, "two CTAs per SM");
 
 }  // namespace
 
+template <class Segs>
 __global__ void __launch_bounds__(kThreads, 2)
 k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_do,
                  const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                  const __grid_constant__ CUtensorMap map_dq, const uint16_t* __restrict__ O,
                  const float* __restrict__ LSE, const int32_t* __restrict__ group_idx,
-                 const int32_t* __restrict__ n_groups, Dims dm,
-                 float* __restrict__ dK, float* __restrict__ dV, int32_t* status_word) {
+                 const int32_t* __restrict__ n_groups, const Dims dm,
+                 float* __restrict__ dK, float* __restrict__ dV, int32_t* status_word, const __grid_constant__ Segs segs) {
   constexpr uint32_t kColS = 0, kColDP = 64, kColDQ = 128;
   extern __shared__ uint8_t smem_raw[];
   SweepSmem& sm = *reinterpret_cast<SweepSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -87,12 +88,13 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
   const int n_mt_item = (dm.rows + 127) / 128;
   // Launch order: late query blocks first.  They have the most routed keys inside the active segment (the
   // expensive dK/dV tiles), early ones none, so the cheapest CTAs are the ones that fill the last wave.
-  const int unit = blockIdx.x / n_mt_item, n_bh = dm.B * dm.Hkv;
-  const int item = (unit % n_bh) * dm.NQB + (dm.NQB - 1 - unit / n_bh);
-  const int mt = blockIdx.x % n_mt_item;
-  int b, h, qb;
-  item_coords(dm, item, b, h, qb);
-  const Window w = window_of(dm, qb);
+  int cta;
+  const Segment sg = segment_of(dm, segs, blockIdx.x, cta);
+  const int unit = cta / n_mt_item, n_bh = dm.B * dm.Hkv, mt = cta % n_mt_item;
+  const int qb = sg.S / dm.Bq - 1 - unit / n_bh, b = unit % n_bh / dm.Hkv, h = unit % n_bh % dm.Hkv;
+  const int64_t item = item_base(dm, sg, b) + h * (sg.S / dm.Bq) + qb;
+  const int qrow = sg.q0 + qb * dm.Bq;                  // the block's first row in Q, O, dO and dQ
+  const Window w = window_at(dm, sg.H + qb * dm.Bq);
   const int n_local = w.p0 + dm.Bq - w.ls;              // tokens of the local window and the block (a multiple of 8)
   const int n_lt = (n_local + kKT - 1) / kKT;           // its tiles
   volatile int* abort = &sm.abort;
@@ -106,8 +108,8 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
 #pragma unroll
     for (int i = 0; i < D / 8; ++i) o_row[i] = make_uint4(0, 0, 0, 0);
     if (r < dm.rows) {
-      const int hq = h * dm.G + r / dm.Bq, srow = qb * dm.Bq + r % dm.Bq;
-      row_lse = LSE[((int64_t)b * dm.Hq + hq) * dm.S + srow];
+      const int hq = h * dm.G + r / dm.Bq, srow = qrow + r % dm.Bq;
+      row_lse = LSE[row_base(dm, sg, b) * dm.Hq + (int64_t)hq * sg.S + (srow - sg.q0)];
       const uint4* op = reinterpret_cast<const uint4*>(O + b * dm.os[0] + hq * dm.os[1] + (int64_t)srow * dm.os[2]);
 #pragma unroll
       for (int i = 0; i < D / 8; ++i) o_row[i] = __ldg(op + i);
@@ -117,7 +119,7 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
   const int half = warp == 7 ? 1 : 0;
   auto local_row = [&](int j) {
     const int off = kKT * j + 8 * (4 * half + lane);
-    return off < n_local ? w.ls + off : dm.L;
+    return off < n_local ? sg.k0 + w.ls + off : dm.rows_k;
   };
   auto copy_tile = [&](uint8_t* dst, const CUtensorMap* map, uint64_t* full, int row) {
     if (lane == 0) mbar_arrive_expect_tx(full, 4 * kOct);
@@ -151,7 +153,7 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
         const int r = mt * 128 + 64 * hf;
         const bool real = r < dm.rows;
         tma_load_5d((is_do ? sm.dO : sm.q) + hf * 8192, is_do ? &map_do : &map_q, &sm.q_full, 0,
-                    real ? qb * dm.Bq + r % dm.Bq : dm.S, 0, h * dm.G + (real ? r / dm.Bq : 0), b);
+                    real ? qrow + r % dm.Bq : dm.rows_q, 0, h * dm.G + (real ? r / dm.Bq : 0), b);
       }
     } else {
       const int row = local_row(0);
@@ -163,8 +165,8 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
   if (warp == 1) {
     tmem_alloc(&sm.tmem_base, 256);
     tmem_relinquish();
-    // with bf16 outputs the conversion kernel follows this grid: let its launch overlap this grid's tail
-    if (lane == 0 && (dm.flags & HGA_FLAG_BWD_BF16_GRADS)) pdl_launch_dependents();
+    // the next kernel's launch may overlap this grid's tail (the conversion of bf16 outputs, the next step's summaries)
+    if (lane == 0) pdl_launch_dependents();
   }
   __syncwarp();
   tc_fence_before_sync();
@@ -182,7 +184,7 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
   if (warp == 0 || warp == 7) {
     // ------------------------------------------------------------------ producers
     bool ok = true;
-    FarList far(dm, w, group_idx + (int64_t)item * dm.width);
+    FarList far(dm, w, group_idx + item * dm.width);
     int n = 0, n_a = 0;
     bool known = false;                                   // the list has been checked (warp 6) and its counts read
     auto learn = [&]() {
@@ -197,7 +199,7 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
     auto row_of = [&](int j) {
       if (j < n_lt) return local_row(j);
       const int o = 8 * (j - n_lt) + 4 * half + (lane & 3);
-      return o < far.n_far ? far.row(o) : dm.L;
+      return o < far.n_far ? sg.k0 + far.row(o) : dm.rows_k;
     };
     auto wait_for = [&](uint64_t* bar, uint32_t parity) {
       if (lane == 0) ok = bwd_wait(bar, parity, abort);
@@ -211,7 +213,7 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
     // Rows of the next two tiles, looked up ahead of their use.  Tile j + 1's K has been issued when tile j is
     // handled, except behind a dK/dV tile.
     if (n_lt < 3) learn();
-    int next_row = ok ? row_of(1) : dm.L, after_row = ok ? row_of(2) : dm.L;
+    int next_row = ok ? row_of(1) : dm.rows_k, after_row = ok ? row_of(2) : dm.rows_k;
     if (ok && (n_lt > 1 || n > 1)) copy_k(1, next_row);
     // The events this loop waits for come in this order: dP(j) done, dQ(j) done, dP(j+1) done, ...
     for (int j = 0; ok; ++j) {
@@ -357,12 +359,13 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
     if (ok) mma_commit_w(&sm.dq_done);
   } else if (warp == 6) {
     // ------------------------------------------------------------------ routing list
-    FarList far(dm, w, group_idx + (int64_t)item * dm.width);
-    far.check(dm, n_groups + item, dm.H);      // (the forward call reports invalid lists)
+    FarList far(dm, w, group_idx + item * dm.width);
+    far.check(dm, n_groups + item, sg.H);      // (the forward call reports invalid lists)
     if (lane == 0) {
       sm.n_listed = far.ng; sm.n_far = far.n_far; sm.first_active = far.first_active; sm.clean = far.clean;
       mbar_arrive(&sm.info_full);
     }
+    pdl_wait();      // (the end of this grid has to imply the end of the band kernel's, even where there is nothing to add)
   } else if (warp < 6) {
     // ------------------------------------------------------------------ one thread per query row
     const int quarter = warp & 3;
@@ -503,8 +506,8 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
       auto reduce_rows = [&](float* dst, uint8_t* buf, int hf, uint32_t off) {
         const int o = 8 * (j - n_lt) + 4 * hf + (lane >> 3);
         if (o >= sm.first_active && o < sm.n_far) {
-          const int pos = sm.rows[j & 3][4 * hf + (lane >> 3)] + (lane & 7);
-          bulk_reduce_add_f32(dst + ((int64_t)(b * dm.Hkv + h) * dm.S + (pos - dm.H)) * D, smem_u32(buf) + (uint32_t)lane * 512 + off, D * 4);
+          const int row = sm.rows[j & 3][4 * hf + (lane >> 3)] + (lane & 7) - sg.k0 - sg.H;      // inside the active segment
+          bulk_reduce_add_f32(dst + (row_base(dm, sg, b) * dm.Hkv + (int64_t)h * sg.S + row) * D, smem_u32(buf) + (uint32_t)lane * 512 + off, D * 4);
         }
         tma_store_commit();
       };
@@ -556,7 +559,7 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
       if (warp == 2 && lane < 2 && bwd_wait(&sm.dq_staged, 0, abort)) {      // all 128 rows are in shared memory
         const int r0 = mt * 128 + 64 * lane;
         if (r0 < dm.rows) {
-          tma_store_5d(&map_dq, sm.q + lane * 8192, 0, qb * dm.Bq + r0 % dm.Bq, 0, h * dm.G + r0 / dm.Bq, b);
+          tma_store_5d(&map_dq, sm.q + lane * 8192, 0, qrow + r0 % dm.Bq, 0, h * dm.G + r0 / dm.Bq, b);
           tma_store_commit();
           tma_store_wait_read();      // (the source tile has been read; the writes complete before the grid does)
         }
@@ -583,14 +586,15 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
   if (warp == 1) tmem_dealloc(tmem, 256);
 }
 
-int launch_attn_bwd_d64_sm100(const Dims& dm, const void* Q, const void* K, const void* V, const void* O, const float* LSE,
+template <class Segs>
+static int launch_sweep64(const Dims& dm, SegTable* table, const Segs& segs, int64_t units, const void* Q, const void* K, const void* V, const void* O, const float* LSE,
                               const void* dO, const int32_t* group_idx, const int32_t* n_groups, void* dQ, float* dK,
                               float* dV, int32_t* status_word, cudaStream_t st) {
   CUtensorMap mq, mdo, mk, mv, mdq;
   const uint32_t box[5] = {64, 8, 1, 1, 1};
   const uint32_t box_q[5] = {64, 64, 1, 1, 1};
-  const uint64_t dq[5] = {64, (uint64_t)dm.S, 1, (uint64_t)dm.Hq, (uint64_t)dm.B};
-  const uint64_t dk[5] = {64, (uint64_t)dm.L, 1, (uint64_t)dm.Hkv, (uint64_t)dm.B};
+  const uint64_t dq[5] = {64, (uint64_t)dm.rows_q, 1, (uint64_t)dm.Hq, (uint64_t)dm.B};
+  const uint64_t dk[5] = {64, (uint64_t)dm.rows_k, 1, (uint64_t)dm.Hkv, (uint64_t)dm.B};
   const uint64_t sq[4] = {(uint64_t)dm.qs[2] * 2, 128, (uint64_t)dm.qs[1] * 2, (uint64_t)dm.qs[0] * 2};
   const uint64_t so[4] = {(uint64_t)dm.os[2] * 2, 128, (uint64_t)dm.os[1] * 2, (uint64_t)dm.os[0] * 2};
   const uint64_t sk[4] = {(uint64_t)dm.ks[2] * 2, 128, (uint64_t)dm.ks[1] * 2, (uint64_t)dm.ks[0] * 2};
@@ -603,27 +607,28 @@ int launch_attn_bwd_d64_sm100(const Dims& dm, const void* Q, const void* K, cons
     return HGA_ERR_UNSUPPORTED;
   const size_t smem = sizeof(SweepSmem) + 1024;
   // two CTAs per SM need the largest shared-memory carve-out
-  int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(&k_attn_bwd_d64_sm100), smem, true);
+  int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(&k_attn_bwd_d64_sm100<Segs>), smem, true);
   if (rc) return rc;
   // dK/dV of the local band first: plain stores that cover every row of the active segment; this kernel then adds
   // the contributions of the keys before the band.  Launched with programmatic serialization behind the band kernel: it
   // waits for it only before the first add.
-  rc = launch_attn_bwd_band_sm100(dm, Q, K, V, O, LSE, dO, dK, dV, status_word, st);
+  rc = launch_attn_bwd_band_sm100(dm, table, Q, K, V, O, LSE, dO, dK, dV, status_word, st);
   if (rc != HGA_OK) return rc;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(dm.B * dm.Hkv * dm.NQB * ((dm.rows + 127) / 128)));
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = (dm.flags & kFlagNoPdl) ? 0 : 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_attn_bwd_d64_sm100, mq, mdo, mk, mv, mdq, (const uint16_t*)O, LSE,
-                                           group_idx, n_groups, dm, dK, dV, status_word);
+  if (table) units = number_units(*table, [&](const Segment& g) { return (int64_t)dm.B * dm.Hkv * (g.S / dm.Bq) * ((dm.rows + 127) / 128); });
+  PdlLaunch cfg((unsigned)units, kThreads, smem, st, dm.flags);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg.c, k_attn_bwd_d64_sm100<Segs>, mq, mdo, mk, mv, mdq, (const uint16_t*)O, LSE,
+                                           group_idx, n_groups, dm, dK, dV, status_word, segs);
   count_launch(HGA_KERNELS_BWD_TENSOR);
   return record_cuda(e);
+}
+
+int launch_attn_bwd_d64_sm100(const Dims& dm, SegTable* segs, const void* Q, const void* K, const void* V, const void* O, const float* LSE,
+                              const void* dO, const int32_t* group_idx, const int32_t* n_groups, void* dQ, float* dK,
+                              float* dV, int32_t* status_word, cudaStream_t st) {
+  const int64_t units = (int64_t)dm.B * dm.Hkv * dm.NQB * ((dm.rows + 127) / 128);
+  if (!segs)
+    return launch_sweep64(dm, nullptr, OneSegment{}, units, Q, K, V, O, LSE, dO, group_idx, n_groups, dQ, dK, dV, status_word, st);
+  return launch_sweep64(dm, segs, *segs, units, Q, K, V, O, LSE, dO, group_idx, n_groups, dQ, dK, dV, status_word, st);
 }
 
 }  // namespace hga

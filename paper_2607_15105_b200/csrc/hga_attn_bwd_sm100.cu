@@ -85,13 +85,14 @@ struct BwdSmem {
 static_assert(kPdsTile == kKvTile && offsetof(BwdSmem, ds) == offsetof(BwdSmem, p) + kKvTile,
               "the P and dS tiles double as one pair of V stages");
 
+template <class Segs>
 __global__ void __launch_bounds__(kBwdThreads, 1)
 k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_do,
                  const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                  const __grid_constant__ CUtensorMap map_dq, const uint16_t* __restrict__ O,
                  const float* __restrict__ LSE, const int32_t* __restrict__ group_idx,
-                 const int32_t* __restrict__ n_groups, Dims dm,
-                 float* __restrict__ dK, float* __restrict__ dV, int32_t* status_word) {
+                 const int32_t* __restrict__ n_groups, const Dims dm,
+                 float* __restrict__ dK, float* __restrict__ dV, int32_t* status_word, const __grid_constant__ Segs segs) {
   constexpr int D = kBwdD;
   // TMEM columns.  Regions 0, 1, 2 rotate through the roles S / dP+dS of the paired steps; a dK/dV
   // step keeps S (64 columns) and dP (64) in region 0 and dV^T, dK^T in region 1.
@@ -107,12 +108,13 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   const int n_mt_item = (dm.rows + 127) / 128;           // (the last M-tile may hold 64 rows only)
   // Launch order: late query blocks first.  They have the most routed keys inside the active segment (the
   // expensive dK/dV steps), early ones none, so the cheapest CTAs are the ones that fill the last wave.
-  const int unit = blockIdx.x / n_mt_item, n_bh = dm.B * dm.Hkv;
-  const int item = (unit % n_bh) * dm.NQB + (dm.NQB - 1 - unit / n_bh);
-  const int mt = blockIdx.x % n_mt_item;
-  int b, h, qb;
-  item_coords(dm, item, b, h, qb);
-  const Window w = window_of(dm, qb);
+  int cta;
+  const Segment sg = segment_of(dm, segs, blockIdx.x, cta);
+  const int unit = cta / n_mt_item, n_bh = dm.B * dm.Hkv, mt = cta % n_mt_item;
+  const int qb = sg.S / dm.Bq - 1 - unit / n_bh, b = unit % n_bh / dm.Hkv, h = unit % n_bh % dm.Hkv;
+  const int64_t item = item_base(dm, sg, b) + h * (sg.S / dm.Bq) + qb;
+  const int qrow = sg.q0 + qb * dm.Bq;                   // the block's first row in Q, O, dO and dQ
+  const Window w = window_at(dm, sg.H + qb * dm.Bq);
 
   if (tid == 0) {
     mbar_init(&sm.q_full, 1);
@@ -146,7 +148,7 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       const bool real = r < dm.rows;                     // (rows past the item's last one arrive as zeros)
       const int a = real ? r / dm.Bq : 0, t = r % dm.Bq;
       const uint32_t off = (uint32_t)panel * 16384 + (uint32_t)half * 8192;
-      const int row = real ? qb * dm.Bq + t : dm.S;
+      const int row = real ? qrow + t : dm.rows_q;
       if (warp < 4) tma_load_5d(sm.q + off, &map_q, &sm.q_full, 0, row, panel, h * dm.G + a, b);
       else tma_load_5d(sm.dO + off, &map_do, &sm.q_full, 0, row, panel, h * dm.G + a, b);
     }
@@ -155,13 +157,13 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   if (warp == 1) {
     tmem_alloc(&sm.tmem_base, 512);
     tmem_relinquish();
-    // with bf16 outputs the conversion kernel follows this grid: let its launch overlap this grid's tail
-    if (lane == 0 && (dm.flags & HGA_FLAG_BWD_BF16_GRADS)) pdl_launch_dependents();
+    // the next kernel's launch may overlap this grid's tail (the conversion of bf16 outputs, the next step's summaries)
+    if (lane == 0) pdl_launch_dependents();
   }
   if (warp == 0) {
     if (lane == 0) { prefetch_tensormap(&map_k); prefetch_tensormap(&map_v); }
     bool bad;   // invalid entries are skipped exactly as in the forward kernel (which reports them)
-    const int n_oct = build_octet_table(dm, w, group_idx + (int64_t)item * dm.width, n_groups + item, sm.oct_row, &bad);
+    const int n_oct = build_octet_table(dm, w, group_idx + item * dm.width, n_groups + item, sm.oct_row, &bad);
     // Keys that receive dK/dV from this kernel: positions in [H, hi), where hi is the start of the
     // local band (the key-major band kernel has written that part).
     // Rows ascend, so these octets are a contiguous range [oa, ob) of the list.
@@ -169,7 +171,7 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     int below_h = 0, below_hi = 0;
     for (int o = lane; o < n_oct; o += 32) {
       const int row = sm.oct_row[o];
-      below_h += row + 8 <= dm.H;
+      below_h += row + 8 <= sg.H;
       below_hi += row < hi;
     }
 #pragma unroll
@@ -191,8 +193,8 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   uint4 o_half[8];
   if (warp >= 2 && warp < 10) {
     const int r_own = mt * 128 + (warp & 3) * 32 + lane, r = min(r_own, dm.rows - 1);
-    const int hq = h * dm.G + r / dm.Bq, srow = qb * dm.Bq + r % dm.Bq;
-    row_lse = r_own < dm.rows ? LSE[((int64_t)b * dm.Hq + hq) * dm.S + srow] : INFINITY;   // (padding rows: P = 0)
+    const int hq = h * dm.G + r / dm.Bq, srow = qrow + r % dm.Bq;
+    row_lse = r_own < dm.rows ? LSE[row_base(dm, sg, b) * dm.Hq + (int64_t)hq * sg.S + (srow - sg.q0)] : INFINITY;   // (padding rows: P = 0)
     const uint4* op = reinterpret_cast<const uint4*>(O + b * dm.os[0] + hq * dm.os[1] + (int64_t)srow * dm.os[2]) +
                       8 * ((warp - 2) >> 2);
 #pragma unroll
@@ -243,9 +245,9 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       for (int step = 0; step < n_act && ok; ++step) {
         const int slot = 2 * step + (is_v ? 1 : 0);
         const int st = slot % kBwdKStages;
-        int row = dm.L;                                      // past the list: zeros
+        int row = dm.rows_k;                                 // past the list: zeros
         const int o = 8 * tile_of_step(step) + oct_in_tile;
-        if (o < n_oct) row = sm.oct_row[o];
+        if (o < n_oct) row = sg.k0 + sm.oct_row[o];
         if (lane == 0 && slot >= kBwdKStages) ok = bwd_wait(&sm.k_empty[st], (uint32_t)(slot / kBwdKStages - 1) & 1, abort);
         ok = __shfl_sync(0xffffffffu, ok, 0);
         if (!ok) break;
@@ -270,10 +272,10 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         const int ps = is_v ? (p & 1) : (n_act_even / 2 + p) % n_ps;
         uint64_t* full = is_v ? &sm.vp_full[ps] : &sm.kp_full[ps];
         const int s = n_act + 2 * p + which;                              // step (tile order)
-        int row = dm.L;
+        int row = dm.rows_k;
         if (s < n_tiles) {
           const int o = 8 * tile_of_step(s) + oct_in_tile;
-          if (o < n_oct) row = sm.oct_row[o];
+          if (o < n_oct) row = sg.k0 + sm.oct_row[o];
         }
         if (lane == 0) {
           if (is_v) {
@@ -630,7 +632,7 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         const int half = lane & 1, panel = lane >> 1;
         const int r0 = mt * 128 + 64 * half;
         if (r0 < dm.rows) {
-          tma_store_5d(&map_dq, sm.q + panel * 16384 + half * 8192, 0, qb * dm.Bq + r0 % dm.Bq, panel,
+          tma_store_5d(&map_dq, sm.q + panel * 16384 + half * 8192, 0, qrow + r0 % dm.Bq, panel,
                        h * dm.G + r0 / dm.Bq, b);
           tma_store_commit();
           tma_store_wait_read();    // (the source tile has been read; the writes complete before the grid does)
@@ -642,13 +644,15 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     const int quarter = warp & 3;
     const int e = quarter * 32 + lane;                       // head_dim element = TMEM lane
     const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
-    float* dKb = dK + ((int64_t)(b * dm.Hkv + h) * dm.S) * D + e;
-    float* dVb = dV + ((int64_t)(b * dm.Hkv + h) * dm.S) * D + e;
+    const int64_t kv_base = (row_base(dm, sg, b) * dm.Hkv + (int64_t)h * sg.S) * D + e;
+    float* dKb = dK + kv_base;
+    float* dVb = dV + kv_base;
     bool ok = true;
     // The band kernel, which precedes this one in the stream, stores its dK/dV rows plainly: the adds
     // below must come after it.  Nothing else in this kernel depends on it, so this is the only wait
     // (a no-op unless the launch carried the programmatic-serialization attribute).
-    if (n_act > 0) pdl_wait();
+    // It is executed even where there is nothing to add: the end of this grid has to imply the end of that one.
+    pdl_wait();
     for (int s = 0; s < n_act; ++s) {
       const int j = tile_of_step(s);
       ok = __all_sync(0xffffffffu, bwd_wait(&sm.dkv_full, s & 1, abort));
@@ -670,9 +674,9 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           const int o = 8 * j + half * 4 + (i >> 3);
           if (o < n_oct) {
             const int pos = sm.oct_row[o] + (i & 7);
-            if (pos >= dm.H && pos < red_hi) {   // warp-uniform: a key this kernel owes dK/dV
-              atomicAdd(dVb + (int64_t)(pos - dm.H) * D, __uint_as_float(gv[i]));
-              atomicAdd(dKb + (int64_t)(pos - dm.H) * D, __uint_as_float(gk[i]));
+            if (pos >= sg.H && pos < red_hi) {   // warp-uniform: a key this kernel owes dK/dV
+              atomicAdd(dVb + (int64_t)(pos - sg.H) * D, __uint_as_float(gv[i]));
+              atomicAdd(dKb + (int64_t)(pos - sg.H) * D, __uint_as_float(gk[i]));
             }
           }
         }
@@ -702,17 +706,15 @@ bool attn_bwd_sm100_supported(const Dims& dm) {
   return true;
 }
 
-int launch_attn_bwd_sm100(const Dims& dm, const void* Q, const void* K, const void* V, const void* O,
-                          const float* LSE, const void* dO, const int32_t* group_idx,
-                          const int32_t* n_groups, void* dQ, float* dK, float* dV, int32_t* status_word,
-                          cudaStream_t st) {
-  if (dm.d == 64)
-    return launch_attn_bwd_d64_sm100(dm, Q, K, V, O, LSE, dO, group_idx, n_groups, dQ, dK, dV, status_word, st);
+template <class Segs>
+static int launch_sweep(const Dims& dm, SegTable* table, const Segs& segs, int64_t units, const void* Q, const void* K, const void* V,
+                        const void* O, const float* LSE, const void* dO, const int32_t* group_idx,
+                        const int32_t* n_groups, void* dQ, float* dK, float* dV, int32_t* status_word, cudaStream_t st) {
   CUtensorMap mq, mdo, mk, mv, mdq;
   const uint32_t box[5] = {64, 8, 2, 1, 1};
   const uint32_t box_q[5] = {64, 64, 1, 1, 1};
-  const uint64_t dq[5] = {64, (uint64_t)dm.S, 2, (uint64_t)dm.Hq, (uint64_t)dm.B};
-  const uint64_t dk[5] = {64, (uint64_t)dm.L, 2, (uint64_t)dm.Hkv, (uint64_t)dm.B};
+  const uint64_t dq[5] = {64, (uint64_t)dm.rows_q, 2, (uint64_t)dm.Hq, (uint64_t)dm.B};
+  const uint64_t dk[5] = {64, (uint64_t)dm.rows_k, 2, (uint64_t)dm.Hkv, (uint64_t)dm.B};
   const uint64_t sq[4] = {(uint64_t)dm.qs[2] * 2, 128, (uint64_t)dm.qs[1] * 2, (uint64_t)dm.qs[0] * 2};
   const uint64_t so[4] = {(uint64_t)dm.os[2] * 2, 128, (uint64_t)dm.os[1] * 2, (uint64_t)dm.os[0] * 2};
   const uint64_t sk[4] = {(uint64_t)dm.ks[2] * 2, 128, (uint64_t)dm.ks[1] * 2, (uint64_t)dm.ks[0] * 2};
@@ -726,31 +728,32 @@ int launch_attn_bwd_sm100(const Dims& dm, const void* Q, const void* K, const vo
   // the octet table starts inside the struct's tail padding; 1024 bytes of slack for the manual alignment
   const size_t smem = offsetof(BwdSmem, oct_row) + sizeof(int) * (max_routed_tokens(dm) / 8 + 8) + 1024;
   if (smem > 227 * 1024) return HGA_ERR_UNSUPPORTED;
-  int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(&k_attn_bwd_sm100), smem);
+  int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(&k_attn_bwd_sm100<Segs>), smem);
   if (rc) return rc;
-  cudaError_t e;
   // dK/dV of the local band: written once per key tile by the key-major kernel, with plain stores that
   // cover every row of the active segment (so nothing has to be zero-filled); this kernel then adds the
-  // contributions of the keys before the band atomically.
-  rc = launch_attn_bwd_band_sm100(dm, Q, K, V, O, LSE, dO, dK, dV, status_word, st);
+  // contributions of the keys before the band atomically.  It may start on SMs the band kernel leaves idle (programmatic
+  // serialization; it waits for it only before adding to dK/dV).
+  rc = launch_attn_bwd_band_sm100(dm, table, Q, K, V, O, LSE, dO, dK, dV, status_word, st);
   if (rc != HGA_OK) return rc;
-  const int units = dm.B * dm.Hkv * dm.NQB * ((dm.rows + 127) / 128);
-  // The sweep is launched with programmatic serialization behind the band kernel: its CTAs may start on
-  // SMs the band kernel leaves idle (they wait for it only before adding to dK/dV).
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)units);
-  cfg.blockDim = dim3(kBwdThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = (dm.flags & kFlagNoPdl) ? 0 : 1;
-  e = cudaLaunchKernelEx(&cfg, k_attn_bwd_sm100, mq, mdo, mk, mv, mdq, (const uint16_t*)O, LSE, group_idx, n_groups,
-                         dm, dK, dV, status_word);
+  if (table) units = number_units(*table, [&](const Segment& g) { return (int64_t)dm.B * dm.Hkv * (g.S / dm.Bq) * ((dm.rows + 127) / 128); });
+  PdlLaunch cfg((unsigned)units, kBwdThreads, smem, st, dm.flags);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg.c, k_attn_bwd_sm100<Segs>, mq, mdo, mk, mv, mdq, (const uint16_t*)O, LSE, group_idx,
+                                           n_groups, dm, dK, dV, status_word, segs);
   count_launch(HGA_KERNELS_BWD_TENSOR);
   return record_cuda(e);
+}
+
+int launch_attn_bwd_sm100(const Dims& dm, SegTable* segs, const void* Q, const void* K, const void* V, const void* O,
+                          const float* LSE, const void* dO, const int32_t* group_idx,
+                          const int32_t* n_groups, void* dQ, float* dK, float* dV, int32_t* status_word,
+                          cudaStream_t st) {
+  if (dm.d == 64)
+    return launch_attn_bwd_d64_sm100(dm, segs, Q, K, V, O, LSE, dO, group_idx, n_groups, dQ, dK, dV, status_word, st);
+  const int64_t units = (int64_t)dm.B * dm.Hkv * dm.NQB * ((dm.rows + 127) / 128);
+  if (!segs)
+    return launch_sweep(dm, nullptr, OneSegment{}, units, Q, K, V, O, LSE, dO, group_idx, n_groups, dQ, dK, dV, status_word, st);
+  return launch_sweep(dm, segs, *segs, units, Q, K, V, O, LSE, dO, group_idx, n_groups, dQ, dK, dV, status_word, st);
 }
 
 }  // namespace hga

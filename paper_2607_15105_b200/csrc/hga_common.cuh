@@ -150,6 +150,8 @@ int record_cuda(cudaError_t e);  // returns HGA_OK or HGA_ERR_CUDA and remembers
 // Kernel launchers, one per translation unit.  All return an HGA status.
 int launch_build_summaries(const Dims& dm, const void* K, int tok_begin, int tok_end,
                            void* chunk_sum, void* group_sum, cudaStream_t st);
+// the active chunks of every segment of the table
+int launch_build_active_summaries(const Dims& dm, SegTable& segs, const void* K, void* chunk_sum, void* group_sum, cudaStream_t st);
 int launch_route_generic(const Dims& dm, const void* Q, const void* chunk_sum,
                          const void* group_sum, int32_t* chunk_idx, int32_t* group_idx,
                          int32_t* n_groups, float* chunk_scores, float* group_scores,
@@ -179,17 +181,17 @@ int launch_route_sm100(const Dims& dm, SegTable* segs, const void* Q, const void
                        int32_t* chunk_idx, int32_t* group_idx, int32_t* n_groups, float* chunk_scores,
                        float* group_scores, cudaStream_t st);
 bool attn_bwd_sm100_supported(const Dims& dm);
-int launch_attn_bwd_sm100(const Dims& dm, const void* Q, const void* K, const void* V, const void* O,
+int launch_attn_bwd_sm100(const Dims& dm, SegTable* segs, const void* Q, const void* K, const void* V, const void* O,
                           const float* LSE, const void* dO, const int32_t* group_idx,
                           const int32_t* n_groups, void* dQ, float* dK, float* dV, int32_t* status_word,
                           cudaStream_t st);
-int launch_attn_bwd_d64_sm100(const Dims& dm, const void* Q, const void* K, const void* V, const void* O,   // head_dim 64, called by the above
+int launch_attn_bwd_d64_sm100(const Dims& dm, SegTable* segs, const void* Q, const void* K, const void* V, const void* O,   // head_dim 64, called by the above
                               const float* LSE, const void* dO, const int32_t* group_idx,
                               const int32_t* n_groups, void* dQ, float* dK, float* dV, int32_t* status_word,
                               cudaStream_t st);
 // Key-major dK/dV of the local band (plain stores covering every active-segment row); launched by the above.
 bool attn_bwd_band_sm100_supported(const Dims& dm);
-int launch_attn_bwd_band_sm100(const Dims& dm, const void* Q, const void* K, const void* V, const void* O,
+int launch_attn_bwd_band_sm100(const Dims& dm, SegTable* segs, const void* Q, const void* K, const void* V, const void* O,
                                const float* LSE, const void* dO, float* dK, float* dV, int32_t* status_word,
                                cudaStream_t st);
 

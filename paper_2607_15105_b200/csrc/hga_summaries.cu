@@ -6,8 +6,11 @@
 // One CTA per (chunk, batch*kv_head), one warp per group; the chunk sum is the sum of its
 // group sums (exact in fp64, so the order does not matter).
 #include "hga_common.cuh"
+#include "hga_sm100.cuh"
 
 namespace hga {
+
+using namespace sm100;
 
 // Round a double to bf16, nearest-even, with a single rounding: truncate to fp32, fold
 // everything lost into the last fp32 bit (round-to-odd), then let the fp32 -> bf16
@@ -22,20 +25,24 @@ __device__ inline uint16_t f64_to_bf16_once(double x) {
 // CTA has warps).  A warp's 32 lanes cover 32 / (D/8) consecutive rows per load instruction, 16 bytes per
 // lane, and request up to four such row sets before the first sum: the kernel is one round trip to memory
 // deep, which is what bounds a 4 MB stream spread over the whole GPU.
-template <int D>
+template <int D, class Segs>
 __global__ void __launch_bounds__(256, 3)
-k_build_summaries(const uint16_t* __restrict__ K, Dims dm, int chunk_begin,
-                  uint16_t* __restrict__ chunk_sum, uint16_t* __restrict__ group_sum) {
+k_build_summaries(const uint16_t* __restrict__ K, const Dims dm, int chunk_begin,
+                  uint16_t* __restrict__ chunk_sum, uint16_t* __restrict__ group_sum, const __grid_constant__ Segs segs) {
   constexpr int VEC = D / 8;                  // lanes across one row
   constexpr int RPI = 32 / VEC;               // rows per load instruction
   extern __shared__ double part[];            // [warps][D]: per-warp sums of the groups it handled
-  const int j = chunk_begin + blockIdx.x;     // chunk id
+  int i_chunk;                                // of the segment's active range (or of the range from chunk_begin on)
+  const Segment sg = segment_of(dm, segs, blockIdx.x, i_chunk);
+  const int j = chunk_begin + (chunk_begin < 0 ? 1 + (sg.k0 + sg.H) / dm.c : 0) + i_chunk;      // row in the chunk table
   const int bh = blockIdx.y;
   const int b = bh / dm.Hkv, h = bh % dm.Hkv;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
   const int v = lane % VEC, sub = lane / VEC;
   const uint16_t* Kb = K + b * dm.ks[0] + h * dm.ks[1] + v * 8;
 
+  pdl_wait();
+  pdl_launch_dependents();
   double csum[8];
 #pragma unroll
   for (int e = 0; e < 8; ++e) csum[e] = 0.0;
@@ -100,25 +107,29 @@ k_build_summaries(const uint16_t* __restrict__ K, Dims dm, int chunk_begin,
   }
 }
 
+template <class Segs>
+static int launch_summaries(const Dims& dm, const Segs& segs, int64_t chunks, const void* K, int chunk_begin, void* chunk_sum,
+                            void* group_sum, cudaStream_t st) {
+  auto* kernel = dm.d == 128 ? k_build_summaries<128, Segs> : k_build_summaries<64, Segs>;
+  const int n_warps = dm.per < 8 ? dm.per : 8;
+  const size_t smem = (size_t)n_warps * dm.d * sizeof(double);
+  // (the shared-memory carve-out of the other kernels of the path: an SM has to drain before it changes)
+  const int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), smem, true);
+  if (rc) return rc;
+  PdlLaunch cfg(dim3((unsigned)chunks, dm.B * dm.Hkv), n_warps * 32, smem, st, dm.flags);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg.c, kernel, (const uint16_t*)K, dm, chunk_begin, (uint16_t*)chunk_sum, (uint16_t*)group_sum, segs);
+  count_launch(HGA_KERNELS_SUMMARIES);
+  return record_cuda(e);
+}
+
 int launch_build_summaries(const Dims& dm, const void* K, int tok_begin, int tok_end,
                            void* chunk_sum, void* group_sum, cudaStream_t st) {
-  const int n_warps = dm.per < 8 ? dm.per : 8;
-  dim3 grid((tok_end - tok_begin) / dm.c, dm.B * dm.Hkv);
-  dim3 block(n_warps * 32);
-  size_t smem = (size_t)n_warps * dm.d * sizeof(double);
-  auto Kp = (const uint16_t*)K;
-  auto cs = (uint16_t*)chunk_sum;
-  auto gs = (uint16_t*)group_sum;
-  // (the shared-memory carve-out of the other kernels of the path: an SM has to drain before it changes)
-  const int rc = ensure_dynamic_smem(dm.d == 128 ? reinterpret_cast<const void*>(&k_build_summaries<128>)
-                                                 : reinterpret_cast<const void*>(&k_build_summaries<64>), smem, true);
-  if (rc) return rc;
-  if (dm.d == 128)
-    k_build_summaries<128><<<grid, block, smem, st>>>(Kp, dm, tok_begin / dm.c, cs, gs);
-  else
-    k_build_summaries<64><<<grid, block, smem, st>>>(Kp, dm, tok_begin / dm.c, cs, gs);
-  count_launch(HGA_KERNELS_SUMMARIES);
-  return record_cuda(cudaGetLastError());
+  return launch_summaries(dm, OneSegment{}, (tok_end - tok_begin) / dm.c, K, tok_begin / dm.c, chunk_sum, group_sum, st);
+}
+
+int launch_build_active_summaries(const Dims& dm, SegTable& segs, const void* K, void* chunk_sum, void* group_sum, cudaStream_t st) {
+  const int64_t chunks = number_units(segs, [&](const Segment& g) { return (int64_t)(g.S / dm.c); });
+  return launch_summaries(dm, segs, chunks, K, -1, chunk_sum, group_sum, st);
 }
 
 }  // namespace hga

@@ -31,7 +31,7 @@
 
 namespace hga {
 void count_launch(int, int) {}
-int launch_attn_bwd_d64_sm100(const Dims&, const void*, const void*, const void*, const void*, const float*, const void*, const int32_t*,
+int launch_attn_bwd_d64_sm100(const Dims&, SegTable*, const void*, const void*, const void*, const void*, const float*, const void*, const int32_t*,
                               const int32_t*, void*, float*, float*, int32_t*, cudaStream_t) { return HGA_ERR_UNSUPPORTED; }   // (head_dim 128 only here)
 int record_cuda(cudaError_t e) { if (e != cudaSuccess) printf("cuda error %s\n", cudaGetErrorString(e)); return e == cudaSuccess ? 0 : -6; }
 }
@@ -84,7 +84,7 @@ int main(int argc, char** argv) {
     { void* p_; cudaGetSymbolAddress(&p_, g_trace_log); cudaMemsetAsync(p_, 0, sizeof(unsigned) * HGA_TRACE_WARPS * HGA_TRACE_SLOTS); }
     cudaEventRecord(e0);
     int rc = fwd_mode ? launch_attn_fwd_sm100(dm, nullptr, dq, dk, dv, dgi, dng, dO, dlse, dst, 0)
-                      : launch_attn_bwd_sm100(dm, dq, dk, dv, dO, dlse, ddO, dgi, dng, ddQ, ddK, ddV, dst, 0);
+                      : launch_attn_bwd_sm100(dm, nullptr, dq, dk, dv, dO, dlse, ddO, dgi, dng, ddQ, ddK, ddV, dst, 0);
     cudaEventRecord(e1);
     cudaError_t ce = cudaDeviceSynchronize();
     float ms; cudaEventElapsedTime(&ms, e0, e1);
