@@ -54,6 +54,7 @@ using namespace sm100;
 
 constexpr int kBwdThreads = 512;                // 16 warps: 128 registers per thread
 constexpr int kBwdKStages = 6;                  // K ring: three pairs (a K tile is held until its dQ GEMM)
+constexpr int kActStages = 4;                   // ... of which the dK/dV steps use two; the third stages their dK/dV rows
 constexpr int kBwdVStages = 2;                  // V ring of the dK/dV steps; the paired steps add the P / dS tiles as a second pair
 constexpr int kBwdD = 128;
 constexpr int kKT = 64;                         // keys per tile
@@ -69,7 +70,7 @@ struct BwdSmem {
   alignas(1024) uint8_t p[kPdsTile];            // [16 row octets][8 rows][128 B], 128-byte swizzle
   alignas(1024) uint8_t ds[kPdsTile];           // (P and dS pass through shared memory only for dK/dV tiles)
   uint64_t q_full, k_full[kBwdKStages], k_empty[kBwdKStages];   // (dK/dV steps: even stages hold K tiles, odd ones V tiles)
-  uint64_t sdp_full, pds_full, dkv_full, dkv_free;      // dK/dV steps
+  uint64_t sdp_full, pds_full, dkv_full, dkv_free, staged, stage_free;   // dK/dV steps
   uint64_t s_full[2], dp_full[4], ds_full[2], s_read[2];   // paired steps (S(u+1) is committed before step u is over: two barriers;
                                                         // dP: four, so that a copy item taken ahead of time cannot mistake an older phase)
   uint64_t phase_a_done;                                // every GEMM of the dK/dV steps is complete
@@ -120,7 +121,7 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     mbar_init(&sm.q_full, 1);
     for (int s = 0; s < kBwdKStages; ++s) { mbar_init(&sm.k_full[s], (s & 1) ? 2 : 1); mbar_init(&sm.k_empty[s], 1); }   // (two V producers)
     mbar_init(&sm.sdp_full, 1); mbar_init(&sm.pds_full, 256);
-    mbar_init(&sm.dkv_full, 1); mbar_init(&sm.dkv_free, 128);
+    mbar_init(&sm.dkv_full, 1); mbar_init(&sm.dkv_free, 128); mbar_init(&sm.staged, 128); mbar_init(&sm.stage_free, 4);
     mbar_init(&sm.s_full[0], 1); mbar_init(&sm.s_full[1], 1);
     // (two barriers each, used alternately: S(u+1) and dP(u+1) are issued before the MMA warp waits for the row
     // threads' arrivals of pair u, so the row threads may finish pair u+1 -- and arrive again -- before that wait
@@ -215,7 +216,9 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   // Ring slots: dK/dV step s takes TWO slots of the K ring, 2s for its K tile and 2s+1 for its V tile, so that
   // the V ring proper stays free and the first V pair of the paired steps is copied while the dK/dV steps
   // still run; the paired steps continue the slot numbering (a pair of stages is one contiguous operand).
-  const int n_act_even = 2 * n_act;
+  // Pair p of the paired steps takes pair-stage (ps_base + p) % 3: after one dK/dV step, which has used the first
+  // pair-stage only, the free one first; the third, where dK/dV rows were staged, last.
+  const int ps_base = n_act == 1 ? 1 : 0;
   const int red_hi = w.ls;
   // Step order: the dK/dV tiles first (descending), so their atomics drain while the rest is
   // computed; then every other tile, descending.
@@ -244,11 +247,11 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       const uint32_t my_bytes = (uint32_t)(is_v ? 4 : 8) * kOct;
       for (int step = 0; step < n_act && ok; ++step) {
         const int slot = 2 * step + (is_v ? 1 : 0);
-        const int st = slot % kBwdKStages;
+        const int st = slot % kActStages;
         int row = dm.rows_k;                                 // past the list: zeros
         const int o = 8 * tile_of_step(step) + oct_in_tile;
         if (o < n_oct) row = sg.k0 + sm.oct_row[o];
-        if (lane == 0 && slot >= kBwdKStages) ok = bwd_wait(&sm.k_empty[st], (uint32_t)(slot / kBwdKStages - 1) & 1, abort);
+        if (lane == 0 && slot >= kActStages) ok = bwd_wait(&sm.k_empty[st], (uint32_t)(slot / kActStages - 1) & 1, abort);
         ok = __shfl_sync(0xffffffffu, ok, 0);
         if (!ok) break;
         if (lane == 0) mbar_arrive_expect_tx(&sm.k_full[st], my_bytes);
@@ -269,7 +272,7 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         // K: three pairs of stages, continuing the slot numbering.  V: two pairs, pair p in slot p & 1; slot 0
         // is the V ring, slot 1 the P and dS tiles (adjacent, one K/V tile each), which only the dK/dV steps
         // use otherwise.  A V pair is free once its dP GEMM is done, a K pair only after its dQ GEMM.
-        const int ps = is_v ? (p & 1) : (n_act_even / 2 + p) % n_ps;
+        const int ps = is_v ? (p & 1) : (ps_base + p) % n_ps;
         uint64_t* full = is_v ? &sm.vp_full[ps] : &sm.kp_full[ps];
         const int s = n_act + 2 * p + which;                              // step (tile order)
         int row = dm.rows_k;
@@ -284,10 +287,12 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             if (p < 2) { if (p == 1 && n_act > 0) ok = bwd_wait(&sm.phase_a_done, 0, abort); }
             else ok = bwd_wait(&sm.dp_full[(p - 2) & 3], (uint32_t)((p - 2) >> 2) & 1, abort);
           } else if (p < n_ps) {
-            // first paired use of these stages: if a dK/dV step used them, those steps must be over
-            if (2 * ps < n_act_even) ok = bwd_wait(&sm.phase_a_done, 0, abort);
+            // first paired use of these stages: if a dK/dV step used them, those steps must be over, and what
+            // was staged in the third pair on its way
+            if (ps == 2 && n_act > 0) ok = bwd_wait(&sm.stage_free, 0, abort);
+            else if (ps < n_act) ok = bwd_wait(&sm.phase_a_done, 0, abort);
           } else {
-            ok = bwd_wait(&sm.kp_empty[(n_act_even / 2 + p - 3) % kBwdKStages], (uint32_t)((p - 3) / kBwdKStages) & 1, abort);   // dQ of pair p-3 is done
+            ok = bwd_wait(&sm.kp_empty[(ps_base + p - 3) % kBwdKStages], (uint32_t)((p - 3) / kBwdKStages) & 1, abort);   // dQ of pair p-3 is done
           }
         }
         ok = __shfl_sync(0xffffffffu, ok, 0);
@@ -330,7 +335,7 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       const uint64_t dsd = smem_desc_sw128(smem_u32(sm.ds), 16, 1024);       // dS: K-major A (dQ) and MN-major B (dK^T)
       const uint64_t pd = smem_desc_sw128(smem_u32(sm.p), 16, 1024);         // P : MN-major B (dV^T)
       // (arguments are ring slots)
-      auto wait_k = [&](int s) { return mma_wait(&sm.k_full[s % kBwdKStages], (s / kBwdKStages) & 1, abort); };
+      auto wait_k = [&](int s) { return mma_wait(&sm.k_full[s % kActStages], (s / kActStages) & 1, abort); };
       // acc (128 rows x N keys) = a (Q or dO, K-major) x b^T (key tiles at ring stage st, K-major)
       auto issue_qk = [&](uint32_t acc, uint64_t a, uint64_t b0, int st, uint32_t idesc) {   // st: ring stage
         const uint64_t bd = desc_advance(b0, (uint32_t)st * kKvTile);
@@ -347,7 +352,7 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       // issue order and a commit covers everything issued before it, so sdp_full of step s+1 also
       // tells the row threads that the GEMMs reading P/dS of step s are done.
       for (int s = 0; s < n_act && ok; ++s) {
-        const int st = (2 * s) % kBwdKStages, vst = (2 * s + 1) % kBwdKStages;      // K tile, V tile
+        const int st = (2 * s) % kActStages, vst = (2 * s + 1) % kActStages;      // K tile, V tile
         ok = wait_k(2 * s);
         HGA_TRACE_POINT(41);
         ok = ok && wait_k(2 * s + 1);
@@ -387,8 +392,8 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       // ---- paired steps.  Step u covers ring stages st, st+1 (contiguous); S(u) lives in region
       // (2u)%3, dP(u) and later dS(u) in region (2u+1)%3.
       if (ok && n_pairs > 0) {
-        if (ok && n_act_even > 0) mma_commit_w(&sm.phase_a_done);
-        const int ps0 = (n_act_even / 2) % (kBwdKStages / 2);
+        if (ok && n_act > 0) mma_commit_w(&sm.phase_a_done);
+        const int ps0 = ps_base;
         if (ok) ok = mma_wait(&sm.kp_full[ps0], 0, abort);
         HGA_TRACE_POINT(43);
         if (ok) {
@@ -407,7 +412,7 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       int rs = 0;                                     // region of S(u)
       for (int u = 0; u < n_pairs && ok; ++u) {
         constexpr int kPs = kBwdKStages / 2;
-        const int ps = (n_act_even / 2 + u) % kPs, ps_n = (ps + 1) % kPs;     // pair stages of steps u, u+1
+        const int ps = (ps_base + u) % kPs, ps_n = (ps + 1) % kPs;     // pair stages of steps u, u+1
         const int rp = rs == 2 ? 0 : rs + 1;          // region of dP(u), dS(u)
         const int rs_n = rp == 2 ? 0 : rp + 1;        // region of S(u+1): two steps ago it held dP(u-1)
         if (u + 1 < n_pairs) {
@@ -443,7 +448,7 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           mma_ts_w(tmem + kColDQ, ds_base + (kk < 4 ? 8 * kk : 64 + 8 * (kk - 4)), desc_advance(kmn, kk * 2 * kOct),
                  idesc_dq, (dq_started || kk > 0));
         dq_started = true;
-        mma_commit_w(&sm.kp_empty[(n_act_even / 2 + u) % kBwdKStages]);
+        mma_commit_w(&sm.kp_empty[(ps_base + u) % kBwdKStages]);
         HGA_TRACE_POINT(7);
         rs = rs_n;
       }
@@ -644,44 +649,68 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     const int quarter = warp & 3;
     const int e = quarter * 32 + lane;                       // head_dim element = TMEM lane
     const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
-    const int64_t kv_base = (row_base(dm, sg, b) * dm.Hkv + (int64_t)h * sg.S) * D + e;
-    float* dKb = dK + kv_base;
-    float* dVb = dV + kv_base;
+    const int64_t kv_base = (row_base(dm, sg, b) * dm.Hkv + (int64_t)h * sg.S) * D;
     bool ok = true;
     // The band kernel, which precedes this one in the stream, stores its dK/dV rows plainly: the adds
     // below must come after it.  Nothing else in this kernel depends on it, so this is the only wait
     // (a no-op unless the launch carried the programmatic-serialization attribute).
     // It is executed even where there is nothing to add: the end of this grid has to imply the end of that one.
     pdl_wait();
-    for (int s = 0; s < n_act; ++s) {
+    // The transposed accumulators (lane = element, column = key) go to shared memory as key rows of 512 bytes, 32 keys at a
+    // time in two buffers of 16 KB (the K ring's third pair); an octet of them is 4 KB of consecutive memory on both
+    // sides and is added by one bulk reduction.  (As 128-byte red.global requests, 512 per step, the adds took the SM
+    // 6k cycles to send off, longer than the step's GEMMs: 2K layer, hga_attn_bwd 115 us.)
+    uint32_t staged_phase = 0;
+    auto all_here = [&]() {                 // the 128 threads meet (bounded: one of them may have given up)
+      mbar_arrive(&sm.staged);
+      ok = __all_sync(0xffffffffu, bwd_wait(&sm.staged, staged_phase, abort));
+      staged_phase ^= 1u;
+      return ok;
+    };
+    for (int s = 0; s < n_act && ok; ++s) {
       const int j = tile_of_step(s);
       ok = __all_sync(0xffffffffu, bwd_wait(&sm.dkv_full, s & 1, abort));
       if (!ok) break;
       tc_fence_after_sync();
       HGA_TRACE_POINT(16);
-#pragma unroll
-      for (int half = 0; half < 2; ++half) {
-        uint32_t gv[32], gk[32];
-        tmem_ld32(lane_base + kColDV + half * 32, gv);
-        tmem_ld32(lane_base + kColDK + half * 32, gk);
+#pragma unroll 1
+      for (int c = 0; c < 4; ++c) {         // dV keys 0-31, 32-63, dK keys 0-31, 32-63
+        const int half = c & 1;
+        uint8_t* const buf = sm.k[kActStages + half];
+        uint32_t x[32];
+        tmem_ld32(lane_base + (c < 2 ? kColDV : kColDK) + half * 32, x);
         tmem_wait_ld();
-        if (half == 1) {
+        if (c == 3) {
           tc_fence_before_sync();
           mbar_arrive(&sm.dkv_free);
         }
+        if (s > 0 || c > 1) {
+          // the buffer's last contents have been read (this thread's reduction before the last one)
+          if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+          __syncwarp();
+          if (!all_here()) break;
+        }
+        const uint32_t dst = smem_u32(buf) + (uint32_t)e * 4;
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const int o = 8 * j + half * 4 + (i >> 3);
-          if (o < n_oct) {
-            const int pos = sm.oct_row[o] + (i & 7);
-            if (pos >= sg.H && pos < red_hi) {   // warp-uniform: a key this kernel owes dK/dV
-              atomicAdd(dVb + (int64_t)(pos - sg.H) * D, __uint_as_float(gv[i]));
-              atomicAdd(dKb + (int64_t)(pos - sg.H) * D, __uint_as_float(gk[i]));
-            }
-          }
+        for (int i = 0; i < 32; ++i) st_shared_b32(dst + (uint32_t)i * 512, x[i]);
+        fence_proxy_async_smem();
+        if (!all_here()) break;
+        if (lane == 0) {                    // warp = octet (its rows are all in the active segment before the band, or none is)
+          const int o = 8 * j + half * 4 + quarter;
+          const int pos = o < n_oct ? sm.oct_row[o] : -1;
+          if (pos >= sg.H && pos < red_hi)
+            bulk_reduce_add_f32((c < 2 ? dV : dK) + kv_base + (int64_t)(pos - sg.H) * D, smem_u32(buf) + quarter * 4096, 4096);
+          tma_store_commit();
         }
       }
       HGA_TRACE_POINT(18);
+    }
+    if (n_act > 0) {
+      if (lane == 0) {
+        tma_store_wait_read();
+        mbar_arrive(&sm.stage_free);
+      }
+      __syncwarp();
     }
   }
   HGA_TRACE_POINT(30);
