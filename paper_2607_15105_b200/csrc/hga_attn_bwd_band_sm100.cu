@@ -112,9 +112,9 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
     for (int s = 0; s < 4; ++s) {
       mbar_init(&sm.qdo_full[s >> 1][s & 1], 1); mbar_init(&sm.qdo_empty[s >> 1][s & 1], 1);
     }
-    mbar_init(&sm.o_full, 1); mbar_init(&sm.o_empty, 128);
+    mbar_init(&sm.o_full, 1); mbar_init(&sm.o_empty, 4);
     for (int s = 0; s < 2; ++s) {
-      mbar_init(&sm.stat_full[s], 64); mbar_init(&sm.sdp_full[s], 1); mbar_init(&sm.pds_full[s], 256);
+      mbar_init(&sm.stat_full[s], 2); mbar_init(&sm.sdp_full[s], 1); mbar_init(&sm.pds_full[s], 8);
     }
     mbar_init(&sm.acc_done, 1); mbar_init(&sm.drain, 1);
     sm.abort = 0;
@@ -382,7 +382,7 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
       }
       tmem_wait_st();
       tc_fence_before_sync();
-      mbar_arrive(&sm.pds_full[hf]);
+      mbar_arrive_warp(&sm.pds_full[hf]);
       HGA_TRACE_POINT(14);
       sp.next(dm, qb_last);
     }
@@ -457,7 +457,7 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
           acc[e] = fmaf(__uint_as_float(xs[e] & 0xffff0000u), __uint_as_float(ys[e] & 0xffff0000u), acc[e]);
         }
       }
-      mbar_arrive(&sm.o_empty);                      // the O tile may be overwritten by the next step's
+      mbar_arrive_warp(&sm.o_empty);                      // the O tile may be overwritten by the next step's
       if (warp == 13 && m + 1 < n_steps) {
         // ... which this warp -- the one whose rows of dO arrive last -- fetches as soon as all four
         // statistics warps have read this one
@@ -476,7 +476,7 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
       if (!ok) break;
       sm.nlse[j] = -lse * 1.4426950408889634f;
       sm.nds[j] = -delta * dm.scale;
-      mbar_arrive(&sm.stat_full[j >> 6]);
+      mbar_arrive_warp(&sm.stat_full[j >> 6]);
       HGA_TRACE_POINT(14);
     }
     // giving up: let the O copy still in flight land before shared memory is released

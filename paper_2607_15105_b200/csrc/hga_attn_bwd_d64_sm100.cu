@@ -133,10 +133,10 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
     mbar_init(&sm.q_full, 1);
     for (int s = 0; s < 2; ++s) { mbar_init(&sm.k_full[s], 2); mbar_init(&sm.k_empty[s], 1); }
     mbar_init(&sm.v_full, 2);
-    mbar_init(&sm.s_full, 1); mbar_init(&sm.s_read, 128);
-    mbar_init(&sm.dp_full, 1); mbar_init(&sm.ds_full, 128);
-    mbar_init(&sm.dkv_full, 1); mbar_init(&sm.staged, 128); mbar_init(&sm.dk_read, 128);
-    mbar_init(&sm.info_full, 1); mbar_init(&sm.dq_done, 1); mbar_init(&sm.dq_staged, 128); mbar_init(&sm.drain, 1);
+    mbar_init(&sm.s_full, 1); mbar_init(&sm.s_read, 4);
+    mbar_init(&sm.dp_full, 1); mbar_init(&sm.ds_full, 4);
+    mbar_init(&sm.dkv_full, 1); mbar_init(&sm.staged, 4); mbar_init(&sm.dk_read, 4);
+    mbar_init(&sm.info_full, 1); mbar_init(&sm.dq_done, 1); mbar_init(&sm.dq_staged, 4); mbar_init(&sm.drain, 1);
     sm.abort = 0;
     fence_barrier_init();
   }
@@ -435,7 +435,7 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
       const bool kind3 = j >= n_lt && j >= n_a;
       if (!kind3) {
         tc_fence_before_sync();
-        mbar_arrive(&sm.s_read);                      // S(j) has been read: S(j+1) may take its place
+        mbar_arrive_warp(&sm.s_read);                      // S(j) has been read: S(j+1) may take its place
       }
       ok = __all_sync(0xffffffffu, bwd_wait(&sm.dp_full, j & 1, abort));
       if (!ok) break;
@@ -471,14 +471,14 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
       if (!kind3) {
         tmem_wait_st();
         tc_fence_before_sync();
-        mbar_arrive(&sm.ds_full);
+        mbar_arrive_warp(&sm.ds_full);
         HGA_TRACE_POINT(14);
         continue;
       }
       // ---- dK/dV tile
       tc_fence_before_sync();
       fence_proxy_async_smem();
-      mbar_arrive(&sm.ds_full);
+      mbar_arrive_warp(&sm.ds_full);
       HGA_TRACE_POINT(17);
       ok = __all_sync(0xffffffffu, bwd_wait(&sm.dkv_full, (j - n_a) & 1, abort));
       if (!ok) break;
@@ -513,12 +513,12 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
       };
       auto hand_over = [&]() {             // what this thread has written is complete and visible to bulk copies
         fence_proxy_async_smem();
-        mbar_arrive(&sm.staged);
+        mbar_arrive_warp(&sm.staged);
         return wait_staged();
       };
       auto have_read = [&](uint64_t* bar) {
         tc_fence_before_sync();
-        mbar_arrive(bar);
+        mbar_arrive_warp(bar);
       };
       const uint32_t col = quarter < 2 ? kColS : kColDP;      // lanes 0-63: dV^T, lanes 64-127: dK^T
       stage(sm.p, col);
@@ -529,7 +529,7 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
       reduce_rows((quarter & 1) ? dK : dV, quarter < 2 ? sm.p : sm.ds, quarter >> 1, (quarter & 1) * 256u);
       tma_store_wait_read();
       __syncwarp();
-      mbar_arrive(&sm.staged);
+      mbar_arrive_warp(&sm.staged);
       if (!wait_staged()) break;                      // P and dS may be written again
       HGA_TRACE_POINT(18);
     }
@@ -555,7 +555,7 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
                        pack_bf16(__uint_as_float(x[c][8 * i + 4]), __uint_as_float(x[c][8 * i + 5])),
                        pack_bf16(__uint_as_float(x[c][8 * i + 6]), __uint_as_float(x[c][8 * i + 7])));
       fence_proxy_async_smem();
-      mbar_arrive(&sm.dq_staged);
+      mbar_arrive_warp(&sm.dq_staged);
       if (warp == 2 && lane < 2 && bwd_wait(&sm.dq_staged, 0, abort)) {      // all 128 rows are in shared memory
         const int r0 = mt * 128 + 64 * lane;
         if (r0 < dm.rows) {

@@ -47,7 +47,11 @@
 #include "hga_sm100.cuh"
 
 #include <cstddef>
+#include <type_traits>
 
+#ifndef HGA_POLY
+#define HGA_POLY 0
+#endif
 namespace hga {
 
 using namespace sm100;
@@ -70,7 +74,7 @@ struct BwdSmem {
   alignas(1024) uint8_t p[kPdsTile];            // [16 row octets][8 rows][128 B], 128-byte swizzle
   alignas(1024) uint8_t ds[kPdsTile];           // (P and dS pass through shared memory only for dK/dV tiles)
   uint64_t q_full, k_full[kBwdKStages], k_empty[kBwdKStages];   // (dK/dV steps: even stages hold K tiles, odd ones V tiles)
-  uint64_t sdp_full, pds_full, dkv_full, dkv_free, staged, stage_free;   // dK/dV steps
+  uint64_t sdp_full, pds_full, dkv_full, dkv_free, stage_free;   // dK/dV steps
   uint64_t s_full[2], dp_full[4], ds_full[2], s_read[2];   // paired steps (S(u+1) is committed before step u is over: two barriers;
                                                         // dP: four, so that a copy item taken ahead of time cannot mistake an older phase)
   uint64_t phase_a_done;                                // every GEMM of the dK/dV steps is complete
@@ -120,19 +124,19 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   if (tid == 0) {
     mbar_init(&sm.q_full, 1);
     for (int s = 0; s < kBwdKStages; ++s) { mbar_init(&sm.k_full[s], (s & 1) ? 2 : 1); mbar_init(&sm.k_empty[s], 1); }   // (two V producers)
-    mbar_init(&sm.sdp_full, 1); mbar_init(&sm.pds_full, 256);
-    mbar_init(&sm.dkv_full, 1); mbar_init(&sm.dkv_free, 128); mbar_init(&sm.staged, 128); mbar_init(&sm.stage_free, 4);
+    mbar_init(&sm.sdp_full, 1); mbar_init(&sm.pds_full, 8);
+    mbar_init(&sm.dkv_full, 1); mbar_init(&sm.dkv_free, 4); mbar_init(&sm.stage_free, 4);
     mbar_init(&sm.s_full[0], 1); mbar_init(&sm.s_full[1], 1);
     // (two barriers each, used alternately: S(u+1) and dP(u+1) are issued before the MMA warp waits for the row
     // threads' arrivals of pair u, so the row threads may finish pair u+1 -- and arrive again -- before that wait
     // has observed pair u; with one barrier its phase would then be missed.  Pair u+2 cannot start before.)
-    for (int s = 0; s < 2; ++s) { mbar_init(&sm.ds_full[s], 256); mbar_init(&sm.s_read[s], 256); }
+    for (int s = 0; s < 2; ++s) { mbar_init(&sm.ds_full[s], 8); mbar_init(&sm.s_read[s], 8); }
     for (int s = 0; s < 4; ++s) mbar_init(&sm.dp_full[s], 1);
     mbar_init(&sm.phase_a_done, 1);
     for (int s = 0; s < kBwdKStages / 2; ++s) mbar_init(&sm.kp_full[s], 1);
     for (int s = 0; s < kBwdKStages; ++s) mbar_init(&sm.kp_empty[s], 1);
     mbar_init(&sm.vp_full[0], 2); mbar_init(&sm.vp_full[1], 2);
-    mbar_init(&sm.dq_done, 1); mbar_init(&sm.dq_staged, 256);
+    mbar_init(&sm.dq_done, 1); mbar_init(&sm.dq_staged, 8);
     sm.abort = 0;
     fence_barrier_init();
   }
@@ -216,9 +220,9 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   // Ring slots: dK/dV step s takes TWO slots of the K ring, 2s for its K tile and 2s+1 for its V tile, so that
   // the V ring proper stays free and the first V pair of the paired steps is copied while the dK/dV steps
   // still run; the paired steps continue the slot numbering (a pair of stages is one contiguous operand).
-  // Pair p of the paired steps takes pair-stage (ps_base + p) % 3: after one dK/dV step, which has used the first
-  // pair-stage only, the free one first; the third, where dK/dV rows were staged, last.
-  const int ps_base = n_act == 1 ? 1 : 0;
+  // Pair-stage of pair p of the paired steps: after one dK/dV step, which has used the first pair-stage only, the free one
+  // first and the third, where dK/dV rows are still staged for a while, last; after more of them in order, for the same reason.
+  auto pair_stage = [&](int p) { return n_act == 1 ? (1 + 2 * p) % 3 : p % 3; };
   const int red_hi = w.ls;
   // Step order: the dK/dV tiles first (descending), so their atomics drain while the rest is
   // computed; then every other tile, descending.
@@ -228,6 +232,7 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     return j >= dkv_hi ? j : j - n_act;
   };
   volatile int* abort = &sm.abort;
+  bool ok = true;
   HGA_TRACE_POINT(1);
 
   if (warp == 0 || warp >= 14) {
@@ -239,7 +244,6 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // different warps issue in parallel.
     const bool is_v = warp != 0;
     const CUtensorMap* map = is_v ? &map_v : &map_k;
-    bool ok = true;
     // ---- slots of the dK/dV steps: one tile per slot, one full/empty barrier pair per stage
     {
       const int oct_in_tile = is_v ? (warp == 14 ? lane : 4 + lane) : lane;
@@ -259,57 +263,6 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         if (copy_lane) tma_load_5d(sm.k[st] + oct_in_tile * kOct, map, &sm.k_full[st], 0, row, 0, h, b);
         HGA_TRACE_POINT(2);
       }
-    }
-    // ---- paired steps: pair p fills stages 2*ps, 2*ps+1 (ps continues the slot numbering) and
-    // completes ONE barrier per operand, so the MMA thread observes one barrier per operand and
-    // pair.  Lanes 0-7 (K) / 0-3 (V): first tile, lanes 8-15 / 4-7: second tile.
-    {
-      const int n_ps = kBwdKStages / 2;
-      const int which = is_v ? lane >> 2 : lane >> 3;                     // tile of the pair
-      const int oct_in_tile = is_v ? (warp == 14 ? 0 : 4) + (lane & 3) : lane & 7;
-      const bool copy_lane = is_v ? lane < 8 : lane < 16;
-      for (int p = 0; p < n_pairs && ok; ++p) {
-        // K: three pairs of stages, continuing the slot numbering.  V: two pairs, pair p in slot p & 1; slot 0
-        // is the V ring, slot 1 the P and dS tiles (adjacent, one K/V tile each), which only the dK/dV steps
-        // use otherwise.  A V pair is free once its dP GEMM is done, a K pair only after its dQ GEMM.
-        const int ps = is_v ? (p & 1) : (ps_base + p) % n_ps;
-        uint64_t* full = is_v ? &sm.vp_full[ps] : &sm.kp_full[ps];
-        const int s = n_act + 2 * p + which;                              // step (tile order)
-        int row = dm.rows_k;
-        if (s < n_tiles) {
-          const int o = 8 * tile_of_step(s) + oct_in_tile;
-          if (o < n_oct) row = sg.k0 + sm.oct_row[o];
-        }
-        if (lane == 0) {
-          if (is_v) {
-            // first pair: the V ring is free from the start; second: the dK/dV steps (which use the P and dS
-            // tiles) must be over; later: dP of pair p-2 is done
-            if (p < 2) { if (p == 1 && n_act > 0) ok = bwd_wait(&sm.phase_a_done, 0, abort); }
-            else ok = bwd_wait(&sm.dp_full[(p - 2) & 3], (uint32_t)((p - 2) >> 2) & 1, abort);
-          } else if (p < n_ps) {
-            // first paired use of these stages: if a dK/dV step used them, those steps must be over, and what
-            // was staged in the third pair on its way
-            if (ps == 2 && n_act > 0) ok = bwd_wait(&sm.stage_free, 0, abort);
-            else if (ps < n_act) ok = bwd_wait(&sm.phase_a_done, 0, abort);
-          } else {
-            ok = bwd_wait(&sm.kp_empty[(ps_base + p - 3) % kBwdKStages], (uint32_t)((p - 3) / kBwdKStages) & 1, abort);   // dQ of pair p-3 is done
-          }
-        }
-        ok = __shfl_sync(0xffffffffu, ok, 0);
-        if (!ok) break;
-        if (lane == 0) mbar_arrive_expect_tx(full, (uint32_t)(is_v ? 8 : 16) * kOct);
-        __syncwarp();
-        if (copy_lane)
-          tma_load_5d((is_v ? (ps == 0 ? sm.v[0] : sm.p) + which * kKvTile : sm.k[2 * ps + which]) + oct_in_tile * kOct, map, full,
-                      0, row, 0, h, b);
-        HGA_TRACE_POINT(2);
-      }
-    }
-    if (*abort && lane == 0) {
-      // giving up: give the copies still in flight time to land before shared memory is released
-      // (the full barriers may never complete once another role has stopped, hence a bounded sleep)
-      if (warp == 0) mbar_wait(&sm.q_full, 0);
-      for (int it = 0; it < 64; ++it) __nanosleep(1000);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
@@ -345,7 +298,7 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           mma_ss_w(acc, desc_advance(a, a_off), desc_advance(bd, b_off), idesc, kk > 0);
         }
       };
-      bool ok = mma_wait(&sm.q_full, 0, abort);
+      ok = mma_wait(&sm.q_full, 0, abort);
       HGA_TRACE_POINT(40);
       bool dq_started = false;
       // ---- dK/dV steps: one at a time, every operand from shared memory.  The tensor pipe runs in
@@ -393,7 +346,7 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       // (2u)%3, dP(u) and later dS(u) in region (2u+1)%3.
       if (ok && n_pairs > 0) {
         if (ok && n_act > 0) mma_commit_w(&sm.phase_a_done);
-        const int ps0 = ps_base;
+        const int ps0 = pair_stage(0);
         if (ok) ok = mma_wait(&sm.kp_full[ps0], 0, abort);
         HGA_TRACE_POINT(43);
         if (ok) {
@@ -410,49 +363,32 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         HGA_TRACE_POINT(3);
       }
       int rs = 0;                                     // region of S(u)
-      for (int u = 0; u < n_pairs && ok; ++u) {
-        constexpr int kPs = kBwdKStages / 2;
-        const int ps = (ps_base + u) % kPs, ps_n = (ps + 1) % kPs;     // pair stages of steps u, u+1
+      for (int u = 0; u + 1 < n_pairs && ok; ++u) {
+        const int ps_n = pair_stage(u + 1);
         const int rp = rs == 2 ? 0 : rs + 1;          // region of dP(u), dS(u)
         const int rs_n = rp == 2 ? 0 : rp + 1;        // region of S(u+1): two steps ago it held dP(u-1)
-        if (u + 1 < n_pairs) {
-          ok = mma_wait(&sm.kp_full[ps_n], (uint32_t)((u + 1) / kPs) & 1, abort);
-          // S(1) is the first to use the region that aliases the dK^T/dV^T accumulators: the
-          // reduction warps must have read the last ones
-          if (ok && u == 0 && n_act > 0) ok = mma_wait(&sm.dkv_free, (n_act - 1) & 1, abort);
-          if (!ok) break;
-          tc_fence_after_sync();
-          issue_qk(tmem + region(rs_n), q_k, k_k0, 2 * ps_n, idesc_sdp2);
-          mma_commit_w(&sm.s_full[(u + 1) & 1]);
-          HGA_TRACE_POINT(6);
-          // dP(u+1) goes into the region of S(u) as soon as the row threads have read S(u) (they keep P in
-          // registers): it is then complete long before they finish dS(u) and P(u+1) and ask for it
-          ok = mma_wait(&sm.s_read[u & 1], (uint32_t)(u >> 1) & 1, abort) &&
-               mma_wait(&sm.vp_full[(u + 1) & 1], (uint32_t)((u + 1) >> 1) & 1, abort);
-          if (!ok) break;
-          tc_fence_after_sync();
-          issue_qk(tmem + region(rs), do_k, ((u + 1) & 1) ? v_k1 : v_k0, 0, idesc_sdp2);
-          mma_commit_w(&sm.dp_full[(u + 1) & 3]);
-          HGA_TRACE_POINT(8);
-        }
-        ok = mma_wait(&sm.ds_full[u & 1], (uint32_t)(u >> 1) & 1, abort);     // the row threads are done with dP(u): dS(u) is in its place
+        ok = mma_wait(&sm.kp_full[ps_n], (uint32_t)((u + 1) / (kBwdKStages / 2)) & 1, abort);
+        // S(1) is the first to use the region that aliases the dK^T/dV^T accumulators: the reduction warps must have
+        // read the last ones; a later S(u+1) overwrites dS(u-1), which dQ(u-1) must have read
+        if (ok && u == 0 && n_act > 0) ok = mma_wait(&sm.dkv_free, (n_act - 1) & 1, abort);
+        if (ok && u > 0) ok = mma_wait(&sm.kp_empty[(u - 1) % kBwdKStages], (uint32_t)((u - 1) / kBwdKStages) & 1, abort);
         if (!ok) break;
         tc_fence_after_sync();
-        HGA_TRACE_POINT(5);
-        // dQ += dS K over 128 keys: bf16 dS from TMEM (first tile at columns 0-31 of its region,
-        // second tile at 64-95), the two K stages as one MN-major B operand
-        const uint64_t kmn = desc_advance(k_mn0, (uint32_t)(2 * ps) * kKvTile);
-        const uint32_t ds_base = tmem + region(rp);
-#pragma unroll
-        for (int kk = 0; kk < 2 * kKT / 16; ++kk)
-          mma_ts_w(tmem + kColDQ, ds_base + (kk < 4 ? 8 * kk : 64 + 8 * (kk - 4)), desc_advance(kmn, kk * 2 * kOct),
-                 idesc_dq, (dq_started || kk > 0));
-        dq_started = true;
-        mma_commit_w(&sm.kp_empty[(ps_base + u) % kBwdKStages]);
-        HGA_TRACE_POINT(7);
+        issue_qk(tmem + region(rs_n), q_k, k_k0, 2 * ps_n, idesc_sdp2);
+        mma_commit_w(&sm.s_full[(u + 1) & 1]);
+        HGA_TRACE_POINT(6);
+        // dP(u+1) goes into the region of S(u) as soon as the row threads have read S(u) (they keep P in
+        // registers): it is then complete long before they finish dS(u) and P(u+1) and ask for it
+        ok = mma_wait(&sm.s_read[u & 1], (uint32_t)(u >> 1) & 1, abort) &&
+             mma_wait(&sm.vp_full[(u + 1) & 1], (uint32_t)((u + 1) >> 1) & 1, abort);
+        if (!ok) break;
+        tc_fence_after_sync();
+        issue_qk(tmem + region(rs), do_k, ((u + 1) & 1) ? v_k1 : v_k0, 0, idesc_sdp2);
+        mma_commit_w(&sm.dp_full[(u + 1) & 3]);
+        HGA_TRACE_POINT(8);
         rs = rs_n;
       }
-      if (ok) mma_commit_w(&sm.dq_done);
+      if (ok && n_pairs == 0) mma_commit_w(&sm.dq_done);
     }
   } else if (warp < 10) {
     // ------------------------------------------------------------------ one thread per query row
@@ -466,7 +402,7 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     const float neg_lse2 = -row_lse * 1.4426950408889634f;
     // delta: this warpgroup's 64-element half of the row's dot product (dO from the tile in shared memory:
     // panel wg, 128-byte line of the row, 16-byte chunks XOR-swizzled), then the sum of the two halves
-    bool ok = __all_sync(0xffffffffu, bwd_wait(&sm.q_full, 0, abort));
+    ok = __all_sync(0xffffffffu, bwd_wait(&sm.q_full, 0, abort));
     {
       float acc[4] = {0.f, 0.f, 0.f, 0.f};
       if (ok) {
@@ -543,7 +479,7 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         }
         tc_fence_before_sync();
         fence_proxy_async_smem();
-        mbar_arrive(&sm.pds_full);
+        mbar_arrive_warp(&sm.pds_full);
         HGA_TRACE_POINT(17);
       }
     }
@@ -562,25 +498,37 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       if (!ok) break;
       tc_fence_after_sync();
       HGA_TRACE_POINT(11);
+      // (the masked copy of the code is for the tiles at the diagonal and the list's end only: with the two comparisons and
+      // selections per element in the common copy, phase 1 was bound by instruction issue)
+      auto phase1 = [&](auto masked) {
 #pragma unroll
-      for (int q4 = 0; q4 < 4; ++q4) {
-        uint32_t sv[16];
-        tmem_ld16(s_addr + q4 * 16, sv);
-        tmem_wait_ld();
+        for (int q4 = 0; q4 < 4; ++q4) {
+          uint32_t sv[16];
+          tmem_ld16(s_addr + q4 * 16, sv);
+          tmem_wait_ld();
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          float a0, a1;            // packed fp32 pairs: one FMA for the two exponent arguments
-          unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(sv[2 * i]), __uint_as_float(sv[2 * i + 1])), sl2_2, neg_lse2_2), a0, a1);
-          float p0 = fast_exp2(a0), p1 = fast_exp2(a1);
-          if (vis < kKT) {
-            if (q4 * 16 + 2 * i >= vis) p0 = 0.f;
-            if (q4 * 16 + 2 * i + 1 >= vis) p1 = 0.f;
+          for (int i = 0; i < 8; ++i) {
+            float p0, p1;            // packed fp32 pairs: one FMA for the two exponent arguments
+            const uint64_t a = fma_f32x2(pack_f32x2(__uint_as_float(sv[2 * i]), __uint_as_float(sv[2 * i + 1])), sl2_2, neg_lse2_2);
+            if (HGA_POLY >> i & 1) {
+              exp2_fma_x2(a, p0, p1);
+            } else {
+              unpack_f32x2(a, p0, p1);
+              p0 = fast_exp2(p0);
+              p1 = fast_exp2(p1);
+            }
+            if (decltype(masked)::value) {
+              if (q4 * 16 + 2 * i >= vis) p0 = 0.f;
+              if (q4 * 16 + 2 * i + 1 >= vis) p1 = 0.f;
+            }
+            pk[8 * q4 + i] = pack_bf16(p0, p1);
           }
-          pk[8 * q4 + i] = pack_bf16(p0, p1);
         }
-      }
+      };
+      if (__any_sync(0xffffffffu, vis < kKT)) phase1(std::true_type{});
+      else phase1(std::false_type{});
       tc_fence_before_sync();
-      mbar_arrive(&sm.s_read[u & 1]);                 // S(u) has been read: its region may take dP(u+1)
+      mbar_arrive_warp(&sm.s_read[u & 1]);                 // S(u) has been read: its region may take dP(u+1)
       ok = __all_sync(0xffffffffu, bwd_wait(&sm.dp_full[u & 3], (u >> 2) & 1, abort));
       if (!ok) break;
       tc_fence_after_sync();
@@ -603,7 +551,7 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       }
       tmem_wait_st();
       tc_fence_before_sync();
-      mbar_arrive(&sm.ds_full[u & 1]);
+      mbar_arrive_warp(&sm.ds_full[u & 1]);
       HGA_TRACE_POINT(14);
       rs = rp == 2 ? 0 : rp + 1;
     }
@@ -632,7 +580,7 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                        pack_bf16(__uint_as_float(x[c][8 * i + 4]), __uint_as_float(x[c][8 * i + 5])),
                        pack_bf16(__uint_as_float(x[c][8 * i + 6]), __uint_as_float(x[c][8 * i + 7])));
       fence_proxy_async_smem();
-      mbar_arrive(&sm.dq_staged);
+      mbar_arrive_warp(&sm.dq_staged);
       if (warp == 2 && lane < 4 && bwd_wait(&sm.dq_staged, 0, abort)) {      // all 256 rows are in shared memory
         const int half = lane & 1, panel = lane >> 1;
         const int r0 = mt * 128 + 64 * half;
@@ -650,58 +598,60 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     const int e = quarter * 32 + lane;                       // head_dim element = TMEM lane
     const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
     const int64_t kv_base = (row_base(dm, sg, b) * dm.Hkv + (int64_t)h * sg.S) * D;
-    bool ok = true;
     // The band kernel, which precedes this one in the stream, stores its dK/dV rows plainly: the adds
     // below must come after it.  Nothing else in this kernel depends on it, so this is the only wait
     // (a no-op unless the launch carried the programmatic-serialization attribute).
     // It is executed even where there is nothing to add: the end of this grid has to imply the end of that one.
     pdl_wait();
-    // The transposed accumulators (lane = element, column = key) go to shared memory as key rows of 512 bytes, 32 keys at a
-    // time in two buffers of 16 KB (the K ring's third pair); an octet of them is 4 KB of consecutive memory on both
+    // The transposed accumulators (lane = element, column = key) go to shared memory as key rows of 512 bytes, 32 keys to
+    // a buffer of 16 KB (the K ring's third pair): dV, then dK; an octet of them is 4 KB of consecutive memory on both
     // sides and is added by one bulk reduction.  (As 128-byte red.global requests, 512 per step, the adds took the SM
-    // 6k cycles to send off, longer than the step's GEMMs: 2K layer, hga_attn_bwd 115 us.)
-    uint32_t staged_phase = 0;
-    auto all_here = [&]() {                 // the 128 threads meet (bounded: one of them may have given up)
-      mbar_arrive(&sm.staged);
-      ok = __all_sync(0xffffffffu, bwd_wait(&sm.staged, staged_phase, abort));
-      staged_phase ^= 1u;
-      return ok;
-    };
-    for (int s = 0; s < n_act && ok; ++s) {
-      const int j = tile_of_step(s);
-      ok = __all_sync(0xffffffffu, bwd_wait(&sm.dkv_full, s & 1, abort));
-      if (!ok) break;
-      tc_fence_after_sync();
-      HGA_TRACE_POINT(16);
-#pragma unroll 1
-      for (int c = 0; c < 4; ++c) {         // dV keys 0-31, 32-63, dK keys 0-31, 32-63
-        const int half = c & 1;
-        uint8_t* const buf = sm.k[kActStages + half];
-        uint32_t x[32];
-        tmem_ld32(lane_base + (c < 2 ? kColDV : kColDK) + half * 32, x);
-        tmem_wait_ld();
-        if (c == 3) {
-          tc_fence_before_sync();
-          mbar_arrive(&sm.dkv_free);
-        }
-        if (s > 0 || c > 1) {
-          // the buffer's last contents have been read (this thread's reduction before the last one)
-          if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-          __syncwarp();
-          if (!all_here()) break;
-        }
-        const uint32_t dst = smem_u32(buf) + (uint32_t)e * 4;
+    // 6k cycles to send off, longer than the step's GEMMs: 2K layer, hga_attn_bwd 115 us.)  dK waits in registers for the
+    // buffers, so that the accumulators are free -- for the next step's GEMMs, and for S of the second pair -- early on.
+    // The four warps meet at hardware barriers, which each of them reaches on every path: a warp that has given up goes
+    // on doing nothing.
+    const uint32_t dst = smem_u32(sm.k[kActStages]) + (uint32_t)e * 4;
+    auto meet = []() { asm volatile("bar.sync 4, 128;" ::: "memory"); };
+    auto reduce = [&](float* to, int j) {
+      if (lane == 0) {                      // two octets per warp (an octet's rows are all in the active segment before the band, or none is)
 #pragma unroll
-        for (int i = 0; i < 32; ++i) st_shared_b32(dst + (uint32_t)i * 512, x[i]);
-        fence_proxy_async_smem();
-        if (!all_here()) break;
-        if (lane == 0) {                    // warp = octet (its rows are all in the active segment before the band, or none is)
+        for (int half = 0; half < 2; ++half) {
           const int o = 8 * j + half * 4 + quarter;
           const int pos = o < n_oct ? sm.oct_row[o] : -1;
-          if (pos >= sg.H && pos < red_hi)
-            bulk_reduce_add_f32((c < 2 ? dV : dK) + kv_base + (int64_t)(pos - sg.H) * D, smem_u32(buf) + quarter * 4096, 4096);
-          tma_store_commit();
+          if (ok && pos >= sg.H && pos < red_hi)
+            bulk_reduce_add_f32(to + kv_base + (int64_t)(pos - sg.H) * D, smem_u32(sm.k[kActStages + half]) + quarter * 4096, 4096);
         }
+        tma_store_commit();
+      }
+    };
+    for (int s = 0; s < n_act; ++s) {
+      const int j = tile_of_step(s);
+      ok = ok && __all_sync(0xffffffffu, bwd_wait(&sm.dkv_full, s & 1, abort));
+      tc_fence_after_sync();
+      HGA_TRACE_POINT(16);
+      uint32_t x[2][32];
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {         // dV, dK
+        if (ok) {
+          tmem_ld32(lane_base + (c ? kColDK : kColDV), x[0]);
+          tmem_ld32(lane_base + (c ? kColDK : kColDV) + 32, x[1]);
+          tmem_wait_ld();
+        }
+        if (c == 1) {
+          tc_fence_before_sync();
+          mbar_arrive_warp(&sm.dkv_free);
+        }
+        // the buffers' last contents have been read
+        if (lane == 0) tma_store_wait_read();
+        __syncwarp();
+        meet();
+#pragma unroll
+        for (int half = 0; half < 2; ++half)
+#pragma unroll
+          for (int i = 0; i < 32; ++i) st_shared_b32(dst + (uint32_t)(half * kKvTile + i * 512), x[half][i]);
+        fence_proxy_async_smem();
+        meet();
+        reduce(c ? dK : dV, j);
       }
       HGA_TRACE_POINT(18);
     }
@@ -711,6 +661,88 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         mbar_arrive(&sm.stage_free);
       }
       __syncwarp();
+    }
+    if (warp == 10 && n_pairs > 0) {
+      // ---- dQ += dS K of the paired steps.  One warp issuing all three GEMMs of a step took longer over it (waits, commits and
+      // 24 instructions, some 60-100 cycles each, one after the other: 3.0k cycles) than the tensor pipe (1.6k) or
+      // the row threads (2.2k) do, so this one, which no other warp waits for within a step, is issued from here.
+      auto mma_wait = [&](uint64_t* bar, uint32_t parity) { return __all_sync(0xffffffffu, bwd_wait(bar, parity, abort)); };
+      constexpr uint32_t idesc_dq = idesc_bf16_f32(128, D, 0, 1);          // dS K-major, K tile MN-major
+      const uint64_t k_mn0 = smem_desc_sw128(smem_u32(sm.k[0]), 1024, kOct);
+      if (ok && n_act > 0) ok = mma_wait(&sm.phase_a_done, 0);              // the accumulator's first GEMMs come from warp 1
+      bool dq_started = n_act > 0;
+      int rp = 1;                                     // region of dS(u)
+      for (int u = 0; u < n_pairs && ok; ++u) {
+        ok = mma_wait(&sm.ds_full[u & 1], (uint32_t)(u >> 1) & 1);          // the row threads are done with dP(u): dS(u) is in its place
+        if (!ok) break;
+        tc_fence_after_sync();
+        HGA_TRACE_POINT(5);
+        // 128 keys: bf16 dS from TMEM (first tile at columns 0-31 of its region, second tile at 64-95), the two K stages
+        // as one MN-major B operand
+        const uint64_t kmn = desc_advance(k_mn0, (uint32_t)(2 * pair_stage(u)) * kKvTile);
+        const uint32_t ds_base = tmem + region(rp);
+#pragma unroll
+        for (int kk = 0; kk < 2 * kKT / 16; ++kk)
+          mma_ts_w(tmem + kColDQ, ds_base + (kk < 4 ? 8 * kk : 64 + 8 * (kk - 4)), desc_advance(kmn, kk * 2 * kOct), idesc_dq,
+                   (dq_started || kk > 0));
+        dq_started = true;
+        mma_commit_w(&sm.kp_empty[u % kBwdKStages]);
+        HGA_TRACE_POINT(7);
+        rp = rp == 0 ? 2 : rp - 1;                    // (two regions on)
+      }
+      if (ok) mma_commit_w(&sm.dq_done);
+    }
+  }
+  if (warp == 0 || warp > 10) {
+    // ------------------------------------------------------------------ producers of the paired steps
+    // Pair p fills stages 2*ps, 2*ps+1 (ps continues the slot numbering) and completes ONE barrier per operand, so the
+    // MMA thread observes one barrier per operand and pair.  The first two pairs are copied by warp 0 (K: 16 boxes) and
+    // warps 14 and 15 (V: 8 each) while the dK/dV steps run; from then on the reduction warps, idle by now, share the
+    // issuing (K: warps 0 and 11, V: warps 14, 15, 12, 13): a K pair can be asked for only when dQ of the pair three
+    // before it is done, and one warp took 1.3-1.9k cycles over its 16 boxes, more than half of a step.
+    const bool is_v = warp > 11, helper = warp != 0 && warp < 14;
+    const CUtensorMap* map = is_v ? &map_v : &map_k;
+    const int part = warp == 0 ? 0 : (warp == 11 ? 1 : (warp - 14) & 3);     // of the boxes of a pair
+    for (int p = helper ? 2 : 0; p < n_pairs && ok; ++p) {
+      // K: three pairs of stages, continuing the slot numbering.  V: two pairs, pair p in slot p & 1; slot 0
+      // is the V ring, slot 1 the P and dS tiles (adjacent, one K/V tile each), which only the dK/dV steps
+      // use otherwise.  A V pair is free once its dP GEMM is done, a K pair only after its dQ GEMM.
+      const int ps = is_v ? (p & 1) : pair_stage(p);
+      uint64_t* full = is_v ? &sm.vp_full[ps] : &sm.kp_full[ps];
+      const int n_mine = (is_v ? 8 : 16) >> (p < 2 ? 0 : 1);           // boxes of this warp
+      const int box = part * n_mine + lane;                            // octet of the pair
+      int row = dm.rows_k;
+      const int o = box < 16 ? 8 * tile_of_step(n_act + 2 * p + (box >> 3)) + (box & 7) : n_oct;
+      if (n_act + 2 * p + (box >> 3) < n_tiles && o < n_oct) row = sg.k0 + sm.oct_row[o];
+      if (lane == 0) {
+        if (is_v) {
+          // first pair: the V ring is free from the start; second: the dK/dV steps (which use the P and dS
+          // tiles) must be over; later: dP of pair p-2 is done
+          if (p < 2) { if (p == 1 && n_act > 0) ok = bwd_wait(&sm.phase_a_done, 0, abort); }
+          else ok = bwd_wait(&sm.dp_full[(p - 2) & 3], (uint32_t)((p - 2) >> 2) & 1, abort);
+        } else if (p < kBwdKStages / 2) {
+          // first paired use of these stages: if a dK/dV step used them, those steps must be over, and what
+          // was staged in the third pair on its way
+          if (ps == 2 && n_act > 0) ok = bwd_wait(&sm.stage_free, 0, abort);
+          else if (ps < n_act) ok = bwd_wait(&sm.phase_a_done, 0, abort);
+        } else {
+          ok = bwd_wait(&sm.kp_empty[(p - 3) % kBwdKStages], (uint32_t)((p - 3) / kBwdKStages) & 1, abort);   // dQ of pair p-3 is done
+        }
+      }
+      ok = __shfl_sync(0xffffffffu, ok, 0);
+      if (!ok) break;
+      // (the helpers' bytes are expected by the others: a phase cannot complete without those arrivals)
+      if (lane == 0 && !helper) mbar_arrive_expect_tx(full, (uint32_t)(is_v ? 8 : 16) * kOct);
+      __syncwarp();
+      if (lane < n_mine)
+        tma_load_5d((is_v ? (ps == 0 ? sm.v[0] : sm.p) : sm.k[2 * ps]) + box * kOct, map, full, 0, row, 0, h, b);
+      HGA_TRACE_POINT(2);
+    }
+    if (*abort && lane == 0) {
+      // giving up: give the copies still in flight time to land before shared memory is released
+      // (the full barriers may never complete once another role has stopped, hence a bounded sleep)
+      if (warp == 0) mbar_wait(&sm.q_full, 0);
+      for (int it = 0; it < 64; ++it) __nanosleep(1000);
     }
   }
   HGA_TRACE_POINT(30);

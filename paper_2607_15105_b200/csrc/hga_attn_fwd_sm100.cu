@@ -147,8 +147,8 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   if (warp == 0 && lane == 0) {
     mbar_init(&sm.q_full, 1);
     mbar_init(&sm.k_full, 2); mbar_init(&sm.v_full, 2); mbar_init(&sm.v_empty, 1);
-    mbar_init(&sm.s_full, 1); mbar_init(&sm.p_full[0], 256); mbar_init(&sm.p_full[1], 256);
-    mbar_init(&sm.info_full, 1); mbar_init(&sm.o_done, 1); mbar_init(&sm.o_staged, 256); mbar_init(&sm.drain, 1);
+    mbar_init(&sm.s_full, 1); mbar_init(&sm.p_full[0], 8); mbar_init(&sm.p_full[1], 8);
+    mbar_init(&sm.info_full, 1); mbar_init(&sm.o_done, 1); mbar_init(&sm.o_staged, 8); mbar_init(&sm.drain, 1);
     sm.abort = 0;
     fence_barrier_init();
   }
@@ -415,7 +415,7 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           tmem_wait_st();
         }
         tc_fence_before_sync();
-        mbar_arrive(&sm.p_full[c]);
+        mbar_arrive_warp(&sm.p_full[c]);
       }
       float x0, x1;
       unpack_f32x2(lsum, x0, x1);
@@ -489,7 +489,7 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     }
     if (boxes) {
       fence_proxy_async_smem();
-      mbar_arrive(&sm.o_staged);
+      mbar_arrive_warp(&sm.o_staged);
       if (ok && warp == 4 && lane < 2 * kPanels && bwd_wait(&sm.o_staged, 0, abort)) {      // all rows are in shared memory
         const int hf = lane & 1, panel = lane >> 1, r0 = mt0 * 128 + 64 * hf;
         if (r0 < dm.rows) {

@@ -151,7 +151,7 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
     if (lane == 0) {
       mbar_init(&sm.q_full, 1);
       for (int s = 0; s < NSTG; ++s) { mbar_init(&sm.a_full[s], 1); mbar_init(&sm.a_empty[s], 1); }
-      for (int s = 0; s < ACCS; ++s) { mbar_init(&sm.acc_full[s], 1); mbar_init(&sm.acc_free[s], 128); }
+      for (int s = 0; s < ACCS; ++s) { mbar_init(&sm.acc_full[s], 1); mbar_init(&sm.acc_free[s], 4); }
       mbar_init(&sm.drain, 1);
       sm.abort = 0;
       fence_barrier_init();
@@ -336,7 +336,7 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
               }
             }
             tc_fence_before_sync();
-            mbar_arrive(&sm.acc_free[acc]);
+            mbar_arrive_warp(&sm.acc_free[acc]);
           }
           if (!ok) break;
           if (agg == 1) best = sum * (1.f / (float)dm.rows);

@@ -30,6 +30,13 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
+// One arrival for a whole (converged) warp, after all its lanes: 32 arrivals of one instruction are 32 updates of the barrier
+// in turn, which kept whoever waited for eight warps waiting for a few hundred cycles more.
+__device__ __forceinline__ void mbar_arrive_warp(uint64_t* bar) {
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
+}
+
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
                : "memory");
@@ -369,6 +376,28 @@ __device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
   uint64_t d;
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
+}
+
+// 2^x of two values on the FMA pipe, for kernels whose exponentials would otherwise queue for the special-function unit (16 a
+// cycle and SM): x = n + f with n the nearest integer (found by adding and subtracting 1.5 * 2^23) and |f| <= 1/2; 2^f by its
+// degree-5 minimax polynomial (Remez exchange for the relative error: 7.5e-8, 2.1e-7 evaluated in fp32, as accurate as
+// ex2.approx); n is added to the exponent field.  x must be at most 127; below -126 the result is that of -126.
+__device__ __forceinline__ void exp2_fma_x2(uint64_t x, float& p0, float& p1) {
+  float x0, x1, t0, t1;
+  unpack_f32x2(x, x0, x1);
+  x = pack_f32x2(fmaxf(x0, -126.f), fmaxf(x1, -126.f));
+  const uint64_t t = add_f32x2(x, pack_f32x2(12582912.f, 12582912.f));
+  const uint64_t n = add_f32x2(t, pack_f32x2(-12582912.f, -12582912.f));
+  const uint64_t f = fma_f32x2(n, pack_f32x2(-1.f, -1.f), x);
+  uint64_t p = fma_f32x2(pack_f32x2(0.00132764725f, 0.00132764725f), f, pack_f32x2(0.00967554096f, 0.00967554096f));
+  p = fma_f32x2(p, f, pack_f32x2(0.0555071309f, 0.0555071309f));
+  p = fma_f32x2(p, f, pack_f32x2(0.240221202f, 0.240221202f));
+  p = fma_f32x2(p, f, pack_f32x2(0.693146944f, 0.693146944f));
+  p = fma_f32x2(p, f, pack_f32x2(1.00000012f, 1.00000012f));
+  unpack_f32x2(p, p0, p1);
+  unpack_f32x2(t, t0, t1);
+  p0 = __uint_as_float(__float_as_uint(p0) + (__float_as_uint(t0) << 23));
+  p1 = __uint_as_float(__float_as_uint(p1) + (__float_as_uint(t1) << 23));
 }
 
 }  // namespace sm100
