@@ -221,6 +221,7 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
     // The whole warp runs this branch converged (waits included) and one elected lane issues: see mma_ss_w.
+    const uint32_t lead = elect_one();
     {
       auto mma_wait = [&](uint64_t* bar, uint32_t parity, volatile int* ab) {
         return __all_sync(0xffffffffu, bwd_wait(bar, parity, ab));
@@ -241,7 +242,7 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
 #pragma unroll
         for (int kk = 0; kk < kD / 16; ++kk) {
           const uint32_t off = (kk >> 2) * 16384 + (kk & 3) * 32;       // panel, then 32-byte K step
-          mma_ss_w(acc, desc_advance(a, off), desc_advance(bq, off), idesc_t, kk > 0);
+          mma_ss_w(lead, acc, desc_advance(a, off), desc_advance(bq, off), idesc_t, kk > 0);
         }
       };
       // acc (keys x head_dim) += a (keys x 64 rows, bf16 in TMEM: rows 0-31 at columns 0-15, rows 32-63 at
@@ -249,7 +250,7 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
       auto issue_g = [&](uint32_t acc, uint32_t a_tmem, uint64_t bmn, bool accumulate) {
 #pragma unroll
         for (int kk = 0; kk < 64 / 16; ++kk)
-          mma_ts_w(acc, a_tmem + (kk < 2 ? 8 * kk : 32 + 8 * (kk - 2)), desc_advance(bmn, kk * 2048), idesc_g,
+          mma_ts_w(lead, acc, a_tmem + (kk < 2 ? 8 * kk : 32 + 8 * (kk - 2)), desc_advance(bmn, kk * 2048), idesc_g,
                    (accumulate || kk > 0));
       };
       // S^T and dP^T of half-step hf of the M-tile in ring stage st, into region hf
@@ -257,7 +258,7 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
         const uint32_t region = tmem + hf * kRegion, off = st * kTile + hf * 8192;
         issue_t(region + kColS, k_k, desc_advance(q_k0, off));
         issue_t(region + kColDP, v_k, desc_advance(do_k0, off));
-        mma_commit_w(&sm.sdp_full[hf]);
+        mma_commit_w(lead, &sm.sdp_full[hf]);
       };
       const int n_half = 2 * n_steps;
       bool ok = mma_wait(&sm.kv_full, 0, abort);
@@ -278,7 +279,7 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
         const uint32_t region = tmem + hf * kRegion, off = st * kTile + hf * 8192;
         issue_g(tmem + kColDV, region + kColS, desc_advance(do_mn0, off), hs > 0);
         issue_g(tmem + kColDK, region + kColDP, desc_advance(q_mn0, off), hs > 0);
-        mma_commit_w(&sm.qdo_empty[st][hf]);                     // these 64 rows of Q and dO are consumed
+        mma_commit_w(lead, &sm.qdo_empty[st][hf]);                     // these 64 rows of Q and dO are consumed
         if (hs + 2 < n_half) {
           // the same half of the next M-tile reuses this region: the in-order tensor pipe runs its GEMMs after
           // the two above, which read P^T and dS^T from it
@@ -290,7 +291,7 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
         }
         HGA_TRACE_POINT(7);
       }
-      if (ok) mma_commit_w(&sm.acc_done);
+      if (ok) mma_commit_w(lead, &sm.acc_done);
     }
   } else if (warp < 10) {
     // ------------------------------------------------------------------ one thread per key
@@ -490,7 +491,7 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
   if (warp == 1 && sm.abort) {
     // giving up: GEMMs already issued may still be writing tensor memory; wait (bounded) until the
     // tensor pipe has run dry before the columns are given back
-    mma_commit_w(&sm.drain);
+    mma_commit_w(elect_one(), &sm.drain);
     mbar_wait(&sm.drain, 0);
   }
   __syncwarp();

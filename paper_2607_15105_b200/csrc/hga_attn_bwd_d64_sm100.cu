@@ -246,6 +246,7 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
     // The whole warp runs this branch converged (waits included) and one elected lane issues: see mma_ss_w.
+    const uint32_t lead = elect_one();
     auto mma_wait = [&](uint64_t* bar, uint32_t parity) {
       return __all_sync(0xffffffffu, bwd_wait(bar, parity, abort));
     };
@@ -266,16 +267,16 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
     auto issue_qk = [&](uint32_t acc, uint64_t a, uint64_t bd) {
 #pragma unroll
       for (int kk = 0; kk < D / 16; ++kk) {
-        mma_ss_w(acc, desc_advance(a, kk * 32), desc_advance(bd, kk * 32), idesc_sdp, kk > 0);
+        mma_ss_w(lead, acc, desc_advance(a, kk * 32), desc_advance(bd, kk * 32), idesc_sdp, kk > 0);
       }
     };
     auto issue_s = [&](int j) {
       issue_qk(tmem + kColS, q_k, desc_advance(k_k0, (uint32_t)(j & 1) * kKv));
-      mma_commit_w(&sm.s_full);
+      mma_commit_w(lead, &sm.s_full);
     };
     auto issue_dp = [&]() {
       issue_qk(tmem + kColDP, do_k, v_k);
-      mma_commit_w(&sm.dp_full);           // also tells the producers that the V tile is free
+      mma_commit_w(lead, &sm.dp_full);           // also tells the producers that the V tile is free
     };
     bool ok = mma_wait(&sm.q_full, 0) && mma_wait(&sm.k_full[0], 0);
     HGA_TRACE_POINT(40);
@@ -311,8 +312,8 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
         HGA_TRACE_POINT(5);
 #pragma unroll
         for (int kk = 0; kk < kKT / 16; ++kk)     // 16 keys per MMA: 8 TMEM columns of dS, two octets of the K tile
-          mma_ts_w(tmem + kColDQ, tmem + kColDP + 8 * kk, desc_advance(kmn, kk * 2 * kOct), idesc_dq, (j > 0 || kk > 0));
-        mma_commit_w(&sm.k_empty[j & 1]);
+          mma_ts_w(lead, tmem + kColDQ, tmem + kColDP + 8 * kk, desc_advance(kmn, kk * 2 * kOct), idesc_dq, (j > 0 || kk > 0));
+        mma_commit_w(lead, &sm.k_empty[j & 1]);
         HGA_TRACE_POINT(7);
         if (j + 1 < n) {
           if (!s_ahead) {
@@ -334,14 +335,14 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
         HGA_TRACE_POINT(45);
 #pragma unroll
         for (int kk = 0; kk < kKT / 16; ++kk)
-          mma_ss_w(tmem + kColDQ, desc_advance(dsd, kk * 32), desc_advance(kmn, kk * 2 * kOct), idesc_dq, (j > 0 || kk > 0));
+          mma_ss_w(lead, tmem + kColDQ, desc_advance(dsd, kk * 32), desc_advance(kmn, kk * 2 * kOct), idesc_dq, (j > 0 || kk > 0));
 #pragma unroll
         for (int kk = 0; kk < 128 / 16; ++kk)     // 16 query rows per MMA (2 row octets)
-          mma_ss_w(tmem + kColS, desc_advance(doq_mn, kk * 2048), desc_advance(pd, kk * 2048), idesc_dkv, kk > 0);
+          mma_ss_w(lead, tmem + kColS, desc_advance(doq_mn, kk * 2048), desc_advance(pd, kk * 2048), idesc_dkv, kk > 0);
 #pragma unroll
         for (int kk = 0; kk < 128 / 16; ++kk)
-          mma_ss_w(tmem + kColDP, desc_advance(doq_mn, kk * 2048), desc_advance(dsd, kk * 2048), idesc_dkv, kk > 0);
-        mma_commit_w(&sm.dkv_full);
+          mma_ss_w(lead, tmem + kColDP, desc_advance(doq_mn, kk * 2048), desc_advance(dsd, kk * 2048), idesc_dkv, kk > 0);
+        mma_commit_w(lead, &sm.dkv_full);
         HGA_TRACE_POINT(4);
         if (j + 1 < n) {
           // the row threads have read dV^T: S(j+1) may take its place; then dK^T: dP(j+1)
@@ -356,7 +357,7 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
         }
       }
     }
-    if (ok) mma_commit_w(&sm.dq_done);
+    if (ok) mma_commit_w(lead, &sm.dq_done);
   } else if (warp == 6) {
     // ------------------------------------------------------------------ routing list
     FarList far(dm, w, group_idx + item * dm.width);
@@ -574,7 +575,7 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
   if (warp == 1 && sm.abort) {
     // giving up: GEMMs already issued may still be writing tensor memory; wait (bounded) until the tensor pipe has run
     // dry before the columns are given back
-    mma_commit_w(&sm.drain);
+    mma_commit_w(elect_one(), &sm.drain);
     mbar_wait(&sm.drain, 0);
   }
   __syncwarp();

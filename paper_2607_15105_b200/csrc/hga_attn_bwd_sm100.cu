@@ -49,9 +49,6 @@
 #include <cstddef>
 #include <type_traits>
 
-#ifndef HGA_POLY
-#define HGA_POLY 0
-#endif
 namespace hga {
 
 using namespace sm100;
@@ -267,6 +264,7 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
     // The whole warp runs this branch converged (waits included) and one elected lane issues: see mma_ss_w.
+    const uint32_t lead = elect_one();
     {
       auto mma_wait = [&](uint64_t* bar, uint32_t parity, volatile int* ab) {
         return __all_sync(0xffffffffu, bwd_wait(bar, parity, ab));
@@ -295,7 +293,7 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk) {
           const uint32_t a_off = (kk >> 2) * 16384 + (kk & 3) * 32, b_off = (kk >> 2) * 1024 + (kk & 3) * 32;
-          mma_ss_w(acc, desc_advance(a, a_off), desc_advance(bd, b_off), idesc, kk > 0);
+          mma_ss_w(lead, acc, desc_advance(a, a_off), desc_advance(bd, b_off), idesc, kk > 0);
         }
       };
       ok = mma_wait(&sm.q_full, 0, abort);
@@ -314,8 +312,8 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         tc_fence_after_sync();
         issue_qk(tmem + region(0), q_k, k_k0, st, idesc_sdp);
         issue_qk(tmem + region(0) + 64, do_k, k_k0, vst, idesc_sdp);
-        mma_commit_w(&sm.sdp_full);
-        mma_commit_w(&sm.k_empty[vst]);
+        mma_commit_w(lead, &sm.sdp_full);
+        mma_commit_w(lead, &sm.k_empty[vst]);
         HGA_TRACE_POINT(44);
         ok = mma_wait(&sm.pds_full, s & 1, abort);
         if (!ok) break;
@@ -324,7 +322,7 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         const uint64_t kmn = desc_advance(k_mn0, (uint32_t)st * kKvTile);
 #pragma unroll
         for (int kk = 0; kk < kKT / 16; ++kk)   // dQ += dS K : 16 keys per MMA
-          mma_ss_w(tmem + kColDQ, desc_advance(dsd, kk * 32), desc_advance(kmn, kk * 2 * kOct), idesc_dq,
+          mma_ss_w(lead, tmem + kColDQ, desc_advance(dsd, kk * 32), desc_advance(kmn, kk * 2 * kOct), idesc_dq,
                  (dq_started || kk > 0));
         dq_started = true;
         if (s > 0) {
@@ -334,31 +332,31 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         }
 #pragma unroll
         for (int kk = 0; kk < 128 / 16; ++kk)    // 16 query rows per MMA (2 row octets)
-          mma_ss_w(tmem + kColDV, desc_advance(do_mn, kk * 2048), desc_advance(pd, kk * 2048), idesc_dkv, kk > 0);
+          mma_ss_w(lead, tmem + kColDV, desc_advance(do_mn, kk * 2048), desc_advance(pd, kk * 2048), idesc_dkv, kk > 0);
 #pragma unroll
         for (int kk = 0; kk < 128 / 16; ++kk)
-          mma_ss_w(tmem + kColDK, desc_advance(q_mn, kk * 2048), desc_advance(dsd, kk * 2048), idesc_dkv, kk > 0);
-        mma_commit_w(&sm.dkv_full);
-        mma_commit_w(&sm.k_empty[st]);
+          mma_ss_w(lead, tmem + kColDK, desc_advance(q_mn, kk * 2048), desc_advance(dsd, kk * 2048), idesc_dkv, kk > 0);
+        mma_commit_w(lead, &sm.dkv_full);
+        mma_commit_w(lead, &sm.k_empty[st]);
         HGA_TRACE_POINT(4);
       }
       // ---- paired steps.  Step u covers ring stages st, st+1 (contiguous); S(u) lives in region
       // (2u)%3, dP(u) and later dS(u) in region (2u+1)%3.
       if (ok && n_pairs > 0) {
-        if (ok && n_act > 0) mma_commit_w(&sm.phase_a_done);
+        if (ok && n_act > 0) mma_commit_w(lead, &sm.phase_a_done);
         const int ps0 = pair_stage(0);
         if (ok) ok = mma_wait(&sm.kp_full[ps0], 0, abort);
         HGA_TRACE_POINT(43);
         if (ok) {
           tc_fence_after_sync();
           issue_qk(tmem + region(0), q_k, k_k0, 2 * ps0, idesc_sdp2);
-          mma_commit_w(&sm.s_full[0]);
+          mma_commit_w(lead, &sm.s_full[0]);
         }
         if (ok) ok = mma_wait(&sm.vp_full[0], 0, abort);
         if (ok) {
           tc_fence_after_sync();
           issue_qk(tmem + region(1), do_k, v_k0, 0, idesc_sdp2);
-          mma_commit_w(&sm.dp_full[0]);    // also tells the V producers that the V pair is free
+          mma_commit_w(lead, &sm.dp_full[0]);    // also tells the V producers that the V pair is free
         }
         HGA_TRACE_POINT(3);
       }
@@ -375,7 +373,7 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         if (!ok) break;
         tc_fence_after_sync();
         issue_qk(tmem + region(rs_n), q_k, k_k0, 2 * ps_n, idesc_sdp2);
-        mma_commit_w(&sm.s_full[(u + 1) & 1]);
+        mma_commit_w(lead, &sm.s_full[(u + 1) & 1]);
         HGA_TRACE_POINT(6);
         // dP(u+1) goes into the region of S(u) as soon as the row threads have read S(u) (they keep P in
         // registers): it is then complete long before they finish dS(u) and P(u+1) and ask for it
@@ -384,11 +382,11 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         if (!ok) break;
         tc_fence_after_sync();
         issue_qk(tmem + region(rs), do_k, ((u + 1) & 1) ? v_k1 : v_k0, 0, idesc_sdp2);
-        mma_commit_w(&sm.dp_full[(u + 1) & 3]);
+        mma_commit_w(lead, &sm.dp_full[(u + 1) & 3]);
         HGA_TRACE_POINT(8);
         rs = rs_n;
       }
-      if (ok && n_pairs == 0) mma_commit_w(&sm.dq_done);
+      if (ok && n_pairs == 0) mma_commit_w(lead, &sm.dq_done);
     }
   } else if (warp < 10) {
     // ------------------------------------------------------------------ one thread per query row
@@ -510,13 +508,9 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           for (int i = 0; i < 8; ++i) {
             float p0, p1;            // packed fp32 pairs: one FMA for the two exponent arguments
             const uint64_t a = fma_f32x2(pack_f32x2(__uint_as_float(sv[2 * i]), __uint_as_float(sv[2 * i + 1])), sl2_2, neg_lse2_2);
-            if (HGA_POLY >> i & 1) {
-              exp2_fma_x2(a, p0, p1);
-            } else {
-              unpack_f32x2(a, p0, p1);
-              p0 = fast_exp2(p0);
-              p1 = fast_exp2(p1);
-            }
+            unpack_f32x2(a, p0, p1);
+            p0 = fast_exp2(p0);
+            p1 = fast_exp2(p1);
             if (decltype(masked)::value) {
               if (q4 * 16 + 2 * i >= vis) p0 = 0.f;
               if (q4 * 16 + 2 * i + 1 >= vis) p1 = 0.f;
@@ -666,6 +660,7 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       // ---- dQ += dS K of the paired steps.  One warp issuing all three GEMMs of a step took longer over it (waits, commits and
       // 24 instructions, some 60-100 cycles each, one after the other: 3.0k cycles) than the tensor pipe (1.6k) or
       // the row threads (2.2k) do, so this one, which no other warp waits for within a step, is issued from here.
+      const uint32_t lead = elect_one();
       auto mma_wait = [&](uint64_t* bar, uint32_t parity) { return __all_sync(0xffffffffu, bwd_wait(bar, parity, abort)); };
       constexpr uint32_t idesc_dq = idesc_bf16_f32(128, D, 0, 1);          // dS K-major, K tile MN-major
       const uint64_t k_mn0 = smem_desc_sw128(smem_u32(sm.k[0]), 1024, kOct);
@@ -683,14 +678,14 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         const uint32_t ds_base = tmem + region(rp);
 #pragma unroll
         for (int kk = 0; kk < 2 * kKT / 16; ++kk)
-          mma_ts_w(tmem + kColDQ, ds_base + (kk < 4 ? 8 * kk : 64 + 8 * (kk - 4)), desc_advance(kmn, kk * 2 * kOct), idesc_dq,
+          mma_ts_w(lead, tmem + kColDQ, ds_base + (kk < 4 ? 8 * kk : 64 + 8 * (kk - 4)), desc_advance(kmn, kk * 2 * kOct), idesc_dq,
                    (dq_started || kk > 0));
         dq_started = true;
-        mma_commit_w(&sm.kp_empty[u % kBwdKStages]);
+        mma_commit_w(lead, &sm.kp_empty[u % kBwdKStages]);
         HGA_TRACE_POINT(7);
         rp = rp == 0 ? 2 : rp - 1;                    // (two regions on)
       }
-      if (ok) mma_commit_w(&sm.dq_done);
+      if (ok) mma_commit_w(lead, &sm.dq_done);
     }
   }
   if (warp == 0 || warp > 10) {

@@ -255,6 +255,7 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
     // The whole warp runs this branch converged (waits included) and one elected lane issues: see mma_ss_w.
+    const uint32_t lead = elect_one();
     auto mma_wait = [&](uint64_t* bar, uint32_t parity) {
       return __all_sync(0xffffffffu, bwd_wait(bar, parity, abort));
     };
@@ -270,15 +271,15 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       const uint32_t idesc = whole ? idesc_s : idesc_s_half;
 #pragma unroll
       for (int kk = 0; kk < D / 16; ++kk)
-        mma_ss_w(tmem, desc_advance(q_desc, (kk >> 2) * q_panel + (kk & 3) * 32), desc_advance(k_desc, (kk >> 2) * 1024 + (kk & 3) * 32),
+        mma_ss_w(lead, tmem, desc_advance(q_desc, (kk >> 2) * q_panel + (kk & 3) * 32), desc_advance(k_desc, (kk >> 2) * 1024 + (kk & 3) * 32),
                  idesc, kk > 0);
-      mma_commit_w(&sm.s_full);                    // also tells the producers that the K tile is free
+      mma_commit_w(lead, &sm.s_full);                    // also tells the producers that the K tile is free
     };
     // half hf of a tile: 16 keys per step; P of keys 32i .. 32i+31 sits at columns 32i .. 32i+15
     auto issue_pv = [&](int hf, bool accumulate) {
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk)
-        mma_ts_w(o_acc, tmem + 64 * hf + (kk >> 1) * 32 + (kk & 1) * 8, desc_advance(v_desc, (uint32_t)(4 * hf + kk) * 2 * kOct), idesc_o,
+        mma_ts_w(lead, o_acc, tmem + 64 * hf + (kk >> 1) * 32 + (kk & 1) * 8, desc_advance(v_desc, (uint32_t)(4 * hf + kk) * 2 * kOct), idesc_o,
                  (accumulate || kk > 0));
     };
     int n_oct = 16 * n_pre + 1;                    // (enough until the list is known)
@@ -311,7 +312,7 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         tc_fence_after_sync();
         issue_pv(1, true);
       }
-      mma_commit_w(more ? &sm.v_empty : &sm.o_done);
+      mma_commit_w(lead, more ? &sm.v_empty : &sm.o_done);
       HGA_TRACE_POINT(7);
       if (!more) break;
       ok = mma_wait(&sm.k_full, (j + 1) & 1);      // S(j+1) takes the columns P(j) sat in: ordered after P V of tile j
@@ -508,7 +509,7 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   if (warp == 1 && sm.abort) {
     // giving up: GEMMs already issued may still be writing tensor memory; wait (bounded) until the tensor pipe has run
     // dry before the columns are given back
-    mma_commit_w(&sm.drain);
+    mma_commit_w(elect_one(), &sm.drain);
     mbar_wait(&sm.drain, 0);
   }
   __syncwarp();

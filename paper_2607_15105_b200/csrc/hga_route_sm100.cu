@@ -240,6 +240,7 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
       } else if (warp == 1) {
         // ---------------------------------------------------------------- MMA issuer
         // The whole warp runs this branch converged (waits included) and one elected lane issues: see mma_ss_w.
+        const uint32_t lead = elect_one();
         auto mma_wait = [&](uint64_t* bar, uint32_t parity) {
           return __all_sync(0xffffffffu, rt_wait(bar, parity, abort));
         };
@@ -267,10 +268,10 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
                 const uint64_t bd = desc_advance(b_desc, (uint32_t)part * part_bytes + pn * q_panel);
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk)
-                  mma_ss_w(tmem + acc * 128, desc_advance(ad, kk * 32), desc_advance(bd, kk * 32), idesc, (pn > 0 || kk > 0));
-                if (pn == kPanels - 1) mma_commit_w(&sm.acc_full[acc]);
+                  mma_ss_w(lead, tmem + acc * 128, desc_advance(ad, kk * 32), desc_advance(bd, kk * 32), idesc, (pn > 0 || kk > 0));
+                if (pn == kPanels - 1) mma_commit_w(lead, &sm.acc_full[acc]);
               }
-              if (ok && p1 == lay.parts) mma_commit_w(&sm.a_empty[s]);
+              if (ok && p1 == lay.parts) mma_commit_w(lead, &sm.a_empty[s]);
             }
           }
         }
@@ -515,7 +516,7 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
     if (warp == 1) {
       // GEMMs the warp's issuing lane started may still be writing tensor memory: a commit completes once
       // every earlier MMA of that lane has, so wait for one (bounded) before the columns are given back
-      mma_commit_w(&sm.drain);
+      mma_commit_w(elect_one(), &sm.drain);
       mbar_wait(&sm.drain, 0);
     }
   }

@@ -283,68 +283,51 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N, int a_mn_maj
          ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-// D[tmem] (+)= A[smem] * B[smem]; issued by one thread.
-__device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                       uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
-// D[tmem] (+)= A[tmem] * B[smem]; A is K-major in tensor memory (lane = row, 2 bf16 per column).
-__device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
-                                       uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
-// Warp-wide forms: called by ALL 32 lanes of the issuing warp (converged); one elected lane issues the
-// instruction.  Because every lane computes the (identical) descriptors, the compiler keeps them in the
-// warp-uniform datapath, which is where the tensor-core instructions take their operands from; a lone
-// thread inside a divergent branch pays a register-file-to-uniform transfer for every operand of every MMA.
-__device__ __forceinline__ void mma_ss_w(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                         uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p, e;\n\t"
-      "elect.sync _|e, 0xffffffff;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-__device__ __forceinline__ void mma_ts_w(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
-                                         uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p, e;\n\t"
-      "elect.sync _|e, 0xffffffff;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-// (the elected lane is the same one every time for a full, converged warp, so this commit covers the
-// MMAs issued through the two wrappers above)
-__device__ __forceinline__ void mma_commit_w(uint64_t* bar) {
+// Tensor-core instructions are issued by ALL 32 lanes of a converged warp, predicated on one elected lane (`lead`): because
+// every lane computes the (identical) descriptors, the compiler keeps them in the warp-uniform datapath, which is where
+// the instructions take their operands from; a lone thread inside a divergent branch pays a register-file-to-uniform
+// transfer for every operand.  The lane is elected once per role: with an election per instruction an MMA took its warp 77
+// cycles to issue next to 16 busy warps, more than the 64 it keeps the tensor pipe busy for (128 x 128 x 16); now 49.
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t lead;
   asm volatile(
       "{\n\t.reg .pred e;\n\t"
       "elect.sync _|e, 0xffffffff;\n\t"
-      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
-      ::"r"(smem_u32(bar))
-      : "memory");
+      "selp.b32 %0, 1, 0, e;\n\t}"
+      : "=r"(lead));
+  return lead;
 }
 
-// Make `bar` complete (one arrival) when every MMA issued so far by this thread has finished.
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                   smem_u32(bar))
-               : "memory");
+// D[tmem] (+)= A[smem] * B[smem]
+__device__ __forceinline__ void mma_ss_w(uint32_t lead, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                         uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p, e;\n\t"
+      "setp.ne.b32 e, %5, 0;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(lead)
+      : "memory");
+}
+// D[tmem] (+)= A[tmem] * B[smem]; A is K-major in tensor memory (lane = row, 2 bf16 per column).
+__device__ __forceinline__ void mma_ts_w(uint32_t lead, uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
+                                         uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p, e;\n\t"
+      "setp.ne.b32 e, %5, 0;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(lead)
+      : "memory");
+}
+// makes the mbarrier track completion of all MMAs this lane has issued so far
+__device__ __forceinline__ void mma_commit_w(uint32_t lead, uint64_t* bar) {
+  asm volatile(
+      "{\n\t.reg .pred e;\n\t"
+      "setp.ne.b32 e, %1, 0;\n\t"
+      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+      ::"r"(smem_u32(bar)), "r"(lead)
+      : "memory");
 }
 
 __device__ __forceinline__ float fast_exp2(float x) {
@@ -376,28 +359,6 @@ __device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
   uint64_t d;
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
-}
-
-// 2^x of two values on the FMA pipe, for kernels whose exponentials would otherwise queue for the special-function unit (16 a
-// cycle and SM): x = n + f with n the nearest integer (found by adding and subtracting 1.5 * 2^23) and |f| <= 1/2; 2^f by its
-// degree-5 minimax polynomial (Remez exchange for the relative error: 7.5e-8, 2.1e-7 evaluated in fp32, as accurate as
-// ex2.approx); n is added to the exponent field.  x must be at most 127; below -126 the result is that of -126.
-__device__ __forceinline__ void exp2_fma_x2(uint64_t x, float& p0, float& p1) {
-  float x0, x1, t0, t1;
-  unpack_f32x2(x, x0, x1);
-  x = pack_f32x2(fmaxf(x0, -126.f), fmaxf(x1, -126.f));
-  const uint64_t t = add_f32x2(x, pack_f32x2(12582912.f, 12582912.f));
-  const uint64_t n = add_f32x2(t, pack_f32x2(-12582912.f, -12582912.f));
-  const uint64_t f = fma_f32x2(n, pack_f32x2(-1.f, -1.f), x);
-  uint64_t p = fma_f32x2(pack_f32x2(0.00132764725f, 0.00132764725f), f, pack_f32x2(0.00967554096f, 0.00967554096f));
-  p = fma_f32x2(p, f, pack_f32x2(0.0555071309f, 0.0555071309f));
-  p = fma_f32x2(p, f, pack_f32x2(0.240221202f, 0.240221202f));
-  p = fma_f32x2(p, f, pack_f32x2(0.693146944f, 0.693146944f));
-  p = fma_f32x2(p, f, pack_f32x2(1.00000012f, 1.00000012f));
-  unpack_f32x2(p, p0, p1);
-  unpack_f32x2(t, t0, t1);
-  p0 = __uint_as_float(__float_as_uint(p0) + (__float_as_uint(t0) << 23));
-  p1 = __uint_as_float(__float_as_uint(p1) + (__float_as_uint(t1) << 23));
 }
 
 }  // namespace sm100

@@ -11,7 +11,7 @@
 #pragma once
 
 #ifdef HGA_TRACE
-#define HGA_TRACE_WARPS 16
+#define HGA_TRACE_WARPS 24
 #define HGA_TRACE_SLOTS 96
 __device__ int g_trace_threads;
 __device__ int g_trace_blk;
