@@ -32,7 +32,8 @@ namespace {
 constexpr int kRtThreads = 256;     // warp 0 producer, warp 1 MMA, warps 2-5 readers, 6-7 help in select
 constexpr int kRtWarps = kRtThreads / 32, kRtCopyWarps = kRtWarps - 2;
 constexpr int kSlab = 128 * 128;    // bytes of 128 summaries x 64 elements
-constexpr int kRankMax = 640;       // up to here a candidate's rank is counted directly
+constexpr int kRankMax = kRtThreads;      // up to here a candidate's rank is counted directly, by a thread each
+constexpr int kMostFinal = 64;            // up to so many chunks to select the warps pick their best first
 
 template <int NSTG, int ACCS>
 struct RouteSmem {
@@ -41,23 +42,22 @@ struct RouteSmem {
   uint64_t drain;              // give-up path only: completes when the tensor pipe has run dry
   uint32_t tmem_base;
   volatile int abort;
-  int count[2][kRtWarps];
   // dynamic tail (see RouteLayout): Q rows (B operand, 1024-aligned), scores, bitmap, selected chunks, group scores
 };
 
 // Query rows of an item on the MMA N dimension: equal parts of at most 128 columns, each a multiple of 32
 struct RouteLayout {
-  int parts, part_cols, q_bytes, n_keys, n_flags;
+  int parts, part_cols, q_bytes, n_keys, n_final;
   __host__ __device__ RouteLayout(const Dims& dm, int max_cand) {
     const int rows = rows_padded(dm);
     parts = (rows + 127) / 128;
     part_cols = ((rows + parts - 1) / parts + 31) & ~31;
     q_bytes = parts * part_cols * dm.d * 2;
     n_keys = (max_cand + 7) & ~3;
-    n_flags = max_cand > 4096 ? (max_cand + 31) / 32 : 128;
+    n_final = max_cand > kRankMax && dm.kc <= kMostFinal ? kRtWarps * dm.kc : 0;
   }
   size_t tail(const Dims& dm) const {
-    return 1024 + (size_t)q_bytes + 4 * ((size_t)n_keys + n_flags + dm.kc + (size_t)dm.kc * dm.per + 8);
+    return 1024 + (size_t)q_bytes + 4 * ((size_t)n_keys + 2 * n_final + 128 + dm.kc + (size_t)dm.kc * dm.per + 8);
   }
 };
 
@@ -68,6 +68,64 @@ __device__ __forceinline__ bool rt_wait(uint64_t* bar, uint32_t parity, volatile
 __device__ __forceinline__ uint32_t rt_orderable(float f) {
   const uint32_t u = __float_as_uint(f);
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+
+// The k largest of n keys (k <= n), ties to the lowest position, by one warp: emit(position, rank by position, key) for each.  The
+// k-th largest is found bit by bit below the bits that all keys share.  KPL: keys that a lane keeps in registers
+// (n <= 32 KPL), 0 = they are read again in every round.
+template <int KPL, class F>
+__device__ __forceinline__ void warp_select(const uint32_t* keys, int n, int k, F emit) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  uint32_t own[KPL > 0 ? KPL : 1];
+  if constexpr (KPL > 0) {
+#pragma unroll
+    for (int q = 0; q < KPL; ++q) own[q] = 32 * q + lane < n ? keys[32 * q + lane] : 0u;
+  }
+  auto each = [&](auto f) {              // f(key), padding keys among them as 0
+    if constexpr (KPL > 0) {
+#pragma unroll
+      for (int q = 0; q < KPL; ++q) f(own[q]);
+    } else {
+#pragma unroll 4
+      for (int i = lane; i < n; i += 32) f(keys[i]);
+    }
+  };
+  uint32_t hi = 0, both = 0xffffffffu, any = 0;      // bits that are one / not zero in all keys
+  each([&](uint32_t key) { hi = max(hi, key); });
+  for (int i = lane; i < n; i += 32) {
+    const uint32_t key = keys[i];
+    both &= key;
+    any |= key;
+  }
+  hi = __reduce_max_sync(full, hi);
+  const uint32_t differ = __reduce_or_sync(full, any) ^ __reduce_and_sync(full, both);
+  uint32_t kth = hi;                    // in the end the largest value that at least k keys reach
+  if (differ != 0) {
+    uint32_t bit = 0x80000000u >> __clz(differ);
+    kth = hi & ~(2 * bit - 1);          // (2 * bit wraps to 0 at the top bit: nothing is shared)
+    for (int reach = n; bit != 0 && reach != k; bit >>= 1) {
+      const uint32_t t = kth | bit;
+      int c = 0;
+      each([&](uint32_t key) { c += key >= t ? 1 : 0; });
+      c = __reduce_add_sync(full, c);
+      if (c >= k) { kth = t; reach = c; }
+    }
+  }
+  int above = 0;
+  each([&](uint32_t key) { above += key > kth ? 1 : 0; });
+  int ties = k - __reduce_add_sync(full, above), rank = 0;      // of the keys equal to it, how many are still to be taken
+  const uint32_t below = (1u << lane) - 1u;
+  for (int base = 0; base < n; base += 32) {
+    const int i = base + lane;
+    const uint32_t key = i < n ? keys[i] : 0u;
+    const uint32_t equal = __ballot_sync(full, i < n && key == kth);
+    const bool sel = i < n && (key > kth || (key == kth && __popc(equal & below) < ties));
+    ties -= min(ties, __popc(equal));
+    const uint32_t word = __ballot_sync(full, sel);
+    if (sel) emit(i, rank + __popc(word & below), key);
+    rank += __popc(word);
+  }
 }
 
 }  // namespace
@@ -87,8 +145,10 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
   Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* q_smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(&sm + 1) + 1023) & ~uintptr_t(1023));
   uint32_t* okeys = reinterpret_cast<uint32_t*>(q_smem + lay.q_bytes);       // orderable candidate scores
-  uint32_t* flags = okeys + lay.n_keys;                                      // bit i: candidate (slot) i selected
-  int* sorted = reinterpret_cast<int*>(flags + lay.n_flags);                 // selected chunks, ascending
+  uint32_t* fkeys = okeys + lay.n_keys;                                      // the warps' best candidates
+  int* fidx = reinterpret_cast<int*>(fkeys + lay.n_final);
+  uint32_t* flags = reinterpret_cast<uint32_t*>(fidx + lay.n_final);         // bit i: slot i selected
+  int* sorted = reinterpret_cast<int*>(flags + 128);                         // selected chunks, ascending
   float* gscore = reinterpret_cast<float*>(sorted + dm.kc);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -360,82 +420,69 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
     // ---------------------------------------------------------------------- chunk top-k
     // Scores compare as 32-bit orderable integers; equal scores are told apart by their index (lowest first).
     if (!sm.abort && k_sel > 0) {
-      if (n_cand <= kRankMax) {
-        // Few candidates: a candidate is selected when fewer than k_sel others beat it; counted for every one, four
+      // Many candidates: every warp first picks the best k_sel of its share, without meeting the others.  (Counting every
+      // candidate's rank, up to 640, and a block-wide search beyond took 17k cycles at 512 candidates and 22k at 2048, a
+      // quarter of the item's time.)
+      const uint32_t* keys = okeys;
+      int n = n_cand;
+      const bool shares = lay.n_final > 0 && n_cand > kRankMax;
+      if (shares) {
+        const int share = (n_cand + kRtWarps - 1) / kRtWarps, last = (n_cand - 1) / share;     // (all whole but the last)
+        const int first = warp * share, mine = min(share, n_cand - first), each = min(k_sel, share);
+        auto keep = [&](int i, int rank, uint32_t key) {
+          fkeys[warp * each + rank] = key;
+          fidx[warp * each + rank] = first + i;
+        };
+        if (mine > 0) {
+          if (share <= 64) warp_select<2>(okeys + first, mine, min(k_sel, mine), keep);
+          else if (share <= 256) warp_select<8>(okeys + first, mine, min(k_sel, mine), keep);
+          else warp_select<0>(okeys + first, mine, min(k_sel, mine), keep);
+        }
+        n = last * each + min(k_sel, n_cand - last * share);
+        keys = fkeys;
+        __syncthreads();
+      }
+      if (n <= kRankMax) {
+        // A key is selected when fewer than k_sel others beat it; counted for every one, a thread each, four
         // keys per 16-byte load.  Equal scores share a rank at first; that only matters when a tie straddles the k-th place,
-        // which shows as a selection of the wrong size and is redone with the index as the second criterion.
+        // which shows as a selection of the wrong size and is redone with the position as the second criterion.
         auto rank_select = [&](bool exact) {
-          for (int base = 0; base < n_cand; base += kRtThreads) {   // warp-uniform trip count (ballots below)
-            const int i = base + tid;
-            bool sel = false;
-            if (i < n_cand) {
-              int beat = 0, q = 0;
-              const uint32_t mine = okeys[i];
-              if (!exact) {
-                const uint4* k4 = reinterpret_cast<const uint4*>(okeys);
+          bool sel = false;
+          if (tid < n) {
+            int beat = 0, q = 0;
+            const uint32_t mine = keys[tid];
+            if (!exact) {
+              const uint4* k4 = reinterpret_cast<const uint4*>(keys);
 #pragma unroll 4
-                for (; q + 4 <= n_cand; q += 4) {
-                  const uint4 kk = k4[q >> 2];
-                  beat += (int)(kk.x > mine) + (int)(kk.y > mine) + (int)(kk.z > mine) + (int)(kk.w > mine);
-                }
-                for (; q < n_cand; ++q) beat += okeys[q] > mine;
-              } else {
-                for (; q < n_cand; ++q) beat += okeys[q] > mine || (okeys[q] == mine && q < i);
+              for (; q + 4 <= n; q += 4) {
+                const uint4 kk = k4[q >> 2];
+                beat += (int)(kk.x > mine) + (int)(kk.y > mine) + (int)(kk.z > mine) + (int)(kk.w > mine);
               }
-              sel = beat < k_sel;
+              for (; q < n; ++q) beat += keys[q] > mine;
+            } else {
+              for (; q < n; ++q) beat += keys[q] > mine || (keys[q] == mine && q < tid);
             }
-            const uint32_t word = __ballot_sync(0xffffffffu, sel);
-            if (lane == 0 && base + warp * 32 < n_cand) flags[(base + warp * 32) >> 5] = word;
+            sel = beat < k_sel;
           }
+          const uint32_t word = __ballot_sync(0xffffffffu, sel);
+          if (lane == 0) flags[warp] = word;
+        };
+        auto picked_below = [&](int words) {
+          int c = 0;
+          for (int q = 0; q < words; ++q) c += __popc(flags[q]);
+          return c;
         };
         rank_select(false);
         __syncthreads();
-        int n_picked = 0;
-        for (int q = 0; q < (n_cand + 31) / 32; ++q) n_picked += __popc(flags[q]);
-        if (n_picked != k_sel) {          // same value in every thread
+        if (picked_below(kRtWarps) != k_sel) {          // same value in every thread
           __syncthreads();
           rank_select(true);
           __syncthreads();
         }
-      } else {
-        // Many candidates: the k_sel-th largest key bit by bit from the top -- at most 32 rounds of one pass over a thread's
-        // few keys and one block-wide count, fewer when a prefix already splits off exactly k_sel.
-        uint32_t kth = 0;                 // largest value that at least k_sel keys reach, once the loop has ended
-        int reach = n_cand;               // how many keys reach it
-        int turn = 0;
-        for (uint32_t bit = 0x80000000u; bit != 0 && reach != k_sel; bit >>= 1, turn ^= 1) {
-          const uint32_t t = kth | bit;
-          int n = 0;
-          for (int i = tid; i < n_cand; i += kRtThreads) n += okeys[i] >= t ? 1 : 0;
-          n = __reduce_add_sync(0xffffffffu, n);
-          if (lane == 0) sm.count[turn][warp] = n;
-          __syncthreads();
-          n = 0;
-#pragma unroll
-          for (int q = 0; q < kRtWarps; ++q) n += sm.count[turn][q];
-          if (n >= k_sel) { kth = t; reach = n; }
-        }
-        for (int base = 0; base < n_cand; base += kRtThreads) {
-          const int i = base + tid;
-          const uint32_t word = __ballot_sync(0xffffffffu, i < n_cand && okeys[i] >= kth);
-          if (lane == 0 && base + warp * 32 < n_cand) flags[(base + warp * 32) >> 5] = word;
-        }
-        __syncthreads();
-        if (reach != k_sel && tid == 0) {
-          // ties at the k-th place: the last reach - k_sel of the keys equal to it, in index order, are not selected
-          int left = reach - k_sel;
-          for (int i = n_cand - 1; i >= 0 && left > 0; --i)
-            if (okeys[i] == kth) { flags[i >> 5] &= ~(1u << (i & 31)); --left; }
-        }
-        __syncthreads();
-      }
-      for (int i = tid; i < n_cand; i += kRtThreads) {
-        const uint32_t word = flags[i >> 5];
-        if ((word >> (i & 31)) & 1u) {
-          int pos = __popc(word & ((1u << (i & 31)) - 1u));
-          for (int q = 0; q < (i >> 5); ++q) pos += __popc(flags[q]);
-          sorted[pos] = j0 + i;
-        }
+        const uint32_t word = flags[warp];
+        if ((word >> lane) & 1u) sorted[picked_below(warp) + __popc(word & ((1u << lane) - 1u))] = j0 + (shares ? fidx[tid] : tid);
+      } else if (warp == 0) {
+        warp_select<0>(keys, n, k_sel, [&](int i, int rank, uint32_t) { sorted[rank] = j0 + (shares ? fidx[i] : i); });
       }
       __syncthreads();
     }
