@@ -357,7 +357,7 @@ def time_varlen(args, stream):
     torch.cuda.synchronize()
     ms = float(np.median([a.elapsed_time(b) for a, b in ev]))
     return {"sequences": n_seq, "tokens": n_q, "resident_tokens": n_k, "ms_per_step": round(ms, 4),
-            "tokens_per_s": round(n_q / (ms * 1e-3), 1), "launch": "eager, two library streams",
+            "tokens_per_s": round(n_q / (ms * 1e-3), 1), "launch": "eager, one launch per step",
             "device_status_word": int(status.item()),
             "note": "16 packed sequences, 512 new tokens behind 1536 resident ones each; summaries of the active "
                     "ranges + route + attention fwd + bwd per sequence"}

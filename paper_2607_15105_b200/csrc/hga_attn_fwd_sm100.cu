@@ -15,8 +15,11 @@
 // so S = Q K^T over 64-key tiles bound the kernel (24 instructions a tile for the two CTAs of an SM, 1.9k cycles).
 // S is single-buffered (128 of the 256 columns; O takes the rest); the chain S -> exponentials -> P V -> next S of
 // one CTA is covered by the other CTA's, and kept short by TWO threads per row.  hga_attn_fwd, 64-key tiles with one
-// thread per row and a running maximum -> this: 16K layer (512 CTAs of 768 keys) 45.2 -> 39.0 us, 2K layer 31.0 -> 27.9,
-// 4 x 64K (2560 keys) 865 -> 842.
+// thread per row and a running maximum -> this: 16K layer (512 CTAs of 768 keys) 45.2 -> 39.3 us, 2K layer 31.0 -> 27.3,
+// 4 x 64K (2560 keys) 865 -> 830.
+//
+// What bounds it: a tile's chain takes ~4.3k cycles, of which the exponentials of both CTAs need 2.0k of the special-function
+// unit and their GEMMs 2.0k of the tensor pipe, half overlapped.  At 4 x 64K the board's power limit on top.
 //
 // Warp roles (384 threads, 80 registers per thread):
 //   warps 0, 2   producers: octets 0-7 / 8-15 of every K and V tile (a box costs its issuing warp ~100 cycles)
