@@ -10,8 +10,8 @@
 //    runs first and stores every row of dK/dV).  They come first:
 //      S = Q K^T, dP = dO V^T -> TMEM;  P, dS by one thread per row -> shared memory;
 //      dQ += dS K;  dV^T = dO^T P, dK^T = Q^T dS (M = head_dim, N = 64 keys, K = 128 rows) -> TMEM,
-//    then four reduction warps add the transposed tiles to global memory (a warp's 32 lanes hold 32
-//    consecutive elements of one key row: one coalesced 128-byte red.global.add.f32 request).
+//    then four reduction warps transpose the two accumulators through shared memory and add them to global
+//    memory octet by octet (4 KB bulk reductions).
 //
 //  * all other steps run on PAIRS of tiles (128 keys), because a tcgen05.mma with N = 64 runs at
 //    little more than half the rate of one with N = 128:
@@ -29,12 +29,14 @@
 // Warp roles (512 threads): warp 0 copies K tiles and runs up to three pairs ahead, warps 14 and 15
 // copy V tiles (half of each tile; in the paired steps V has room for two pairs -- its own two stages and
 // the P / dS tiles, idle by then -- each refilled as soon as the dP GEMM that read it is done: with one
-// pair only, the copy's latency sat between consecutive dP GEMMs), warp 1 MMA issuer, warps 2-5 and 6-9
-// one thread per query row (warpgroup 0: first tile of a pair and all dK/dV steps; warpgroup 1:
-// second tile of a pair; both write the dQ epilogue), warps 10-13 dK/dV reduction.
-// Every barrier hand-off costs the MMA thread a few hundred cycles and every tcgen05.commit about a
-// hundred, so a paired step has one full barrier per operand and pair, and the dP commit doubles as
-// the V stages' release.
+// pair only, the copy's latency sat between consecutive dP GEMMs), warp 1 MMA issuer (all GEMMs of a dK/dV step, S and dP of a
+// pair), warps 2-5 and 6-9 one thread per query row (warpgroup 0: first tile of a pair and half of every dK/dV step's keys;
+// warpgroup 1: the others; both write the dQ epilogue), warps 10-13 dK/dV reduction, then dQ of the pairs (10) and a share of the
+// copies (11 K, 12 and 13 V).
+// What bounds it: the row threads, 2.4k cycles per pair (1.0k of exponentials, the rest tensor-memory loads and barrier
+// hand-offs of 200-400 cycles each; the pair's GEMMs take the tensor pipe 1.5k), at 4 x 64K the power limit; at 2K tokens
+// without history (every routed key is differentiable) the dK/dV steps, ~4k cycles each.  hga_attn_bwd with the band
+// kernel: 2K layer 104 us, 16K layer 100 us, 4 x 64K 1.55 ms.
 // TMEM (512 columns): region 0 | region 2 (aliased by dV^T, dK^T during the dK/dV steps) | dQ |
 // region 1.  Shared memory: Q, dO (32 KB each), K ring of six 16 KB stages, V ring of two, P and dS
 // (16 KB each, used by the dK/dV steps only).
