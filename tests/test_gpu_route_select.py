@@ -1,4 +1,4 @@
-"""The router's chunk selection where it changes method: rank counting up to 640 candidates, bit-by-bit search beyond;
+"""The router's chunk selection where it changes method: rank counting for few candidates, bit-by-bit search for many;
 ties that straddle the k-th place on both sides of that line (lowest index wins); and query-row counts that need more
 accumulators than a CTA has (several passes over a summary tile)."""
 import numpy as np
@@ -48,6 +48,22 @@ def test_candidate_counts(n_cand, ties):
     ci, gi, ng = routed(cfg, x, cs, gs)
     if ties:      # equal bits give equal scores on both sides, so even tied selections agree exactly
         assert np.array_equal(ci, ref["chunk_idx"])
+    check_routing(cfg, ref, ci, gi, ng)
+
+
+@pytest.mark.parametrize("n_cand,k", [(255, 7), (256, 64), (257, 7), (257, 64), (512, 32), (513, 40), (2048, 16), (2049, 33), (257, 65), (300, 200)])
+def test_selection_by_shares(n_cand, k):
+    """A thread per candidate up to 256, each warp's share first beyond (2, 8 or any number of keys per lane), one warp where
+    more than 64 chunks are opened; ties inside a share and across shares."""
+    cfg = cfg_of(total_len=(n_cand + 1) * 64, topk_chunks=k)
+    x = make_inputs(cfg)
+    cs, gs = oracle.build_summaries(cfg, x["K"])
+    cs = cs.copy()
+    for j in range(0, n_cand, 9):
+        cs[0, 0, j:j + 9] = cs[0, 0, j % 63]
+    ref = oracle.route(cfg, x["Q"], cs, gs, want_scores=True)
+    ci, gi, ng = routed(cfg, x, cs, gs)
+    assert np.array_equal(ci, ref["chunk_idx"])
     check_routing(cfg, ref, ci, gi, ng)
 
 
