@@ -16,7 +16,7 @@
 // S is single-buffered (128 of the 256 columns; O takes the rest); the chain S -> exponentials -> P V -> next S of
 // one CTA is covered by the other CTA's, and kept short by TWO threads per row.  hga_attn_fwd, 64-key tiles with one
 // thread per row and a running maximum -> this: 16K layer (512 CTAs of 768 keys) 45.2 -> 39.3 us, 2K layer 31.0 -> 27.3,
-// 4 x 64K (2560 keys) 865 -> 830.
+// 4 x 64K (2560 keys) 865 -> 830 (before the second terms, see below).
 //
 // What bounds it: a tile's chain takes ~4.3k cycles, of which the exponentials of both CTAs need 2.0k of the special-function
 // unit and their GEMMs 2.0k of the tensor pipe, half overlapped.  At 4 x 64K the board's power limit on top.
@@ -26,12 +26,20 @@
 //   warp 1       MMA issuer: S = Q K^T (smem x smem), O += P V (P from TMEM)
 //   warp 3       Q, then the check of the routing list
 //   warps 4-11   softmax, two threads per row (TMEM lane = row), 32 keys each of both halves of a tile; the epilogue
-// TMEM (256 columns): S (128), P (bf16) over the first half of each 32 columns just read | O.
+// TMEM (256 columns): S (128), P (bf16) over the S columns just read, per 16 keys 8 columns and 8 of second terms | O.
 //
 // Softmax: every exponential of a row is taken against ONE reference, the row's maximum over the first tile (which holds
 // the start of the local window, visible to every row).  bf16 and fp32 share an exponent range of 2^127 and O is divided
 // by the sum in the end, so a later, larger logit costs no precision until it exceeds the reference by tens of binary
-// orders; no maximum is looked for in later tiles, and no sum is ever rescaled.  A row whose sum does grow past
+// orders; no maximum is looked for in later tiles, and no sum is ever rescaled.
+// What the one reference does cost is the exactness of a dominant weight: against its own tile's maximum, which a running
+// reference is raised to, it is 1, here it has a rounding error of 2^-9 like any other.  Where 32 keys of some row
+// outweigh the reference by more than 64, that half of the tile gets P in TWO bf16 terms (value and remainder, 2^-17), the
+// second ones a GEMM of their own; every warp stores the second terms, zeros elsewhere.  16K layer (needles in one block
+// of eight: 1 % of the half-tiles): error of O against fp64 2.11e-3 with one term, 1.82e-3 so, 2.06e-3 with a running
+// reference; hga_attn_fwd 39.8 -> 41.3 us (two terms everywhere: 1.66e-3, which is O's own rounding, and 43.5 us).
+// kTwoTerms kernels use them everywhere (see two_terms()).
+// A row whose sum does grow past
 // 2^80 (a logit 55 nats above the first tile's) is recomputed at the end by its warp with a running maximum.
 #include "hga_bwd_sm100.cuh"
 #include "hga_common.cuh"
@@ -50,6 +58,7 @@ namespace {
 constexpr int kFwdThreads = 384;
 constexpr int kFT = 128;                      // keys per tile
 constexpr float kSumLimit = 1.2e24f;          // 2^80
+constexpr float kTwoTermSum = 64.f;           // 32 keys that together outweigh the reference by so much get two terms
 
 template <int D>
 struct FwdSmem {
@@ -63,6 +72,7 @@ struct FwdSmem {
   uint32_t tmem_base;
   int n_far, n_listed;
   bool clean;
+  volatile int second_terms[2];                // number (from 1) of the last tile whose half needs the weights' second terms
   volatile int abort;
 };
 
@@ -108,7 +118,7 @@ __device__ __forceinline__ float row_with_running_maximum(const FarList& far, co
 
 }  // namespace
 
-template <int D, class Segs>
+template <int D, bool kTwoTerms, class Segs>
 __global__ void __launch_bounds__(kFwdThreads, 2)
 k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                  const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_o,
@@ -152,6 +162,7 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     mbar_init(&sm.k_full, 2); mbar_init(&sm.v_full, 2); mbar_init(&sm.v_empty, 1);
     mbar_init(&sm.s_full, 1); mbar_init(&sm.p_full[0], 8); mbar_init(&sm.p_full[1], 8);
     mbar_init(&sm.info_full, 1); mbar_init(&sm.o_done, 1); mbar_init(&sm.o_staged, 8); mbar_init(&sm.drain, 1);
+    sm.second_terms[0] = sm.second_terms[1] = 0;
     sm.abort = 0;
     fence_barrier_init();
   }
@@ -278,12 +289,17 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                  idesc, kk > 0);
       mma_commit_w(lead, &sm.s_full);                    // also tells the producers that the K tile is free
     };
-    // half hf of a tile: 16 keys per step; P of keys 32i .. 32i+31 sits at columns 32i .. 32i+15
-    auto issue_pv = [&](int hf, bool accumulate) {
+    // half hf of tile j: 16 keys per step; P of keys 16i .. 16i+15 sits at columns 16i .. 16i+7, its second terms behind it
+    auto issue_pv = [&](int hf, int j, bool accumulate) {
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk)
-        mma_ts_w(lead, o_acc, tmem + 64 * hf + (kk >> 1) * 32 + (kk & 1) * 8, desc_advance(v_desc, (uint32_t)(4 * hf + kk) * 2 * kOct), idesc_o,
+        mma_ts_w(lead, o_acc, tmem + 64 * hf + 16 * kk, desc_advance(v_desc, (uint32_t)(4 * hf + kk) * 2 * kOct), idesc_o,
                  (accumulate || kk > 0));
+      if (kTwoTerms || sm.second_terms[hf] == j + 1) {
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)
+          mma_ts_w(lead, o_acc, tmem + 64 * hf + 16 * kk + 8, desc_advance(v_desc, (uint32_t)(4 * hf + kk) * 2 * kOct), idesc_o, 1);
+      }
     };
     int n_oct = 16 * n_pre + 1;                    // (enough until the list is known)
     bool ok = true;
@@ -308,12 +324,12 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       if (!ok) break;
       tc_fence_after_sync();
       HGA_TRACE_POINT(5);
-      issue_pv(0, j > 0);
+      issue_pv(0, j, j > 0);
       if (whole) {
         ok = mma_wait(&sm.p_full[1], j & 1);
         if (!ok) break;
         tc_fence_after_sync();
-        issue_pv(1, true);
+        issue_pv(1, j, true);
       }
       mma_commit_w(lead, more ? &sm.v_empty : &sm.o_done);
       HGA_TRACE_POINT(7);
@@ -396,23 +412,74 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           const uint32_t s_addr = lane_base + 64 * c + 32 * hw;
           // (two copies of the code: a compare per element in the common one doubled its time)
           auto exponentials = [&](auto masked) {
-            uint32_t x[32], pk[16];
-            tmem_ld32(s_addr, x);
-            tmem_wait_ld();
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
+            // weights of keys k and k + 1 of the 32
+            auto weights = [&](int k, uint32_t x0, uint32_t x1, float& p0, float& p1) {
               float a0, a1;
-              unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1])), sl2_2, neg_m2), a0, a1);
-              float p0 = fast_exp2(a0), p1 = fast_exp2(a1);
+              unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(x0), __uint_as_float(x1)), sl2_2, neg_m2), a0, a1);
+              p0 = fast_exp2(a0);
+              p1 = fast_exp2(a1);
               if constexpr (decltype(masked)::value) {
-                if (!((2 * i < lo_c || 2 * i >= hi_c) && 2 * i < end_c)) p0 = 0.f;
-                if (!((2 * i + 1 < lo_c || 2 * i + 1 >= hi_c) && 2 * i + 1 < end_c)) p1 = 0.f;
+                if (!((k < lo_c || k >= hi_c) && k < end_c)) p0 = 0.f;
+                if (!((k + 1 < lo_c || k + 1 >= hi_c) && k + 1 < end_c)) p1 = 0.f;
               }
-              lsum = add_f32x2(lsum, pack_f32x2(p0, p1));
-              pk[i] = pack_bf16(p0, p1);
-              rsum = add_f32x2(rsum, pack_f32x2(__uint_as_float(pk[i] << 16), __uint_as_float(pk[i] & 0xffff0000u)));
+            };
+            auto sum_of = [](uint32_t pk) { return pack_f32x2(__uint_as_float(pk << 16), __uint_as_float(pk & 0xffff0000u)); };
+            [[maybe_unused]] bool two = kTwoTerms;
+            if constexpr (!kTwoTerms) {
+              uint32_t x[32], pk[16];
+              uint64_t sum = pack_f32x2(0.f, 0.f);
+              tmem_ld32(s_addr, x);
+              tmem_wait_ld();
+#pragma unroll
+              for (int i = 0; i < 16; ++i) {
+                float p0, p1;
+                weights(2 * i, x[2 * i], x[2 * i + 1], p0, p1);
+                sum = add_f32x2(sum, pack_f32x2(p0, p1));
+                pk[i] = pack_bf16(p0, p1);
+                rsum = add_f32x2(rsum, sum_of(pk[i]));
+              }
+              lsum = add_f32x2(lsum, sum);
+              float x0, x1;
+              unpack_f32x2(sum, x0, x1);
+              two = __any_sync(0xffffffffu, x0 + x1 > kTwoTermSum);
+              if (!two) {
+                const uint32_t out[32] = {pk[0], pk[1], pk[2], pk[3], pk[4], pk[5], pk[6], pk[7], 0, 0, 0, 0, 0, 0, 0, 0,
+                                          pk[8], pk[9], pk[10], pk[11], pk[12], pk[13], pk[14], pk[15], 0, 0, 0, 0, 0, 0, 0, 0};
+                tmem_st32(s_addr, out);
+              } else if (lane == 0) {
+                sm.second_terms[c] = j + 1;
+              }
             }
-            tmem_st16(s_addr, pk);
+            // 16 keys with two terms each (S is fetched again rather than kept)
+            auto two_terms_of = [&](int k0, const uint32_t (&x)[16]) {
+              uint32_t out[16];
+#pragma unroll
+              for (int i = 0; i < 8; ++i) {
+                float p0, p1;
+                weights(k0 + 2 * i, x[2 * i], x[2 * i + 1], p0, p1);
+                out[i] = pack_bf16(p0, p1);
+                out[8 + i] = pack_bf16(p0 - __uint_as_float(out[i] << 16), p1 - __uint_as_float(out[i] & 0xffff0000u));
+                if constexpr (kTwoTerms) lsum = add_f32x2(lsum, pack_f32x2(p0, p1));
+                else rsum = add_f32x2(rsum, sum_of(out[8 + i]));
+              }
+              tmem_st16(s_addr + k0, out);
+            };
+            if constexpr (kTwoTerms) {
+              uint32_t x[2][16];
+              tmem_ld16(s_addr, x[0]);
+              tmem_ld16(s_addr + 16, x[1]);
+              tmem_wait_ld();
+              two_terms_of(0, x[0]);
+              two_terms_of(16, x[1]);
+            } else if (two) {
+#pragma unroll 1
+              for (int k0 = 0; k0 < 32; k0 += 16) {
+                uint32_t x[16];
+                tmem_ld16(s_addr + k0, x);
+                tmem_wait_ld();
+                two_terms_of(k0, x);
+              }
+            }
           };
           if (__all_sync(0xffffffffu, (lo_c >= 32 || hi_c <= 0) && end_c >= 32)) exponentials(std::false_type{});
           else exponentials(std::true_type{});
@@ -424,8 +491,10 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       float x0, x1;
       unpack_f32x2(lsum, x0, x1);
       l += x0 + x1;
-      unpack_f32x2(rsum, x0, x1);
-      l_mma += x0 + x1;
+      if constexpr (!kTwoTerms) {
+        unpack_f32x2(rsum, x0, x1);
+        l_mma += x0 + x1;
+      }
       HGA_TRACE_POINT(14);
     }
     if (ok) ok = __all_sync(0xffffffffu, bwd_wait(&sm.o_done, 0, abort));
@@ -433,10 +502,11 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // the row's two sums meet (every GEMM has read the K tile); ok or not, every softmax thread meets here once
     float* const xchg = reinterpret_cast<float*>(sm.k);
     xchg[hw * 256 + row] = l;
-    xchg[hw * 256 + 128 + row] = l_mma;
+    if constexpr (!kTwoTerms) xchg[hw * 256 + 128 + row] = l_mma;
     asm volatile("bar.sync 1, 256;" ::: "memory");
     l += xchg[(hw ^ 1) * 256 + row];
-    l_mma += xchg[(hw ^ 1) * 256 + 128 + row];
+    if constexpr (!kTwoTerms) l_mma += xchg[(hw ^ 1) * 256 + 128 + row];
+    else l_mma = l;                                     // (two terms leave 2^-17 of a weight: its sum needs no counterpart)
     if (ok && warp_real) {
       tc_fence_after_sync();
       const float inv = 1.f / l_mma;
@@ -532,7 +602,16 @@ bool attn_fwd_sm100_supported(const Dims& dm) {
   return dm.g % 8 == 0;
 }
 
-template <int D, class Segs>
+// Row counts that do not fill M-tiles: until these kernels took them they had the warp-per-row kernel, which weighs V with
+// fp32 probabilities, and they keep that precision: error of O against fp64 (head_dim 128, 64 rows) 1.66e-3, which is the
+// rounding of O itself, with two terms; 2.3e-3 with one.
+static bool two_terms(const Dims& dm) {
+  const int rows_pad = rows_padded(dm);
+  if (rows_pad > 128) return rows_pad % 128 != 0 || rows_pad != dm.rows;
+  return rows_pad < 128 && !(dm.flags & HGA_FLAG_DECODE);
+}
+
+template <int D, bool kTwoTerms, class Segs>
 static int launch_fwd(const Dims& dm, const Segs& segs, int64_t units, const void* Q, const void* K, const void* V,
                       const int32_t* group_idx, const int32_t* n_groups, void* O, float* LSE, int32_t* status_word, cudaStream_t st) {
   CUtensorMap mq, mk, mv, mo;
@@ -552,10 +631,10 @@ static int launch_fwd(const Dims& dm, const Segs& segs, int64_t units, const voi
   const size_t smem = sizeof(FwdSmem<D>) + 1024;
   static_assert(sizeof(FwdSmem<D>) + 1024 <= 113 * 1024, "two CTAs per SM");
   // two CTAs per SM need the largest shared-memory carve-out
-  const int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(&k_attn_fwd_sm100<D, Segs>), smem, true);
+  const int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(&k_attn_fwd_sm100<D, kTwoTerms, Segs>), smem, true);
   if (rc) return rc;
   PdlLaunch cfg((unsigned)units, kFwdThreads, smem, st, dm.flags);
-  const cudaError_t e = cudaLaunchKernelEx(&cfg.c, k_attn_fwd_sm100<D, Segs>, mq, mk, mv, mo, (const uint16_t*)Q, (const uint16_t*)K,
+  const cudaError_t e = cudaLaunchKernelEx(&cfg.c, k_attn_fwd_sm100<D, kTwoTerms, Segs>, mq, mk, mv, mo, (const uint16_t*)Q, (const uint16_t*)K,
                                            (const uint16_t*)V, group_idx, n_groups, dm, (uint16_t*)O, LSE, status_word, segs);
   count_launch(HGA_KERNELS_FWD_TENSOR);
   return record_cuda(e);
@@ -565,14 +644,15 @@ int launch_attn_fwd_sm100(const Dims& dm, SegTable* segs, const void* Q, const v
                           const int32_t* group_idx, const int32_t* n_groups, void* O, float* LSE,
                           int32_t* status_word, cudaStream_t st) {
   const int n_mt = (rows_padded(dm) + 127) / 128;
-  if (!segs) {
-    const int64_t units = (int64_t)dm.B * dm.Hkv * dm.NQB * n_mt;
-    if (dm.d == 128) return launch_fwd<128>(dm, OneSegment{}, units, Q, K, V, group_idx, n_groups, O, LSE, status_word, st);
-    return launch_fwd<64>(dm, OneSegment{}, units, Q, K, V, group_idx, n_groups, O, LSE, status_word, st);
-  }
+#define HGA_FWD_ARGS(segs, units) dm, segs, units, Q, K, V, group_idx, n_groups, O, LSE, status_word, st
+#define HGA_FWD(segs, units)                                                                                            \
+  (two_terms(dm) ? (dm.d == 128 ? launch_fwd<128, true>(HGA_FWD_ARGS(segs, units)) : launch_fwd<64, true>(HGA_FWD_ARGS(segs, units))) \
+                 : (dm.d == 128 ? launch_fwd<128, false>(HGA_FWD_ARGS(segs, units)) : launch_fwd<64, false>(HGA_FWD_ARGS(segs, units))))
+  if (!segs) return HGA_FWD(OneSegment{}, (int64_t)dm.B * dm.Hkv * dm.NQB * n_mt);
   const int64_t units = number_units(*segs, [&](const Segment& s) { return (int64_t)dm.B * dm.Hkv * (s.S / dm.Bq) * n_mt; });
-  if (dm.d == 128) return launch_fwd<128>(dm, *segs, units, Q, K, V, group_idx, n_groups, O, LSE, status_word, st);
-  return launch_fwd<64>(dm, *segs, units, Q, K, V, group_idx, n_groups, O, LSE, status_word, st);
+  return HGA_FWD(*segs, units);
+#undef HGA_FWD
+#undef HGA_FWD_ARGS
 }
 
 }  // namespace hga
