@@ -25,11 +25,14 @@
 // ahead), so the backward needs no separate pass over O and dO.
 //
 // Work unit (one CTA): (batch, kv head, 128-key tile of the active segment); keys past the end of the
-// segment arrive as zeros, are masked by causality and are not stored.
+// segment arrive as zeros (or are the next segment's, where a launch covers several), are masked and not stored.
 // Warp roles (448 threads): warp 0 producer (K, V once; Q, dO tiles through a two-stage ring, O tiles one at a time),
 // warp 1 MMA issuer, warps 2-5 and 6-9 one thread per key (warpgroup w: query rows 32w .. 32w+31 of
 // every half-step), warps 10-13 row statistics (LSE, delta).
 // TMEM (512 columns): two regions of [S^T / P^T (64) | dP^T / dS^T (64)], then dV and dK, 128 columns each.
+// For the shapes of k_attn_bwd_terms_sm100 (see there why), P^T has three bf16 terms here and dS^T two, each term a GEMM of
+// its own: two lie over the columns just read, 8 per 16 rows each, P's third apart (at head_dim 128 in the place of the
+// second region, so the half-steps follow one another).
 #include "hga_bwd_sm100.cuh"
 #include "hga_common.cuh"
 #include "hga_sm100.cuh"
@@ -51,7 +54,7 @@ struct BandSmem {
   alignas(1024) uint8_t q[2][kTile];
   alignas(1024) uint8_t dO[2][kTile];
   alignas(1024) uint8_t o[kTile];                // (q, dO and o, contiguous, also stage the dV / dK tiles on their way out)
-  alignas(16) float nlse[128];                   // per query row of the current M-tile: -LSE * log2(e)
+  alignas(16) float nlse[128];                   // per query row of the current M-tile: -LSE * log2(e) (in terms: -LSE)
   alignas(16) float nds[128];                    //                                      -delta * scale
   uint64_t kv_full, qdo_full[2][2], qdo_empty[2][2], o_full, o_empty;   // Q/dO: [ring stage][half of the M-tile's rows]
   // per half of the M-tile (= per region of tensor memory), so that every barrier completes once per step and
@@ -76,13 +79,20 @@ struct HalfStep {
 
 }  // namespace
 
-template <int D, class Segs>
+template <int D, bool kTerms, class Segs>
 __global__ void __launch_bounds__(kBandThreads, 1)
 k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_do,
                       const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                       const __grid_constant__ CUtensorMap map_o, const float* __restrict__ LSE, const Dims dm,
                       float* __restrict__ dK, float* __restrict__ dV, int32_t* status_word, const __grid_constant__ Segs segs) {
-  constexpr uint32_t kColS = 0, kColDP = 64, kRegion = 128, kColDV = 256, kColDK = 384;   // (S^T, dP^T: inside a region)
+  // (S^T, dP^T: inside a region; in terms at head_dim 128 one region only: the other's place takes P's third terms)
+  constexpr uint32_t kColS = 0, kColDP = 64, kRegions = kTerms && D == 128 ? 1 : 2, kRegion = kRegions == 2 ? 128 : 0, kColDV = 256, kColDK = 384;
+  constexpr uint32_t kColP3 = D == 128 ? 128 : kColDV + 64, kP3Region = kRegions == 2 ? 32 : 0;
+  // The tensor pipe cuts its fp32 sums off rather than rounding them, an error that grows with the length of the chain (12
+  // additions a half-step with P's three terms): at head_dim 64 a half-step's dV is a sum by itself, in a buffer per
+  // region, and the key threads add them up in registers.
+  constexpr bool kShortChains = kTerms && D == 64;
+  constexpr uint32_t kColDV1 = kColDK + 64;
   constexpr int kD = D, kPanels = D / 64, kTile = BandSmem<D>::kTile;
   constexpr int kHalfBoxes = 2 * kPanels;          // boxes (64 rows x 64 elements) of one half-step's Q and dO, or of one 128-row tile
   extern __shared__ uint8_t smem_raw[];
@@ -245,13 +255,12 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
           mma_ss_w(lead, acc, desc_advance(a, off), desc_advance(bq, off), idesc_t, kk > 0);
         }
       };
-      // acc (keys x head_dim) += a (keys x 64 rows, bf16 in TMEM: rows 0-31 at columns 0-15, rows 32-63 at
-      // columns 32-47 of its S^T or dP^T part) x b (64 rows of the Q or dO tile: rows along K, 16 per instruction)
-      auto issue_g = [&](uint32_t acc, uint32_t a_tmem, uint64_t bmn, bool accumulate) {
+      // acc (keys x head_dim) += a (keys x 64 rows, bf16 in TMEM) x b (64 rows of the Q or dO tile: rows along K, 16 per
+      // instruction).  a_col: columns of rows 16 kk .. of a
+      auto issue_g = [&](uint32_t acc, uint64_t bmn, bool accumulate, auto a_col) {
 #pragma unroll
         for (int kk = 0; kk < 64 / 16; ++kk)
-          mma_ts_w(lead, acc, a_tmem + (kk < 2 ? 8 * kk : 32 + 8 * (kk - 2)), desc_advance(bmn, kk * 2048), idesc_g,
-                   (accumulate || kk > 0));
+          mma_ts_w(lead, acc, a_col(kk), desc_advance(bmn, kk * 2048), idesc_g, (accumulate || kk > 0));
       };
       // S^T and dP^T of half-step hf of the M-tile in ring stage st, into region hf
       auto issue_sdp = [&](uint32_t st, uint32_t hf) {
@@ -262,7 +271,7 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
       };
       const int n_half = 2 * n_steps;
       bool ok = mma_wait(&sm.kv_full, 0, abort);
-      for (uint32_t hf = 0; hf < 2 && ok; ++hf) {
+      for (uint32_t hf = 0; hf < kRegions && ok; ++hf) {
         ok = mma_wait(&sm.qdo_full[0][hf], 0, abort);
         if (!ok) break;
         tc_fence_after_sync();
@@ -277,17 +286,30 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
         tc_fence_after_sync();
         HGA_TRACE_POINT(5);
         const uint32_t region = tmem + hf * kRegion, off = st * kTile + hf * 8192;
-        issue_g(tmem + kColDV, region + kColS, desc_advance(do_mn0, off), hs > 0);
-        issue_g(tmem + kColDK, region + kColDP, desc_advance(q_mn0, off), hs > 0);
+        const uint64_t do_mn = desc_advance(do_mn0, off), q_mn = desc_advance(q_mn0, off);
+        if constexpr (!kTerms) {
+          // rows 0-31 at columns 0-15, rows 32-63 at columns 32-47 of the S^T or dP^T part
+          issue_g(tmem + kColDV, do_mn, hs > 0, [&](int kk) { return region + kColS + (kk < 2 ? 8 * kk : 32 + 8 * (kk - 2)); });
+          issue_g(tmem + kColDK, q_mn, hs > 0, [&](int kk) { return region + kColDP + (kk < 2 ? 8 * kk : 32 + 8 * (kk - 2)); });
+        } else {
+          // per 16 rows 8 columns of the first terms and 8 of the second
+          const uint32_t dv_acc = tmem + (kShortChains && hf ? kColDV1 : kColDV);
+          issue_g(dv_acc, do_mn, !kShortChains && hs > 0, [&](int kk) { return region + kColS + 16 * kk; });
+          issue_g(dv_acc, do_mn, true, [&](int kk) { return region + kColS + 16 * kk + 8; });
+          issue_g(dv_acc, do_mn, true, [&](int kk) { return tmem + kColP3 + hf * kP3Region + 8 * kk; });
+          issue_g(tmem + kColDK, q_mn, hs > 0, [&](int kk) { return region + kColDP + 16 * kk; });
+          issue_g(tmem + kColDK, q_mn, true, [&](int kk) { return region + kColDP + 16 * kk + 8; });
+        }
         mma_commit_w(lead, &sm.qdo_empty[st][hf]);                     // these 64 rows of Q and dO are consumed
-        if (hs + 2 < n_half) {
-          // the same half of the next M-tile reuses this region: the in-order tensor pipe runs its GEMMs after
-          // the two above, which read P^T and dS^T from it
-          const uint32_t st_n = st ^ 1u;
-          ok = mma_wait(&sm.qdo_full[st_n][hf], ((m + 1) >> 1) & 1, abort);
+        if (hs + (int)kRegions < n_half) {
+          // the next half-step that uses this region (the same half of the next M-tile, with two of them): the in-order
+          // tensor pipe runs its GEMMs after those above, which read P^T and dS^T from it
+          const int hs_n = hs + kRegions, m_n = hs_n >> 1;
+          const uint32_t st_n = (uint32_t)(m_n & 1), hf_n = (uint32_t)(hs_n & 1);
+          ok = mma_wait(&sm.qdo_full[st_n][hf_n], (m_n >> 1) & 1, abort);
           if (!ok) break;
           tc_fence_after_sync();
-          issue_sdp(st_n, hf);
+          issue_sdp(st_n, hf_n);
         }
         HGA_TRACE_POINT(7);
       }
@@ -302,8 +324,20 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
     const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
     const float sl2 = dm.scale * 1.4426950408889634f;
     const uint64_t sl2_2 = pack_f32x2(sl2, sl2), scale_2 = pack_f32x2(dm.scale, dm.scale);
+    const uint64_t log2e_2 = pack_f32x2(1.4426950408889634f, 1.4426950408889634f);
     bool ok = true;
     HalfStep sp = first[0];
+    float dv_sum[kShortChains ? 32 : 1];             // this key's dV, columns 32*wg ..
+#pragma unroll
+    for (float& x : dv_sum) x = 0.f;
+    auto add_dv = [&](int hf) {
+      uint32_t x[32];
+      tmem_ld32(lane_base + (hf ? kColDV1 : kColDV) + 32 * wg, x);
+      tmem_wait_ld();
+      if constexpr (kShortChains)
+#pragma unroll
+        for (int i = 0; i < 32; ++i) dv_sum[i] += __uint_as_float(x[i]);
+    };
     for (int hs = 0; hs < 2 * n_steps; ++hs) {
       const int m = hs >> 1, hf = hs & 1;
       const Window w = window_at(dm, sg.H + sp.qb * dm.Bq);
@@ -317,12 +351,62 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
       const uint32_t nlse_a = smem_u32(&sm.nlse[r_first]), nds_a = smem_u32(&sm.nds[r_first]);
       const uint32_t s_addr = lane_base + hf * kRegion + kColS + 32 * wg;
       const uint32_t dp_addr = lane_base + hf * kRegion + kColDP + 32 * wg;
-      uint32_t pk[16];                               // P of this key against 32 query rows, packed bf16
       ok = __all_sync(0xffffffffu, bwd_wait(&sm.sdp_full[hf], m & 1, abort));
       if (ok) ok = __all_sync(0xffffffffu, bwd_wait(&sm.stat_full[hf], m & 1, abort));
       if (!ok) break;
       tc_fence_after_sync();
       HGA_TRACE_POINT(11);
+      // (S^T of this half-step was issued behind the GEMMs of the one before it in this region: that one's dV is complete)
+      if (kShortChains && hs >= 2) add_dv(hf);
+      if constexpr (kTerms) {
+        // 16 query rows at a time: P = e^(S*scale - LSE) in three terms, dS = scale * P o (dP - delta) in two
+        const uint32_t p3_addr = lane_base + kColP3 + hf * kP3Region + 16 * wg;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          uint32_t pt[16], p3[8], dt[16];
+          if (none) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) pt[i] = dt[i] = 0u;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) p3[i] = 0u;
+          } else {
+            uint32_t x[16], y[16];
+            tmem_ld16(s_addr + 16 * c, x);
+            tmem_ld16(dp_addr + 16 * c, y);
+            tmem_wait_ld();
+#pragma unroll
+            for (int i = 0; i < 8; i += 2) {
+              uint32_t ls[4], dl[4];                       // -LSE and -delta*scale of four consecutive columns
+              ld_shared_v4(nlse_a + (16 * c + 2 * i) * 4, ls[0], ls[1], ls[2], ls[3]);
+              ld_shared_v4(nds_a + (16 * c + 2 * i) * 4, dl[0], dl[1], dl[2], dl[3]);
+#pragma unroll
+              for (int u = 0; u < 2; ++u) {
+                const int w2 = i + u, col = 16 * c + 2 * w2;
+                float a0, a1;
+                unpack_f32x2(mul_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(x[2 * w2]), __uint_as_float(x[2 * w2 + 1])), scale_2,
+                                                 pack_f32x2(__uint_as_float(ls[2 * u]), __uint_as_float(ls[2 * u + 1]))), log2e_2), a0, a1);
+                float p0 = fast_exp2(a0), p1 = fast_exp2(a1), d0, d1;
+                if (masked) {
+                  if (col < imin) p0 = 0.f;
+                  if (col + 1 < imin) p1 = 0.f;
+                }
+                const uint64_t g = fma_f32x2(pack_f32x2(__uint_as_float(y[2 * w2]), __uint_as_float(y[2 * w2 + 1])), scale_2,
+                                             pack_f32x2(__uint_as_float(dl[2 * u]), __uint_as_float(dl[2 * u + 1])));
+                unpack_f32x2(mul_f32x2(pack_f32x2(p0, p1), g), d0, d1);
+                pt[w2] = next_term(p0, p1);
+                pt[8 + w2] = next_term(p0, p1);
+                p3[w2] = pack_bf16(p0, p1);
+                dt[w2] = next_term(d0, d1);
+                dt[8 + w2] = pack_bf16(d0, d1);
+              }
+            }
+          }
+          tmem_st16(s_addr + 16 * c, pt);                  // over the columns just read
+          tmem_st8(p3_addr + 8 * c, p3);
+          tmem_st16(dp_addr + 16 * c, dt);
+        }
+      } else {
+      uint32_t pk[16];                               // P of this key against 32 query rows, packed bf16
       if (none) {
         // no key of this warp is visible to any of the 32 rows: zeros, no exponentials
 #pragma unroll
@@ -381,6 +465,7 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
         }
         tmem_st16(dp_addr, out);                     // dS^T (bf16) over the first 16 of the dP^T columns just read
       }
+      }
       tmem_wait_st();
       tc_fence_before_sync();
       mbar_arrive_warp(&sm.pds_full[hf]);
@@ -390,29 +475,52 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
     if (ok) ok = __all_sync(0xffffffffu, bwd_wait(&sm.acc_done, 0, abort));
     HGA_TRACE_POINT(20);
     if (ok) {
-      // epilogue: thread = key row; warpgroup 0 sends dV, warpgroup 1 dK.  A row (512 bytes) goes through
+      // epilogue: thread = key row; warpgroup 0 sends dV, warpgroup 1 dK.  A row (4 head_dim bytes) goes through
       // shared memory (the Q / dO / O tiles, free now: every GEMM and every copy into them is complete) and
-      // leaves as one bulk copy, or one bulk add with the accumulate flag; rows are 528 bytes apart so that
+      // leaves as one bulk copy, or one bulk add with the accumulate flag; rows are 16 bytes further apart so that
       // the 16-byte stores of a quarter warp fall into different banks
       tc_fence_after_sync();
       constexpr uint32_t kRowPitch = kD * 4 + 16;
       static_assert(2 * 128 * kRowPitch <= 5 * kTile, "staging area: q, dO and o tiles");
       const int srow = kt * kKeys + key;
-      float* dst = (wg == 0 ? dV : dK) + (row_base(dm, sg, b) * dm.Hkv + (int64_t)h * sg.S + srow) * kD;
-      const uint32_t col = wg == 0 ? kColDV : kColDK;
-      const uint32_t stage = smem_u32(sm.q[0]) + (uint32_t)(wg * 128 + key) * kRowPitch;
-#pragma unroll
-      for (int c = 0; c < kD / 32; ++c) {
+      const int64_t out = (row_base(dm, sg, b) * dm.Hkv + (int64_t)h * sg.S + srow) * kD;
+      const uint32_t stage = smem_u32(sm.q[0]) + (uint32_t)key * kRowPitch;          // (dK's rows behind dV's)
+      auto send = [&](float* dst, uint32_t from, uint32_t bytes) {
+        if (dm.flags & HGA_FLAG_BWD_ACCUMULATE) bulk_reduce_add_f32(dst, from, bytes);
+        else bulk_store(dst, from, bytes);
+      };
+      if constexpr (kShortChains) {
+        // a thread holds half of its key's dV, and sends that half of dK as well
+        add_dv(0);
+        add_dv(1);
         uint32_t x[32];
-        tmem_ld32(lane_base + col + 32 * c, x);
+        tmem_ld32(lane_base + kColDK + 32 * wg, x);
         tmem_wait_ld();
+        const uint32_t mine = stage + (uint32_t)wg * 128;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) st_shared_v4(stage + (uint32_t)(32 * c + 4 * i) * 4, x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3]);
+        for (int i = 0; i < 8; ++i) {
+          st_shared_v4(mine + 16 * i, __float_as_uint(dv_sum[4 * i]), __float_as_uint(dv_sum[4 * i + 1]), __float_as_uint(dv_sum[4 * i + 2]), __float_as_uint(dv_sum[4 * i + 3]));
+          st_shared_v4(mine + 128 * kRowPitch + 16 * i, x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3]);
+        }
+        fence_proxy_async_smem();
+        if (srow < sg.S) {
+          send(dV + out + 32 * wg, mine, 128);
+          send(dK + out + 32 * wg, mine + 128 * kRowPitch, 128);
+        }
+      } else {
+        const uint32_t col = wg == 0 ? kColDV : kColDK, mine = stage + (uint32_t)wg * 128 * kRowPitch;
+#pragma unroll
+        for (int c = 0; c < kD / 32; ++c) {
+          uint32_t x[32];
+          tmem_ld32(lane_base + col + 32 * c, x);
+          tmem_wait_ld();
+#pragma unroll
+          for (int i = 0; i < 8; ++i) st_shared_v4(mine + (uint32_t)(32 * c + 4 * i) * 4, x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3]);
+        }
+        fence_proxy_async_smem();
+        if (srow < sg.S) send((wg == 0 ? dV : dK) + out, mine, kD * 4);
       }
-      fence_proxy_async_smem();
       if (srow < sg.S) {
-        if (dm.flags & HGA_FLAG_BWD_ACCUMULATE) bulk_reduce_add_f32(dst, stage, kD * 4);
-        else bulk_store(dst, stage, kD * 4);
         tma_store_commit();
         tma_store_wait_read();
       }
@@ -475,7 +583,7 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
       // the key threads read the previous step's statistics of this half until they hand its P^T and dS^T over
       if (m > 0) ok = __all_sync(0xffffffffu, bwd_wait(&sm.pds_full[j >> 6], (m - 1) & 1, abort));
       if (!ok) break;
-      sm.nlse[j] = -lse * 1.4426950408889634f;
+      sm.nlse[j] = kTerms ? -lse : -lse * 1.4426950408889634f;
       sm.nds[j] = -delta * dm.scale;
       mbar_arrive_warp(&sm.stat_full[j >> 6]);
       HGA_TRACE_POINT(14);
@@ -508,7 +616,7 @@ bool attn_bwd_band_sm100_supported(const Dims& dm) {
   return dm.d == 128 || dm.d == 64;
 }
 
-template <int D, class Segs>
+template <int D, bool kTerms, class Segs>
 static int launch_band(const Dims& dm, const Segs& segs, int64_t units, const void* Q, const void* K, const void* V, const void* O,
                        const float* LSE, const void* dO, float* dK, float* dV, int32_t* status_word, cudaStream_t st) {
   CUtensorMap mq, mdo, mk, mv, mo;
@@ -526,10 +634,10 @@ static int launch_band(const Dims& dm, const Segs& segs, int64_t units, const vo
       encode_tensor_map_bf16(&mv, V, 5, dk, sv, box, true))
     return HGA_ERR_UNSUPPORTED;
   const size_t smem = sizeof(BandSmem<D>) + 1024;
-  const int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(&k_attn_bwd_band_sm100<D, Segs>), smem);
+  const int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(&k_attn_bwd_band_sm100<D, kTerms, Segs>), smem);
   if (rc) return rc;
   PdlLaunch cfg((unsigned)units, kBandThreads, smem, st, dm.flags);
-  const cudaError_t e = cudaLaunchKernelEx(&cfg.c, k_attn_bwd_band_sm100<D, Segs>, mq, mdo, mk, mv, mo, LSE, dm, dK, dV, status_word, segs);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg.c, k_attn_bwd_band_sm100<D, kTerms, Segs>, mq, mdo, mk, mv, mo, LSE, dm, dK, dV, status_word, segs);
   count_launch(HGA_KERNELS_BWD_TENSOR);
   return record_cuda(e);
 }
@@ -538,12 +646,14 @@ int launch_attn_bwd_band_sm100(const Dims& dm, SegTable* segs, const void* Q, co
                                const float* LSE, const void* dO, float* dK, float* dV, int32_t* status_word,
                                cudaStream_t st) {
   auto tiles = [&](int S) { return (int64_t)dm.B * dm.Hkv * ((S + kKeys - 1) / kKeys); };
-  if (!segs)
-    return dm.d == 128 ? launch_band<128>(dm, OneSegment{}, tiles(dm.S), Q, K, V, O, LSE, dO, dK, dV, status_word, st)
-                       : launch_band<64>(dm, OneSegment{}, tiles(dm.S), Q, K, V, O, LSE, dO, dK, dV, status_word, st);
+#define HGA_BAND(segs, units)                                                                                                        \
+  (dm.d == 64 ? launch_band<64, true>(dm, segs, units, Q, K, V, O, LSE, dO, dK, dV, status_word, st)                                  \
+   : bwd_in_terms(dm) ? launch_band<128, true>(dm, segs, units, Q, K, V, O, LSE, dO, dK, dV, status_word, st)                          \
+                      : launch_band<128, false>(dm, segs, units, Q, K, V, O, LSE, dO, dK, dV, status_word, st))
+  if (!segs) return HGA_BAND(OneSegment{}, tiles(dm.S));
   const int64_t units = number_units(*segs, [&](const Segment& g) { return tiles(g.S); });
-  return dm.d == 128 ? launch_band<128>(dm, *segs, units, Q, K, V, O, LSE, dO, dK, dV, status_word, st)
-                     : launch_band<64>(dm, *segs, units, Q, K, V, O, LSE, dO, dK, dV, status_word, st);
+  return HGA_BAND(*segs, units);
+#undef HGA_BAND
 }
 
 }  // namespace hga

@@ -1,4 +1,4 @@
-// hga_attn_bwd for sm_100a (head_dim 128): backward of routed exact-token attention with the
+// hga_attn_bwd for sm_100a (head_dim 128, items of whole 128-row M-tiles): backward of routed exact-token attention with the
 // routing frozen (Section 2.1, last paragraph) and history K/V detached (Section 2.2).
 //
 // Work unit (one CTA): one 128-row M-tile of one item, swept over the item's routed keys, which
@@ -109,7 +109,7 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   HGA_TRACE_DECL(512);
-  const int n_mt_item = (dm.rows + 127) / 128;           // (the last M-tile may hold 64 rows only)
+  const int n_mt_item = dm.rows / 128;
   // Launch order: late query blocks first.  They have the most routed keys inside the active segment (the
   // expensive dK/dV steps), early ones none, so the cheapest CTAs are the ones that fill the last wave.
   int cta;
@@ -149,12 +149,10 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       // four boxes of 64 rows x one 64-element panel per tensor, laid out [panel][128 rows][128 B]
       const int half = warp & 1, panel = (warp >> 1) & 1;
       const int r = mt * 128 + 64 * half;
-      const bool real = r < dm.rows;                     // (rows past the item's last one arrive as zeros)
-      const int a = real ? r / dm.Bq : 0, t = r % dm.Bq;
+      const int a = r / dm.Bq, t = r % dm.Bq;
       const uint32_t off = (uint32_t)panel * 16384 + (uint32_t)half * 8192;
-      const int row = real ? qrow + t : dm.rows_q;
-      if (warp < 4) tma_load_5d(sm.q + off, &map_q, &sm.q_full, 0, row, panel, h * dm.G + a, b);
-      else tma_load_5d(sm.dO + off, &map_do, &sm.q_full, 0, row, panel, h * dm.G + a, b);
+      if (warp < 4) tma_load_5d(sm.q + off, &map_q, &sm.q_full, 0, qrow + t, panel, h * dm.G + a, b);
+      else tma_load_5d(sm.dO + off, &map_do, &sm.q_full, 0, qrow + t, panel, h * dm.G + a, b);
     }
     __syncwarp();
   }
@@ -196,9 +194,9 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   float row_lse = 0.f;
   uint4 o_half[8];
   if (warp >= 2 && warp < 10) {
-    const int r_own = mt * 128 + (warp & 3) * 32 + lane, r = min(r_own, dm.rows - 1);
+    const int r = mt * 128 + (warp & 3) * 32 + lane;
     const int hq = h * dm.G + r / dm.Bq, srow = qrow + r % dm.Bq;
-    row_lse = r_own < dm.rows ? LSE[row_base(dm, sg, b) * dm.Hq + (int64_t)hq * sg.S + (srow - sg.q0)] : INFINITY;   // (padding rows: P = 0)
+    row_lse = LSE[row_base(dm, sg, b) * dm.Hq + (int64_t)hq * sg.S + (srow - sg.q0)];
     const uint4* op = reinterpret_cast<const uint4*>(O + b * dm.os[0] + hq * dm.os[1] + (int64_t)srow * dm.os[2]) +
                       8 * ((warp - 2) >> 2);
 #pragma unroll
@@ -580,12 +578,10 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       if (warp == 2 && lane < 4 && bwd_wait(&sm.dq_staged, 0, abort)) {      // all 256 rows are in shared memory
         const int half = lane & 1, panel = lane >> 1;
         const int r0 = mt * 128 + 64 * half;
-        if (r0 < dm.rows) {
-          tma_store_5d(&map_dq, sm.q + panel * 16384 + half * 8192, 0, qrow + r0 % dm.Bq, panel,
-                       h * dm.G + r0 / dm.Bq, b);
-          tma_store_commit();
-          tma_store_wait_read();    // (the source tile has been read; the writes complete before the grid does)
-        }
+        tma_store_5d(&map_dq, sm.q + panel * 16384 + half * 8192, 0, qrow + r0 % dm.Bq, panel,
+                     h * dm.G + r0 / dm.Bq, b);
+        tma_store_commit();
+        tma_store_wait_read();    // (the source tile has been read; the writes complete before the grid does)
       }
     }
   } else {
@@ -794,7 +790,7 @@ static int launch_sweep(const Dims& dm, SegTable* table, const Segs& segs, int64
   // serialization; it waits for it only before adding to dK/dV).
   rc = launch_attn_bwd_band_sm100(dm, table, Q, K, V, O, LSE, dO, dK, dV, status_word, st);
   if (rc != HGA_OK) return rc;
-  if (table) units = number_units(*table, [&](const Segment& g) { return (int64_t)dm.B * dm.Hkv * (g.S / dm.Bq) * ((dm.rows + 127) / 128); });
+  if (table) units = number_units(*table, [&](const Segment& g) { return (int64_t)dm.B * dm.Hkv * (g.S / dm.Bq) * (dm.rows / 128); });
   PdlLaunch cfg((unsigned)units, kBwdThreads, smem, st, dm.flags);
   const cudaError_t e = cudaLaunchKernelEx(&cfg.c, k_attn_bwd_sm100<Segs>, mq, mdo, mk, mv, mdq, (const uint16_t*)O, LSE, group_idx,
                                            n_groups, dm, dK, dV, status_word, segs);
@@ -806,9 +802,9 @@ int launch_attn_bwd_sm100(const Dims& dm, SegTable* segs, const void* Q, const v
                           const float* LSE, const void* dO, const int32_t* group_idx,
                           const int32_t* n_groups, void* dQ, float* dK, float* dV, int32_t* status_word,
                           cudaStream_t st) {
-  if (dm.d == 64)
-    return launch_attn_bwd_d64_sm100(dm, segs, Q, K, V, O, LSE, dO, group_idx, n_groups, dQ, dK, dV, status_word, st);
-  const int64_t units = (int64_t)dm.B * dm.Hkv * dm.NQB * ((dm.rows + 127) / 128);
+  if (bwd_in_terms(dm))
+    return launch_attn_bwd_terms_sm100(dm, segs, Q, K, V, O, LSE, dO, group_idx, n_groups, dQ, dK, dV, status_word, st);
+  const int64_t units = (int64_t)dm.B * dm.Hkv * dm.NQB * (dm.rows / 128);
   if (!segs)
     return launch_sweep(dm, nullptr, OneSegment{}, units, Q, K, V, O, LSE, dO, group_idx, n_groups, dQ, dK, dV, status_word, st);
   return launch_sweep(dm, segs, *segs, units, Q, K, V, O, LSE, dO, group_idx, n_groups, dQ, dK, dV, status_word, st);

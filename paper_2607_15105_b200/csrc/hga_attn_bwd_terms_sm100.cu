@@ -1,13 +1,21 @@
-// hga_attn_bwd for sm_100a, head_dim 64: the query-major sweep (routing frozen, Section 2.1 last paragraph; history K/V
-// detached, Section 2.2).
+// hga_attn_bwd for sm_100a with fp32-grade probabilities: the query-major sweep (routing frozen, Section 2.1 last paragraph;
+// history K/V detached, Section 2.2) of the shapes that the CUDA-core backward, which holds P and dS in fp32, used to take:
+// head_dim 64, and query-row counts that do not fill 128-row M-tiles.
+//
+// bf16 operands hold P and dS to 2^-9.  Here P enters its products in three bf16 terms (p = p1 + p2 + p3, each the rounding
+// of what the ones before it leave: 24 bits) and dS in two (16 bits; its error is that of delta = rowsum(dO o O), which
+// comes from the rounded O, 2^-9 of a sum of many, and dQ is rounded to bf16).  Every term is a GEMM of its own.  Errors
+// against fp64 (head_dim 64, 64 rows; relative, dQ / dK / dV): 1.68e-3 / 1.33e-4 / 5.0e-7, on CUDA cores 1.68e-3 / 1.33e-4 /
+// 3.8e-7 (the tensor pipe cuts S and its sums off at 2^-24), with one term 2.9e-3 / 2.1e-3 / 1.6e-3; at head_dim 128 dV
+// is off by 0.8e-6 to 1.8e-6 (see k_attn_bwd_band_sm100 for why not less).
+// hga_attn_bwd, 16 heads of 64 rows, 512 items of 768 keys: head_dim 64 98 us (one term 68, CUDA cores 918), head_dim 128
+// 160 us (99, 1970).  What bounds it: the row threads, with twice the instructions per weight, and the hand-offs.
 //
 // Work unit (one CTA): one 128-row M-tile of one item (b, kv head, query block), swept over the item's routed
 // keys in 64-key tiles (eight octets of 8 consecutive tokens, one TMA box each).  At head_dim 64 a CTA takes less than
 // half of an SM (88 KB of shared memory, 256 TMEM columns, 256 threads), so two CTAs run on an SM: a tile is
-// a chain of hand-offs (copy -> S -> P -> dS -> dQ), and while one CTA is in its exponentials, its set-up, its
-// dK/dV reduction or its epilogue, the other one has the tensor pipe.  (At head_dim 128 the same layout was slower than
-// the pairs of tiles of k_attn_bwd_sm100, 3.3k against 3.0k cycles per 128 keys and SM: its GEMMs have twice the K
-// steps and an N = 64 instruction costs nearly as much as one with N = 128, so the pipe itself was the bound.)
+// a chain of hand-offs (copy -> S -> dS -> dQ), and while one CTA is in its exponentials, its set-up, its
+// dK/dV reduction or its epilogue, the other one has the tensor pipe.  At head_dim 128 it has the SM to itself.
 //
 // Order of the tiles of an item:
 //   1. the local window and the causal block, [ls, p0 + Bq): known without the routing list, so their copies
@@ -15,21 +23,22 @@
 //   2. "far" keys (sink, then the selected groups, ascending) of the detached history: dQ only;
 //   3. far keys of the active segment, which also get dK/dV from this kernel (the local band's dK/dV are written by
 //      the key-major kernel k_attn_bwd_band_sm100, which precedes this one and stores every row).
-// Per tile: S = Q K^T, dP = dO V^T (smem x smem -> TMEM); one thread per query row turns them into
-// P = 2^(S*c - LSE*log2e) (packed bf16 in registers) and dS = scale * P o (dP - delta);
-//   kinds 1, 2:  dS (bf16) goes over the dP columns just read; dQ += dS K with A from TMEM
-//   kind 3:      P and dS go to shared memory; dQ += dS K; dV^T = dO^T P over S's columns, dK^T = Q^T dS over dP's, both
-//                with M = 128: A = [dO^T ; Q^T] (the two tiles are neighbours), of whose products with P and dS one half
-//                each is wanted; the row threads stage the transposed tiles in shared memory as key rows (dV | dK) and
-//                add them to global memory with bulk reductions, one 256-byte row per instruction.
-// S(j+1) is issued as soon as the rows have read S(j), dP(j+1) behind dQ(j): the in-order tensor pipe makes every
-// reuse of a region safe.  A wait on S(j+1)'s K tile never holds up dQ(j), which frees the stage of K(j+2).
+// Per tile: S = Q K^T, dP = dO V^T (smem x smem -> TMEM); one thread per query row turns them, 16 keys at a time, into
+// P = e^(S*scale - LSE) and dS = scale * P o (dP - delta), and the two terms of dS go over the dP columns just read:
+// dQ += dS K with A from TMEM.  Tiles of kind 3 go through shared memory in three rounds besides: p1 and p2; p3 and dS's
+// first term; dS's second.  dV^T = dO^T P (over the other S buffer) and dK^T = Q^T dS (over this tile's S, dead by then) sum
+// them up; the row threads stage the transposed tiles in shared memory as key rows and add them to global memory with bulk
+// reductions.  At head_dim 64 one instruction does both halves, M = 128: A = [dO^T ; Q^T] (the two tiles are neighbours), of
+// whose products with P and dS one half each is wanted, and a staged row is dV | dK.
+// S has two buffers: S(j+1) is issued ahead of dQ(j) if its K tile is already there, dP(j+1) behind dQ(j): the in-order
+// tensor pipe makes every reuse of a region safe.  A wait on S(j+1)'s K tile never holds up dQ(j), which frees the stage of
+// K(j+2).
 //
 // Warp roles (256 threads):
 //   warps 0, 7   producers: octets 0-3 / 4-7 of every K and V tile (a box costs its issuing warp ~100 cycles)
 //   warp 6       Q and dO tiles, then the check of the routing list       warp 1   MMA issuer
 //   warps 2-5    one thread per query row (TMEM lane = row); delta = rowsum(dO o O) of its own row
-// TMEM (256 columns): S 64 | dP / dS 64 | dQ 64.
+// TMEM: S 64 | dP / dS 64 | dQ head_dim | S 64.
 #include "hga_bwd_sm100.cuh"
 #include "hga_common.cuh"
 #include "hga_octets.cuh"
@@ -42,24 +51,22 @@ using namespace sm100;
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int D = 64;
 constexpr int kKT = 64;                         // keys per tile
-constexpr int kPdsTile = 128 * kKT * 2;         // bytes of one P or dS tile: [16 row octets][8 rows][128 B], 128-byte swizzle
+constexpr int kPdsTile = 128 * kKT * 2;         // bytes of one term of P or dS: [16 row octets][8 rows][128 B], 128-byte swizzle
 
-constexpr int kQBytes = 128 * D * 2;            // the Q or dO tile: [128 rows][128 B]
-constexpr int kKv = kKT * D * 2;                // one K or V tile: [octet][8 rows][128 B]
-constexpr int kOct = 8 * D * 2;
-
+template <int D>
 struct SweepSmem {
-  alignas(1024) uint8_t dO[kQBytes];            // (dO and Q adjacent: one MN-major operand of 128 rows, see above)
+  static constexpr int kQBytes = 128 * D * 2;   // the Q or dO tile: [panel][128 rows][128 B]
+  static constexpr int kKv = kKT * D * 2;       // one K or V tile: [octet][panel][8 rows][128 B]
+  alignas(1024) uint8_t dO[kQBytes];            // (dO and Q adjacent: at head_dim 64 one MN-major operand of 128 rows, see above)
   alignas(1024) uint8_t q[kQBytes];
   alignas(1024) uint8_t k[2][kKv];
   alignas(1024) uint8_t v[kKv];
-  alignas(1024) uint8_t p[kPdsTile];            // dK/dV tiles: P and dS, then the staged dV | dK rows of 32 keys each
-  alignas(1024) uint8_t ds[kPdsTile];
+  alignas(1024) uint8_t a[kPdsTile];            // dK/dV tiles: two terms at a time, then the staged key rows
+  alignas(1024) uint8_t b[kPdsTile];
   uint64_t q_full, k_full[2], k_empty[2], v_full;
-  uint64_t s_full, s_read, dp_full, ds_full;            // per tile
-  uint64_t dkv_full, staged, dk_read;                   // per dK/dV tile
+  uint64_t s_full[2], dp_full, ds_full;                 // per tile (S(j+1) may be complete before S(j) has been looked for)
+  uint64_t round_full, round_done, acc_read, staged;    // dK/dV tiles
   uint64_t info_full, dq_done, dq_staged, drain;
   uint32_t tmem_base;
   int n_far, first_active, n_listed;                    // far octets; the first of them that belongs to the active segment; list entries (see FarList)
@@ -67,21 +74,24 @@ struct SweepSmem {
   volatile int abort;
   int rows[4][8];                                       // token rows of the last four tiles' octets (dK/dV tiles read them back)
 };
-static_assert(sizeof(SweepSmem) + 1024 <= 113 * 1024, "two CTAs per SM");
+static_assert(sizeof(SweepSmem<64>) + 1024 <= 113 * 1024, "two CTAs per SM");
 
 }  // namespace
 
-template <class Segs>
-__global__ void __launch_bounds__(kThreads, 2)
-k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_do,
+template <int D, class Segs>
+__global__ void __launch_bounds__(kThreads, D == 64 ? 2 : 1)
+k_attn_bwd_terms_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_do,
                  const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                  const __grid_constant__ CUtensorMap map_dq, const uint16_t* __restrict__ O,
                  const float* __restrict__ LSE, const int32_t* __restrict__ group_idx,
                  const int32_t* __restrict__ n_groups, const Dims dm,
                  float* __restrict__ dK, float* __restrict__ dV, int32_t* status_word, const __grid_constant__ Segs segs) {
-  constexpr uint32_t kColS = 0, kColDP = 64, kColDQ = 128;
+  using Smem = SweepSmem<D>;
+  constexpr int kOct = 8 * D * 2, kPanels = D / 64, kQBytes = Smem::kQBytes, kKv = Smem::kKv;
+  constexpr uint32_t kColDP = 64, kColDQ = 128, kTmemCols = D == 64 ? 256 : 512;
+  auto s_col = [](int j) -> uint32_t { return (j & 1) ? 128 + D : 0; };      // S of tile j
   extern __shared__ uint8_t smem_raw[];
-  SweepSmem& sm = *reinterpret_cast<SweepSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   HGA_TRACE_DECL(64);
@@ -133,9 +143,9 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
     mbar_init(&sm.q_full, 1);
     for (int s = 0; s < 2; ++s) { mbar_init(&sm.k_full[s], 2); mbar_init(&sm.k_empty[s], 1); }
     mbar_init(&sm.v_full, 2);
-    mbar_init(&sm.s_full, 1); mbar_init(&sm.s_read, 4);
+    mbar_init(&sm.s_full[0], 1); mbar_init(&sm.s_full[1], 1);
     mbar_init(&sm.dp_full, 1); mbar_init(&sm.ds_full, 4);
-    mbar_init(&sm.dkv_full, 1); mbar_init(&sm.staged, 4); mbar_init(&sm.dk_read, 4);
+    mbar_init(&sm.round_full, 4); mbar_init(&sm.round_done, 1); mbar_init(&sm.acc_read, 4); mbar_init(&sm.staged, 4);
     mbar_init(&sm.info_full, 1); mbar_init(&sm.dq_done, 1); mbar_init(&sm.dq_staged, 4); mbar_init(&sm.drain, 1);
     sm.abort = 0;
     fence_barrier_init();
@@ -147,13 +157,13 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
     if (warp == 6) {
       if (lane == 0) mbar_arrive_expect_tx(&sm.q_full, 2 * kQBytes);
       __syncwarp();
-      if (lane < 4) {
-        // boxes of 64 rows, Q first, then dO; rows past the item's last one (an M-tile may hold 64 rows only) arrive as zeros
-        const int is_do = lane >> 1, hf = lane & 1;
+      if (lane < 4 * kPanels) {
+        // boxes of 64 rows x one panel, Q first, then dO; rows past the item's last one (an M-tile may hold 64 rows only) arrive as zeros
+        const int is_do = lane / (2 * kPanels), hf = lane & 1, panel = (lane >> 1) % kPanels;
         const int r = mt * 128 + 64 * hf;
         const bool real = r < dm.rows;
-        tma_load_5d((is_do ? sm.dO : sm.q) + hf * 8192, is_do ? &map_do : &map_q, &sm.q_full, 0,
-                    real ? qrow + r % dm.Bq : dm.rows_q, 0, h * dm.G + (real ? r / dm.Bq : 0), b);
+        tma_load_5d((is_do ? sm.dO : sm.q) + panel * 16384 + hf * 8192, is_do ? &map_do : &map_q, &sm.q_full, 0,
+                    real ? qrow + r % dm.Bq : dm.rows_q, panel, h * dm.G + (real ? r / dm.Bq : 0), b);
       }
     } else {
       const int row = local_row(0);
@@ -163,7 +173,7 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
     __syncwarp();
   }
   if (warp == 1) {
-    tmem_alloc(&sm.tmem_base, 256);
+    tmem_alloc(&sm.tmem_base, kTmemCols);
     tmem_relinquish();
     // the next kernel's launch may overlap this grid's tail (the conversion of bf16 outputs, the next step's summaries)
     if (lane == 0) pdl_launch_dependents();
@@ -210,8 +220,7 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
       note_rows(j, row);
       copy_tile(sm.k[j & 1], &map_k, &sm.k_full[j & 1], row);
     };
-    // Rows of the next two tiles, looked up ahead of their use.  Tile j + 1's K has been issued when tile j is
-    // handled, except behind a dK/dV tile.
+    // Rows of the next two tiles, looked up ahead of their use.  Tile j + 1's K has been issued when tile j is handled.
     if (n_lt < 3) learn();
     int next_row = ok ? row_of(1) : dm.rows_k, after_row = ok ? row_of(2) : dm.rows_k;
     if (ok && (n_lt > 1 || n > 1)) copy_k(1, next_row);
@@ -219,22 +228,13 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
     for (int j = 0; ok; ++j) {
       if (!known && j + 3 >= n_lt && !learn()) break;
       if (known && j + 1 >= n) break;
-      if (!known || j < n_a) {
-        if (!wait_for(&sm.dp_full, j & 1)) break;                           // V(j) has been read
-        copy_tile(sm.v, &map_v, &sm.v_full, next_row);                       // V(j+1)
-        next_row = after_row;
-        after_row = row_of(j + 3);
-        if (!known || (j + 2 < n && j + 2 <= n_a)) {
-          if (!wait_for(&sm.k_empty[j & 1], (j >> 1) & 1)) break;           // dQ(j) is done
-          copy_k(j + 2, next_row);
-        }
-      } else {
-        // behind a dK/dV tile both stages are free
-        if (!wait_for(&sm.dkv_full, (j - n_a) & 1)) break;
-        copy_k(j + 1, next_row);
-        copy_tile(sm.v, &map_v, &sm.v_full, next_row);
-        next_row = after_row;
-        after_row = row_of(j + 3);
+      if (!wait_for(&sm.dp_full, j & 1)) break;                           // V(j) has been read
+      copy_tile(sm.v, &map_v, &sm.v_full, next_row);                       // V(j+1)
+      next_row = after_row;
+      after_row = row_of(j + 3);
+      if (!known || j + 2 < n) {
+        if (!wait_for(&sm.k_empty[j & 1], (j >> 1) & 1)) break;           // dQ(j) is done
+        copy_k(j + 2, next_row);
       }
       HGA_TRACE_POINT(2);
     }
@@ -254,29 +254,35 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
     constexpr uint32_t idesc_dq = idesc_bf16_f32(128, D, 0, 1);          // dS K-major, K tile MN-major
     constexpr uint32_t idesc_dkv = idesc_bf16_f32(128, kKT, 1, 1);       // both MN-major
     // Descriptors are built once; inside the loops an MMA costs two integer adds.
-    // Q, dO: [128 rows][128 B] (8-row groups 1024 B apart)
+    // Q, dO: [panel][128 rows][128 B] (8-row groups 1024 B apart, panels 16 KB apart)
     const uint64_t q_k = smem_desc_sw128(smem_u32(sm.q), 16, 1024);         // Q  as K-major A   (S)
     const uint64_t do_k = smem_desc_sw128(smem_u32(sm.dO), 16, 1024);       // dO as K-major A   (dP)
-    // MN-major A of dV^T and dK^T: dO, and Q 16 KB on, as the two 64-element atoms
-    const uint64_t doq_mn = smem_desc_sw128(smem_u32(sm.dO), 16384, 1024);
+    // MN-major A of dV^T and of dK^T (two 64-element atoms 16 KB apart: the panels, or at head_dim 64 dO and Q for both)
+    const uint64_t do_mn = smem_desc_sw128(smem_u32(sm.dO), 16384, 1024);
+    const uint64_t q_mn = D == 64 ? do_mn : smem_desc_sw128(smem_u32(sm.q), 16384, 1024);
     const uint64_t k_k0 = smem_desc_sw128(smem_u32(sm.k[0]), 16, kOct);     // K tile, K-major B  (S)
     const uint64_t v_k = smem_desc_sw128(smem_u32(sm.v), 16, kOct);         // V tile, K-major B  (dP)
     const uint64_t k_mn0 = smem_desc_sw128(smem_u32(sm.k[0]), 1024, kOct);  // K tile, MN-major B (dQ)
-    const uint64_t dsd = smem_desc_sw128(smem_u32(sm.ds), 16, 1024);       // dS: K-major A (dQ) and MN-major B (dK^T)
-    const uint64_t pd = smem_desc_sw128(smem_u32(sm.p), 16, 1024);          // P : MN-major B (dV^T)
-    auto issue_qk = [&](uint32_t acc, uint64_t a, uint64_t bd) {
+    const uint64_t ad = smem_desc_sw128(smem_u32(sm.a), 16, 1024);          // a term of P or dS: MN-major B
+    const uint64_t bd = smem_desc_sw128(smem_u32(sm.b), 16, 1024);
+    auto issue_qk = [&](uint32_t acc, uint64_t a, uint64_t b) {
 #pragma unroll
-      for (int kk = 0; kk < D / 16; ++kk) {
-        mma_ss_w(lead, acc, desc_advance(a, kk * 32), desc_advance(bd, kk * 32), idesc_sdp, kk > 0);
-      }
+      for (int kk = 0; kk < D / 16; ++kk)
+        mma_ss_w(lead, acc, desc_advance(a, (kk >> 2) * 16384 + (kk & 3) * 32), desc_advance(b, (kk >> 2) * 1024 + (kk & 3) * 32), idesc_sdp, kk > 0);
     };
     auto issue_s = [&](int j) {
-      issue_qk(tmem + kColS, q_k, desc_advance(k_k0, (uint32_t)(j & 1) * kKv));
-      mma_commit_w(lead, &sm.s_full);
+      issue_qk(tmem + s_col(j), q_k, desc_advance(k_k0, (uint32_t)(j & 1) * kKv));
+      mma_commit_w(lead, &sm.s_full[j & 1]);
     };
     auto issue_dp = [&]() {
       issue_qk(tmem + kColDP, do_k, v_k);
       mma_commit_w(lead, &sm.dp_full);           // also tells the producers that the V tile is free
+    };
+    // dV^T or dK^T: 16 query rows per MMA (2 row octets)
+    auto issue_t = [&](uint32_t acc, uint64_t amn, uint64_t term, bool accumulate) {
+#pragma unroll
+      for (int kk = 0; kk < 128 / 16; ++kk)
+        mma_ss_w(lead, acc, desc_advance(amn, kk * 2048), desc_advance(term, kk * 2048), idesc_dkv, accumulate || kk > 0);
     };
     bool ok = mma_wait(&sm.q_full, 0) && mma_wait(&sm.k_full[0], 0);
     HGA_TRACE_POINT(40);
@@ -291,70 +297,63 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
         if (!ok) break;
         counts(sm.n_far, sm.first_active, n, n_a);
       }
-      const uint64_t kmn = desc_advance(k_mn0, (uint32_t)(j & 1) * kKv);
-      if (j < n_a) {
-        // S(j+1) goes ahead of dQ(j) if its K tile is already there; waiting for it first would hold up dQ(j), and with
-        // it the copy of K(j+2) into the stage that dQ(j) reads
-        bool s_ahead = false;
-        if (j + 1 < n) {
-          ok = mma_wait(&sm.s_read, j & 1);
-          if (!ok) break;
-          s_ahead = __all_sync(0xffffffffu, mbar_test_wait(&sm.k_full[(j + 1) & 1], k_parity(j + 1)));
-          if (s_ahead) {
-            tc_fence_after_sync();
-            issue_s(j + 1);
-            HGA_TRACE_POINT(6);
-          }
-        }
-        ok = mma_wait(&sm.ds_full, j & 1);
-        if (!ok) break;
-        tc_fence_after_sync();
-        HGA_TRACE_POINT(5);
-#pragma unroll
-        for (int kk = 0; kk < kKT / 16; ++kk)     // 16 keys per MMA: 8 TMEM columns of dS, two octets of the K tile
-          mma_ts_w(lead, tmem + kColDQ, tmem + kColDP + 8 * kk, desc_advance(kmn, kk * 2 * kOct), idesc_dq, (j > 0 || kk > 0));
-        mma_commit_w(lead, &sm.k_empty[j & 1]);
-        HGA_TRACE_POINT(7);
-        if (j + 1 < n) {
-          if (!s_ahead) {
-            ok = mma_wait(&sm.k_full[(j + 1) & 1], k_parity(j + 1));
-            if (!ok) break;
-            tc_fence_after_sync();
-            issue_s(j + 1);
-          }
-          ok = mma_wait(&sm.v_full, (j + 1) & 1);
-          if (!ok) break;
+      const bool dkv = j >= n_a;
+      // S(j+1) goes ahead of dQ(j) if its K tile is already there (its buffer held S(j-1), which the rows are done with); waiting
+      // for the tile first would hold up dQ(j), and with it the copy of K(j+2) into the stage that dQ(j) reads
+      bool s_ahead = false;
+      if (!dkv && j + 1 < n) {
+        s_ahead = __all_sync(0xffffffffu, mbar_test_wait(&sm.k_full[(j + 1) & 1], k_parity(j + 1)));
+        if (s_ahead) {
           tc_fence_after_sync();
-          issue_dp();
-          HGA_TRACE_POINT(8);
+          issue_s(j + 1);
+          HGA_TRACE_POINT(6);
         }
-      } else {
-        ok = mma_wait(&sm.ds_full, j & 1);        // P and dS are in shared memory, S and dP have been read
+      }
+      ok = mma_wait(&sm.ds_full, j & 1);
+      if (!ok) break;
+      tc_fence_after_sync();
+      HGA_TRACE_POINT(5);
+      const uint64_t kmn = desc_advance(k_mn0, (uint32_t)(j & 1) * kKv);
+#pragma unroll
+      for (int kk = 0; kk < 2 * (kKT / 16); ++kk)     // 16 keys (two octets of the K tile): 8 TMEM columns of each of dS's terms
+        mma_ts_w(lead, tmem + kColDQ, tmem + kColDP + 8 * kk, desc_advance(kmn, (kk >> 1) * 2 * kOct), idesc_dq, (j > 0 || kk > 0));
+      mma_commit_w(lead, &sm.k_empty[j & 1]);
+      HGA_TRACE_POINT(7);
+      if (dkv) {
+        const uint32_t dv_acc = tmem + s_col(j + 1), dk_acc = tmem + s_col(j);
+        const uint32_t phase = (uint32_t)(j - n_a) * 2;
+        issue_t(dv_acc, do_mn, ad, false);                              // p1, p2
+        issue_t(dv_acc, do_mn, bd, true);
+        mma_commit_w(lead, &sm.round_done);
+        ok = mma_wait(&sm.round_full, phase & 1);
         if (!ok) break;
         tc_fence_after_sync();
-        HGA_TRACE_POINT(45);
-#pragma unroll
-        for (int kk = 0; kk < kKT / 16; ++kk)
-          mma_ss_w(lead, tmem + kColDQ, desc_advance(dsd, kk * 32), desc_advance(kmn, kk * 2 * kOct), idesc_dq, (j > 0 || kk > 0));
-#pragma unroll
-        for (int kk = 0; kk < 128 / 16; ++kk)     // 16 query rows per MMA (2 row octets)
-          mma_ss_w(lead, tmem + kColS, desc_advance(doq_mn, kk * 2048), desc_advance(pd, kk * 2048), idesc_dkv, kk > 0);
-#pragma unroll
-        for (int kk = 0; kk < 128 / 16; ++kk)
-          mma_ss_w(lead, tmem + kColDP, desc_advance(doq_mn, kk * 2048), desc_advance(dsd, kk * 2048), idesc_dkv, kk > 0);
-        mma_commit_w(lead, &sm.dkv_full);
+        issue_t(dv_acc, do_mn, ad, true);                               // p3, dS's first term (S(j) has been read)
+        issue_t(dk_acc, q_mn, bd, false);
+        mma_commit_w(lead, &sm.round_done);
+        ok = mma_wait(&sm.round_full, (phase + 1) & 1);
+        if (!ok) break;
+        tc_fence_after_sync();
+        issue_t(dk_acc, q_mn, ad, true);                                // dS's second term
+        mma_commit_w(lead, &sm.round_done);
         HGA_TRACE_POINT(4);
         if (j + 1 < n) {
-          // the row threads have read dV^T: S(j+1) may take its place; then dK^T: dP(j+1)
-          ok = mma_wait(&sm.s_read, j & 1) && mma_wait(&sm.k_full[(j + 1) & 1], k_parity(j + 1));
+          ok = mma_wait(&sm.acc_read, (uint32_t)(j - n_a) & 1);         // S(j+1) takes the place of dV^T
+          if (!ok) break;
+        }
+      }
+      if (j + 1 < n) {
+        if (!s_ahead) {
+          ok = mma_wait(&sm.k_full[(j + 1) & 1], k_parity(j + 1));
           if (!ok) break;
           tc_fence_after_sync();
           issue_s(j + 1);
-          ok = mma_wait(&sm.dk_read, (j - n_a) & 1) && mma_wait(&sm.v_full, (j + 1) & 1);
-          if (!ok) break;
-          tc_fence_after_sync();
-          issue_dp();
         }
+        ok = mma_wait(&sm.v_full, (j + 1) & 1);
+        if (!ok) break;
+        tc_fence_after_sync();
+        issue_dp();
+        HGA_TRACE_POINT(8);
       }
     }
     if (ok) mma_commit_w(lead, &sm.dq_done);
@@ -374,8 +373,6 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
     const int r = mt * 128 + row_in_tile;
     const int limit = w.p0 - w.ls + r % dm.Bq + 1;          // visible keys of the local tiles (causal inside the block)
     const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
-    const float sl2 = dm.scale * 1.4426950408889634f;
-    const float neg_lse2 = -row_lse * 1.4426950408889634f;
     const uint32_t key7 = (uint32_t)(row_in_tile & 7);
     bool ok = __all_sync(0xffffffffu, bwd_wait(&sm.q_full, 0, abort));
     // delta (dO from the tile in shared memory: 128-byte lines of 16-byte chunks, XOR-swizzled)
@@ -386,7 +383,7 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
 #pragma unroll
       for (int i = 0; i < D / 8; ++i) {
         uint32_t ys[4];
-        ld_shared_v4(line + (((uint32_t)i ^ key7) * 16), ys[0], ys[1], ys[2], ys[3]);
+        ld_shared_v4(line + (uint32_t)(i >> 3) * 16384 + (((uint32_t)(i & 7) ^ key7) * 16), ys[0], ys[1], ys[2], ys[3]);
         const uint32_t xs[4] = {o_row[i].x, o_row[i].y, o_row[i].z, o_row[i].w};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
@@ -398,10 +395,19 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
     }
     HGA_TRACE_POINT(10);
     int n = n_lt + 1, n_a = n_lt, n_far_keys = 0;      // (bounds that do until the list is known)
-    const uint64_t sl2_2 = pack_f32x2(sl2, sl2), neg_lse2_2 = pack_f32x2(neg_lse2, neg_lse2);
-    const uint64_t scale_2 = pack_f32x2(dm.scale, dm.scale), neg_delta_s_2 = pack_f32x2(neg_delta_s, neg_delta_s);
-    const uint32_t s_addr = lane_base + kColS, dp_addr = lane_base + kColDP;
-    uint32_t staged_phase = 0;
+    // (e^x as 2^(x log2 e), x = S*scale - LSE rounded once: no common factor of log2 e rounds S and LSE apart)
+    const uint64_t scale_2 = pack_f32x2(dm.scale, dm.scale), neg_lse_2 = pack_f32x2(-row_lse, -row_lse);
+    const uint64_t neg_delta_s_2 = pack_f32x2(neg_delta_s, neg_delta_s);
+    const uint64_t log2e_2 = pack_f32x2(1.4426950408889634f, 1.4426950408889634f);
+    const uint32_t dp_addr = lane_base + kColDP;
+    const uint32_t a_line = smem_u32(sm.a) + (uint32_t)row_in_tile * 128, b_line = smem_u32(sm.b) + (uint32_t)row_in_tile * 128;
+    // this row's 16 keys of chunk c (four to a tile) in a term's tile: two 16-byte pieces, XOR-swizzled
+    auto put = [&](uint32_t line, int c, const uint32_t* w) {
+#pragma unroll
+      for (int q = 0; q < 2; ++q)
+        st_shared_v4(line + (((uint32_t)(2 * c + q) ^ key7) * 16), w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+    };
+    uint32_t staged_phase = 0, rounds = 0;
     for (int j = 0; j < n && ok; ++j) {
       if (j == n_lt) {
         ok = __all_sync(0xffffffffu, bwd_wait(&sm.info_full, 0, abort));
@@ -411,127 +417,179 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
         if (j >= n) break;
       }
       const int vis = j < n_lt ? limit - kKT * j : n_far_keys - kKT * (j - n_lt);
-      uint32_t pk[32];                                // P of this row, 64 keys, packed bf16
-      ok = __all_sync(0xffffffffu, bwd_wait(&sm.s_full, j & 1, abort));
-      if (!ok) break;
-      tc_fence_after_sync();
-      HGA_TRACE_POINT(11);
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        uint32_t sv[32];
-        tmem_ld32(s_addr + 32 * c, sv);
-        tmem_wait_ld();
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          float a0, a1;            // packed fp32 pairs: one FMA for the two exponent arguments
-          unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(sv[2 * i]), __uint_as_float(sv[2 * i + 1])), sl2_2, neg_lse2_2), a0, a1);
-          float p0 = fast_exp2(a0), p1 = fast_exp2(a1);
-          if (vis < kKT) {         // diagonal / ragged tile only
-            if (32 * c + 2 * i >= vis) p0 = 0.f;
-            if (32 * c + 2 * i + 1 >= vis) p1 = 0.f;
-          }
-          pk[16 * c + i] = pack_bf16(p0, p1);
+      const bool dkv = j >= n_lt && j >= n_a;
+      const uint32_t s_addr = lane_base + s_col(j);
+      // P of two neighbouring keys
+      auto weights = [&](int key, uint32_t s0, uint32_t s1, float& p0, float& p1) {
+        float a0, a1;
+        unpack_f32x2(mul_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(s0), __uint_as_float(s1)), scale_2, neg_lse_2), log2e_2), a0, a1);
+        p0 = fast_exp2(a0);
+        p1 = fast_exp2(a1);
+        if (vis < kKT) {           // diagonal / ragged tile only
+          if (key >= vis) p0 = 0.f;
+          if (key + 1 >= vis) p1 = 0.f;
         }
-      }
-      const bool kind3 = j >= n_lt && j >= n_a;
-      if (!kind3) {
-        tc_fence_before_sync();
-        mbar_arrive_warp(&sm.s_read);                      // S(j) has been read: S(j+1) may take its place
-      }
-      ok = __all_sync(0xffffffffu, bwd_wait(&sm.dp_full, j & 1, abort));
+      };
+      ok = __all_sync(0xffffffffu, bwd_wait(&sm.s_full[j & 1], (j >> 1) & 1, abort));
+      HGA_TRACE_POINT(11);
+      if (ok) ok = __all_sync(0xffffffffu, bwd_wait(&sm.dp_full, j & 1, abort));
       if (!ok) break;
       tc_fence_after_sync();
       HGA_TRACE_POINT(13);
-      const uint32_t p_line = smem_u32(sm.p) + (uint32_t)row_in_tile * 128, ds_line = smem_u32(sm.ds) + (uint32_t)row_in_tile * 128;
 #pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        uint32_t dp[32], dk[16];
-        tmem_ld32(dp_addr + 32 * c, dp);
+      for (int c = 0; c < 4; ++c) {          // 16 keys at a time
+        uint32_t sv[16], dp[16], out[16], p1[8], p2[8];
+        tmem_ld16(s_addr + 16 * c, sv);
+        tmem_ld16(dp_addr + 16 * c, dp);
         tmem_wait_ld();
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const uint32_t pp = pk[16 * c + i];
-          const uint64_t p2 = pack_f32x2(__uint_as_float(pp << 16), __uint_as_float(pp & 0xffff0000u));
+        for (int i = 0; i < 8; ++i) {
+          float x0, x1, d0, d1;
+          weights(16 * c + 2 * i, sv[2 * i], sv[2 * i + 1], x0, x1);
           const uint64_t g2 = fma_f32x2(pack_f32x2(__uint_as_float(dp[2 * i]), __uint_as_float(dp[2 * i + 1])), scale_2, neg_delta_s_2);
-          float d0, d1;
-          unpack_f32x2(mul_f32x2(p2, g2), d0, d1);
-          dk[i] = pack_bf16(d0, d1);
-        }
-        if (!kind3) {
-          // bf16 dS over the dP columns already read (8 columns per 16 keys): the A operand of dQ
-          tmem_st16(dp_addr + 16 * c, dk);
-        } else {
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {               // 16-byte chunks (8 keys each), XOR-swizzled
-            const uint32_t off = ((uint32_t)(4 * c + q) ^ key7) * 16;
-            st_shared_v4(p_line + off, pk[16 * c + 4 * q], pk[16 * c + 4 * q + 1], pk[16 * c + 4 * q + 2], pk[16 * c + 4 * q + 3]);
-            st_shared_v4(ds_line + off, dk[4 * q], dk[4 * q + 1], dk[4 * q + 2], dk[4 * q + 3]);
+          unpack_f32x2(mul_f32x2(pack_f32x2(x0, x1), g2), d0, d1);
+          out[i] = next_term(d0, d1);
+          out[8 + i] = pack_bf16(d0, d1);
+          if (dkv) {
+            p1[i] = next_term(x0, x1);
+            p2[i] = pack_bf16(x0, x1);
           }
         }
+        // dS's two terms over the dP columns just read (8 columns each): the A operands of dQ
+        tmem_st16(dp_addr + 16 * c, out);
+        if (dkv) {
+          put(a_line, c, p1);
+          put(b_line, c, p2);
+        }
       }
-      if (!kind3) {
-        tmem_wait_st();
-        tc_fence_before_sync();
+      tmem_wait_st();
+      tc_fence_before_sync();
+      if (!dkv) {
         mbar_arrive_warp(&sm.ds_full);
         HGA_TRACE_POINT(14);
         continue;
       }
       // ---- dK/dV tile
-      tc_fence_before_sync();
       fence_proxy_async_smem();
       mbar_arrive_warp(&sm.ds_full);
       HGA_TRACE_POINT(17);
-      ok = __all_sync(0xffffffffu, bwd_wait(&sm.dkv_full, (j - n_a) & 1, abort));
-      if (!ok) break;
-      tc_fence_after_sync();
+      auto round_done = [&]() {
+        ok = __all_sync(0xffffffffu, bwd_wait(&sm.round_done, rounds, abort));
+        rounds ^= 1u;
+        if (ok) tc_fence_after_sync();
+        return ok;
+      };
+      auto hand_over_round = [&]() {
+        tc_fence_before_sync();
+        fence_proxy_async_smem();
+        mbar_arrive_warp(&sm.round_full);
+      };
+      // a term of dS from tensor memory into a tile
+      auto put_ds = [&](uint32_t line, int term) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          uint32_t ds[8];
+          tmem_ld8(dp_addr + 16 * c + 8 * term, ds);
+          tmem_wait_ld();
+          put(line, c, ds);
+        }
+      };
+      {
+        uint32_t p3[32];                     // ready when the first round is over
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          uint32_t sv[16];
+          tmem_ld16(s_addr + 16 * c, sv);
+          tmem_wait_ld();
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            float x0, x1;
+            weights(16 * c + 2 * i, sv[2 * i], sv[2 * i + 1], x0, x1);
+            next_term(x0, x1);
+            next_term(x0, x1);
+            p3[8 * c + i] = pack_bf16(x0, x1);
+          }
+        }
+        if (!round_done()) break;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) put(a_line, c, p3 + 8 * c);
+      }
+      put_ds(b_line, 0);
+      hand_over_round();
+      if (!round_done()) break;
+      put_ds(a_line, 1);
+      hand_over_round();
+      if (!round_done()) break;
       HGA_TRACE_POINT(16);
       // (the band kernel, which precedes this one in the stream, stores its dK/dV rows plainly: the adds below must
       // come after it; a no-op unless the launch carried the programmatic-serialization attribute)
       if (j == n_a) pdl_wait();
-      // All GEMMs are done, the P and dS tiles are free: each takes 32 keys x (64 floats of dV | 64 of dK); thread =
-      // element of that row, so a warp writes 128 consecutive bytes per key.
       auto wait_staged = [&]() {           // all 128 row threads have arrived
         ok = __all_sync(0xffffffffu, bwd_wait(&sm.staged, staged_phase, abort));
         staged_phase ^= 1u;
         return ok;
       };
-      auto stage = [&](uint8_t* buf, uint32_t col) {
+      // the lane's 32 columns (keys) of an accumulator, as element `row_in_tile` of key rows of 512 bytes
+      auto stage = [&](uint32_t buf, uint32_t col) {
         uint32_t x[32];
         tmem_ld32(lane_base + col, x);
         tmem_wait_ld();
-        const uint32_t base = smem_u32(buf) + (uint32_t)row_in_tile * 4;
+        const uint32_t base = buf + (uint32_t)row_in_tile * 4;
 #pragma unroll
         for (int i = 0; i < 32; ++i) st_shared_b32(base + (uint32_t)i * 512, x[i]);
-      };
-      // adds the rows of one chunk (lane = key) to dst; `off` = byte offset inside the chunk's rows
-      auto reduce_rows = [&](float* dst, uint8_t* buf, int hf, uint32_t off) {
-        const int o = 8 * (j - n_lt) + 4 * hf + (lane >> 3);
-        if (o >= sm.first_active && o < sm.n_far) {
-          const int row = sm.rows[j & 3][4 * hf + (lane >> 3)] + (lane & 7) - sg.k0 - sg.H;      // inside the active segment
-          bulk_reduce_add_f32(dst + (row_base(dm, sg, b) * dm.Hkv + (int64_t)h * sg.S + row) * D, smem_u32(buf) + (uint32_t)lane * 512 + off, D * 4);
-        }
-        tma_store_commit();
       };
       auto hand_over = [&]() {             // what this thread has written is complete and visible to bulk copies
         fence_proxy_async_smem();
         mbar_arrive_warp(&sm.staged);
         return wait_staged();
       };
-      auto have_read = [&](uint64_t* bar) {
-        tc_fence_before_sync();
-        mbar_arrive_warp(bar);
+      auto buffers_read = [&]() {          // the terms' tiles may be written again
+        tma_store_wait_read();
+        __syncwarp();
+        mbar_arrive_warp(&sm.staged);
+        return wait_staged();
       };
-      const uint32_t col = quarter < 2 ? kColS : kColDP;      // lanes 0-63: dV^T, lanes 64-127: dK^T
-      stage(sm.p, col);
-      stage(sm.ds, col + 32);
-      have_read(&sm.s_read);
-      have_read(&sm.dk_read);
-      if (!hand_over()) break;
-      reduce_rows((quarter & 1) ? dK : dV, quarter < 2 ? sm.p : sm.ds, quarter >> 1, (quarter & 1) * 256u);
-      tma_store_wait_read();
-      __syncwarp();
-      mbar_arrive_warp(&sm.staged);
-      if (!wait_staged()) break;                      // P and dS may be written again
+      const uint32_t dv_col = s_col(j + 1), dk_col = s_col(j), buf_a = smem_u32(sm.a), buf_b = smem_u32(sm.b);
+      // row of octet o (of this tile) in the segment's dK and dV, -1: gets nothing from here
+      auto grad_row = [&](int o) {
+        const int far_o = 8 * (j - n_lt) + o;
+        return far_o >= sm.first_active && far_o < sm.n_far ? sm.rows[j & 3][o] - sg.k0 - sg.H : -1;
+      };
+      const int64_t kv_base = row_base(dm, sg, b) * dm.Hkv + (int64_t)h * sg.S;
+      if constexpr (D == 64) {
+        // every GEMM is done, the terms' tiles are free: each takes 32 keys x (64 floats of dV | 64 of dK) (lanes 0-63 hold dV^T,
+        // lanes 64-127 dK^T); a warp adds its half of each buffer's rows, 256 bytes per instruction
+        const uint32_t col = quarter < 2 ? dv_col : dk_col;
+        stage(buf_a, col);
+        stage(buf_b, col + 32);
+        tc_fence_before_sync();
+        mbar_arrive_warp(&sm.acc_read);
+        if (!hand_over()) break;
+        const int hf = quarter >> 1, row = grad_row(4 * hf + (lane >> 3));
+        if (row >= 0)
+          bulk_reduce_add_f32(((quarter & 1) ? dK : dV) + (kv_base + row + (lane & 7)) * D, (hf ? buf_b : buf_a) + (uint32_t)lane * 512 + (quarter & 1) * 256, D * 4);
+        tma_store_commit();
+        if (!buffers_read()) break;
+      } else {
+        // dV, then dK: 64 key rows over both tiles; an octet of them is 4 KB of consecutive memory on both sides
+#pragma unroll
+        for (int which = 0; which < 2; ++which) {
+          stage(buf_a, which ? dk_col : dv_col);
+          stage(buf_b, (which ? dk_col : dv_col) + 32);
+          if (which == 1) {
+            tc_fence_before_sync();
+            mbar_arrive_warp(&sm.acc_read);
+          }
+          if (!hand_over()) break;
+          if (lane < 2) {
+            const int o = 2 * quarter + lane, row = grad_row(o);
+            if (row >= 0) bulk_reduce_add_f32((which ? dK : dV) + (kv_base + row) * D, buf_a + (uint32_t)o * 4096, 4096);
+            tma_store_commit();
+          }
+          if (!buffers_read()) break;
+        }
+        if (!ok) break;
+      }
       HGA_TRACE_POINT(18);
     }
     if (ok) ok = __all_sync(0xffffffffu, bwd_wait(&sm.dq_done, 0, abort));
@@ -541,26 +599,26 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
       // 16-byte stores would touch 32 different sectors per instruction.  The rows go into Q's shared memory (all
       // GEMMs that read it are complete) in the swizzled [panel][128 rows][128 B] layout and leave as boxes.
       tc_fence_after_sync();
-      uint32_t x[2][32];
-      tmem_ld32(lane_base + kColDQ, x[0]);
-      tmem_ld32(lane_base + kColDQ + 32, x[1]);
-      tmem_wait_ld();
-      const uint32_t line = smem_u32(sm.q) + (uint32_t)row_in_tile * 128;
 #pragma unroll
-      for (int c = 0; c < 2; ++c)
+      for (int c = 0; c < D / 32; ++c) {
+        uint32_t x[32];
+        tmem_ld32(lane_base + kColDQ + 32 * c, x);
+        tmem_wait_ld();
+        const uint32_t line = smem_u32(sm.q) + (uint32_t)(c >> 1) * 16384 + (uint32_t)row_in_tile * 128;
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-          st_shared_v4(line + (((uint32_t)(4 * c + i) ^ key7) * 16),
-                       pack_bf16(__uint_as_float(x[c][8 * i]), __uint_as_float(x[c][8 * i + 1])),
-                       pack_bf16(__uint_as_float(x[c][8 * i + 2]), __uint_as_float(x[c][8 * i + 3])),
-                       pack_bf16(__uint_as_float(x[c][8 * i + 4]), __uint_as_float(x[c][8 * i + 5])),
-                       pack_bf16(__uint_as_float(x[c][8 * i + 6]), __uint_as_float(x[c][8 * i + 7])));
+          st_shared_v4(line + (((uint32_t)(4 * (c & 1) + i) ^ key7) * 16),
+                       pack_bf16(__uint_as_float(x[8 * i]), __uint_as_float(x[8 * i + 1])),
+                       pack_bf16(__uint_as_float(x[8 * i + 2]), __uint_as_float(x[8 * i + 3])),
+                       pack_bf16(__uint_as_float(x[8 * i + 4]), __uint_as_float(x[8 * i + 5])),
+                       pack_bf16(__uint_as_float(x[8 * i + 6]), __uint_as_float(x[8 * i + 7])));
+      }
       fence_proxy_async_smem();
       mbar_arrive_warp(&sm.dq_staged);
-      if (warp == 2 && lane < 2 && bwd_wait(&sm.dq_staged, 0, abort)) {      // all 128 rows are in shared memory
-        const int r0 = mt * 128 + 64 * lane;
+      if (warp == 2 && lane < 2 * kPanels && bwd_wait(&sm.dq_staged, 0, abort)) {      // all 128 rows are in shared memory
+        const int hf = lane & 1, panel = lane >> 1, r0 = mt * 128 + 64 * hf;
         if (r0 < dm.rows) {
-          tma_store_5d(&map_dq, sm.q + lane * 8192, 0, qrow + r0 % dm.Bq, 0, h * dm.G + r0 / dm.Bq, b);
+          tma_store_5d(&map_dq, sm.q + panel * 16384 + hf * 8192, 0, qrow + r0 % dm.Bq, panel, h * dm.G + r0 / dm.Bq, b);
           tma_store_commit();
           tma_store_wait_read();      // (the source tile has been read; the writes complete before the grid does)
         }
@@ -584,18 +642,18 @@ k_attn_bwd_d64_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_con
   HGA_TRACE_POINT(31);
   HGA_TRACE_DUMP;
   if (tid == 0 && sm.abort && status_word) atomicOr(status_word, HGA_ABORT_CODE(3, sm.abort));
-  if (warp == 1) tmem_dealloc(tmem, 256);
+  if (warp == 1) tmem_dealloc(tmem, kTmemCols);
 }
 
-template <class Segs>
-static int launch_sweep64(const Dims& dm, SegTable* table, const Segs& segs, int64_t units, const void* Q, const void* K, const void* V, const void* O, const float* LSE,
+template <int D, class Segs>
+static int launch_terms(const Dims& dm, SegTable* table, const Segs& segs, int64_t units, const void* Q, const void* K, const void* V, const void* O, const float* LSE,
                               const void* dO, const int32_t* group_idx, const int32_t* n_groups, void* dQ, float* dK,
                               float* dV, int32_t* status_word, cudaStream_t st) {
   CUtensorMap mq, mdo, mk, mv, mdq;
-  const uint32_t box[5] = {64, 8, 1, 1, 1};
+  const uint32_t box[5] = {64, 8, (uint32_t)(D / 64), 1, 1};
   const uint32_t box_q[5] = {64, 64, 1, 1, 1};
-  const uint64_t dq[5] = {64, (uint64_t)dm.rows_q, 1, (uint64_t)dm.Hq, (uint64_t)dm.B};
-  const uint64_t dk[5] = {64, (uint64_t)dm.rows_k, 1, (uint64_t)dm.Hkv, (uint64_t)dm.B};
+  const uint64_t dq[5] = {64, (uint64_t)dm.rows_q, (uint64_t)(D / 64), (uint64_t)dm.Hq, (uint64_t)dm.B};
+  const uint64_t dk[5] = {64, (uint64_t)dm.rows_k, (uint64_t)(D / 64), (uint64_t)dm.Hkv, (uint64_t)dm.B};
   const uint64_t sq[4] = {(uint64_t)dm.qs[2] * 2, 128, (uint64_t)dm.qs[1] * 2, (uint64_t)dm.qs[0] * 2};
   const uint64_t so[4] = {(uint64_t)dm.os[2] * 2, 128, (uint64_t)dm.os[1] * 2, (uint64_t)dm.os[0] * 2};
   const uint64_t sk[4] = {(uint64_t)dm.ks[2] * 2, 128, (uint64_t)dm.ks[1] * 2, (uint64_t)dm.ks[0] * 2};
@@ -606,9 +664,9 @@ static int launch_sweep64(const Dims& dm, SegTable* table, const Segs& segs, int
       encode_tensor_map_bf16(&mk, K, 5, dk, sk, box, true) ||
       encode_tensor_map_bf16(&mv, V, 5, dk, sv, box, true))
     return HGA_ERR_UNSUPPORTED;
-  const size_t smem = sizeof(SweepSmem) + 1024;
-  // two CTAs per SM need the largest shared-memory carve-out
-  int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(&k_attn_bwd_d64_sm100<Segs>), smem, true);
+  const size_t smem = sizeof(SweepSmem<D>) + 1024;
+  // (two CTAs per SM need the largest shared-memory carve-out)
+  int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(&k_attn_bwd_terms_sm100<D, Segs>), smem, true);
   if (rc) return rc;
   // dK/dV of the local band first: plain stores that cover every row of the active segment; this kernel then adds
   // the contributions of the keys before the band.  Launched with programmatic serialization behind the band kernel: it
@@ -617,19 +675,21 @@ static int launch_sweep64(const Dims& dm, SegTable* table, const Segs& segs, int
   if (rc != HGA_OK) return rc;
   if (table) units = number_units(*table, [&](const Segment& g) { return (int64_t)dm.B * dm.Hkv * (g.S / dm.Bq) * ((dm.rows + 127) / 128); });
   PdlLaunch cfg((unsigned)units, kThreads, smem, st, dm.flags);
-  const cudaError_t e = cudaLaunchKernelEx(&cfg.c, k_attn_bwd_d64_sm100<Segs>, mq, mdo, mk, mv, mdq, (const uint16_t*)O, LSE,
+  const cudaError_t e = cudaLaunchKernelEx(&cfg.c, k_attn_bwd_terms_sm100<D, Segs>, mq, mdo, mk, mv, mdq, (const uint16_t*)O, LSE,
                                            group_idx, n_groups, dm, dK, dV, status_word, segs);
   count_launch(HGA_KERNELS_BWD_TENSOR);
   return record_cuda(e);
 }
 
-int launch_attn_bwd_d64_sm100(const Dims& dm, SegTable* segs, const void* Q, const void* K, const void* V, const void* O, const float* LSE,
+int launch_attn_bwd_terms_sm100(const Dims& dm, SegTable* segs, const void* Q, const void* K, const void* V, const void* O, const float* LSE,
                               const void* dO, const int32_t* group_idx, const int32_t* n_groups, void* dQ, float* dK,
                               float* dV, int32_t* status_word, cudaStream_t st) {
   const int64_t units = (int64_t)dm.B * dm.Hkv * dm.NQB * ((dm.rows + 127) / 128);
+#define HGA_TERMS_ARGS(table, segs) dm, table, segs, units, Q, K, V, O, LSE, dO, group_idx, n_groups, dQ, dK, dV, status_word, st
   if (!segs)
-    return launch_sweep64(dm, nullptr, OneSegment{}, units, Q, K, V, O, LSE, dO, group_idx, n_groups, dQ, dK, dV, status_word, st);
-  return launch_sweep64(dm, segs, *segs, units, Q, K, V, O, LSE, dO, group_idx, n_groups, dQ, dK, dV, status_word, st);
+    return dm.d == 64 ? launch_terms<64>(HGA_TERMS_ARGS(nullptr, OneSegment{})) : launch_terms<128>(HGA_TERMS_ARGS(nullptr, OneSegment{}));
+  return dm.d == 64 ? launch_terms<64>(HGA_TERMS_ARGS(segs, *segs)) : launch_terms<128>(HGA_TERMS_ARGS(segs, *segs));
+#undef HGA_TERMS_ARGS
 }
 
 }  // namespace hga

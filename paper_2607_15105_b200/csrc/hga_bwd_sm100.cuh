@@ -56,4 +56,12 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
+// x0, x1 -> their bf16 roundings (packed), and what those leave in x0, x1
+__device__ __forceinline__ uint32_t next_term(float& x0, float& x1) {
+  const uint32_t t = pack_bf16(x0, x1);
+  x0 -= __uint_as_float(t << 16);
+  x1 -= __uint_as_float(t & 0xffff0000u);
+  return t;
+}
+
 }  // namespace hga

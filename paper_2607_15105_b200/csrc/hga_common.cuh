@@ -185,10 +185,13 @@ int launch_attn_bwd_sm100(const Dims& dm, SegTable* segs, const void* Q, const v
                           const float* LSE, const void* dO, const int32_t* group_idx,
                           const int32_t* n_groups, void* dQ, float* dK, float* dV, int32_t* status_word,
                           cudaStream_t st);
-int launch_attn_bwd_d64_sm100(const Dims& dm, SegTable* segs, const void* Q, const void* K, const void* V, const void* O,   // head_dim 64, called by the above
-                              const float* LSE, const void* dO, const int32_t* group_idx,
-                              const int32_t* n_groups, void* dQ, float* dK, float* dV, int32_t* status_word,
-                              cudaStream_t st);
+// The backward keeps P and dS in several bf16 terms, i.e. at fp32's precision, for the shapes that used to have the CUDA-core
+// kernel; they have a sweep of their own, called by the above
+inline bool bwd_in_terms(const Dims& dm) { return dm.d == 64 || dm.rows % 128 != 0; }
+int launch_attn_bwd_terms_sm100(const Dims& dm, SegTable* segs, const void* Q, const void* K, const void* V, const void* O,
+                                const float* LSE, const void* dO, const int32_t* group_idx,
+                                const int32_t* n_groups, void* dQ, float* dK, float* dV, int32_t* status_word,
+                                cudaStream_t st);
 // Key-major dK/dV of the local band (plain stores covering every active-segment row); launched by the above.
 bool attn_bwd_band_sm100_supported(const Dims& dm);
 int launch_attn_bwd_band_sm100(const Dims& dm, SegTable* segs, const void* Q, const void* K, const void* V, const void* O,

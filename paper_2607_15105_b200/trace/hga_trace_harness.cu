@@ -31,7 +31,7 @@
 
 namespace hga {
 void count_launch(int, int) {}
-int launch_attn_bwd_d64_sm100(const Dims&, SegTable*, const void*, const void*, const void*, const void*, const float*, const void*, const int32_t*,
+int launch_attn_bwd_terms_sm100(const Dims&, SegTable*, const void*, const void*, const void*, const void*, const float*, const void*, const int32_t*,
                               const int32_t*, void*, float*, float*, int32_t*, cudaStream_t) { return HGA_ERR_UNSUPPORTED; }   // (head_dim 128 only here)
 int record_cuda(cudaError_t e) { if (e != cudaSuccess) printf("cuda error %s\n", cudaGetErrorString(e)); return e == cudaSuccess ? 0 : -6; }
 }

@@ -60,3 +60,38 @@ def test_forward_keeps_dominant_weights(name):
     err = forward(DOMINANT[name])[-1]
     print(name, "O %.3e" % err)
     assert err <= 1.9e-3
+
+
+# backward: the CUDA-core kernel holds P and dS in fp32; every shape that tensor-core kernels took over from it (head_dim 64,
+# row counts that do not fill M-tiles) must come as close to fp64.  Many and few differentiable far keys, a ragged last
+# key tile (S = 576), sequences without history.
+GRADIENTS = dict(UNFILLED, d64_rows128=cfg_of(head_dim=64, n_q_heads=4), d64_no_history=cfg_of(head_dim=64, total_len=1024, seg_len=1024),
+                 d128_no_history=cfg_of(total_len=1024, seg_len=1024), d64_ragged=cfg_of(head_dim=64, seg_len=576, total_len=1600, n_q_heads=6),
+                 d128_needles=cfg_of(needles=16), d64_needles=cfg_of(head_dim=64, needles=16, n_q_heads=4),
+                 d64_wide=cfg_of(head_dim=64, topk_chunks=16, topk_groups=8, sink=128, local=256))
+
+
+@pytest.mark.parametrize("name", list(GRADIENTS))
+def test_gradients_are_as_exact_as_the_cuda_core_kernels(name):
+    cfg = GRADIENTS[name]
+    x, dev, gi, ng, gid, ngd, buf, _ = forward(cfg)
+    ref = oracle.attn_bwd(cfg, x["Q"], x["K"], x["V"], x["dO"], gi, ng)
+    errs = []
+    for flags in (0, binding.HGA_FLAG_GENERIC_KERNELS):
+        other = binding.HgaLayerBuffers(cfg, flags=flags)
+        other.O.copy_(buf.O)
+        other.LSE.copy_(buf.LSE)
+        before = binding.hga_kernel_launch_counts()
+        other.attn_bwd(dev["Q"], dev["K"], dev["V"], dev["dO"], gid, ngd)
+        torch.cuda.synchronize()
+        ran = [b - a for a, b in zip(before, binding.hga_kernel_launch_counts())]
+        assert (ran[binding.HGA_KERNELS_BWD_TENSOR] == 2) == (flags == 0 and cfg.q_block % 64 == 0), ran
+        assert int(other.status.item()) == 0
+        got = (bf16_to_f64(other.dQ), other.dK.cpu().numpy().astype(np.float64), other.dV.cpu().numpy().astype(np.float64))
+        errs.append([rel_fro(a, r) for a, r in zip(got, ref)])
+    print(name, " ".join("%s %.2e (CUDA cores %.2e)" % (n, a, b) for n, a, b in zip(("dQ", "dK", "dV"), *errs)))
+    for n, a, b in zip(("dQ", "dK", "dV"), *errs):
+        # fp32 sums in other orders: a part in 10 of the error.  At head_dim 128 the tensor pipe sums dV, of 12 products per
+        # 64 rows and cut off at 2^-24 each, without interruption: up to 4 query blocks (window and tile) of 3 heads there
+        chain = 12 * 4 * cfg.gqa * 2.0 ** -24 if n == "dV" and cfg.head_dim == 128 else 1e-7
+        assert a <= 1.1 * b + chain, (n, a, b)
