@@ -152,7 +152,6 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   const int n_pre = n_loc_oct / 16;                     // tiles that hold local octets only
   // 64 rows of an M-tile are 64 rows of one head: Q and O travel in boxes of 64 rows x one panel
   const bool boxes = dm.Bq % 64 == 0;
-  const bool chained = (dm.flags & kFlagChained) != 0;
   volatile int* abort = &sm.abort;
   FarList far(dm, w, group_idx + item * dm.width);
   auto n_octets = [&](int n_far) { return n_loc_oct + n_far; };
@@ -186,7 +185,7 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // Q and a first tile of local octets do not depend on the routing: their copies start before the CTA meets.  Barrier 2
     // makes the mbarrier initialisation above visible to the issuing warps.
     asm volatile("bar.sync 2, 96;" ::: "memory");
-    if (!chained) pdl_wait();
+    pdl_wait();
     if (warp == 3) {
       const int q_oct = min(16, rows_pad / 8 - 16 * mt0);   // octets of real rows in this M-tile
       if (lane == 0) mbar_arrive_expect_tx(&sm.q_full, (uint32_t)q_oct * kOct);
@@ -259,7 +258,6 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     }
   } else if (warp == 3) {
     // ------------------------------------------------------------------ routing list
-    if (chained) pdl_wait();
     const bool bad = far.check(dm, n_groups + item, sg.H);
     if (lane == 0) {
       sm.n_listed = far.ng; sm.n_far = far.n_far; sm.clean = far.clean;

@@ -20,12 +20,6 @@ __host__ __device__ inline int score_agg_of(int flags) {
 // kernels.
 constexpr int kFlagNoPdl = 1 << 30;
 
-// Kernels of the path are launched with programmatic serialization (they may start before their predecessor in the
-// stream has ended) and execute griddepcontrol.wait before they touch memory and before they end, so "the
-// predecessor has ended" includes all work before it.  Internal flag kFlagChained: the predecessor is the library's
-// own kernel of the step before, which writes neither Q, K, V nor dO; copies of those may start ahead of the wait.
-constexpr int kFlagChained = 1 << 29;
-
 // Resolved problem description handed to kernels by value.
 struct Dims {
   int B, Hq, Hkv, G, d;
@@ -123,7 +117,9 @@ __host__ __device__ inline int max_routed_tokens(const Dims& dm) {
   return dm.sink + dm.width * dm.g + dm.local + dm.Bq + dm.c;
 }
 
-// A launch with programmatic serialization (see kFlagChained), or a plain one with kFlagNoPdl.
+// A launch with programmatic serialization, or a plain one with kFlagNoPdl.  The kernel may start before its predecessor in
+// the stream has ended; it executes griddepcontrol.wait before it touches memory that the predecessor may write, and before
+// it ends, so that "the predecessor has ended" includes all work before it.
 struct PdlLaunch {
   cudaLaunchConfig_t c = {};
   cudaLaunchAttribute attr;
