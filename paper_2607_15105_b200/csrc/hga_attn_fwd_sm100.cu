@@ -39,8 +39,12 @@
 // of eight: 1 % of the half-tiles): error of O against fp64 2.11e-3 with one term, 1.82e-3 so, 2.06e-3 with a running
 // reference; hga_attn_fwd 39.8 -> 41.3 us (two terms everywhere: 1.66e-3, which is O's own rounding, and 43.5 us).
 // kTwoTerms kernels use them everywhere (see two_terms()).
-// A row whose sum does grow past
-// 2^80 (a logit 55 nats above the first tile's) is recomputed at the end by its warp with a running maximum.
+// Where that does not hold for some row of
+// the M-tile (a sum past 2^80, i.e. a logit 55 nats above the first tile's; a weight past 2^16 that took V out of the fp32
+// range; no finite logit in the first tile) the CTA goes over its keys again, twice: for the rows' true maxima, then
+// with those as references.  That is one tile after another with nothing overlapped, but on the tensor cores and for all
+// rows at once, so its cost is bounded by a small multiple of the first pass whatever the inputs are.  A row whose sum is
+// not a number has no finite answer and is written as it is.
 #include "hga_bwd_sm100.cuh"
 #include "hga_common.cuh"
 #include "hga_octets.cuh"
@@ -58,62 +62,290 @@ namespace {
 constexpr int kFwdThreads = 384;
 constexpr int kFT = 128;                      // keys per tile
 constexpr float kSumLimit = 1.2e24f;          // 2^80
+constexpr float kWeightLimit = 65536.f;       // (a smaller sum means that no weight exceeded it)
 constexpr float kTwoTermSum = 64.f;           // 32 keys that together outweigh the reference by so much get two terms
 
 template <int D>
 struct FwdSmem {
   static constexpr int kQBytes = 128 * D * 2;
   static constexpr int kTileBytes = kFT * D * 2;
+  static constexpr uint32_t kColO = 128;       // TMEM: S at 0, O at 128
   alignas(1024) uint8_t q[kQBytes];            // (the epilogue stages O here)
   alignas(1024) uint8_t k[kTileBytes];         // (and exchanges the row sums here)
   alignas(1024) uint8_t v[kTileBytes];
   float mx[2][128];                            // first tile: the two threads' maxima of a row
   uint64_t q_full, k_full, v_full, v_empty, s_full, p_full[2], info_full, o_done, o_staged, drain;
+  uint64_t again_copied, again_multiplied;     // second passes
   uint32_t tmem_base;
   int n_far, n_listed;
   bool clean;
   volatile int second_terms[2];                // number (from 1) of the last tile whose half needs the weights' second terms
+  volatile int again;                          // some row asks for the second passes
   volatile int abort;
 };
 
-// One row against its visible keys with a running maximum, by a whole warp (lane: D/32 elements): rows whose exponentials
-// left the range of the first tile's reference.  Returns log2 of the sum; o: the normalised output elements.
-template <int D>
-__device__ __forceinline__ float row_with_running_maximum(const FarList& far, const uint16_t* q, const uint16_t* K, const uint16_t* V,
-                                                       int64_t k_stride, int64_t v_stride, int pos, float sl2, float (&o)[D / 32]) {
-  constexpr int E = D / 32;
-  const int lane = threadIdx.x & 31;
-  auto frag = [&](const uint16_t* p, float (&x)[E]) {
-#pragma unroll
-    for (int e = 0; e < E; ++e) x[e] = __uint_as_float((uint32_t)p[lane * E + e] << 16);
-  };
-  float qf[E], m = -INFINITY, l = 0.f;
-  frag(q, qf);
-#pragma unroll
-  for (int e = 0; e < E; ++e) o[e] = 0.f;
-  auto key = [&](int64_t tok) {
-    float kf[E], vf[E], s = 0.f;
-    frag(K + tok * k_stride, kf);
-    frag(V + tok * v_stride, vf);
-#pragma unroll
-    for (int e = 0; e < E; ++e) s = fmaf(qf[e], kf[e], s);
-#pragma unroll
-    for (int i = 16; i > 0; i >>= 1) s += __shfl_xor_sync(0xffffffffu, s, i);
-    s *= sl2;
-    const float m_new = fmaxf(m, s), corr = fast_exp2(m - m_new), p = fast_exp2(s - m_new);
-    l = fmaf(l, corr, p);
-#pragma unroll
-    for (int e = 0; e < E; ++e) o[e] = fmaf(o[e], corr, p * vf[e]);
-    m = m_new;
-  };
-  for (int t = far.ls; t <= pos; ++t) key(t);
-  for (int i = 0; i < far.n_far; ++i) {
-    const int r = far.row(i);
-    for (int u = 0; u < 8; ++u) key(r + u);
+// What a CTA works on
+struct Place {
+  Segment sg;
+  int mt, b, h, qb, qrow;               // M-tile inside the item, item; the block's first row in Q and O
+  Window w;
+  template <class Segs>
+  __device__ Place(const Dims& dm, const Segs& segs, int cta_id) {
+    // Launch order: late query blocks first -- where the history is short they see the most keys, so the cheapest CTAs are
+    // the ones that fill the last wave.
+    const int n_mt_item = (rows_padded(dm) + 127) / 128, n_bh = dm.B * dm.Hkv;
+    int cta;
+    sg = segment_of(dm, segs, cta_id, cta);
+    const int unit = cta / n_mt_item;
+    mt = cta % n_mt_item;
+    qb = sg.S / dm.Bq - 1 - unit / n_bh;
+    b = unit % n_bh / dm.Hkv;
+    h = unit % n_bh % dm.Hkv;
+    qrow = sg.q0 + qb * dm.Bq;
+    w = window_at(dm, sg.H + qb * dm.Bq);
   }
+  __device__ int64_t item(const Dims& dm) const { return item_base(dm, sg, b) + h * (sg.S / dm.Bq) + qb; }
+};
+
+// The row of a softmax thread: rows of the item are every head's Bq rows padded to whole octets (padding rows compute
+// garbage in their own TMEM lanes and are never stored)
+struct Row {
+  int hw, row, r, a, t;                 // which half of every 64 keys; TMEM lane; row inside the item = (query head, token)
+  bool real;
+  __device__ Row(const Dims& dm, const Place& pl, int tid) {
+    const int warp = tid >> 5;
+    hw = (warp - 4) >> 2;
+    row = (warp & 3) * 32 + (tid & 31);
+    r = pl.mt * 128 + row;
+    a = r / bq_padded(dm);
+    t = r % bq_padded(dm);
+    real = r < rows_padded(dm) && t < dm.Bq;
+  }
+};
+
+// A thread index or block number that the compiler does not know to be the one it has already worked with: what follows
+// from it is worked out afresh, instead of being kept in registers through the main loop
+__device__ __forceinline__ int again_tid() { int x; asm volatile("mov.u32 %0, %%tid.x;" : "=r"(x)); return x; }
+__device__ __forceinline__ int again_cta() { int x; asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(x)); return x; }
+
+// A softmax thread's half of its row of O = (accumulators) / l_mma, and LSE from l and the reference m (log2 units).  O's columns
+// (D/2)*hw .. are at head_dim 128 a panel each; rows go through Q's shared memory ([panel][128 rows][128 B], swizzled; every
+// GEMM that reads Q is complete) and leave as boxes, or are stored directly where boxes do not fit.  Returns whether
+// the accumulators are finite.
+template <int D>
+__device__ __forceinline__ bool store_row(FwdSmem<D>& sm, const Dims& dm, const Place& pl, const Row& rw, uint32_t tmem, float l, float l_mma, float m,
+                                          uint16_t* O, float* LSE) {
+  constexpr int kCols = D / 2;
+  const bool boxes = dm.Bq % 64 == 0;
+  const uint32_t lane_base = tmem + ((uint32_t)(rw.row & 96) << 16);
+  const float inv = 1.f / l_mma;
+  const int hq = pl.h * dm.G + rw.a;
+  uint16_t* const orow = O + pl.b * dm.os[0] + (int64_t)hq * dm.os[1] + (int64_t)(pl.qrow + rw.t) * dm.os[2];
+  if (rw.real && rw.hw == 0)
+    LSE[row_base(dm, pl.sg, pl.b) * dm.Hq + (int64_t)hq * pl.sg.S + pl.qb * dm.Bq + rw.t] = (log2f(l) + m) * 0.6931471805599453f;
+  const uint32_t line = smem_u32(sm.q) + (uint32_t)(kCols * rw.hw / 64) * 16384 + (uint32_t)rw.row * 128;
+  uint64_t finite = pack_f32x2(0.f, 0.f);                 // stays zero as long as every element is finite
+#pragma unroll 1
+  for (int c = 0; c < kCols / 32; ++c) {
+    const int col = kCols * rw.hw + 32 * c;
+    uint32_t y[32];
+    tmem_ld32(lane_base + FwdSmem<D>::kColO + col, y);
+    tmem_wait_ld();
 #pragma unroll
-  for (int e = 0; e < E; ++e) o[e] /= l;
-  return m + log2f(l);
+    for (int i = 0; i < 16; ++i)
+      finite = fma_f32x2(pack_f32x2(__uint_as_float(y[2 * i]), __uint_as_float(y[2 * i + 1])), pack_f32x2(0.f, 0.f), finite);
+    if (rw.real) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        uint32_t pk[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) pk[e] = pack_bf16(__uint_as_float(y[8 * i + 2 * e]) * inv, __uint_as_float(y[8 * i + 2 * e + 1]) * inv);
+        if (boxes) st_shared_v4(line + (((uint32_t)((col & 63) / 8 + i) ^ (uint32_t)(rw.row & 7)) * 16), pk[0], pk[1], pk[2], pk[3]);
+        else *reinterpret_cast<uint4*>(orow + col + 8 * i) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+      }
+    }
+  }
+  float x0, x1;
+  unpack_f32x2(finite, x0, x1);
+  return x0 + x1 == 0.f;
+}
+
+// The staged M-tile as boxes of 64 rows x one panel (the first lanes of one warp, after every row has been staged)
+template <int D>
+__device__ __forceinline__ void store_boxes(FwdSmem<D>& sm, const Dims& dm, const Place& pl, const CUtensorMap& map_o, int lane) {
+  const int hf = lane & 1, panel = lane >> 1, r0 = pl.mt * 128 + 64 * hf;
+  if (lane < 2 * (D / 64) && r0 < dm.rows) {
+    tma_store_5d(&map_o, sm.q + panel * 16384 + hf * 8192, 0, pl.qrow + r0 % dm.Bq, panel, pl.h * dm.G + r0 / dm.Bq, pl.b);
+    tma_store_commit();
+    tma_store_wait_read();      // (the source has been read; the writes complete before the grid does)
+  }
+}
+
+// Q's rows: boxes of 64 rows x one panel, [panel][128 rows][128 B], or octets, [octet][panel][8 rows][128 B]; `lane`s of one
+// warp, bytes announced by the caller
+template <int D>
+__device__ __forceinline__ void copy_q(FwdSmem<D>& sm, const Dims& dm, const Place& pl, const CUtensorMap& map_q, uint64_t* bar, int q_oct, int lane) {
+  constexpr int kOct = 8 * D * 2, kPanels = D / 64;
+  if (dm.Bq % 64 == 0) {
+    if (lane < 2 * kPanels && 8 * (lane & 1) < q_oct) {
+      const int hf = lane & 1, panel = lane >> 1, r = pl.mt * 128 + 64 * hf;
+      tma_load_5d(sm.q + panel * 16384 + hf * 8192, &map_q, bar, 0, pl.qrow + r % dm.Bq, panel, pl.h * dm.G + r / dm.Bq, pl.b);
+    }
+  } else if (lane < q_oct) {
+    const int bq_pad = bq_padded(dm), r = pl.mt * 128 + 8 * lane;
+    tma_load_5d(sm.q + lane * kOct, &map_q, bar, 0, pl.qrow + r % bq_pad, 0, pl.h * dm.G + r / bq_pad, pl.b);
+  }
+}
+
+// The M-tile once more, for rows whose exponentials left the range of the first tile's reference: all 384 threads, one tile
+// at a time (a block barrier behind every hand-off), first S alone for the rows' maxima, then everything against those.
+// The main pass is complete: no copy, GEMM or store of it is in flight, and sm.n_far etc. hold the checked list.
+template <int D, class Segs>
+__device__ __forceinline__ void passes_with_true_maxima(FwdSmem<D>& sm, const CUtensorMap& map_q, const CUtensorMap& map_k, const CUtensorMap& map_v,
+                                                        const CUtensorMap& map_o, const int32_t* group_idx, const Dims& dm, uint16_t* O, float* LSE,
+                                                        const Segs& segs, uint32_t tmem) {
+  constexpr int kOct = 8 * D * 2;
+  const int tid = again_tid(), warp = tid >> 5, lane = tid & 31;
+  const Place pl(dm, segs, again_cta());
+  const Window& w = pl.w;
+  const int n_loc_oct = (w.p0 + dm.Bq - w.ls + 7) / 8, n_oct = n_loc_oct + sm.n_far, n_tiles = (n_oct + 15) / 16;
+  const bool boxes = dm.Bq % 64 == 0;
+  volatile int* abort = &sm.abort;
+  const bool softmax = warp >= 4;
+  const Row rw(dm, pl, tid);
+  const int hw = rw.hw, row = rw.row;
+  const uint32_t lane_base = tmem + ((uint32_t)(row & 96) << 16);
+  const float sl2 = dm.scale * 1.4426950408889634f;
+  const int limit = w.p0 - w.ls + rw.t + 1;
+
+  uint32_t copies = 0, multiplications = 0;          // phases of the two barriers
+  bool ok = true;
+  auto copied = [&]() { ok = ok && __all_sync(0xffffffffu, bwd_wait(&sm.again_copied, copies++ & 1, abort)); };
+  auto multiplied = [&]() { ok = ok && __all_sync(0xffffffffu, bwd_wait(&sm.again_multiplied, multiplications++ & 1, abort)); };
+  // a thread that gave up has the others leave behind the next barrier, and the copies in flight a bounded time to land
+  auto all_fine = [&]() {
+    if (!__syncthreads_or(!ok)) return true;
+    if (warp == 0 && lane == 0)
+      for (int it = 0; it < 64; ++it) __nanosleep(1000);
+    return false;
+  };
+  // the copies below overwrite what the epilogue has written into Q's and K's place
+  fence_proxy_async_smem();
+  __syncthreads();
+  float m = -INFINITY, l = 0.f, l_mma = 0.f;
+#pragma unroll 1
+  for (int step = 0; step < 2 * n_tiles; ++step) {
+    const bool sums = step >= n_tiles;
+    const int j = sums ? step - n_tiles : step;
+    if (step == n_tiles) {
+      // the row's true maximum, in log2 units
+      if (softmax) sm.mx[hw][row] = m;
+      __syncthreads();
+      if (softmax) m = fmaxf(m, sm.mx[hw ^ 1][row]) * sl2;
+    }
+    if (warp == 0) {
+      const int q_oct = min(16, rows_padded(dm) / 8 - 16 * pl.mt);
+      if (lane == 0) mbar_arrive_expect_tx(&sm.again_copied, (uint32_t)(16 * (sums ? 2 : 1) + (step == 0 ? q_oct : 0)) * kOct);
+      __syncwarp();
+      if (lane < 16) {
+        FarList far(dm, w, group_idx + pl.item(dm) * dm.width);
+        far.ng = sm.n_listed; far.n_far = sm.n_far; far.clean = sm.clean;
+        const int o = 16 * j + lane;
+        const int krow = o < n_loc_oct ? pl.sg.k0 + w.ls + 8 * o : o < n_oct ? pl.sg.k0 + far.row(o - n_loc_oct) : dm.rows_k;
+        tma_load_5d(sm.k + lane * kOct, &map_k, &sm.again_copied, 0, krow, 0, pl.h, pl.b);
+        if (sums) tma_load_5d(sm.v + lane * kOct, &map_v, &sm.again_copied, 0, krow, 0, pl.h, pl.b);
+      }
+      if (step == 0) copy_q(sm, dm, pl, map_q, &sm.again_copied, q_oct, lane);       // (O may have been staged over Q)
+      __syncwarp();
+    }
+    copied();
+    if (warp == 1 && ok) {
+      tc_fence_after_sync();
+      const uint32_t lead = elect_one();
+      const uint64_t q_desc = smem_desc_sw128(smem_u32(sm.q), 16, boxes ? 1024 : kOct), k_desc = smem_desc_sw128(smem_u32(sm.k), 16, kOct);
+      const uint32_t q_panel = boxes ? 16384 : 1024;
+#pragma unroll 1
+      for (int kk = 0; kk < D / 16; ++kk)
+        mma_ss_w(lead, tmem, desc_advance(q_desc, (kk >> 2) * q_panel + (kk & 3) * 32), desc_advance(k_desc, (kk >> 2) * 1024 + (kk & 3) * 32),
+                 idesc_bf16_f32(128, kFT, 0, 0), kk > 0);
+      mma_commit_w(lead, &sm.again_multiplied);
+    }
+    multiplied();
+    if (softmax && ok) {
+      tc_fence_after_sync();
+      float tile_l = 0.f, tile_l_mma = 0.f;
+#pragma unroll 1
+      for (int c = 0; c < 2; ++c) {
+        const int first = 64 * c + 32 * hw;
+        const int lo = limit - kFT * j - first, hi = 8 * n_loc_oct - kFT * j - first, end = 8 * n_oct - kFT * j - first;
+        uint32_t x[32];
+        tmem_ld32(lane_base + first, x);
+        tmem_wait_ld();
+        if (!sums) {
+#pragma unroll
+          for (int i = 0; i < 32; ++i)
+            if ((i < lo || i >= hi) && i < end) m = fmaxf(m, __uint_as_float(x[i]));
+        } else {
+#pragma unroll
+          for (int k0 = 0; k0 < 32; k0 += 16) {      // (two terms per weight, see the main pass)
+            uint32_t pk[16];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              float p[2];
+#pragma unroll
+              for (int u = 0; u < 2; ++u) {
+                const int k = k0 + 2 * i + u;
+                p[u] = (k < lo || k >= hi) && k < end ? fast_exp2(fmaf(__uint_as_float(x[k]), sl2, -m)) : 0.f;
+                tile_l += p[u];
+              }
+              pk[i] = pack_bf16(p[0], p[1]);
+              pk[8 + i] = pack_bf16(p[0] - __uint_as_float(pk[i] << 16), p[1] - __uint_as_float(pk[i] & 0xffff0000u));
+#pragma unroll
+              for (int u = 0; u < 2; ++u) tile_l_mma += __uint_as_float(pk[8 * u + i] << 16) + __uint_as_float(pk[8 * u + i] & 0xffff0000u);
+            }
+            tmem_st16(lane_base + first + k0, pk);
+          }
+        }
+      }
+      l += tile_l;
+      l_mma += tile_l_mma;
+      if (sums) tmem_wait_st();
+      tc_fence_before_sync();
+    }
+    // (also: S has been read, K may be overwritten)
+    if (!all_fine()) return;
+    if (!sums) continue;
+    if (warp == 1) {
+      tc_fence_after_sync();
+      const uint32_t lead = elect_one();
+      const uint64_t v_desc = smem_desc_sw128(smem_u32(sm.v), 1024, kOct);
+#pragma unroll 1
+      for (int kk = 0; kk < 2 * (kFT / 16); ++kk)
+        mma_ts_w(lead, tmem + FwdSmem<D>::kColO, tmem + 8 * kk, desc_advance(v_desc, (uint32_t)(kk >> 1) * 2 * kOct),
+                 idesc_bf16_f32(128, D, 0, 1), j > 0 || kk > 0);
+      mma_commit_w(lead, &sm.again_multiplied);
+    }
+    multiplied();
+    if (!all_fine()) return;
+  }
+  // the row's two sums meet, then the epilogue of the main pass
+  float* const xchg = reinterpret_cast<float*>(sm.k);
+  if (softmax) {
+    xchg[hw * 256 + row] = l;
+    xchg[hw * 256 + 128 + row] = l_mma;
+  }
+  __syncthreads();
+  if (softmax) {
+    tc_fence_after_sync();
+    l += xchg[(hw ^ 1) * 256 + row];
+    l_mma += xchg[(hw ^ 1) * 256 + 128 + row];
+    store_row(sm, dm, pl, rw, tmem, l, l_mma, m, O, LSE);
+    fence_proxy_async_smem();
+    tc_fence_before_sync();
+  }
+  __syncthreads();
+  if (boxes && warp == 4) store_boxes(sm, dm, pl, map_o, lane);
+  __syncwarp();
 }
 
 }  // namespace
@@ -122,38 +354,26 @@ template <int D, bool kTwoTerms, class Segs>
 __global__ void __launch_bounds__(kFwdThreads, 2)
 k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                  const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_o,
-                 const uint16_t* __restrict__ Q, const uint16_t* __restrict__ K, const uint16_t* __restrict__ V,
                  const int32_t* __restrict__ group_idx, const int32_t* __restrict__ n_groups, const Dims dm,
                  uint16_t* __restrict__ O, float* __restrict__ LSE, int32_t* status_word, const __grid_constant__ Segs segs) {
-  constexpr int kOct = 8 * D * 2, kPanels = D / 64;
-  constexpr uint32_t kColO = 128;                 // TMEM: S at 0, O at 128
+  constexpr int kOct = 8 * D * 2;
   constexpr uint32_t kTmemCols = 256;
   extern __shared__ uint8_t smem_raw[];
   FwdSmem<D>& sm = *reinterpret_cast<FwdSmem<D>*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   HGA_TRACE_DECL(256);
-  // rows of the item: every head's Bq rows padded to whole octets (padding rows compute garbage
-  // in their own TMEM lanes and are never stored)
-  const int bq_pad = bq_padded(dm), rows_pad = rows_padded(dm);
-  const int n_mt_item = (rows_pad + 127) / 128;
-  // Launch order: late query blocks first -- where the history is short they see the most keys, so the
-  // cheapest CTAs are the ones that fill the last wave.
-  int cta;
-  const Segment sg = segment_of(dm, segs, blockIdx.x, cta);
-  const int unit = cta / n_mt_item, n_bh = dm.B * dm.Hkv;
-  const int mt0 = cta % n_mt_item;                      // this CTA's M-tile inside the item
-  const int qb = sg.S / dm.Bq - 1 - unit / n_bh, b = unit % n_bh / dm.Hkv, h = unit % n_bh % dm.Hkv;
-  const int64_t item = item_base(dm, sg, b) + h * (sg.S / dm.Bq) + qb;
-  const int qrow = sg.q0 + qb * dm.Bq;                  // the block's first row in Q and O
-  const Window w = window_at(dm, sg.H + qb * dm.Bq);
+  const Place pl(dm, segs, blockIdx.x);
+  const Segment& sg = pl.sg;
+  const Window& w = pl.w;
+  const int b = pl.b, h = pl.h;
   const int n_local = w.p0 + dm.Bq - w.ls;              // tokens of the local window and the block
   const int n_loc_oct = (n_local + 7) / 8;              // (the last octet may be partial in generation shapes)
   const int n_pre = n_loc_oct / 16;                     // tiles that hold local octets only
   // 64 rows of an M-tile are 64 rows of one head: Q and O travel in boxes of 64 rows x one panel
   const bool boxes = dm.Bq % 64 == 0;
   volatile int* abort = &sm.abort;
-  FarList far(dm, w, group_idx + item * dm.width);
+  FarList far(dm, w, group_idx + pl.item(dm) * dm.width);
   auto n_octets = [&](int n_far) { return n_loc_oct + n_far; };
 
   if (warp == 0 && lane == 0) {
@@ -161,7 +381,9 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     mbar_init(&sm.k_full, 2); mbar_init(&sm.v_full, 2); mbar_init(&sm.v_empty, 1);
     mbar_init(&sm.s_full, 1); mbar_init(&sm.p_full[0], 8); mbar_init(&sm.p_full[1], 8);
     mbar_init(&sm.info_full, 1); mbar_init(&sm.o_done, 1); mbar_init(&sm.o_staged, 8); mbar_init(&sm.drain, 1);
+    mbar_init(&sm.again_copied, 1); mbar_init(&sm.again_multiplied, 1);
     sm.second_terms[0] = sm.second_terms[1] = 0;
+    sm.again = 0;
     sm.abort = 0;
     fence_barrier_init();
   }
@@ -187,18 +409,10 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     asm volatile("bar.sync 2, 96;" ::: "memory");
     pdl_wait();
     if (warp == 3) {
-      const int q_oct = min(16, rows_pad / 8 - 16 * mt0);   // octets of real rows in this M-tile
+      const int q_oct = min(16, rows_padded(dm) / 8 - 16 * pl.mt);   // octets of real rows in this M-tile
       if (lane == 0) mbar_arrive_expect_tx(&sm.q_full, (uint32_t)q_oct * kOct);
       __syncwarp();
-      if (boxes) {                                          // [panel][128 rows][128 B]
-        if (lane < 2 * kPanels && 8 * (lane & 1) < q_oct) {
-          const int hf = lane & 1, panel = lane >> 1, r = mt0 * 128 + 64 * hf;
-          tma_load_5d(sm.q + panel * 16384 + hf * 8192, &map_q, &sm.q_full, 0, qrow + r % dm.Bq, panel, h * dm.G + r / dm.Bq, b);
-        }
-      } else if (lane < q_oct) {                            // [octet][panel][8 rows][128 B]
-        const int r = mt0 * 128 + 8 * lane;
-        tma_load_5d(sm.q + lane * kOct, &map_q, &sm.q_full, 0, qrow + r % bq_pad, 0, h * dm.G + r / bq_pad, b);
-      }
+      copy_q(sm, dm, pl, map_q, &sm.q_full, q_oct, lane);
     } else if (n_pre > 0) {
       const int row = row_of(0);
       copy_tile(sm.k, &map_k, &sm.k_full, row, true);
@@ -258,7 +472,7 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     }
   } else if (warp == 3) {
     // ------------------------------------------------------------------ routing list
-    const bool bad = far.check(dm, n_groups + item, sg.H);
+    const bool bad = far.check(dm, n_groups + pl.item(dm), sg.H);
     if (lane == 0) {
       sm.n_listed = far.ng; sm.n_far = far.n_far; sm.clean = far.clean;
       mbar_arrive(&sm.info_full);
@@ -278,7 +492,7 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     const uint32_t q_panel = boxes ? 16384 : 1024;
     const uint64_t k_desc = smem_desc_sw128(smem_u32(sm.k), 16, kOct);         // K-major B of S = Q K^T
     const uint64_t v_desc = smem_desc_sw128(smem_u32(sm.v), 1024, kOct);       // MN-major B of O += P V
-    const uint32_t o_acc = tmem + kColO;
+    const uint32_t o_acc = tmem + FwdSmem<D>::kColO;
     auto issue_s = [&](bool whole) {
       const uint32_t idesc = whole ? idesc_s : idesc_s_half;
 #pragma unroll
@@ -340,22 +554,19 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     }
   } else {
     // ------------------------------------------------------------------ softmax + epilogue
-    const int hw = (warp - 4) >> 2;                     // keys 32*hw .. and 64 + 32*hw .. of every tile
-    const int quarter = warp & 3;                       // TMEM lanes this warp may touch
-    const int row = quarter * 32 + lane;
-    const int r = mt0 * 128 + row;                      // row inside the item
-    const int a = r / bq_pad, t = r % bq_pad;
-    const bool real_row = r < rows_pad && t < dm.Bq;
+    const Row rw(dm, pl, tid);
+    const int hw = rw.hw, row = rw.row;                 // keys 32*hw .. and 64 + 32*hw .. of every tile
     // a warp whose 32 lanes are all padding only keeps the barriers moving
-    const bool warp_real = __any_sync(0xffffffffu, real_row);
-    const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
+    const bool warp_real = __any_sync(0xffffffffu, rw.real);
+    const uint32_t lane_base = tmem + ((uint32_t)(row & 96) << 16);      // the TMEM lanes this warp may touch
     const float sl2 = dm.scale * 1.4426950408889634f;   // softmax scale in log2 units
     const uint64_t sl2_2 = pack_f32x2(sl2, sl2);
     // Column c of tile j is slot 128*j + c of the set: visible below `limit` (causal), masked from there to the end of the
     // local octets, visible again up to the end of the set.
-    const int limit = w.p0 - w.ls + t + 1;
+    const int limit = w.p0 - w.ls + rw.t + 1;
     int n_oct = 16 * n_pre + 1;                         // (enough until the list is known)
-    float neg_m = 0.f, l = 0.f, l_mma = 0.f;
+    uint64_t neg_m2 = pack_f32x2(0.f, 0.f);             // minus the reference (log2 units), twice
+    float l = 0.f, l_mma = 0.f;
     bool ok = true;
     for (int j = 0; 16 * j < n_oct; ++j) {
       if (j == n_pre) {
@@ -367,8 +578,6 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       if (!ok && j > 0) break;
       tc_fence_after_sync();
       HGA_TRACE_POINT(11);
-      // slots relative to the first column of this thread's 32 in each half
-      const int lo = limit - kFT * j - 32 * hw, hi = 8 * n_loc_oct - kFT * j - 32 * hw, end = 8 * n_oct - kFT * j - 32 * hw;
       const bool whole = 8 * n_oct - kFT * j > 64;
       if (j == 0) {
         // the row's reference: its maximum over the first tile (ok or not, every softmax thread meets here once)
@@ -379,7 +588,8 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             uint32_t x[32];
             tmem_ld32(lane_base + 64 * c + 32 * hw, x);
             tmem_wait_ld();
-            const int lo_c = lo - 64 * c, hi_c = hi - 64 * c, end_c = end - 64 * c;
+            // slots relative to the first of this thread's 32 columns
+            const int first = kFT * j + 64 * c + 32 * hw, lo_c = limit - first, hi_c = 8 * n_loc_oct - first, end_c = 8 * n_oct - first;
             if (__all_sync(0xffffffffu, (lo_c >= 32 || hi_c <= 0) && end_c >= 32)) {
 #pragma unroll
               for (int i = 0; i < 32; ++i) mx[i & 1] = fmaxf(mx[i & 1], __uint_as_float(x[i]));
@@ -393,20 +603,20 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         const float m = fmaxf(mx[0], mx[1]);
         sm.mx[hw][row] = m;
         asm volatile("bar.sync 1, 256;" ::: "memory");
-        neg_m = -fmaxf(m, sm.mx[hw ^ 1][row]) * sl2;
+        const float neg_m = -fmaxf(m, sm.mx[hw ^ 1][row]) * sl2;
+        neg_m2 = pack_f32x2(neg_m, neg_m);
         HGA_TRACE_POINT(13);
         if (!ok) break;
       }
       // p = 2^(x*c - m), bf16, over columns already read.  l sums the exact probabilities (for LSE), l_mma the rounded ones
       // the MMA really applies: normalising O by THEIR sum makes the rounding of a dominant weight cancel.
-      const uint64_t neg_m2 = pack_f32x2(neg_m, neg_m);
       uint64_t lsum = pack_f32x2(0.f, 0.f), rsum = pack_f32x2(0.f, 0.f);
       // (one copy of the code for both halves: a CTA of a few tiles pays for every line of it once in instruction-cache misses)
 #pragma unroll 1
       for (int c = 0; c < 2; ++c) {
         if (c == 1 && !whole) break;
         if (warp_real) {
-          const int lo_c = lo - 64 * c, hi_c = hi - 64 * c, end_c = end - 64 * c;
+          const int first = kFT * j + 64 * c + 32 * hw, lo_c = limit - first, hi_c = 8 * n_loc_oct - first, end_c = 8 * n_oct - first;
           const uint32_t s_addr = lane_base + 64 * c + 32 * hw;
           // (two copies of the code: a compare per element in the common one doubled its time)
           auto exponentials = [&](auto masked) {
@@ -495,101 +705,60 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       }
       HGA_TRACE_POINT(14);
     }
+    // the place once more (while the last GEMM runs)
+    const int tid2 = again_tid();
+    const Place pl2(dm, segs, again_cta());
+    const Row rw2(dm, pl2, tid2);
     if (ok) ok = __all_sync(0xffffffffu, bwd_wait(&sm.o_done, 0, abort));
     HGA_TRACE_POINT(20);
     // the row's two sums meet (every GEMM has read the K tile); ok or not, every softmax thread meets here once
+    float neg_m, unused;
+    unpack_f32x2(neg_m2, neg_m, unused);
     float* const xchg = reinterpret_cast<float*>(sm.k);
-    xchg[hw * 256 + row] = l;
-    if constexpr (!kTwoTerms) xchg[hw * 256 + 128 + row] = l_mma;
+    xchg[rw2.hw * 256 + rw2.row] = l;
+    if constexpr (!kTwoTerms) xchg[rw2.hw * 256 + 128 + rw2.row] = l_mma;
     asm volatile("bar.sync 1, 256;" ::: "memory");
-    l += xchg[(hw ^ 1) * 256 + row];
-    if constexpr (!kTwoTerms) l_mma += xchg[(hw ^ 1) * 256 + 128 + row];
+    l += xchg[(rw2.hw ^ 1) * 256 + rw2.row];
+    if constexpr (!kTwoTerms) l_mma += xchg[(rw2.hw ^ 1) * 256 + 128 + rw2.row];
     else l_mma = l;                                     // (two terms leave 2^-17 of a weight: its sum needs no counterpart)
-    if (ok && warp_real) {
+    if (ok && __any_sync(0xffffffffu, rw2.real)) {
       tc_fence_after_sync();
-      const float inv = 1.f / l_mma;
-      const int hq = h * dm.G + a;
-      uint16_t* const orow = O + b * dm.os[0] + (int64_t)hq * dm.os[1] + (int64_t)(qrow + t) * dm.os[2];
-      float* const lse = LSE + row_base(dm, sg, b) * dm.Hq + (int64_t)hq * sg.S + qb * dm.Bq + t;
-      const bool lost = real_row && !(l < kSumLimit);         // (also a sum that is infinite or not a number)
-      if (real_row && hw == 0 && !lost) *lse = (log2f(l) - neg_m) * 0.6931471805599453f;
-      // O, columns (D/2)*hw ..: at head_dim 128 a panel each.  Rows go through Q's shared memory ([panel][128 rows][128 B],
-      // swizzled; every GEMM that reads Q is complete) and leave as boxes, or are stored directly where boxes do not fit.
-      constexpr int kCols = D / 2;
-      const uint32_t line = smem_u32(sm.q) + (uint32_t)(kCols * hw / 64) * 16384 + (uint32_t)row * 128;
-      const uint32_t key7 = (uint32_t)(row & 7);
-#pragma unroll
-      for (int c = 0; c < kCols / 32; ++c) {
-        const int col = kCols * hw + 32 * c;
-        uint32_t y[32];
-        tmem_ld32(lane_base + kColO + col, y);
-        tmem_wait_ld();
-        if (real_row && !lost) {
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            uint32_t pk[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) pk[e] = pack_bf16(__uint_as_float(y[8 * i + 2 * e]) * inv, __uint_as_float(y[8 * i + 2 * e + 1]) * inv);
-            if (boxes) st_shared_v4(line + (((uint32_t)((col & 63) / 8 + i) ^ key7) * 16), pk[0], pk[1], pk[2], pk[3]);
-            else *reinterpret_cast<uint4*>(orow + col + 8 * i) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-          }
-        }
-      }
-      unsigned todo = hw == 0 ? __ballot_sync(0xffffffffu, lost) : 0u;
-      if (todo) {
-        far.ng = sm.n_listed; far.n_far = sm.n_far; far.clean = sm.clean;
-      }
-      while (todo) {
-        const int src = __ffs(todo) - 1;
-        todo &= todo - 1;
-        const int r2 = __shfl_sync(0xffffffffu, r, src), row2 = quarter * 32 + src;
-        const int hq2 = h * dm.G + r2 / bq_pad, t2 = r2 % bq_pad;
-        float o[D / 32];
-        const float lse2 = row_with_running_maximum<D>(
-            far, Q + b * dm.qs[0] + hq2 * dm.qs[1] + (int64_t)(qrow + t2) * dm.qs[2], K + b * dm.ks[0] + h * dm.ks[1] + sg.k0 * dm.ks[2],
-            V + b * dm.vs[0] + h * dm.vs[1] + sg.k0 * dm.vs[2], dm.ks[2], dm.vs[2], w.p0 + t2, sl2, o);
-        if (lane == 0) LSE[row_base(dm, sg, b) * dm.Hq + (int64_t)hq2 * sg.S + qb * dm.Bq + t2] = lse2 * 0.6931471805599453f;
-#pragma unroll
-        for (int e = 0; e < D / 32; e += 2) {
-          const int col = lane * (D / 32) + e;
-          const uint32_t v2 = pack_bf16(o[e], o[e + 1]);
-          if (boxes) st_shared_b32(smem_u32(sm.q) + (uint32_t)(col >> 6) * 16384 + (uint32_t)row2 * 128 +
-                                   ((((uint32_t)(col & 63) >> 3) ^ (uint32_t)(row2 & 7)) * 16) + (uint32_t)(col & 7) * 2, v2);
-          else *reinterpret_cast<uint32_t*>(O + b * dm.os[0] + hq2 * dm.os[1] + (int64_t)(qrow + t2) * dm.os[2] + col) = v2;
-        }
-      }
+      const bool finite = store_row(sm, dm, pl2, rw2, tmem, l, l_mma, -neg_m, O, LSE);
+      // (a sum that is not a number passes none of these tests)
+      if (rw2.real && (l >= kSumLimit || neg_m == INFINITY || (l > kWeightLimit && !finite))) sm.again = 1;
     }
-    if (boxes) {
+    if (dm.Bq % 64 == 0) {
       fence_proxy_async_smem();
       mbar_arrive_warp(&sm.o_staged);
-      if (ok && warp == 4 && lane < 2 * kPanels && bwd_wait(&sm.o_staged, 0, abort)) {      // all rows are in shared memory
-        const int hf = lane & 1, panel = lane >> 1, r0 = mt0 * 128 + 64 * hf;
-        if (r0 < dm.rows) {
-          tma_store_5d(&map_o, sm.q + panel * 16384 + hf * 8192, 0, qrow + r0 % dm.Bq, panel, h * dm.G + r0 / dm.Bq, b);
-          tma_store_commit();
-          tma_store_wait_read();      // (the source has been read; the writes complete before the grid does)
-        }
-      }
+      if (ok && warp == 4 && bwd_wait(&sm.o_staged, 0, abort) && !sm.again) store_boxes(sm, dm, pl2, map_o, lane);   // all rows are in shared memory
     }
     HGA_TRACE_POINT(21);
   }
 
-  // common exit: every role has either finished or given up; tensor memory is released
+  // common exit: every role has either finished or given up
   HGA_TRACE_POINT(30);
-  __syncwarp();
-  if (warp == 1 && sm.abort) {
-    // giving up: GEMMs already issued may still be writing tensor memory; wait (bounded) until the tensor pipe has run
-    // dry before the columns are given back
-    mma_commit_w(elect_one(), &sm.drain);
-    mbar_wait(&sm.drain, 0);
-  }
   __syncwarp();
   tc_fence_before_sync();
   __syncthreads();
   HGA_TRACE_POINT(31);
+  if (sm.again && !sm.abort) {
+    passes_with_true_maxima<D>(sm, map_q, map_k, map_v, map_o, group_idx, dm, O, LSE, segs, sm.tmem_base);
+    tc_fence_before_sync();
+    __syncthreads();
+  }
   HGA_TRACE_DUMP;
   if (tid == 0 && sm.abort && status_word) atomicOr(status_word, HGA_ABORT_CODE(1, sm.abort));
-  if (warp == 1) tmem_dealloc(tmem, kTmemCols);
+  if (warp == 1) {
+    __syncwarp();
+    if (sm.abort) {
+      // given up (known for certain behind the barrier): GEMMs already issued may still be writing tensor memory; wait
+      // (bounded) until the tensor pipe has run dry before the columns are given back
+      mma_commit_w(elect_one(), &sm.drain);
+      mbar_wait(&sm.drain, 0);
+      __syncwarp();
+    }
+    tmem_dealloc(sm.tmem_base, kTmemCols);
+  }
 }
 
 bool attn_fwd_sm100_supported(const Dims& dm) {
@@ -632,8 +801,8 @@ static int launch_fwd(const Dims& dm, const Segs& segs, int64_t units, const voi
   const int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(&k_attn_fwd_sm100<D, kTwoTerms, Segs>), smem, true);
   if (rc) return rc;
   PdlLaunch cfg((unsigned)units, kFwdThreads, smem, st, dm.flags);
-  const cudaError_t e = cudaLaunchKernelEx(&cfg.c, k_attn_fwd_sm100<D, kTwoTerms, Segs>, mq, mk, mv, mo, (const uint16_t*)Q, (const uint16_t*)K,
-                                           (const uint16_t*)V, group_idx, n_groups, dm, (uint16_t*)O, LSE, status_word, segs);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg.c, k_attn_fwd_sm100<D, kTwoTerms, Segs>, mq, mk, mv, mo, group_idx, n_groups, dm, (uint16_t*)O,
+                                           LSE, status_word, segs);
   count_launch(HGA_KERNELS_FWD_TENSOR);
   return record_cuda(e);
 }
