@@ -206,17 +206,18 @@ __device__ __forceinline__ void passes_with_true_maxima(FwdSmem<D>& sm, const CU
                                                         const Segs& segs, uint32_t tmem) {
   constexpr int kOct = 8 * D * 2;
   const int tid = again_tid(), warp = tid >> 5, lane = tid & 31;
-  const Place pl(dm, segs, again_cta());
-  const Window& w = pl.w;
-  const int n_loc_oct = (w.p0 + dm.Bq - w.ls + 7) / 8, n_oct = n_loc_oct + sm.n_far, n_tiles = (n_oct + 15) / 16;
-  const bool boxes = dm.Bq % 64 == 0;
   volatile int* abort = &sm.abort;
-  const bool softmax = warp >= 4;
-  const Row rw(dm, pl, tid);
-  const int hw = rw.hw, row = rw.row;
+  const bool softmax = warp >= 4, boxes = dm.Bq % 64 == 0;
+  const int hw = (warp - 4) >> 2, row = (warp & 3) * 32 + lane;         // (as in Row)
   const uint32_t lane_base = tmem + ((uint32_t)(row & 96) << 16);
   const float sl2 = dm.scale * 1.4426950408889634f;
-  const int limit = w.p0 - w.ls + rw.t + 1;
+  int n_loc_oct, limit;                              // as in the main pass
+  {
+    const Place pl(dm, segs, again_cta());
+    n_loc_oct = (pl.w.p0 + dm.Bq - pl.w.ls + 7) / 8;
+    limit = pl.w.p0 - pl.w.ls + Row(dm, pl, tid).t + 1;
+  }
+  const int n_oct = n_loc_oct + sm.n_far, n_tiles = (n_oct + 15) / 16;
 
   uint32_t copies = 0, multiplications = 0;          // phases of the two barriers
   bool ok = true;
@@ -244,14 +245,15 @@ __device__ __forceinline__ void passes_with_true_maxima(FwdSmem<D>& sm, const CU
       if (softmax) m = fmaxf(m, sm.mx[hw ^ 1][row]) * sl2;
     }
     if (warp == 0) {
+      const Place pl(dm, segs, again_cta());
       const int q_oct = min(16, rows_padded(dm) / 8 - 16 * pl.mt);
       if (lane == 0) mbar_arrive_expect_tx(&sm.again_copied, (uint32_t)(16 * (sums ? 2 : 1) + (step == 0 ? q_oct : 0)) * kOct);
       __syncwarp();
       if (lane < 16) {
-        FarList far(dm, w, group_idx + pl.item(dm) * dm.width);
+        FarList far(dm, pl.w, group_idx + pl.item(dm) * dm.width);
         far.ng = sm.n_listed; far.n_far = sm.n_far; far.clean = sm.clean;
         const int o = 16 * j + lane;
-        const int krow = o < n_loc_oct ? pl.sg.k0 + w.ls + 8 * o : o < n_oct ? pl.sg.k0 + far.row(o - n_loc_oct) : dm.rows_k;
+        const int krow = o < n_loc_oct ? pl.sg.k0 + pl.w.ls + 8 * o : o < n_oct ? pl.sg.k0 + far.row(o - n_loc_oct) : dm.rows_k;
         tma_load_5d(sm.k + lane * kOct, &map_k, &sm.again_copied, 0, krow, 0, pl.h, pl.b);
         if (sums) tma_load_5d(sm.v + lane * kOct, &map_v, &sm.again_copied, 0, krow, 0, pl.h, pl.b);
       }
@@ -275,41 +277,34 @@ __device__ __forceinline__ void passes_with_true_maxima(FwdSmem<D>& sm, const CU
       tc_fence_after_sync();
       float tile_l = 0.f, tile_l_mma = 0.f;
 #pragma unroll 1
-      for (int c = 0; c < 2; ++c) {
-        const int first = 64 * c + 32 * hw;
-        const int lo = limit - kFT * j - first, hi = 8 * n_loc_oct - kFT * j - first, end = 8 * n_oct - kFT * j - first;
-        uint32_t x[32];
-        tmem_ld32(lane_base + first, x);
+      for (int c = 0; c < 4; ++c) {                   // 16 keys at a time
+        const int first = 64 * (c >> 1) + 32 * hw + 16 * (c & 1), lo = limit - kFT * j - first, hi = 8 * n_loc_oct - kFT * j - first, end = 8 * n_oct - kFT * j - first;
+        uint32_t x[16], pk[16];
+        tmem_ld16(lane_base + first, x);
         tmem_wait_ld();
-        if (!sums) {
 #pragma unroll
-          for (int i = 0; i < 32; ++i)
-            if ((i < lo || i >= hi) && i < end) m = fmaxf(m, __uint_as_float(x[i]));
-        } else {
+        for (int i = 0; i < 8; ++i) {
+          float p[2];
 #pragma unroll
-          for (int k0 = 0; k0 < 32; k0 += 16) {      // (two terms per weight, see the main pass)
-            uint32_t pk[16];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              float p[2];
-#pragma unroll
-              for (int u = 0; u < 2; ++u) {
-                const int k = k0 + 2 * i + u;
-                p[u] = (k < lo || k >= hi) && k < end ? fast_exp2(fmaf(__uint_as_float(x[k]), sl2, -m)) : 0.f;
-                tile_l += p[u];
-              }
-              pk[i] = pack_bf16(p[0], p[1]);
-              pk[8 + i] = pack_bf16(p[0] - __uint_as_float(pk[i] << 16), p[1] - __uint_as_float(pk[i] & 0xffff0000u));
-#pragma unroll
-              for (int u = 0; u < 2; ++u) tile_l_mma += __uint_as_float(pk[8 * u + i] << 16) + __uint_as_float(pk[8 * u + i] & 0xffff0000u);
-            }
-            tmem_st16(lane_base + first + k0, pk);
+          for (int u = 0; u < 2; ++u) {
+            const int k = 2 * i + u;
+            const bool see = (k < lo || k >= hi) && k < end;
+            if (!sums && see) m = fmaxf(m, __uint_as_float(x[k]));
+            p[u] = see ? fast_exp2(fmaf(__uint_as_float(x[k]), sl2, -m)) : 0.f;
+            tile_l += p[u];
           }
+          pk[i] = pack_bf16(p[0], p[1]);                // (two terms per weight, see the main pass)
+          pk[8 + i] = pack_bf16(p[0] - __uint_as_float(pk[i] << 16), p[1] - __uint_as_float(pk[i] & 0xffff0000u));
+#pragma unroll
+          for (int u = 0; u < 2; ++u) tile_l_mma += __uint_as_float(pk[8 * u + i] << 16) + __uint_as_float(pk[8 * u + i] & 0xffff0000u);
         }
+        if (sums) tmem_st16(lane_base + first, pk);
       }
-      l += tile_l;
-      l_mma += tile_l_mma;
-      if (sums) tmem_wait_st();
+      if (sums) {
+        l += tile_l;
+        l_mma += tile_l_mma;
+        tmem_wait_st();
+      }
       tc_fence_before_sync();
     }
     // (also: S has been read, K may be overwritten)
@@ -335,11 +330,12 @@ __device__ __forceinline__ void passes_with_true_maxima(FwdSmem<D>& sm, const CU
     xchg[hw * 256 + 128 + row] = l_mma;
   }
   __syncthreads();
+  const Place pl(dm, segs, again_cta());
   if (softmax) {
     tc_fence_after_sync();
     l += xchg[(hw ^ 1) * 256 + row];
     l_mma += xchg[(hw ^ 1) * 256 + 128 + row];
-    store_row(sm, dm, pl, rw, tmem, l, l_mma, m, O, LSE);
+    store_row(sm, dm, pl, Row(dm, pl, tid), tmem, l, l_mma, m, O, LSE);
     fence_proxy_async_smem();
     tc_fence_before_sync();
   }
