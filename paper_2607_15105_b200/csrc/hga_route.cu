@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(kScoreThreads)
 k_route_groups(const uint16_t* __restrict__ Q, const uint16_t* __restrict__ group_sum, Dims dm,
                const int32_t* __restrict__ chunk_idx, int32_t* __restrict__ group_idx,
                int32_t* __restrict__ n_groups, float* __restrict__ group_scores_out,
-               float* __restrict__ gscratch /* [items][kc * per], global budget only */) {
+               uint32_t* __restrict__ gscratch /* [items][kc * per] orderable scores, global budget only */) {
   extern __shared__ float smem[];
   float* s_sum = smem;
   float* s_q = s_sum + kScoreTile * (D + 1);
@@ -242,7 +242,7 @@ k_route_groups(const uint16_t* __restrict__ Q, const uint16_t* __restrict__ grou
     if (global_budget) {
       // keep the scores: the selection runs over all opened chunks at the end
       if (tid < chunks_per_tile * dm.per && base + tid < total)
-        gscratch[(int64_t)item * dm.kc * dm.per + base + tid] = s_out[tid];
+        gscratch[(int64_t)item * dm.kc * dm.per + base + tid] = orderable(s_out[tid] + 0.f);
     } else if (tid == 0) {
       // one thread per opened chunk of this tile: top-kg_eff of its `per` groups.  Chunks are
       // handled in ascending order by thread 0 so the output list is ascending.
@@ -267,13 +267,13 @@ k_route_groups(const uint16_t* __restrict__ Q, const uint16_t* __restrict__ grou
   if (global_budget) {
     // slot i (chunk-major = ascending group id) is selected when fewer than nsel * kg_eff slots beat
     // it (higher score, or equal score and lower id); its output place is the number of selected
-    // slots below it
-    const float* v = gscratch + (int64_t)item * dm.kc * dm.per;
+    // slots below it.  (Integers, so that a NaN has a place too and exactly so many slots pass.)
+    const uint32_t* v = gscratch + (int64_t)item * dm.kc * dm.per;
     const int want = nsel * dm.kge;
     if (tid < 64) s_flags[tid] = 0;
     __syncthreads();                        // also orders the score writes above before the reads below
     for (int i = tid; i < total; i += blockDim.x) {
-      const float mine = v[i];
+      const uint32_t mine = v[i];
       int beat = 0;
       for (int q = 0; q < total; ++q) beat += v[q] > mine || (v[q] == mine && q < i);
       if (beat < want) atomicOr(&s_flags[i >> 6], 1ull << (i & 63));
@@ -302,7 +302,7 @@ int launch_route_generic(const Dims& dm, const void* Q, const void* chunk_sum,
                          void* workspace, cudaStream_t st) {
   const int items = dm.B * dm.Hkv * dm.NQB;
   float* scores = (float*)workspace;
-  float* gscratch = scores + (size_t)items * dm.Nc;      // behind the chunk scores (global group budget only)
+  uint32_t* gscratch = (uint32_t*)scores + (size_t)items * dm.Nc;      // behind the chunk scores (global group budget only)
   auto Qp = (const uint16_t*)Q;
   auto cs = (const uint16_t*)chunk_sum;
   auto gs = (const uint16_t*)group_sum;

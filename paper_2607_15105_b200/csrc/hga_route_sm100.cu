@@ -69,6 +69,9 @@ __device__ __forceinline__ uint32_t rt_orderable(float f) {
   const uint32_t u = __float_as_uint(f);
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
+__device__ __forceinline__ float rt_score(uint32_t key) {
+  return __uint_as_float((key & 0x80000000u) ? key ^ 0x80000000u : ~key);
+}
 
 // The k largest of n keys (k <= n), ties to the lowest position, by one warp: emit(position, rank by position, key) for each.  The
 // k-th largest is found bit by bit below the bits that all keys share.  KPL: keys that a lane keeps in registers
@@ -149,7 +152,7 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
   int* fidx = reinterpret_cast<int*>(fkeys + lay.n_final);
   uint32_t* flags = reinterpret_cast<uint32_t*>(fidx + lay.n_final);         // bit i: slot i selected
   int* sorted = reinterpret_cast<int*>(flags + 128);                         // selected chunks, ascending
-  float* gscore = reinterpret_cast<float*>(sorted + dm.kc);
+  uint32_t* gkeys = reinterpret_cast<uint32_t*>(sorted + dm.kc);             // orderable scores of the opened chunks' groups
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // (late query blocks first: where the history is short they have the most candidates)
@@ -407,7 +410,7 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
             if (i < n_cand) okeys[i] = rt_orderable(best);
             if (chunk_scores && i < n_cand) chunk_scores[item * dm.Nc + j0 + i] = best;
           } else {
-            if (i < k_sel * dm.per) gscore[i] = best;
+            if (i < k_sel * dm.per) gkeys[i] = rt_orderable(best + 0.f);       // (+ 0: a negative zero equals a positive one)
           }
         }
       }
@@ -502,20 +505,22 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
       // A slot is selected when fewer than `want` slots of its scope beat it (higher score, or equal
       // score and lower id); the scope is its own chunk (want = kg_eff) or, with one budget over all
       // opened chunks, every slot (want = k_sel * kg_eff).  Its place in the ascending output is the
-      // number of selected slots below it.
+      // number of selected slots below it.  (Compared as orderable integers: exactly `want` slots pass whatever the
+      // scores are.  A NaN, which a mean or a log-sum-exp can be, compares with nothing as a float, so that every slot of such
+      // a chunk passed and the list was written past its end.)
       const int total = k_sel * dm.per;
       const int want = global_budget ? k_sel * dm.kge : dm.kge;
       for (int base = 0; base < total; base += kRtThreads) {      // warp-uniform trip count (ballots below)
         const int i = base + tid;
         bool sel = false;
         if (i < total) {
-          const float mine = gscore[i];
+          const uint32_t mine = gkeys[i];
           const int lo = global_budget ? 0 : i - i % dm.per, hi = global_budget ? total : lo + dm.per;
           int beat = 0;
 #pragma unroll 8
-          for (int q = lo; q < hi; ++q) beat += gscore[q] > mine || (gscore[q] == mine && q < i);
+          for (int q = lo; q < hi; ++q) beat += gkeys[q] > mine || (gkeys[q] == mine && q < i);
           sel = beat < want;
-          if (group_scores) group_scores[item * dm.kc * dm.per + i] = mine;
+          if (group_scores) group_scores[item * dm.kc * dm.per + i] = rt_score(mine);
         }
         const uint32_t word = __ballot_sync(0xffffffffu, sel);
         if (lane == 0 && base + warp * 32 < total) flags[(base + warp * 32) >> 5] = word;
@@ -530,7 +535,7 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
     } else
     for (int r = tid; r < dm.kc; r += kRtThreads) {
       if (r < k_sel) {
-        const float* v = gscore + r * dm.per;
+        const uint32_t* v = gkeys + r * dm.per;
         unsigned long long picked = 0;
         for (int q = 0; q < dm.kge; ++q) {
           int bu = -1;
@@ -543,7 +548,7 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
           if ((picked >> u) & 1ull) gi[n++] = sorted[r] * dm.per + u;
         if (group_scores)
           for (int u = 0; u < dm.per; ++u)
-            group_scores[item * dm.kc * dm.per + r * dm.per + u] = v[u];
+            group_scores[item * dm.kc * dm.per + r * dm.per + u] = rt_score(v[u]);
       }
     }
     for (int i = k_sel * dm.kge + tid; i < dm.width; i += kRtThreads) gi[i] = -1;
