@@ -128,7 +128,9 @@ static bool segments_supported(const Dims& dm, const std::vector<Segment>& segs,
 }
 
 // Routing, forward and (dO given) backward of all segments, up to kMaxSegments per launch, longest first.  *bwd_done: the
-// backward was queued too (it is not where its kernels have no room for the widest item).
+// backward was queued too (it is not where its kernels have no room for the widest item).  HGA_ERR_UNSUPPORTED: the routing or
+// the forward of these tensors is not for the tensor-core kernels after all (a stride that no tensor map takes), the same for
+// every group of segments; the caller goes on segment by segment, which repeats what has been queued.
 static int run_segments(const Dims& dm, std::vector<Segment> segs, bool summaries, const void* Q, const void* K, const void* V,
                         const void* dO, void* chunk_sum, void* group_sum, int32_t* chunk_idx, int32_t* group_idx, int32_t* n_groups,
                         void* O, float* LSE, void* dQ, float* dK, float* dV, int32_t* status_word, cudaStream_t st, bool* bwd_done) {
@@ -504,8 +506,10 @@ int hga_tbptt_walk(const hga_params* p, const void* Q, const void* K, const void
       bool bwd_done = false;
       rc = run_segments(dm, segs, false, Q, K, V, dO, chunk_sum, group_sum, chunk_idx, group_idx, n_groups, O, LSE, dQ, (float*)dK,
                         (float*)dV, status_word, st, &bwd_done);
-      if (rc || bwd_done || !bwd) return rc;
-      fwd_done = true;
+      if (rc != HGA_ERR_UNSUPPORTED) {
+        if (rc || bwd_done || !bwd) return rc;
+        fwd_done = true;
+      }
     }
   }
   // Otherwise segment by segment.  The backward of segment s depends on that segment's forward only, and the forward chain
@@ -641,8 +645,10 @@ int hga_varlen_step(const hga_params* p, int32_t n_seq, const int32_t* cu_q, con
       bool bwd_done = false;
       rc = run_segments(dm, segs, true, Q, K, V, dO, chunk_sum, group_sum, chunk_idx, group_idx, n_groups, O, LSE, dQ, (float*)dK,
                         (float*)dV, status_word, st, &bwd_done);
-      if (rc || bwd_done || !bwd) return rc;
-      fwd_done = true;
+      if (rc != HGA_ERR_UNSUPPORTED) {
+        if (rc || bwd_done || !bwd) return rc;
+        fwd_done = true;
+      }
     }
   }
   // Otherwise one sequence after another, alternately on two library-owned streams ("lanes"), each with its own half of the
