@@ -630,19 +630,22 @@ k_attn_bwd_terms_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_c
   // Common exit.  Roles leave their warps diverged, so every warp reconverges first: a block barrier reached by
   // part of a warp would count that warp as arrived.
   __syncwarp();
-  if (warp == 1 && sm.abort) {
-    // giving up: GEMMs already issued may still be writing tensor memory; wait (bounded) until the tensor pipe has run
-    // dry before the columns are given back
-    mma_commit_w(elect_one(), &sm.drain);
-    mbar_wait(&sm.drain, 0);
-  }
-  __syncwarp();
   tc_fence_before_sync();
   __syncthreads();
   HGA_TRACE_POINT(31);
   HGA_TRACE_DUMP;
   if (tid == 0 && sm.abort && status_word) atomicOr(status_word, HGA_ABORT_CODE(3, sm.abort));
-  if (warp == 1) tmem_dealloc(tmem, kTmemCols);
+  if (warp == 1) {
+    __syncwarp();
+    if (sm.abort) {
+      // given up (known for certain behind the barrier): GEMMs already issued may still be writing tensor memory; wait
+      // (bounded) until the tensor pipe has run dry before the columns are given back
+      mma_commit_w(elect_one(), &sm.drain);
+      mbar_wait(&sm.drain, 0);
+      __syncwarp();
+    }
+    tmem_dealloc(tmem, kTmemCols);
+  }
 }
 
 template <int D, class Segs>
