@@ -95,3 +95,20 @@ def test_gradients_are_as_exact_as_the_cuda_core_kernels(name):
         # 64 rows and cut off at 2^-24 each, without interruption: up to 4 query blocks (window and tile) of 3 heads there
         chain = 12 * 4 * cfg.gqa * 2.0 ** -24 if n == "dV" and cfg.head_dim == 128 else 1e-7
         assert a <= 1.1 * b + chain, (n, a, b)
+
+
+@pytest.mark.parametrize("kc,kg,tiles,tensor", [(4, 4, 4, False), (8, 4, 7, False), (9, 4, 7, True), (64, 8, 1, True), (4, 4, 8, True)])
+def test_the_smallest_head_dim_64_layers_keep_the_cuda_core_backward(kc, kg, tiles, tensor):
+    """... on both sides of the line: fewer than eight M-tiles and room for at most 512 routed keys."""
+    cfg = cfg_of(head_dim=64, n_q_heads=tiles, n_kv_heads=tiles, seg_len=64, total_len=4672, topk_chunks=kc, topk_groups=kg, local=64)
+    x, dev, gi, ng, gid, ngd, buf, _ = forward(cfg)
+    before = binding.hga_kernel_launch_counts()
+    buf.attn_bwd(dev["Q"], dev["K"], dev["V"], dev["dO"], gid, ngd)
+    torch.cuda.synchronize()
+    ran = [b - a for a, b in zip(before, binding.hga_kernel_launch_counts())]
+    assert (ran[binding.HGA_KERNELS_BWD_TENSOR], ran[binding.HGA_KERNELS_BWD_GENERIC]) == ((2, 0) if tensor else (0, 2))
+    assert int(buf.status.item()) == 0
+    ref = oracle.attn_bwd(cfg, x["Q"], x["K"], x["V"], x["dO"], gi, ng)
+    got = (bf16_to_f64(buf.dQ), buf.dK.cpu().numpy().astype(np.float64), buf.dV.cpu().numpy().astype(np.float64))
+    for a, r, most in zip(got, ref, (1.8e-3, 1e-3, 1e-6)):
+        assert rel_fro(a, r) <= most
