@@ -79,7 +79,7 @@ struct BwdSmem {
   uint64_t phase_a_done;                                // every GEMM of the dK/dV steps is complete
   uint64_t kp_full[kBwdKStages / 2], kp_empty[kBwdKStages], vp_full[2];    // paired steps: one barrier per pair of stages
                                                         // (kp_empty: indexed by pair number mod 6, see dp_full)
-  uint64_t dq_done, dq_staged, drain[2];
+  uint64_t dq_done, dq_staged;
   uint32_t tmem_base;
   int n_oct, dkv_lo, n_dkv;    // tiles [dkv_lo, dkv_lo + n_dkv) are processed as dK/dV steps
   volatile int abort;
@@ -136,7 +136,6 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     for (int s = 0; s < kBwdKStages; ++s) mbar_init(&sm.kp_empty[s], 1);
     mbar_init(&sm.vp_full[0], 2); mbar_init(&sm.vp_full[1], 2);
     mbar_init(&sm.dq_done, 1); mbar_init(&sm.dq_staged, 8);
-    mbar_init(&sm.drain[0], 1); mbar_init(&sm.drain[1], 1);
     sm.abort = 0;
     fence_barrier_init();
   }
@@ -751,9 +750,17 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   if (sm.abort) {
     // Given up (known for certain behind the barrier, and the same in every thread).  GEMMs already issued, by either issuing
     // warp, may still be reading shared and writing tensor memory: wait (bounded) until the tensor pipe has run dry.
-    if (tid == 0 && status_word) atomicOr(status_word, HGA_ABORT_CODE(3, sm.abort));
+    // The two barriers for that lie in the octet table, which nobody reads any more (it is all the room there is).
+    uint64_t* drain = reinterpret_cast<uint64_t*>((reinterpret_cast<uintptr_t>(sm.oct_row) + 7) & ~uintptr_t(7));
+    if (tid == 0) {
+      if (status_word) atomicOr(status_word, HGA_ABORT_CODE(3, sm.abort));
+      mbar_init(&drain[0], 1);
+      mbar_init(&drain[1], 1);
+      fence_barrier_init();
+    }
+    __syncthreads();
     if (warp == 1 || warp == 10) {
-      uint64_t* drain = &sm.drain[warp == 10 ? 1 : 0];
+      if (warp == 10) ++drain;
       mma_commit_w(elect_one(), drain);
       mbar_wait(drain, 0);
     }

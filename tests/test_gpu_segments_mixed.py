@@ -151,3 +151,26 @@ def test_walk_with_bf16_gradients():
             assert float((a[k].double() - b[k].double()).abs().max()) <= 2.0 ** -7 * float(b[k].double().abs().max()), k
         else:
             assert torch.equal(a[k], b[k]), k
+
+
+@pytest.mark.parametrize("kc,tensor", [(383, True), (384, False)])
+def test_the_widest_items_the_sweep_has_room_for(kc, tensor):
+    """Room for 3327 routed keys per item (sink, groups, window, block and a chunk) beside the tiles; from there on the CUDA cores."""
+    cfg = cfg_of(1024, 256, chunk=64, group=8, q_block=64, topk_chunks=kc, topk_groups=1, sink=64, local=64)
+    gen = torch.Generator(device="cuda").manual_seed(kc)
+    Q, dO = (draw(gen, 1, cfg.n_q_heads, 256, 128) for _ in range(2))
+    K, V = (draw(gen, 1, cfg.n_kv_heads, 1024, 128) for _ in range(2))
+    grads = []
+    for flags in (0, binding.HGA_FLAG_GENERIC_KERNELS):
+        buf = binding.HgaLayerBuffers(cfg, flags=flags)
+        buf.build_summaries(K, 0, 1024)
+        buf.route(Q)
+        buf.attn_fwd(Q, K, V)
+        before = binding.hga_kernel_launch_counts()
+        buf.attn_bwd(Q, K, V, dO)
+        n = ran(before)
+        assert n[binding.HGA_KERNELS_BWD_TENSOR] == (2 if tensor and not flags else 0)
+        grads.append((buf.dQ.float(), buf.dK, buf.dV))
+    torch.cuda.synchronize()
+    for a, b in zip(*grads):          # bf16 P and dS against fp32 ones: 2^-9 per term
+        assert float((a - b).norm()) <= 1e-2 * float(b.norm())
