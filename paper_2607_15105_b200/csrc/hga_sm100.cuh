@@ -145,9 +145,6 @@ __device__ __forceinline__ void tma_store_5d(const CUtensorMap* m, const void* s
       : "memory");
 }
 __device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-// waits until every committed bulk store of this thread has completed (shared memory read AND global written)
-__device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-
 // waits until every committed bulk store of this thread has READ its shared-memory source (the
 // global writes may still be in flight: enough before the source is reused or the CTA exits)
 __device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
