@@ -14,6 +14,10 @@
  *   - Unless a parameter says "host", every data pointer is a DEVICE pointer owned by the
  *     caller.  The library allocates and frees no device memory, never synchronises the
  *     device, and launches on the `stream` it is given (a cudaStream_t passed as void*).
+ *   - Kernels are launched with programmatic serialization: they start early behind a kernel that releases its successor
+ *     early, and release theirs.  Each waits (griddepcontrol.wait) before it touches memory and before it ends, so ordinary
+ *     work around a call sees plain stream order; a caller's own kernel that is launched with that attribute behind
+ *     a call must wait the same way before it reads the call's results or writes its inputs.
  *   - Every call returns an int status: HGA_OK (0) or a negative HGA_ERR_* code.  On an
  *     error nothing has been launched.  hga_status_string() names a code.
  *   - bf16 data are raw 16-bit patterns.  The innermost (head_dim) axis is contiguous.
@@ -193,7 +197,9 @@ HGA_API int hga_attn_fwd(const hga_params* p, const void* Q, const void* K, cons
  * O and LSE are hga_attn_fwd's outputs, dO the upstream gradient (layout of O).
  * dK/dV are fp32 [B,Hkv,S,d] (bf16 with HGA_FLAG_BWD_BF16_GRADS) and are overwritten unless
  * HGA_FLAG_BWD_ACCUMULATE is set.  The sum over query blocks
- * uses floating-point atomics: results may differ in the last bits from run to run.
+ * uses floating-point atomics: results may differ in the last bits from run to run.  At head_dim 128 and whole 128-row
+ * tiles per item (G*Bq a multiple of 128) the tensor-core kernels take items of up to 3327 routed keys (sink + k_c*kg_eff*g +
+ * local + Bq + c); wider ones have the CUDA-core kernel.
  * workspace: device scratch of at least hga_workspace_bytes().bwd bytes. */
 HGA_API int hga_attn_bwd(const hga_params* p, const void* Q, const void* K, const void* V, const void* O,
                  const float* LSE, const void* dO, const int32_t* group_idx,
