@@ -19,6 +19,7 @@
 // counts take a whole SM with four accumulators.
 #include <algorithm>
 #include <cfloat>
+#include <type_traits>
 
 #include "hga_common.cuh"
 #include "hga_sm100.cuh"
@@ -236,8 +237,12 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
   tc_fence_after_sync();
   const uint32_t tmem = sm.tmem_base;
   pdl_wait();            // (every thread: any of them may write results)
-  // the forward kernel, the usual successor, may set itself up meanwhile
-  if (tid == 0) pdl_launch_dependents();
+  // The forward kernel, the usual successor, may set itself up meanwhile.  Released here its CTAs come to lie on the SMs
+  // while this kernel still selects, and fetch their instructions beside it; for one problem, a wave or two of CTAs, that cost
+  // more than it hid (released ahead of the group selection instead: 32 sequences 42.4 -> 39.7 us, 128K 93.6 -> 92.1, 16K layer
+  // 166.5 -> 165.6, all whole steps).  The many CTAs of several segments hide it (walk of 16K: 1155 us so, 1175 late).
+  constexpr bool kReleaseEarly = !std::is_same<Segs, OneSegment>::value;
+  if (kReleaseEarly && tid == 0) pdl_launch_dependents();
 
   // optional output: -inf outside the candidate range
   if (chunk_scores)
@@ -496,6 +501,7 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
     __syncthreads();
   }
 
+  if (!kReleaseEarly && tid == 0) pdl_launch_dependents();
   // ---------------------------------------------------------------------- groups of the opened chunks
   if (!sm.abort) {
     int32_t* gi = group_idx + item * dm.width;
