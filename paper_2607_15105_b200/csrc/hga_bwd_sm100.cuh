@@ -20,7 +20,6 @@ namespace hga {
 static __device__ int g_dbg_fail[64];     // [w] line | parity << 16, [16 + w] barrier address, [32 + w] block | blockDim << 16
 #endif
 __device__ __forceinline__ bool bwd_wait_(uint64_t* bar, uint32_t parity, volatile int* abort, int code) {
-  if (sm100::mbar_test_wait(bar, parity)) return true;    // fast path: the phase is already over
   const bool fine = sm100::mbar_wait_bounded(bar, parity, abort, sm100::kWaitCycles, code);
 #ifdef HGA_DEBUG_WAIT
   if (!fine && g_dbg_fail[threadIdx.x >> 5] == 0) {

@@ -5,7 +5,8 @@
 // group list is validated on the way: an entry must be greater than the last accepted entry
 // and lie wholly between the sink and the local window; other entries are skipped and
 // reported.  The common case (a valid ascending list) is checked with one coalesced load and a
-// warp vote per 32 entries; only a list that fails the vote is walked sequentially.
+// warp vote per 32 entries; only a list that fails the vote is walked sequentially.  (None of these loops is worth
+// unrolling: they are inlined into every role that looks octets up.)
 #pragma once
 
 #include "hga_common.cuh"
@@ -29,6 +30,7 @@ __device__ inline int build_octet_table(const Dims& dm, const Window& w, const i
   const int n_sink = w.se / 8;
   bool all_ok = true;
   int prev = -1;
+#pragma unroll 1
   for (int base = 0; base < ng; base += 32) {
     const int i = base + lane;
     const int m = i >= ng ? 0x7fffffff : base == 0 ? pre0 : base == 32 ? pre1 : __ldcg(gi + i);
@@ -46,6 +48,7 @@ __device__ inline int build_octet_table(const Dims& dm, const Window& w, const i
     int n = n_sink;
     if (lane == 0) {
       int last = -1;
+#pragma unroll 1
       for (int i = 0; i < ng; ++i) {
         const int m = __ldcg(gi + i);
         if (m > last && (int64_t)m * dm.g >= w.se && ((int64_t)m + 1) * dm.g <= w.ls) {
@@ -88,6 +91,7 @@ struct FarList {
     const int listed = __ldcg(ng_ptr);
     ng = listed < 0 ? 0 : listed > dm.width ? dm.width : listed;
     int prev = -1, below = 0;
+#pragma unroll 1
     for (int base = 0; base < ng; base += 32) {
       const int i = base + lane;
       const int m = i >= ng ? 0x7fffffff : base == 0 ? pre0 : base == 32 ? pre1 : __ldcg(gi + i);
@@ -102,6 +106,7 @@ struct FarList {
       n = below = 0;
       if (lane == 0) {
         int last = -1;
+#pragma unroll 1
         for (int i = 0; i < ng; ++i) {
           const int m = __ldcg(gi + i);
           if (fits(m, last)) { ++n; below += (int64_t)m * g < H; last = m; }
@@ -120,6 +125,7 @@ struct FarList {
     const int k = o - n_sink, u = opg == 1 ? k : k / opg, sub = k - u * opg;
     if (clean) return __ldcg(gi + u) * g + 8 * sub;
     int last = -1, n = -1;
+#pragma unroll 1
     for (int i = 0; i < ng; ++i) {
       const int m = __ldcg(gi + i);
       if (fits(m, last)) { last = m; if (++n == u) break; }

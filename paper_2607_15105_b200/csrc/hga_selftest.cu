@@ -10,7 +10,7 @@ namespace hga {
 namespace {
 
 __global__ void __launch_bounds__(64)
-k_selftest_bounded_wait(long long cycle_limit, int32_t* status_word, long long* waited_cycles) {
+k_selftest_bounded_wait(uint32_t cycle_limit, int32_t* status_word, long long* waited_cycles) {
   __shared__ uint64_t never;      // one arrival expected, none ever made
   __shared__ int abort_flag;
   if (threadIdx.x == 0) {
@@ -41,7 +41,7 @@ extern "C" int hga_selftest_bounded_wait(uint32_t cycle_limit, int32_t* status_w
                                          void* stream) {
   if (!status_word) return HGA_ERR_NULL;
   if (cycle_limit < 1 || cycle_limit > (1u << 24)) return HGA_ERR_SHAPE;
-  hga::k_selftest_bounded_wait<<<1, 64, 0, (cudaStream_t)stream>>>((long long)cycle_limit, status_word, waited_cycles);
+  hga::k_selftest_bounded_wait<<<1, 64, 0, (cudaStream_t)stream>>>(cycle_limit, status_word, waited_cycles);
   hga::count_launch(HGA_KERNELS_AUX);
   return hga::record_cuda(cudaGetLastError());
 }
