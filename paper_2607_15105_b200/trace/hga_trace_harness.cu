@@ -5,7 +5,7 @@
 // each warp, cycles counted from the CTA's earliest record.
 //
 //   python -m paper_2607_15105_b200.build --trace          builds paper_2607_15105_b200/hga_trace
-//   ./paper_2607_15105_b200/hga_trace <kernel number: 256 forward, 448 band, 512 sweep> [block index]
+//   ./paper_2607_15105_b200/hga_trace <kernel number: 256 forward, 448 band, 512 sweep> [block index [total length]]
 //
 // Tags (see the kernels): 1 set-up done; 2 a producer issued a tile; 3 first GEMMs issued; 5/6/7/8 the
 // issuing warp (barrier observed / S issued / dQ or PV issued / dP issued); 11/13/14/15 a row or key
@@ -41,7 +41,7 @@ int main(int argc, char** argv) {
   const int trace_threads = argc > 1 ? atoi(argv[1]) : 512;
   const int trace_blk = argc > 2 ? atoi(argv[2]) : 300;
   Dims dm{};
-  dm.B = 1; dm.Hq = 32; dm.Hkv = 8; dm.G = 4; dm.d = 128; dm.L = 16384; dm.S = 2048; dm.H = dm.L - dm.S;
+  dm.B = 1; dm.Hq = 32; dm.Hkv = 8; dm.G = 4; dm.d = 128; dm.L = argc > 3 ? atoi(argv[3]) : 16384; dm.S = 2048; dm.H = dm.L - dm.S;
   dm.c = 64; dm.g = 8; dm.Bq = 64; dm.kc = 16; dm.kg = 4; dm.kge = 4; dm.per = 8; dm.sink = 64; dm.local = 128;
   dm.NQB = dm.S / dm.Bq; dm.Nc = dm.L / dm.c; dm.Ng = dm.L / dm.g; dm.NcS = dm.Nc; dm.NgS = dm.Ng; dm.width = 64; dm.rows = 256; dm.flags = 0; dm.rows_q = dm.S; dm.rows_k = dm.L;
   dm.scale = 1.f / sqrtf(128.f);
@@ -61,10 +61,11 @@ int main(int argc, char** argv) {
     Window w = window_of(dm, qb);
     int lo = w.se / 8, hi = w.ls / 8;
     std::vector<int> pool;
-    // 16 chunks x 4 groups, as the router would select (history mostly)
-    while ((int)pool.size() < 64) { int m = lo + rand() % (hi - lo); if (std::find(pool.begin(), pool.end(), m) == pool.end()) pool.push_back(m); }
+    // 16 chunks x 4 groups, as the router would select (history mostly, if there is any)
+    ng[it] = std::max(0, std::min(64, (hi - lo) / 2));
+    while ((int)pool.size() < ng[it]) { int m = lo + rand() % (hi - lo); if (std::find(pool.begin(), pool.end(), m) == pool.end()) pool.push_back(m); }
     std::sort(pool.begin(), pool.end());
-    for (int i = 0; i < 64; ++i) gi[it * 64 + i] = pool[i];
+    for (int i = 0; i < ng[it]; ++i) gi[it * 64 + i] = pool[i];
   }
   __nv_bfloat16 *dq, *dk, *dv, *dO, *ddO, *ddQ; int *dgi, *dng, *dst; float* dlse; float *ddK, *ddV;
   cudaMalloc(&dq, nq * 2); cudaMalloc(&dk, nk * 2); cudaMalloc(&dv, nk * 2); cudaMalloc(&dO, nq * 2);
@@ -81,7 +82,8 @@ int main(int argc, char** argv) {
   const bool fwd_mode = trace_threads == 256 || trace_threads == 384;
   for (int rep = 0; rep < 4; ++rep) {
     cudaMemsetAsync(flush, rep, 512u << 20);
-    { void* p_; cudaGetSymbolAddress(&p_, g_trace_log); cudaMemsetAsync(p_, 0, sizeof(unsigned) * HGA_TRACE_WARPS * HGA_TRACE_SLOTS); }
+    { void* p_; cudaGetSymbolAddress(&p_, g_trace_log); cudaMemsetAsync(p_, 0, sizeof(unsigned) * HGA_TRACE_WARPS * HGA_TRACE_SLOTS);
+      cudaGetSymbolAddress(&p_, g_trace_cta); cudaMemsetAsync(p_, 0, sizeof(g_trace_cta)); }
     cudaEventRecord(e0);
     int rc = fwd_mode ? launch_attn_fwd_sm100(dm, nullptr, dq, dk, dv, dgi, dng, dO, dlse, dst, 0)
                       : launch_attn_bwd_sm100(dm, nullptr, dq, dk, dv, dO, dlse, ddO, dgi, dng, ddQ, ddK, ddV, dst, 0);
@@ -93,13 +95,20 @@ int main(int argc, char** argv) {
   int st; cudaMemcpy(&st, dst, 4, cudaMemcpyDeviceToHost); printf("status %d\n", st);
   static unsigned long long hc[2048][3]; cudaMemcpyFromSymbol(hc, g_trace_cta, sizeof(hc));
   const int ncta = trace_threads == 448 ? 128 : trace_threads == 384 ? 256 : 512;
+  // (a persistent kernel's CTAs take over most of the grid: those never start)
   unsigned long long t0 = ~0ull, t1 = 0;
-  for (int i = 0; i < ncta; ++i) { t0 = std::min(t0, hc[i][1]); t1 = std::max(t1, hc[i][2]); }
+  int started = 0;
+  double sum = 0;
+  for (int i = 0; i < ncta; ++i)
+    if (hc[i][2]) { ++started; t0 = std::min(t0, hc[i][1]); t1 = std::max(t1, hc[i][2]); sum += (hc[i][2] - hc[i][1]) / 1e3; }
   printf("kernel span by globaltimer: %.1f us\n", (t1 - t0) / 1e3);
-  double sum = 0; for (int i = 0; i < ncta; ++i) sum += (hc[i][2] - hc[i][1]) / 1e3; printf("mean CTA duration %.1f us\n", sum / ncta);
+  printf("%d CTAs, mean duration %.1f us; start .. end:\n", started, sum / started);
+  for (int i = 0; i < ncta; ++i)
+    if (hc[i][2]) printf(" %d:%.1f..%.1f", i, (hc[i][1] - t0) / 1e3, (hc[i][2] - t0) / 1e3);
+  printf("\n");
   { unsigned sm_sel = (unsigned)hc[trace_blk][0];
     std::vector<std::array<unsigned long long, 2>> vv;
-    for (int i = 0; i < ncta; ++i) if (hc[i][0] == sm_sel) vv.push_back({hc[i][1], hc[i][2]});
+    for (int i = 0; i < ncta; ++i) if (hc[i][0] == sm_sel && hc[i][2]) vv.push_back({hc[i][1], hc[i][2]});
     std::sort(vv.begin(), vv.end());
     printf("SM %u:", sm_sel);
     for (auto& x : vv) printf(" [%.1f .. %.1f]", (x[0] - t0) / 1e3, (x[1] - t0) / 1e3);
