@@ -481,7 +481,7 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       for (int u = 0; u < n_pairs; ++u, ++U) {
         const uint32_t s_addr = lane_base + region(rs) + wg * 64, dp_addr = lane_base + region(rp) + wg * 64;
         const Pairs pairs(un);                    // (read again for every pair: registers are short)
-        const bool with_grads = pairs.with_grads(u), grads = with_grads && wg == 0;
+        const bool with_grads = pairs.with_grads(u);
         // how many of this thread's keys are visible: all of the far ones, of the local ones those up to the row's own
         const int see = un.vis + un.pos[row >> 6] + (row & 63);
         const int vis = (wg == 0 ? 8 * pairs.acts(u) : 0) + max(0, see - 8 * pairs.first_other(u, wg));
@@ -489,23 +489,45 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         if (!wait(&sm.s_full[U & 1], U >> 1)) break;
         tc_fence_after_sync();
         HGA_TRACE_POINT(11);
+        auto exponents = [&](uint32_t s0, uint32_t s1, float& a0, float& a1) {       // of two neighbouring keys
+          unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(s0), __uint_as_float(s1)), sl2_2, neg_lse2_2), a0, a1);
+        };
+        if (!with_grads) {
 #pragma unroll
-        for (int q4 = 0; q4 < 4; ++q4) {
-          uint32_t sv[16];
-          tmem_ld16(s_addr + q4 * 16, sv);
-          tmem_wait_ld();
+          for (int q4 = 0; q4 < 4; ++q4) {
+            uint32_t sv[16];
+            tmem_ld16(s_addr + q4 * 16, sv);
+            tmem_wait_ld();
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            float p0, p1;              // packed fp32 pairs: one FMA for the two exponent arguments
-            unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(sv[2 * i]), __uint_as_float(sv[2 * i + 1])), sl2_2, neg_lse2_2), p0, p1);
-            pk[8 * q4 + i] = pack_bf16(fast_exp2(p0), fast_exp2(p1));
+            for (int i = 0; i < 8; ++i) {
+              float a0, a1;
+              exponents(sv[2 * i], sv[2 * i + 1], a0, a1);
+              pk[8 * q4 + i] = pack_bf16(fast_exp2(a0), fast_exp2(a1));
+            }
           }
-        }
-        // (at the diagonal and the list's end only: two comparisons and selections per element in the loop above bound it by
-        // instruction issue, and a copy of it costs more instruction fetch than this)
-        if (__any_sync(0xffffffffu, vis < 64)) {
+          // (at the diagonal and the list's end only: two comparisons and selections per element in the loop above bound it by
+          // instruction issue, and a copy of it costs more instruction fetch than this)
+          if (__any_sync(0xffffffffu, vis < 64)) {
 #pragma unroll
-          for (int i = 0; i < 32; ++i) pk[i] = 2 * i + 1 < vis ? pk[i] : 2 * i < vis ? pk[i] & 0xffffu : 0u;
+            for (int i = 0; i < 32; ++i) pk[i] = 2 * i + 1 < vis ? pk[i] : 2 * i < vis ? pk[i] & 0xffffu : 0u;
+          }
+        } else {
+          // a pair with dK/dV: dS comes from the unrounded P, which takes the place of S (the next dP does not go there)
+#pragma unroll 1
+          for (int q4 = 0; q4 < 4; ++q4) {
+            uint32_t sv[16];
+            tmem_ld16(s_addr + q4 * 16, sv);
+            tmem_wait_ld();
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              float a0, a1;
+              exponents(sv[2 * i], sv[2 * i + 1], a0, a1);
+              sv[2 * i] = 16 * q4 + 2 * i < vis ? __float_as_uint(fast_exp2(a0)) : 0u;
+              sv[2 * i + 1] = 16 * q4 + 2 * i + 1 < vis ? __float_as_uint(fast_exp2(a1)) : 0u;
+            }
+            tmem_st16(s_addr + q4 * 16, sv);
+          }
+          tmem_wait_st();
         }
         tc_fence_before_sync();
         mbar_arrive_warp(&sm.s_read[U & 1]);      // S has been read: its region may take the next pair's dP
@@ -519,36 +541,49 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         HGA_TRACE_POINT(13);
         k.next();
         const uint64_t scale_2 = pack_f32x2(dm.scale, dm.scale), neg_delta_s_2 = pack_f32x2(nds, nds);
-        uint32_t p_line = 0;                      // this row's 128-byte line of P (dS's: 16 KB on), 16-byte chunks XOR-swizzled
-        if (grads) {
-          if (!wait(&sm.k_full[k.at], k.parity)) break;
-          p_line = smem_u32(sm.k[k.at]) + (uint32_t)row * 128;
-        }
+        auto gradient = [&](uint64_t p2, uint32_t dp0, uint32_t dp1) {               // dS of two neighbouring keys, rounded
+          float d0, d1;
+          unpack_f32x2(mul_f32x2(p2, fma_f32x2(pack_f32x2(__uint_as_float(dp0), __uint_as_float(dp1)), scale_2, neg_delta_s_2)), d0, d1);
+          return pack_bf16(d0, d1);
+        };
+        // bf16 dS goes over the dP columns already read (8 columns per 16 keys): the A operand of dQ
+        if (!with_grads) {
 #pragma unroll
-        for (int q4 = 0; q4 < 4; ++q4) {          // 16 keys at a time
-          uint32_t dp[16], dk[8];
-          tmem_ld16(dp_addr + q4 * 16, dp);
-          tmem_wait_ld();
+          for (int q4 = 0; q4 < 4; ++q4) {        // 16 keys at a time
+            uint32_t dp[16], dk[8];
+            tmem_ld16(dp_addr + q4 * 16, dp);
+            tmem_wait_ld();
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const uint64_t p2 = pack_f32x2(__uint_as_float(pk[8 * q4 + i] << 16), __uint_as_float(pk[8 * q4 + i] & 0xffff0000u));
-            const uint64_t g2 = fma_f32x2(pack_f32x2(__uint_as_float(dp[2 * i]), __uint_as_float(dp[2 * i + 1])), scale_2, neg_delta_s_2);
-            float d0, d1;
-            unpack_f32x2(mul_f32x2(p2, g2), d0, d1);
-            dk[i] = pack_bf16(d0, d1);
+            for (int i = 0; i < 8; ++i)
+              dk[i] = gradient(pack_f32x2(__uint_as_float(pk[8 * q4 + i] << 16), __uint_as_float(pk[8 * q4 + i] & 0xffff0000u)), dp[2 * i], dp[2 * i + 1]);
+            tmem_st8(dp_addr + q4 * 8, dk);
           }
-          // bf16 dS over the dP columns already read (8 columns per 16 keys): the A operand of dQ
-          tmem_st8(dp_addr + q4 * 8, dk);
-          if (grads)
+        } else {
+          if (wg == 0 && !wait(&sm.k_full[k.at], k.parity)) break;
+          const uint32_t p_line = smem_u32(sm.k[k.at]) + (uint32_t)row * 128;      // this row's 128-byte line of P (dS's: 16 KB on), 16-byte chunks XOR-swizzled
+#pragma unroll 1
+          for (int q4 = 0; q4 < 4; ++q4) {
+            uint32_t p[16], dp[16], dk[8];
+            tmem_ld16(s_addr + q4 * 16, p);
+            tmem_ld16(dp_addr + q4 * 16, dp);
+            tmem_wait_ld();
 #pragma unroll
-            for (int cc = 0; cc < 2; ++cc) {      // 8 keys
-              const uint32_t at = p_line + ((uint32_t)(2 * q4 + cc) ^ key) * 16;
-              st_shared_v4(at, pk[8 * q4 + 4 * cc], pk[8 * q4 + 4 * cc + 1], pk[8 * q4 + 4 * cc + 2], pk[8 * q4 + 4 * cc + 3]);
-              st_shared_v4(at + 16384, dk[4 * cc], dk[4 * cc + 1], dk[4 * cc + 2], dk[4 * cc + 3]);
+            for (int i = 0; i < 8; ++i)
+              dk[i] = gradient(pack_f32x2(__uint_as_float(p[2 * i]), __uint_as_float(p[2 * i + 1])), dp[2 * i], dp[2 * i + 1]);
+            tmem_st8(dp_addr + q4 * 8, dk);
+            if (wg == 0) {
+#pragma unroll
+              for (int cc = 0; cc < 2; ++cc) {    // 8 keys
+                const uint32_t at = p_line + ((uint32_t)(2 * q4 + cc) ^ key) * 16;
+                auto rounded = [&](int i) { return pack_bf16(__uint_as_float(p[8 * cc + 2 * i]), __uint_as_float(p[8 * cc + 2 * i + 1])); };
+                st_shared_v4(at, rounded(0), rounded(1), rounded(2), rounded(3));
+                st_shared_v4(at + 16384, dk[4 * cc], dk[4 * cc + 1], dk[4 * cc + 2], dk[4 * cc + 3]);
+              }
             }
+          }
+          fence_proxy_async_smem();
         }
         tmem_wait_st();
-        if (grads) fence_proxy_async_smem();
         tc_fence_before_sync();
         mbar_arrive_warp(&sm.ds_full[U & 1]);
         HGA_TRACE_POINT(14);
