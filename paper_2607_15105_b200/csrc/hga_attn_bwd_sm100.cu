@@ -11,7 +11,7 @@
 // block come from k_attn_bwd_band_sm100, which precedes this kernel).  Their octets, eight to a pair, are in the first tiles of
 // n_a pairs; P and dS of such a first tile go to shared memory as well:
 //      dV^T = dO^T P, dK^T = Q^T dS                  (M = head_dim, N = 64 keys, K = 128 rows) over the S columns read by then,
-// and four warps stage the two, as key rows, in the place of P and dS and add them to global memory row by row.
+// and four warps add the two to global memory straight from tensor memory.
 //
 // Persistent CTAs: a CTA takes over the next one of the grid that has not started (cluster launch control), and
 // every role goes on to the next unit by itself, so that its list, Q, dO, K, V, delta and first GEMMs come while the
@@ -29,9 +29,9 @@
 //
 // What bounds it: the row threads, ~2.7k cycles per pair (1.0k of exponentials; tensor-memory loads and barrier hand-offs), a unit's
 // first pair, which waits for dO (its buffer is free only behind the last pair's dP), and a pair with dK/dV, whose place costs the K
-// ring its third stage.  hga_attn_bwd with the band kernel, one CTA per unit -> persistent: 16K layer 99 -> 86 us, whole step 160.7 ->
-// 146.6; walk of 16K 1147 -> 1095; twelve packed sequences 369 -> 342; 2K layer, nearly all of whose pairs have dK/dV (one every
-// 7k cycles, 5k of them the four warps' reduction), 149.4 -> 150.4.
+// ring its third stage.  Whole steps, one CTA per unit -> persistent: 16K layer 161 -> 147 us, walk of 16K 1147 -> 1076; 2K layer,
+// nearly all of whose pairs have dK/dV, 149 -> 139; twelve packed sequences 369 -> 334.  The 2K layer's additions (168 MB of
+// fp32) are what it waits for.
 //
 // Warp roles (640 threads, 96 registers):
 //   0, 3     K octets 0-7 / 8-15 of every pair (a box costs its issuing warp ~100 cycles)      16, 17   the same for V
@@ -104,13 +104,12 @@ struct BwdSmem {
   alignas(16) uint4 cancelled;                  // answer of the launch control
   uint64_t info_full[2], info_empty[2], plan, cancel_full;
   uint64_t q_full, q_empty, do_full, do_empty;
-  // Ring items: full by copy (or, a place of P and dS, as soon as it is free); empty by the GEMMs that read them, or (k_out, a
-  // place of P and dS) by the four warps that staged dV and dK there
-  uint64_t k_full[kKStages], k_empty[kKStages], k_out[kKStages], v_full[kVStages], v_empty[kVStages];
+  // Ring items: full by copy (or, a place of P and dS, as soon as it is free), empty by the GEMMs that read them
+  uint64_t k_full[kKStages], k_empty[kKStages], v_full[kVStages], v_empty[kVStages];
   // Per pair, alternately (every completion has to depend on its waiter having observed the one before on the same barrier:
   // S(u+1) and dP(u+1) are issued before the row threads' arrivals of pair u have been waited for)
   uint64_t s_full[2], dp_full[2], s_read[2], ds_full[2], step_done[2];
-  uint64_t acc_full[2], acc_read[2], staged;    // pairs with dK/dV, counted by themselves
+  uint64_t acc_full[2], acc_read[2];            // pairs with dK/dV, counted by themselves
   uint64_t lse_full, stat_full, stat_empty, dq_done, dq_free;
   uint64_t drain[2];
   uint32_t tmem_base;
@@ -139,16 +138,12 @@ __device__ __forceinline__ int next_cta_of(const void* answer) {
   return given ? (int)x : -1;
 }
 
-__device__ __forceinline__ void red_add_v4(float* to, const uint32_t (&x)[4]) {
-  asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};"
-               ::"l"(__cvta_generic_to_global(to)), "f"(__uint_as_float(x[0])), "f"(__uint_as_float(x[1])), "f"(__uint_as_float(x[2])), "f"(__uint_as_float(x[3]))
-               : "memory");
+__device__ __forceinline__ void red_add(float* to, float x) {
+  asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(__cvta_generic_to_global(to)), "f"(x) : "memory");
 }
 
-__device__ __noinline__ bool wait_out_of_line(uint64_t* bar, uint32_t parity, volatile int* abort) {
-  return __all_sync(0xffffffffu, bwd_wait(bar, parity & 1, abort));
-}
-// Quotients where nothing waits for them
+// A quotient where nothing waits for it (400 bytes of code; called from the set-up of the other kernels, whose CTAs do wait for
+// it, this made the forward 2 us slower)
 __device__ __noinline__ int quotient(int a, int b) { return a / b; }
 
 // The units of a segment in launch order.  The first blocks see no routed key of the active segment: they come first, for the
@@ -194,9 +189,8 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     mbar_init(&sm.q_full, 1); mbar_init(&sm.do_full, 1);
     mbar_init(&sm.q_empty, 2);                    // S of the last pair, and the dK GEMMs
     mbar_init(&sm.do_empty, 6);                   // dP of the last pair, the dV GEMMs, and the four statistics warps
-    for (int s = 0; s < kKStages; ++s) { mbar_init(&sm.k_full[s], 2); mbar_init(&sm.k_empty[s], 1); mbar_init(&sm.k_out[s], 4); }
+    for (int s = 0; s < kKStages; ++s) { mbar_init(&sm.k_full[s], 2); mbar_init(&sm.k_empty[s], 1); }
     for (int s = 0; s < kVStages; ++s) { mbar_init(&sm.v_full[s], 2); mbar_init(&sm.v_empty[s], 1); }
-    mbar_init(&sm.staged, 4);
     mbar_init(&sm.lse_full, 4); mbar_init(&sm.stat_full, 4); mbar_init(&sm.stat_empty, 8);
     mbar_init(&sm.dq_done, 1); mbar_init(&sm.dq_free, 4);
     sm.abort = 0;
@@ -294,15 +288,11 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     if (lane == 0) prefetch_tensormap(map);
     const int n_stages = is_v ? kVStages : kKStages;
     int st = 0;                                   // stage of the next ring item
-    uint32_t used = 0, phase_empty = 0, phase_out = 0, is_place = 0;       // per stage
-    auto take_stage = [&](bool place) {           // waits until it is free
+    uint32_t used = 0, phase = 0;                 // per stage
+    auto take_stage = [&]() {                     // waits until it is free
       const uint32_t bit = 1u << st;
-      if (used & bit) {
-        if (is_place & bit) { wait_by_call(&sm.k_out[st], phase_out >> st); phase_out ^= bit; }
-        else { wait_by_call(&empty[st], phase_empty >> st); phase_empty ^= bit; }
-      }
+      if (used & bit) { wait_by_call(&empty[st], phase >> st); phase ^= bit; }
       used |= bit;
-      is_place = place ? is_place | bit : is_place & ~bit;
       return ok;
     };
     auto next_stage = [&]() { st = st + 1 == n_stages ? 0 : st + 1; };
@@ -325,14 +315,14 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         const int next_row = u + 1 < n_pairs ? row_of(u + 1) : 0;
         if (u >= 0) {
           if (warp == 0 && lane == 0 && u == max(0, n_pairs - 3)) mbar_arrive(&sm.plan);
-          if (!take_stage(false)) break;
+          if (!take_stage()) break;
           if (lane == 0) mbar_arrive_expect_tx(&full[st], 8 * kOct);
           __syncwarp();
           if (lane < 8) tma_load_5d((is_v ? sm.v[st] : sm.k[st]) + (8 * part + lane) * kOct, map, &full[st], 0, row, 0, h, b);
           HGA_TRACE_POINT(2);
           next_stage();
           if (!is_v && pairs.with_grads(u)) {     // the place of P and dS
-            if (!take_stage(true)) break;
+            if (!take_stage()) break;
             mbar_arrive_warp(&full[st]);
             next_stage();
           }
@@ -455,6 +445,7 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             for (int kk = 0; kk < 8; ++kk)        // 16 query rows per instruction
               mma_ss_w(lead, acc + 64 * which, desc_advance(which ? q_mn : do_mn, kk * 2048), desc_advance(p, which * 16384 + kk * 2048), idesc_t, kk > 0);
           mma_commit_w(lead, &sm.acc_full[n_grads++ & 1]);
+          mma_commit_w(lead, &sm.k_empty[k.at]);
           if (u + 1 == pairs.a_begin + pairs.n_a) { mma_commit_w(lead, &sm.q_empty); mma_commit_w(lead, &sm.do_empty); }
           k.next();
         }
@@ -596,8 +587,7 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // ------------------------------------------------------------------ statistics, dK / dV reduction, dQ epilogue
     const int quarter = warp & 3, row = quarter * 32 + lane;
     const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16), key = (uint32_t)(row & 7);
-    uint32_t n_grads = 0, rs = 0, rp = 1, staged_phase = 0;
-    KStage k;
+    uint32_t n_grads = 0, rs = 0, rp = 1;
     bool band_done = false;
     // -LSE and -delta of unit n's rows: a thread each (O from global memory, dO from the tile in shared memory)
     auto statistics = [&](int n, const Unit& un) {
@@ -642,10 +632,6 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       mbar_arrive_warp(&sm.stat_full);
       HGA_TRACE_POINT(10);
     };
-    auto all_staged = [&]() {                     // the four warps meet
-      mbar_arrive_warp(&sm.staged);
-      return wait_by_call(&sm.staged, staged_phase++);
-    };
     for (int n = 0; ok; ++n) {
       const Unit& un = unit_info(n);
       if (!ok) break;
@@ -679,74 +665,51 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       }
       if (!more) break;
 #pragma unroll 1
-      for (int u = 0; u < un.a_begin; ++u) { next_regions(false, rs, rp); k.next(); }
+      for (int u = 0; u < un.a_begin; ++u) next_regions(false, rs, rp);
 #pragma unroll 1
       for (int first = 0; first < un.n_act; first += 8) {
-        k.next();                                 // (the place)
-        // Four octets at a time, one per warp, of dV (into P's place) and of dK (dS's)
-        const int n_rounds = un.n_act - first > 4 ? 2 : 1;
-        int at, at_next;                          // positions of this warp's
+        int mine;                                 // lane = octet: its position, -1 where it gets nothing from here
         {
           FarList far(dm, Window{0, un.ls, un.se}, group_idx + un.list);
           far.ng = un.ng; far.n_far = un.n_hist + un.n_act; far.clean = un.clean;
-          const int o = first + quarter + 4 * (lane & 1);
-          const int mine = o < un.n_act ? far.row(un.n_hist + o) : -1;
-          at = __shfl_sync(0xffffffffu, mine, 0);
-          at_next = __shfl_sync(0xffffffffu, mine, 1);
+          mine = lane < 8 && first + lane < un.n_act ? far.row(un.n_hist + first + lane) : -1;
         }
         if (!wait_by_call(&sm.acc_full[n_grads & 1], n_grads >> 1)) break;
         tc_fence_after_sync();
         HGA_TRACE_POINT(16);
-        // The transposed accumulators (lane = element, column = key) become key rows of 512 bytes, which a warp adds to global
-        // memory with one instruction each.  (As 4 KB bulk reductions they queued up behind the K and V copies and held the place,
-        // and with it the ring, for up to 6k cycles.)
-        const uint32_t place = smem_u32(sm.k[k.at]);
+        // The band kernel, which precedes this one in the stream, stores its dK/dV rows plainly: these additions must come
+        // after it.  Nothing else in this kernel depends on it (what is read was complete when that kernel let this one start).
+        if (!band_done) { pdl_wait(); band_done = true; }
+        // lane = element, column = key: 128 consecutive bytes per warp and addition
+        // (staged in shared memory as key rows and added 512 bytes or 4 KB at a time, the additions held the place of P and
+        // dS, and with it the K ring, for 5k cycles a pair)
 #pragma unroll 1
-        for (int round = 0; round < n_rounds; ++round) {
-          if (round == 1 && !all_staged()) break;                          // the first round's rows have been read
-#pragma unroll 1
-          for (int which = 0; which < 2; ++which) {                        // dV, dK
-            uint32_t x[32];
-            tmem_ld32(lane_base + region(rs) + 64 * which + 32 * round, x);
-            tmem_wait_ld();
-#pragma unroll
-            for (int i = 0; i < 32; ++i) st_shared_b32(place + (uint32_t)(row * 4 + which * 16384 + i * 512), x[i]);
-          }
-          if (round + 1 == n_rounds) {
+        for (int part = 0; part < 4; ++part) {    // dV of octets 0-3 and 4-7, dK of the same
+          uint32_t x[32];
+          tmem_ld32(lane_base + region(rs) + 32 * part, x);
+          tmem_wait_ld();
+          if (part == 3) {
             tc_fence_before_sync();
             mbar_arrive_warp(&sm.acc_read[n_grads & 1]);
           }
-          if (!all_staged()) break;
-          // The band kernel, which precedes this one in the stream, stores its dK/dV rows plainly: these additions must come
-          // after it.  Nothing else in this kernel depends on it (what is read was complete when that kernel let this one start).
-          if (!band_done) { pdl_wait(); band_done = true; }
-          if (at >= 0) {
-            const int64_t to = (un.grad_row + at) * D + 4 * lane;
-#pragma unroll 1
-            for (int which = 0; which < 2; ++which) {
-              float* const out = (which ? dK : dV) + to;
-              const uint32_t from = place + (uint32_t)(which * 16384 + quarter * 4096 + lane * 16);
 #pragma unroll
-              for (int i = 0; i < 8; ++i) {       // rows of the octet
-                uint32_t w[4];
-                ld_shared_v4(from + i * 512, w[0], w[1], w[2], w[3]);
-                red_add_v4(out + 128 * i, w);
-              }
+          for (int o = 0; o < 4; ++o) {
+            const int at = __shfl_sync(0xffffffffu, mine, 4 * (part & 1) + o);
+            if (at >= 0) {
+              float* const to = (part >= 2 ? dK : dV) + (un.grad_row + at) * D + row;
+#pragma unroll
+              for (int i = 0; i < 8; ++i) red_add(to + i * D, __uint_as_float(x[8 * o + i]));
             }
           }
-          at = at_next;
         }
-        fence_proxy_async_smem();                 // (the place is next written by a copy)
-        mbar_arrive_warp(&sm.k_out[k.at]);
         if (!ok) break;
         HGA_TRACE_POINT(18);
         ++n_grads;
-        k.next();
         next_regions(true, rs, rp);
       }
       if (!ok) break;
 #pragma unroll 1
-      for (int u = un.a_begin + un.n_a; u < un.n_pairs; ++u) { next_regions(false, rs, rp); k.next(); }
+      for (int u = un.a_begin + un.n_a; u < un.n_pairs; ++u) next_regions(false, rs, rp);
     }
     // the end of this grid has to imply the end of the band kernel's, even where there was nothing to add
     if (!band_done) pdl_wait();

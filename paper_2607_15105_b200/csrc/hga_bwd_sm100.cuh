@@ -38,6 +38,11 @@ __device__ __forceinline__ bool bwd_wait_(uint64_t* bar, uint32_t parity, volati
 #define HGA_ABORT_CODE(kernel, flag) HGA_STATUS_WAIT_TIMEOUT
 #endif
 
+// The same for a whole warp, all of whose lanes poll, and out of line: for roles that can spare the call
+static __device__ __noinline__ bool wait_out_of_line(uint64_t* bar, uint32_t parity, volatile int* abort) {
+  return __all_sync(0xffffffffu, bwd_wait(bar, parity & 1, abort));
+}
+
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
