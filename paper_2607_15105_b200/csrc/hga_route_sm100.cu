@@ -17,6 +17,10 @@
 // half of this tile's GEMMs.  Where Q, two slabs and the scores fit half of an SM (up to 256 query rows at head_dim 128)
 // two CTAs share it and one's serial phases hide behind the other's GEMMs; four slabs where they fit; larger row
 // counts take a whole SM with four accumulators.
+//
+// Code size: a CTA of a small problem runs most of this once, on instruction caches that other kernels have filled meanwhile, so
+// loops that are not hot are not unrolled (left to itself the compiler made 127 KB of it, now 67): whole steps, 16K layer
+// 147.1 -> 145.6 us, one / 32 tokens of a generation 16.6 -> 15.4 and 36.9 -> 35.1, tiny layer 43.6 -> 42.7, 128K 90.2 -> 89.4.
 #include <algorithm>
 #include <cfloat>
 #include <type_traits>
@@ -97,6 +101,7 @@ __device__ __forceinline__ void warp_select(const uint32_t* keys, int n, int k, 
   };
   uint32_t hi = 0, both = 0xffffffffu, any = 0;      // bits that are one / not zero in all keys
   each([&](uint32_t key) { hi = max(hi, key); });
+#pragma unroll 1
   for (int i = lane; i < n; i += 32) {
     const uint32_t key = keys[i];
     both &= key;
@@ -108,6 +113,7 @@ __device__ __forceinline__ void warp_select(const uint32_t* keys, int n, int k, 
   if (differ != 0) {
     uint32_t bit = 0x80000000u >> __clz(differ);
     kth = hi & ~(2 * bit - 1);          // (2 * bit wraps to 0 at the top bit: nothing is shared)
+#pragma unroll 1
     for (int reach = n; bit != 0 && reach != k; bit >>= 1) {
       const uint32_t t = kth | bit;
       int c = 0;
@@ -120,6 +126,7 @@ __device__ __forceinline__ void warp_select(const uint32_t* keys, int n, int k, 
   each([&](uint32_t key) { above += key > kth ? 1 : 0; });
   int ties = k - __reduce_add_sync(full, above), rank = 0;      // of the keys equal to it, how many are still to be taken
   const uint32_t below = (1u << lane) - 1u;
+#pragma unroll 1
   for (int base = 0; base < n; base += 32) {
     const int i = base + lane;
     const uint32_t key = i < n ? keys[i] : 0u;
@@ -159,8 +166,8 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
   // (late query blocks first: where the history is short they have the most candidates)
   int cta;
   const Segment sg = segment_of(dm, segs, blockIdx.x, cta);
-  const int n_bh = dm.B * dm.Hkv, n_qb = sg.S / dm.Bq;
-  const int qb = n_qb - 1 - cta / n_bh, b = cta % n_bh / dm.Hkv, h = cta % n_bh % dm.Hkv;
+  const int n_bh = dm.B * dm.Hkv, n_qb = sg.S / dm.Bq, i_qb = cta / n_bh, bh = cta - i_qb * n_bh;
+  const int qb = n_qb - 1 - i_qb, b = bh / dm.Hkv, h = bh - b * dm.Hkv;
   const int64_t item = item_base(dm, sg, b) + h * n_qb + qb;
   const Window w = window_at(dm, sg.H + qb * dm.Bq);
   const int j0 = w.se / dm.c, n_cand = (w.ls - w.se) / dm.c;
@@ -181,7 +188,8 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
   uint32_t col_mask = 0xffffffffu;                           // bit i: column i of a block of 32 is a real query row
   if (!all_rows_real) {
     col_mask = 0;
-    for (int i = 0; i < 32; ++i) col_mask |= (uint32_t)((i % bq_pad) < dm.Bq) << i;
+#pragma unroll 1
+    for (int i = 0, t = 0; i < 32; ++i, t = t + 1 == bq_pad ? 0 : t + 1) col_mask |= (uint32_t)(t < dm.Bq) << i;
   }
 
   // Copies slab p of chunk tile t (slab number g overall) into its stage; all lanes of warp 0.  The candidate chunks are
@@ -197,8 +205,8 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
   // Box `oc` of group tile t: one octet of an opened chunk's group summaries, [octet][panel][8 rows][128 B] over the tile's
   // neighbouring slabs; the bytes are announced on the first one's barrier.
   auto copy_group_octet = [&](int tg, int t, int oc_in_tile) {
-    const int s = tg * kPanels % NSTG, oc = 16 * t + oc_in_tile, r = oc / opc;
-    const int row = r < k_sel ? gs0 + sorted[r] * dm.per + 8 * (oc % opc) : dm.Ng;
+    const int s = tg * kPanels % NSTG, oc = 16 * t + oc_in_tile, r = opc == 1 ? oc : oc >> 1;      // (one or two octets)
+    const int row = r < k_sel ? gs0 + sorted[r] * dm.per + 8 * (oc - r * opc) : dm.Ng;
     tma_load_5d(sm.a[s] + oc_in_tile * kOctBytes, &map_gs, &sm.a_full[s], 0, row, 0, h, b);
   };
   auto announce_group_tile = [&](int tg) {
@@ -224,6 +232,7 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
     __syncwarp();
     pdl_wait();
     // the first slabs depend on nothing: their copies start before the CTA meets
+#pragma unroll 1
     for (int g = 0; g < n_pre; ++g) copy_slab(g, g / kPanels, g % kPanels);
     if (lane == 0 && k_sel > 0) mbar_arrive_expect_tx(&sm.q_full, (uint32_t)(rows_pad / 8) * kOctBytes);
   }
@@ -246,9 +255,11 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
 
   // optional output: -inf outside the candidate range
   if (chunk_scores)
+#pragma unroll 1
     for (int j = tid; j < dm.Nc; j += kRtThreads)
       if (j < j0 || j >= j0 + n_cand) chunk_scores[item * dm.Nc + j] = -INFINITY;
   if (group_scores)
+#pragma unroll 1
     for (int i = tid; i < dm.kc * dm.per; i += kRtThreads)
       group_scores[item * dm.kc * dm.per + i] = -INFINITY;
 
@@ -265,13 +276,15 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
         // The item's query rows.  Issuing a box costs its warp a few hundred
         // cycles and warps issue in parallel, so the boxes are spread over the non-producer warps.
         if (boxes) {
+#pragma unroll 1
           for (int i = (warp - 2) + kRtCopyWarps * lane; i < rows_pad / 64 * kPanels; i += 32 * kRtCopyWarps) {
-            const int panel = i % kPanels, r = i / kPanels * 64;
-            tma_load_5d(q_smem + panel * q_panel + r * 128, &map_q, &sm.q_full, 0, sg.q0 + qb * dm.Bq + r % dm.Bq, panel, h * dm.G + r / dm.Bq, b);
+            const int panel = i % kPanels, r = i / kPanels * 64, a = r / dm.Bq;
+            tma_load_5d(q_smem + panel * q_panel + r * 128, &map_q, &sm.q_full, 0, sg.q0 + qb * dm.Bq + r - a * dm.Bq, panel, h * dm.G + a, b);
           }
         } else {
+#pragma unroll 1
           for (int o = (warp - 2) + kRtCopyWarps * lane; o < rows_pad / 8; o += 32 * kRtCopyWarps) {
-            const int r = 8 * o, a = r / bq_pad, t = r % bq_pad;    // rows past the segment arrive as zeros
+            const int r = 8 * o, a = r / bq_pad, t = r - a * bq_pad;    // rows past the segment arrive as zeros
             tma_load_5d(q_smem + o * kOctBytes, &map_q, &sm.q_full, 0, sg.q0 + qb * dm.Bq + t, 0, h * dm.G + a, b);
           }
         }
@@ -290,12 +303,14 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
           return ok;
         };
         if (!phase2) {
+#pragma unroll 1
           for (int g = n_pre; g < n_slabs; ++g) {
             if (!wait_empty(g)) break;
             copy_slab(g, g / kPanels, g % kPanels);
           }
         } else {
           announce_group_tile(t_begin);      // (its boxes come from the other warps, see above)
+#pragma unroll 1
           for (int t = 1; t < n_tiles && ok; ++t) {
             const int tg = t_begin + t;
             for (int p = 0; p < kPanels && ok; ++p) wait_empty(tg * kPanels + p);
@@ -466,8 +481,10 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
                 const uint4 kk = k4[q >> 2];
                 beat += (int)(kk.x > mine) + (int)(kk.y > mine) + (int)(kk.z > mine) + (int)(kk.w > mine);
               }
+#pragma unroll 1
               for (; q < n; ++q) beat += keys[q] > mine;
             } else {
+#pragma unroll 1
               for (; q < n; ++q) beat += keys[q] > mine || (keys[q] == mine && q < tid);
             }
             sel = beat < k_sel;
@@ -477,6 +494,7 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
         };
         auto picked_below = [&](int words) {
           int c = 0;
+#pragma unroll 1
           for (int q = 0; q < words; ++q) c += __popc(flags[q]);
           return c;
         };
@@ -495,6 +513,7 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
       __syncthreads();
     }
     if (!sm.abort) {
+#pragma unroll 1
       for (int i = tid; i < dm.kc; i += kRtThreads)
         chunk_idx[item * dm.kc + i] = i < k_sel ? sorted[i] : -1;
     }
@@ -516,12 +535,14 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
       // a chunk passed and the list was written past its end.)
       const int total = k_sel * dm.per;
       const int want = global_budget ? k_sel * dm.kge : dm.kge;
+#pragma unroll 1
       for (int base = 0; base < total; base += kRtThreads) {      // warp-uniform trip count (ballots below)
         const int i = base + tid;
         bool sel = false;
         if (i < total) {
           const uint32_t mine = gkeys[i];
-          const int lo = global_budget ? 0 : i - i % dm.per, hi = global_budget ? total : lo + dm.per;
+          const int lo = global_budget ? 0 : i & ~(dm.per - 1),       // (8 or 16)
+                    hi = global_budget ? total : lo + dm.per;
           int beat = 0;
 #pragma unroll 8
           for (int q = lo; q < hi; ++q) beat += gkeys[q] > mine || (gkeys[q] == mine && q < i);
@@ -532,31 +553,39 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
         if (lane == 0 && base + warp * 32 < total) flags[(base + warp * 32) >> 5] = word;
       }
       __syncthreads();
+#pragma unroll 1
       for (int i = tid; i < total; i += kRtThreads)
         if ((flags[i >> 5] >> (i & 31)) & 1u) {
           int pos = __popc(flags[i >> 5] & ((1u << (i & 31)) - 1u));
+#pragma unroll 1
           for (int q = 0; q < (i >> 5); ++q) pos += __popc(flags[q]);
-          gi[pos] = sorted[i / dm.per] * dm.per + i % dm.per;
+          gi[pos] = sorted[i >> (dm.per == 8 ? 3 : 4)] * dm.per + (i & (dm.per - 1));
         }
     } else
+#pragma unroll 1
     for (int r = tid; r < dm.kc; r += kRtThreads) {
       if (r < k_sel) {
         const uint32_t* v = gkeys + r * dm.per;
         unsigned long long picked = 0;
+#pragma unroll 1
         for (int q = 0; q < dm.kge; ++q) {
           int bu = -1;
+#pragma unroll 1
           for (int u = 0; u < dm.per; ++u)
             if (!((picked >> u) & 1ull) && (bu < 0 || v[u] > v[bu])) bu = u;     // first wins ties
           picked |= 1ull << bu;
         }
         int n = r * dm.kge;
+#pragma unroll 1
         for (int u = 0; u < dm.per; ++u)
           if ((picked >> u) & 1ull) gi[n++] = sorted[r] * dm.per + u;
         if (group_scores)
+#pragma unroll 1
           for (int u = 0; u < dm.per; ++u)
             group_scores[item * dm.kc * dm.per + r * dm.per + u] = rt_score(v[u]);
       }
     }
+#pragma unroll 1
     for (int i = k_sel * dm.kge + tid; i < dm.width; i += kRtThreads) gi[i] = -1;
     if (tid == 0) n_groups[item] = k_sel * dm.kge;
   }
