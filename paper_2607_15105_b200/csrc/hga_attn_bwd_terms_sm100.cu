@@ -17,6 +17,10 @@
 // a chain of hand-offs (copy -> S -> dS -> dQ), and while one CTA is in its exponentials, its set-up, its
 // dK/dV reduction or its epilogue, the other one has the tensor pipe.  At head_dim 128 it has the SM to itself.
 //
+// An M-tile that holds 64 rows only has them TWICE, in lanes 0-63 and 64-127, and a row's two threads take the first and the
+// last 32 keys of every tile, with zeros in the columns of the others: dQ is the sum of the two lanes' in the end.  (With zero
+// rows in lanes 64-127 two of the four sub-cores of an SM did all the work: 16 heads of 64 159.6 us a whole step, 146.5 so.)
+//
 // Order of the tiles of an item:
 //   1. the local window and the causal block, [ls, p0 + Bq): known without the routing list, so their copies
 //      start at once and the list is fetched and checked behind them;
@@ -100,30 +104,29 @@ k_attn_bwd_terms_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_c
   // expensive dK/dV tiles), early ones none, so the cheapest CTAs are the ones that fill the last wave.
   int cta;
   const Segment sg = segment_of(dm, segs, blockIdx.x, cta);
-  const int unit = cta / n_mt_item, n_bh = dm.B * dm.Hkv, mt = cta % n_mt_item;
-  const int qb = sg.S / dm.Bq - 1 - unit / n_bh, b = unit % n_bh / dm.Hkv, h = unit % n_bh % dm.Hkv;
-  const int64_t item = item_base(dm, sg, b) + h * (sg.S / dm.Bq) + qb;
+  const int n_qb = sg.S / dm.Bq, unit = cta / n_mt_item, n_bh = dm.B * dm.Hkv, mt = cta - unit * n_mt_item;
+  const int i_qb = unit / n_bh, bh = unit - i_qb * n_bh, qb = n_qb - 1 - i_qb, b = bh / dm.Hkv, h = bh - b * dm.Hkv;
+  const int64_t item = item_base(dm, sg, b) + h * n_qb + qb;
+  const bool twice = dm.rows - mt * 128 == 64;          // the M-tile's rows are there twice (Bq is a multiple of 64)
   const int qrow = sg.q0 + qb * dm.Bq;                  // the block's first row in Q, O, dO and dQ
   const Window w = window_at(dm, sg.H + qb * dm.Bq);
   const int n_local = w.p0 + dm.Bq - w.ls;              // tokens of the local window and the block (a multiple of 8)
   const int n_lt = (n_local + kKT - 1) / kKT;           // its tiles
   volatile int* abort = &sm.abort;
 
-  // Row threads: LSE and the O row of the thread's own query row (rows past the item's last one: zeros), requested
+  // Row threads: LSE and the O row of the thread's own query row, requested
   // before anything else so that the latency hides behind the set-up.
   float row_lse = 0.f;
+  int row_pos = 0;                                      // position inside the query block
   uint4 o_row[D / 8];
   if (warp >= 2 && warp < 6) {
-    const int r = mt * 128 + (warp & 3) * 32 + lane;
+    const int r = mt * 128 + (((warp & 3) * 32 + lane) & (twice ? 63 : 127)), a = r / dm.Bq;
+    row_pos = r - a * dm.Bq;
+    const int hq = h * dm.G + a, srow = qrow + row_pos;
+    row_lse = LSE[row_base(dm, sg, b) * dm.Hq + (int64_t)hq * sg.S + (srow - sg.q0)];
+    const uint4* op = reinterpret_cast<const uint4*>(O + b * dm.os[0] + hq * dm.os[1] + (int64_t)srow * dm.os[2]);
 #pragma unroll
-    for (int i = 0; i < D / 8; ++i) o_row[i] = make_uint4(0, 0, 0, 0);
-    if (r < dm.rows) {
-      const int hq = h * dm.G + r / dm.Bq, srow = qrow + r % dm.Bq;
-      row_lse = LSE[row_base(dm, sg, b) * dm.Hq + (int64_t)hq * sg.S + (srow - sg.q0)];
-      const uint4* op = reinterpret_cast<const uint4*>(O + b * dm.os[0] + hq * dm.os[1] + (int64_t)srow * dm.os[2]);
-#pragma unroll
-      for (int i = 0; i < D / 8; ++i) o_row[i] = __ldg(op + i);
-    }
+    for (int i = 0; i < D / 8; ++i) o_row[i] = __ldg(op + i);
   }
   // Octet rows of local tile j for the producers (lane < 4: octet 4 * half + lane); past the window: out of range, zeros
   const int half = warp == 7 ? 1 : 0;
@@ -158,12 +161,11 @@ k_attn_bwd_terms_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_c
       if (lane == 0) mbar_arrive_expect_tx(&sm.q_full, 2 * kQBytes);
       __syncwarp();
       if (lane < 4 * kPanels) {
-        // boxes of 64 rows x one panel, Q first, then dO; rows past the item's last one (an M-tile may hold 64 rows only) arrive as zeros
+        // boxes of 64 rows x one panel, Q first, then dO
         const int is_do = lane / (2 * kPanels), hf = lane & 1, panel = (lane >> 1) % kPanels;
-        const int r = mt * 128 + 64 * hf;
-        const bool real = r < dm.rows;
+        const int r = mt * 128 + (twice ? 0 : 64 * hf), a = r / dm.Bq;
         tma_load_5d((is_do ? sm.dO : sm.q) + panel * 16384 + hf * 8192, is_do ? &map_do : &map_q, &sm.q_full, 0,
-                    real ? qrow + r % dm.Bq : dm.rows_q, panel, h * dm.G + (real ? r / dm.Bq : 0), b);
+                    qrow + r - a * dm.Bq, panel, h * dm.G + a, b);
       }
     } else {
       const int row = local_row(0);
@@ -198,8 +200,7 @@ k_attn_bwd_terms_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_c
     int n = 0, n_a = 0;
     bool known = false;                                   // the list has been checked (warp 6) and its counts read
     auto learn = [&]() {
-      if (lane == 0) ok = bwd_wait(&sm.info_full, 0, abort);
-      ok = __shfl_sync(0xffffffffu, ok, 0);
+      ok = wait_out_of_line(&sm.info_full, 0, abort);
       far.ng = sm.n_listed; far.n_far = sm.n_far; far.first_active = sm.first_active; far.clean = sm.clean;
       counts(far.n_far, far.first_active, n, n_a);
       known = true;
@@ -211,13 +212,10 @@ k_attn_bwd_terms_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_c
       const int o = 8 * (j - n_lt) + 4 * half + (lane & 3);
       return o < far.n_far ? sg.k0 + far.row(o) : dm.rows_k;
     };
-    auto wait_for = [&](uint64_t* bar, uint32_t parity) {
-      if (lane == 0) ok = bwd_wait(bar, parity, abort);
-      ok = __shfl_sync(0xffffffffu, ok, 0);
-      return ok;
-    };
+    auto wait_for = [&](uint64_t* bar, uint32_t parity) { return ok = wait_out_of_line(bar, parity, abort); };
     auto copy_k = [&](int j, int row) {
       note_rows(j, row);
+      __syncwarp();                            // (all of them, before the arrival that publishes them)
       copy_tile(sm.k[j & 1], &map_k, &sm.k_full[j & 1], row);
     };
     // Rows of the next two tiles, looked up ahead of their use.  Tile j + 1's K has been issued when tile j is handled.
@@ -247,9 +245,7 @@ k_attn_bwd_terms_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_c
     // ------------------------------------------------------------------ MMA issuer
     // The whole warp runs this branch converged (waits included) and one elected lane issues: see mma_ss_w.
     const uint32_t lead = elect_one();
-    auto mma_wait = [&](uint64_t* bar, uint32_t parity) {
-      return __all_sync(0xffffffffu, bwd_wait(bar, parity, abort));
-    };
+    auto mma_wait = [&](uint64_t* bar, uint32_t parity) { return wait_out_of_line(bar, parity, abort); };
     constexpr uint32_t idesc_sdp = idesc_bf16_f32(128, kKT, 0, 0);       // rows x 64 keys, both K-major
     constexpr uint32_t idesc_dq = idesc_bf16_f32(128, D, 0, 1);          // dS K-major, K tile MN-major
     constexpr uint32_t idesc_dkv = idesc_bf16_f32(128, kKT, 1, 1);       // both MN-major
@@ -278,11 +274,13 @@ k_attn_bwd_terms_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_c
       issue_qk(tmem + kColDP, do_k, v_k);
       mma_commit_w(lead, &sm.dp_full);           // also tells the producers that the V tile is free
     };
-    // dV^T or dK^T: 16 query rows per MMA (2 row octets)
+    // dV^T or dK^T: 16 query rows per MMA (2 row octets), the rows once where they are there twice
     auto issue_t = [&](uint32_t acc, uint64_t amn, uint64_t term, bool accumulate) {
+#pragma unroll 1
+      for (uint32_t part = 0; part < (twice ? 1 : 2); ++part)
 #pragma unroll
-      for (int kk = 0; kk < 128 / 16; ++kk)
-        mma_ss_w(lead, acc, desc_advance(amn, kk * 2048), desc_advance(term, kk * 2048), idesc_dkv, accumulate || kk > 0);
+        for (int kk = 0; kk < 4; ++kk)
+          mma_ss_w(lead, acc, desc_advance(amn, part * 8192 + kk * 2048), desc_advance(term, part * 8192 + kk * 2048), idesc_dkv, accumulate || part > 0 || kk > 0);
     };
     bool ok = mma_wait(&sm.q_full, 0) && mma_wait(&sm.k_full[0], 0);
     HGA_TRACE_POINT(40);
@@ -369,9 +367,9 @@ k_attn_bwd_terms_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_c
   } else if (warp < 6) {
     // ------------------------------------------------------------------ one thread per query row
     const int quarter = warp & 3;
-    const int row_in_tile = quarter * 32 + lane;
-    const int r = mt * 128 + row_in_tile;
-    const int limit = w.p0 - w.ls + r % dm.Bq + 1;          // visible keys of the local tiles (causal inside the block)
+    const int row_in_tile = quarter * 32 + lane, row_of_item = row_in_tile & (twice ? 63 : 127);
+    const int c_first = twice && row_in_tile >= 64 ? 2 : 0, c_end = twice ? c_first + 2 : 4;      // its 16-key chunks of a tile
+    const int limit = w.p0 - w.ls + row_pos + 1;            // visible keys of the local tiles (causal inside the block)
     const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
     const uint32_t key7 = (uint32_t)(row_in_tile & 7);
     bool ok = __all_sync(0xffffffffu, bwd_wait(&sm.q_full, 0, abort));
@@ -400,7 +398,7 @@ k_attn_bwd_terms_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_c
     const uint64_t neg_delta_s_2 = pack_f32x2(neg_delta_s, neg_delta_s);
     const uint64_t log2e_2 = pack_f32x2(1.4426950408889634f, 1.4426950408889634f);
     const uint32_t dp_addr = lane_base + kColDP;
-    const uint32_t a_line = smem_u32(sm.a) + (uint32_t)row_in_tile * 128, b_line = smem_u32(sm.b) + (uint32_t)row_in_tile * 128;
+    const uint32_t a_line = smem_u32(sm.a) + (uint32_t)row_of_item * 128, b_line = smem_u32(sm.b) + (uint32_t)row_of_item * 128;
     // this row's 16 keys of chunk c (four to a tile) in a term's tile: two 16-byte pieces, XOR-swizzled
     auto put = [&](uint32_t line, int c, const uint32_t* w) {
 #pragma unroll
@@ -436,8 +434,14 @@ k_attn_bwd_terms_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_c
       if (!ok) break;
       tc_fence_after_sync();
       HGA_TRACE_POINT(13);
+      if (twice) {                           // (dS of the keys that the row's other thread takes)
+        const uint32_t zero[32] = {};
+        tmem_st32(dp_addr + 32 - 16 * c_first, zero);
+      }
+#pragma unroll 1
+      for (int c0 = c_first; c0 < c_end; c0 += 2)
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {          // 16 keys at a time
+      for (int c = c0; c < c0 + 2; ++c) {    // 16 keys at a time
         uint32_t sv[16], dp[16], out[16], p1[8], p2[8];
         tmem_ld16(s_addr + 16 * c, sv);
         tmem_ld16(dp_addr + 16 * c, dp);
@@ -486,8 +490,8 @@ k_attn_bwd_terms_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_c
       };
       // a term of dS from tensor memory into a tile
       auto put_ds = [&](uint32_t line, int term) {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
+#pragma unroll 1
+        for (int c = c_first; c < c_end; ++c) {
           uint32_t ds[8];
           tmem_ld8(dp_addr + 16 * c + 8 * term, ds);
           tmem_wait_ld();
@@ -497,7 +501,9 @@ k_attn_bwd_terms_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_c
       {
         uint32_t p3[32];                     // ready when the first round is over
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
+        for (int k = 0; k < 4; ++k) {
+          if (c_first + k >= c_end) break;
+          const int c = c_first + k;
           uint32_t sv[16];
           tmem_ld16(s_addr + 16 * c, sv);
           tmem_wait_ld();
@@ -507,12 +513,13 @@ k_attn_bwd_terms_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_c
             weights(16 * c + 2 * i, sv[2 * i], sv[2 * i + 1], x0, x1);
             next_term(x0, x1);
             next_term(x0, x1);
-            p3[8 * c + i] = pack_bf16(x0, x1);
+            p3[8 * k + i] = pack_bf16(x0, x1);
           }
         }
         if (!round_done()) break;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) put(a_line, c, p3 + 8 * c);
+        for (int k = 0; k < 4; ++k)
+          if (c_first + k < c_end) put(a_line, c_first + k, p3 + 8 * k);
       }
       put_ds(b_line, 0);
       hand_over_round();
@@ -599,11 +606,37 @@ k_attn_bwd_terms_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_c
       // 16-byte stores would touch 32 different sectors per instruction.  The rows go into Q's shared memory (all
       // GEMMs that read it are complete) in the swizzled [panel][128 rows][128 B] layout and leave as boxes.
       tc_fence_after_sync();
+      // the two lanes of a row meet in the terms' tiles (64 rows of 4 D bytes, 16-byte pieces XOR-swizzled)
+      const uint32_t partner = smem_u32(sm.a) + (uint32_t)row_of_item * (4 * D);
+      if (twice) {
+        if (quarter >= 2) {
+#pragma unroll 1
+          for (int c = 0; c < D / 32; ++c) {
+            uint32_t x[32];
+            tmem_ld32(lane_base + kColDQ + 32 * c, x);
+            tmem_wait_ld();
 #pragma unroll
+            for (int i = 0; i < 8; ++i) st_shared_v4(partner + 128 * c + (((uint32_t)i ^ key7) * 16), x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3]);
+          }
+        }
+        mbar_arrive_warp(&sm.staged);
+        ok = __all_sync(0xffffffffu, bwd_wait(&sm.staged, staged_phase, abort));
+      }
+      if (!twice || quarter < 2)
+#pragma unroll 1
       for (int c = 0; c < D / 32; ++c) {
         uint32_t x[32];
         tmem_ld32(lane_base + kColDQ + 32 * c, x);
         tmem_wait_ld();
+        if (twice) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            uint32_t y[4];
+            ld_shared_v4(partner + 128 * c + (((uint32_t)i ^ key7) * 16), y[0], y[1], y[2], y[3]);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) x[4 * i + e] = __float_as_uint(__uint_as_float(x[4 * i + e]) + __uint_as_float(y[e]));
+          }
+        }
         const uint32_t line = smem_u32(sm.q) + (uint32_t)(c >> 1) * 16384 + (uint32_t)row_in_tile * 128;
 #pragma unroll
         for (int i = 0; i < 4; ++i)
@@ -615,10 +648,10 @@ k_attn_bwd_terms_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_c
       }
       fence_proxy_async_smem();
       mbar_arrive_warp(&sm.dq_staged);
-      if (warp == 2 && lane < 2 * kPanels && bwd_wait(&sm.dq_staged, 0, abort)) {      // all 128 rows are in shared memory
-        const int hf = lane & 1, panel = lane >> 1, r0 = mt * 128 + 64 * hf;
+      if (warp == 2 && ok && lane < 2 * kPanels && bwd_wait(&sm.dq_staged, 0, abort)) {      // all 128 rows are in shared memory
+        const int hf = lane & 1, panel = lane >> 1, r0 = mt * 128 + 64 * hf, a = r0 / dm.Bq;
         if (r0 < dm.rows) {
-          tma_store_5d(&map_dq, sm.q + panel * 16384 + hf * 8192, 0, qrow + r0 % dm.Bq, panel, h * dm.G + r0 / dm.Bq, b);
+          tma_store_5d(&map_dq, sm.q + panel * 16384 + hf * 8192, 0, qrow + r0 - a * dm.Bq, panel, h * dm.G + a, b);
           tma_store_commit();
           tma_store_wait_read();      // (the source tile has been read; the writes complete before the grid does)
         }
