@@ -38,7 +38,10 @@
 // second ones a GEMM of their own; every warp stores the second terms, zeros elsewhere.  16K layer (needles in one block
 // of eight: 1 % of the half-tiles): error of O against fp64 2.11e-3 with one term, 1.82e-3 so, 2.06e-3 with a running
 // reference; hga_attn_fwd 39.8 -> 41.3 us (two terms everywhere: 1.66e-3, which is O's own rounding, and 43.5 us).
-// kTwoTerms kernels use them everywhere (see two_terms()).
+// kTwoTerms kernels use them everywhere (see two_terms()).  Their M-tiles of up to 64 rows have the rows TWICE, in lanes 0-63
+// and 64-127; a row's lanes take the first and the second half of every tile, against the same reference, with zeros in
+// the other half's columns, and O and the sums of the two are added in the end.  (With lanes 64-127 empty, half of the SM's
+// sub-cores did all the exponentials: 16 heads of 64 142.3 us a whole step, 138.7 so.)
 // Where that does not hold for some row of
 // the M-tile (a sum past 2^80, i.e. a logit 55 nats above the first tile's; a weight past 2^16 that took V out of the fp32
 // range; no finite logit in the first tile) the CTA goes over its keys again, twice: for the rows' true maxima, then
@@ -107,16 +110,20 @@ struct Place {
   __device__ int64_t item(const Dims& dm) const { return item_base(dm, sg, b) + h * (sg.S / dm.Bq) + qb; }
 };
 
+// Whether an M-tile's rows are there twice
+template <bool kTwoTerms>
+__device__ __forceinline__ bool rows_twice(const Dims& dm, const Place& pl) { return kTwoTerms && rows_padded(dm) - 128 * pl.mt <= 64; }
+
 // The row of a softmax thread: rows of the item are every head's Bq rows padded to whole octets (padding rows compute
 // garbage in their own TMEM lanes and are never stored)
 struct Row {
   int hw, row, r, a, t;                 // which half of every 64 keys; TMEM lane; row inside the item = (query head, token)
   bool real;
-  __device__ Row(const Dims& dm, const Place& pl, int tid) {
+  __device__ Row(const Dims& dm, const Place& pl, int tid, bool twice) {
     const int warp = tid >> 5;
     hw = (warp - 4) >> 2;
     row = (warp & 3) * 32 + (tid & 31);
-    r = pl.mt * 128 + row;
+    r = pl.mt * 128 + (twice ? row & 63 : row);
     a = r / bq_padded(dm);
     t = r % bq_padded(dm);
     real = r < rows_padded(dm) && t < dm.Bq;
@@ -131,10 +138,10 @@ __device__ __forceinline__ int again_cta() { int x; asm volatile("mov.u32 %0, %%
 // A softmax thread's half of its row of O = (accumulators) / l_mma, and LSE from l and the reference m (log2 units).  O's columns
 // (D/2)*hw .. are at head_dim 128 a panel each; rows go through Q's shared memory ([panel][128 rows][128 B], swizzled; every
 // GEMM that reads Q is complete) and leave as boxes, or are stored directly where boxes do not fit.  Returns whether
-// the accumulators are finite.
+// the accumulators are finite.  partner: the other lane's accumulators in shared memory (see share_row), 0 if there are none.
 template <int D>
 __device__ __forceinline__ bool store_row(FwdSmem<D>& sm, const Dims& dm, const Place& pl, const Row& rw, uint32_t tmem, float l, float l_mma, float m,
-                                          uint16_t* O, float* LSE) {
+                                          uint16_t* O, float* LSE, uint32_t partner = 0) {
   constexpr int kCols = D / 2;
   const bool boxes = dm.Bq % 64 == 0;
   const uint32_t lane_base = tmem + ((uint32_t)(rw.row & 96) << 16);
@@ -151,6 +158,15 @@ __device__ __forceinline__ bool store_row(FwdSmem<D>& sm, const Dims& dm, const 
     uint32_t y[32];
     tmem_ld32(lane_base + FwdSmem<D>::kColO + col, y);
     tmem_wait_ld();
+    if (partner) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        uint32_t x[4];
+        ld_shared_v4(partner + 4 * col + (((uint32_t)i ^ (uint32_t)(rw.row & 7)) * 16), x[0], x[1], x[2], x[3]);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) y[4 * i + e] = __float_as_uint(__uint_as_float(y[4 * i + e]) + __uint_as_float(x[e]));
+      }
+    }
 #pragma unroll
     for (int i = 0; i < 16; ++i)
       finite = fma_f32x2(pack_f32x2(__uint_as_float(y[2 * i]), __uint_as_float(y[2 * i + 1])), pack_f32x2(0.f, 0.f), finite);
@@ -170,6 +186,23 @@ __device__ __forceinline__ bool store_row(FwdSmem<D>& sm, const Dims& dm, const 
   return x0 + x1 == 0.f;
 }
 
+// Where a row's two lanes meet: 4 D bytes per row in V's shared memory, 16-byte pieces XOR-swizzled; the thread's half of the columns
+template <int D>
+__device__ __forceinline__ uint32_t shared_row(FwdSmem<D>& sm, const Row& rw) { return smem_u32(sm.v) + (uint32_t)(rw.row & 63) * (4 * D); }
+template <int D>
+__device__ __forceinline__ void share_row(FwdSmem<D>& sm, const Row& rw, uint32_t tmem) {
+#pragma unroll 1
+  for (int c = 0; c < D / 64; ++c) {
+    const int col = D / 2 * rw.hw + 32 * c;
+    uint32_t y[32];
+    tmem_ld32(tmem + ((uint32_t)(rw.row & 96) << 16) + FwdSmem<D>::kColO + col, y);
+    tmem_wait_ld();
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      st_shared_v4(shared_row(sm, rw) + 4 * col + (((uint32_t)i ^ (uint32_t)(rw.row & 7)) * 16), y[4 * i], y[4 * i + 1], y[4 * i + 2], y[4 * i + 3]);
+  }
+}
+
 // The staged M-tile as boxes of 64 rows x one panel (the first lanes of one warp, after every row has been staged)
 template <int D>
 __device__ __forceinline__ void store_boxes(FwdSmem<D>& sm, const Dims& dm, const Place& pl, const CUtensorMap& map_o, int lane) {
@@ -181,19 +214,20 @@ __device__ __forceinline__ void store_boxes(FwdSmem<D>& sm, const Dims& dm, cons
   }
 }
 
-// Q's rows: boxes of 64 rows x one panel, [panel][128 rows][128 B], or octets, [octet][panel][8 rows][128 B]; `lane`s of one
-// warp, bytes announced by the caller
+// Q's rows: boxes of 64 rows x one panel, [panel][128 rows][128 B], or octets, [octet][panel][8 rows][128 B], up to 64 of them
+// twice if asked for; `lane`s of one warp, bytes announced by the caller
 template <int D>
-__device__ __forceinline__ void copy_q(FwdSmem<D>& sm, const Dims& dm, const Place& pl, const CUtensorMap& map_q, uint64_t* bar, int q_oct, int lane) {
+__device__ __forceinline__ void copy_q(FwdSmem<D>& sm, const Dims& dm, const Place& pl, const CUtensorMap& map_q, uint64_t* bar, int q_oct, bool twice, int lane) {
   constexpr int kOct = 8 * D * 2, kPanels = D / 64;
   if (dm.Bq % 64 == 0) {
-    if (lane < 2 * kPanels && 8 * (lane & 1) < q_oct) {
-      const int hf = lane & 1, panel = lane >> 1, r = pl.mt * 128 + 64 * hf;
-      tma_load_5d(sm.q + panel * 16384 + hf * 8192, &map_q, bar, 0, pl.qrow + r % dm.Bq, panel, pl.h * dm.G + r / dm.Bq, pl.b);
+    if (lane < 2 * kPanels && (twice || 8 * (lane & 1) < q_oct)) {
+      const int hf = lane & 1, panel = lane >> 1, r = pl.mt * 128 + (twice ? 0 : 64 * hf), a = r / dm.Bq;
+      tma_load_5d(sm.q + panel * 16384 + hf * 8192, &map_q, bar, 0, pl.qrow + r - a * dm.Bq, panel, pl.h * dm.G + a, pl.b);
     }
-  } else if (lane < q_oct) {
-    const int bq_pad = bq_padded(dm), r = pl.mt * 128 + 8 * lane;
-    tma_load_5d(sm.q + lane * kOct, &map_q, bar, 0, pl.qrow + r % bq_pad, 0, pl.h * dm.G + r / bq_pad, pl.b);
+  } else if (lane < (twice ? 2 : 1) * q_oct) {
+    const int again = lane >= q_oct, oct = lane - again * q_oct;
+    const int bq_pad = bq_padded(dm), r = pl.mt * 128 + 8 * oct, a = r / bq_pad;
+    tma_load_5d(sm.q + (oct + 8 * again) * kOct, &map_q, bar, 0, pl.qrow + r - a * bq_pad, 0, pl.h * dm.G + a, pl.b);
   }
 }
 
@@ -215,7 +249,7 @@ __device__ __forceinline__ void passes_with_true_maxima(FwdSmem<D>& sm, const CU
   {
     const Place pl(dm, segs, again_cta());
     n_loc_oct = (pl.w.p0 + dm.Bq - pl.w.ls + 7) / 8;
-    limit = pl.w.p0 - pl.w.ls + Row(dm, pl, tid).t + 1;
+    limit = pl.w.p0 - pl.w.ls + Row(dm, pl, tid, false).t + 1;
   }
   const int n_oct = n_loc_oct + sm.n_far, n_tiles = (n_oct + 15) / 16;
 
@@ -257,7 +291,7 @@ __device__ __forceinline__ void passes_with_true_maxima(FwdSmem<D>& sm, const CU
         tma_load_5d(sm.k + lane * kOct, &map_k, &sm.again_copied, 0, krow, 0, pl.h, pl.b);
         if (sums) tma_load_5d(sm.v + lane * kOct, &map_v, &sm.again_copied, 0, krow, 0, pl.h, pl.b);
       }
-      if (step == 0) copy_q(sm, dm, pl, map_q, &sm.again_copied, q_oct, lane);       // (O may have been staged over Q)
+      if (step == 0) copy_q(sm, dm, pl, map_q, &sm.again_copied, q_oct, false, lane);       // (O may have been staged over Q)
       __syncwarp();
     }
     copied();
@@ -335,7 +369,7 @@ __device__ __forceinline__ void passes_with_true_maxima(FwdSmem<D>& sm, const CU
     tc_fence_after_sync();
     l += xchg[(hw ^ 1) * 256 + row];
     l_mma += xchg[(hw ^ 1) * 256 + 128 + row];
-    store_row(sm, dm, pl, Row(dm, pl, tid), tmem, l, l_mma, m, O, LSE);
+    store_row(sm, dm, pl, Row(dm, pl, tid, false), tmem, l, l_mma, m, O, LSE);
     fence_proxy_async_smem();
     tc_fence_before_sync();
   }
@@ -369,6 +403,7 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   // 64 rows of an M-tile are 64 rows of one head: Q and O travel in boxes of 64 rows x one panel
   const bool boxes = dm.Bq % 64 == 0;
   volatile int* abort = &sm.abort;
+  const bool twice = rows_twice<kTwoTerms>(dm, pl);
   FarList far(dm, w, group_idx + pl.item(dm) * dm.width);
   auto n_octets = [&](int n_far) { return n_loc_oct + n_far; };
 
@@ -406,9 +441,9 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     pdl_wait();
     if (warp == 3) {
       const int q_oct = min(16, rows_padded(dm) / 8 - 16 * pl.mt);   // octets of real rows in this M-tile
-      if (lane == 0) mbar_arrive_expect_tx(&sm.q_full, (uint32_t)q_oct * kOct);
+      if (lane == 0) mbar_arrive_expect_tx(&sm.q_full, (uint32_t)(twice ? 2 * q_oct : q_oct) * kOct);
       __syncwarp();
-      copy_q(sm, dm, pl, map_q, &sm.q_full, q_oct, lane);
+      copy_q(sm, dm, pl, map_q, &sm.q_full, q_oct, twice, lane);
     } else if (n_pre > 0) {
       const int row = row_of(0);
       copy_tile(sm.k, &map_k, &sm.k_full, row, true);
@@ -550,7 +585,7 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     }
   } else {
     // ------------------------------------------------------------------ softmax + epilogue
-    const Row rw(dm, pl, tid);
+    const Row rw(dm, pl, tid, twice);
     const int hw = rw.hw, row = rw.row;                 // keys 32*hw .. and 64 + 32*hw .. of every tile
     // a warp whose 32 lanes are all padding only keeps the barriers moving
     const bool warp_real = __any_sync(0xffffffffu, rw.real);
@@ -611,7 +646,11 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 #pragma unroll 1
       for (int c = 0; c < 2; ++c) {
         if (c == 1 && !whole) break;
-        if (warp_real) {
+        if (twice && c != row >> 6) {                // (the row's other lane has this half)
+          const uint32_t zero[32] = {};
+          tmem_st32(lane_base + 64 * c + 32 * hw, zero);
+          tmem_wait_st();
+        } else if (warp_real) {
           const int first = kFT * j + 64 * c + 32 * hw, lo_c = limit - first, hi_c = 8 * n_loc_oct - first, end_c = 8 * n_oct - first;
           const uint32_t s_addr = lane_base + 64 * c + 32 * hw;
           // (two copies of the code: a compare per element in the common one doubled its time)
@@ -704,7 +743,8 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // the place once more (while the last GEMM runs)
     const int tid2 = again_tid();
     const Place pl2(dm, segs, again_cta());
-    const Row rw2(dm, pl2, tid2);
+    const bool twice2 = rows_twice<kTwoTerms>(dm, pl2);
+    const Row rw2(dm, pl2, tid2, twice2);
     if (ok) ok = __all_sync(0xffffffffu, bwd_wait(&sm.o_done, 0, abort));
     HGA_TRACE_POINT(20);
     // the row's two sums meet (every GEMM has read the K tile); ok or not, every softmax thread meets here once
@@ -713,13 +753,22 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     float* const xchg = reinterpret_cast<float*>(sm.k);
     xchg[rw2.hw * 256 + rw2.row] = l;
     if constexpr (!kTwoTerms) xchg[rw2.hw * 256 + 128 + rw2.row] = l_mma;
+    if constexpr (kTwoTerms) {
+      if (twice2 && rw2.row >= 64 && ok) {
+        tc_fence_after_sync();
+        share_row(sm, rw2, tmem);
+      }
+    }
     asm volatile("bar.sync 1, 256;" ::: "memory");
     l += xchg[(rw2.hw ^ 1) * 256 + rw2.row];
+    if constexpr (kTwoTerms) {
+      if (twice2) l += xchg[rw2.row ^ 64] + xchg[256 + (rw2.row ^ 64)];
+    }
     if constexpr (!kTwoTerms) l_mma += xchg[(rw2.hw ^ 1) * 256 + 128 + rw2.row];
     else l_mma = l;                                     // (two terms leave 2^-17 of a weight: its sum needs no counterpart)
-    if (ok && __any_sync(0xffffffffu, rw2.real)) {
+    if (ok && __any_sync(0xffffffffu, rw2.real) && !(twice2 && rw2.row >= 64)) {
       tc_fence_after_sync();
-      const bool finite = store_row(sm, dm, pl2, rw2, tmem, l, l_mma, -neg_m, O, LSE);
+      const bool finite = store_row(sm, dm, pl2, rw2, tmem, l, l_mma, -neg_m, O, LSE, twice2 ? shared_row(sm, rw2) : 0);
       // (a sum that is not a number passes none of these tests)
       if (rw2.real && (l >= kSumLimit || neg_m == INFINITY || (l > kWeightLimit && !finite))) sm.again = 1;
     }
