@@ -2,6 +2,8 @@
 // its backward under segment-wise TBPTT (Section 2.2).  Forward: one warp owns one query row, a lane owns
 // d/32 consecutive elements.  Backward: one CTA owns 8 query rows of an item.  These kernels accept
 // every shape hga_params allows and serve as the cross-check of the tensor-core kernels.
+#include <atomic>
+
 #include <cfloat>
 
 #include "hga_common.cuh"
@@ -194,6 +196,8 @@ k_attn_fwd_generic(const uint16_t* __restrict__ Q, const uint16_t* __restrict__ 
 //   dQ += dS K               lane = one row, d/4 elements (registers; the warps' sums meet at the end)
 //   dV = P^T dO, dK = dS^T Q lane = one key, d/4 elements, added to global memory 16 bytes at a time (keys of the
 //                            active segment only: history keys are detached constants)
+// Where that leaves half of the device idle, a cluster of two CTAs owns the rows and each takes every other round of
+// keys; their dQ sums meet through distributed shared memory.
 // Everything is fp32.  Taken for shapes the tensor-core kernels do not cover and for problems too small to fill
 // them, so what counts is the length of one CTA's chain and how many CTAs there are; the work itself is bound by
 // shared-memory reads, 216 per 640 fused multiply-adds of a warp.
@@ -225,6 +229,24 @@ __device__ inline void fma4(float4& acc, float s, float4 x) {
 }
 __device__ inline float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 
+__device__ inline uint32_t cluster_size() {
+  uint32_t n;
+  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(n));
+  return n;
+}
+__device__ inline void cluster_meet() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+}
+// four floats at the same place in the shared memory of CTA `rank` of the cluster
+__device__ inline float4 ld4_of_rank(const float* p, uint32_t rank) {
+  uint32_t at = (uint32_t)__cvta_generic_to_shared(p);
+  float4 x;
+  asm volatile("mapa.shared::cluster.u32 %0, %0, %1;" : "+r"(at) : "r"(rank));
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(at) : "memory");
+  return x;
+}
+
 template <int D>
 __global__ void __launch_bounds__(32 * kBwdWarps)
 k_attn_bwd_generic(const uint16_t* __restrict__ Q, const uint16_t* __restrict__ K, const uint16_t* __restrict__ V,
@@ -239,7 +261,8 @@ k_attn_bwd_generic(const uint16_t* __restrict__ Q, const uint16_t* __restrict__ 
   __shared__ float s_lse[kBwdRows], s_delta[kBwdRows];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int slices = (dm.rows + kBwdRows - 1) / kBwdRows;
-  const int item = blockIdx.x / slices, r0 = (blockIdx.x % slices) * kBwdRows;
+  const int n_split = (int)cluster_size(), split = (int)blockIdx.x % n_split, slice = (int)blockIdx.x / n_split;      // (1 or 2 CTAs)
+  const int item = slice / slices, r0 = (slice % slices) * kBwdRows;
   int b, h, qb;
   item_coords(dm, item, b, h, qb);
   const Window w = window_of(dm, qb);
@@ -268,7 +291,7 @@ k_attn_bwd_generic(const uint16_t* __restrict__ Q, const uint16_t* __restrict__ 
     }
   }
   const int n_far = w.se + dm.g * build_group_list(dm, w, group_idx + (int64_t)item * dm.width, n_groups[item], vg, s_meta,
-                                                   r0 == 0 ? status_word : nullptr);   // (ends with a block barrier)
+                                                   r0 == 0 && split == 0 ? status_word : nullptr);   // (ends with a block barrier)
   const int n_tok = n_far + (w.p0 + dm.Bq - w.ls);
   const uint16_t* Kb = K + b * dm.ks[0] + h * dm.ks[1];
   const uint16_t* Vb = V + b * dm.vs[0] + h * dm.vs[1];
@@ -295,8 +318,9 @@ k_attn_bwd_generic(const uint16_t* __restrict__ Q, const uint16_t* __restrict__ 
   for (int c = 0; c < D / 16; ++c) dq[c] = make_float4(0.f, 0.f, 0.f, 0.f);
   bool waited = false;
 
-  fetch(kBwdKeys * warp);
-  for (int t0 = kBwdKeys * warp; t0 < n_tok; t0 += kBwdKeys * kBwdWarps) {
+  const int round = kBwdKeys * kBwdWarps * n_split;
+  fetch(kBwdKeys * (warp + kBwdWarps * split));
+  for (int t0 = kBwdKeys * (warp + kBwdWarps * split); t0 < n_tok; t0 += round) {
 #pragma unroll
     for (int i = 0; i < kLoads; ++i) {
       const int key = (i * 32 + lane) / kParts, part = (i * 32 + lane) % kParts;
@@ -305,7 +329,7 @@ k_attn_bwd_generic(const uint16_t* __restrict__ Q, const uint16_t* __restrict__ 
       if (part == 0) tile.tok[key] = tok[i];
     }
     __syncwarp();
-    fetch(t0 + kBwdKeys * kBwdWarps);
+    fetch(t0 + round);
     {
       float s[2] = {0.f, 0.f}, dp[2] = {0.f, 0.f};
 #pragma unroll 8
@@ -365,16 +389,23 @@ k_attn_bwd_generic(const uint16_t* __restrict__ Q, const uint16_t* __restrict__ 
   // the warps' dQ sums meet in the K tiles
 #pragma unroll
   for (int c = 0; c < D / 16; ++c) *reinterpret_cast<float4*>(&tile.k[row][16 * c + 4 * quad]) = dq[c];
-  __syncthreads();
-  if (r0 + warp < dm.rows && lane < D / 4) {
+  if (n_split > 1) cluster_meet();
+  else __syncthreads();
+  // (of a cluster every CTA writes its share of the rows)
+  if (r0 + warp < dm.rows && lane < D / 4 && warp % n_split == split) {
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int u = 0; u < kBwdWarps; ++u) fma4(a, 1.f, ld4(&sm.w[u].k[warp][4 * lane]));
+    if (n_split > 1) {
+#pragma unroll
+      for (int u = 0; u < kBwdWarps; ++u) fma4(a, 1.f, ld4_of_rank(&sm.w[u].k[warp][4 * lane], split ^ 1));
+    }
     const int r = r0 + warp, hq = h * dm.G + r / dm.Bq, sr = qb * dm.Bq + r % dm.Bq;
     Frag<4> f;
     f.v[0] = a.x; f.v[1] = a.y; f.v[2] = a.z; f.v[3] = a.w;
     store_frag_bf16<4>(dQ + b * dm.qs[0] + hq * dm.qs[1] + sr * dm.qs[2] + 4 * lane, f);
   }
+  if (n_split > 1) cluster_meet();               // (the other CTA may still be reading this one's shared memory)
 }
 
 // dK and dV to zero, one launch for both tensors (n elements each, a multiple of 8)
@@ -443,6 +474,16 @@ int launch_attn_fwd_generic(const Dims& dm, const void* Q, const void* K, const 
   return record_cuda(cudaGetLastError());
 }
 
+// SMs of the current device
+static int multiprocessors() {
+  static std::atomic<int> known[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev >= 64) return 0;
+  int n = known[dev].load(std::memory_order_relaxed);
+  if (n == 0 && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess) known[dev].store(n, std::memory_order_relaxed);
+  return n;
+}
+
 template <int D>
 static int bwd_generic(const Dims& dm, const uint16_t* Q, const uint16_t* K, const uint16_t* V,
                        const uint16_t* O, const float* LSE, const uint16_t* dO,
@@ -458,16 +499,28 @@ static int bwd_generic(const Dims& dm, const uint16_t* Q, const uint16_t* K, con
     k_zero_grads<<<(unsigned)((n4 + 255) / 256), 256, 0, st>>>((float4*)dK, (float4*)dV, n4);
     count_launch(HGA_KERNELS_BWD_GENERIC);
   }
+  // Two CTAs per eight rows where both fit the device at once and there is more than a round of keys for the second: tiny layer
+  // (64 of them, five rounds) 41.5 -> 38.2 us a whole step.
+  const int64_t slices = (int64_t)dm.B * dm.Hkv * dm.NQB * ((dm.rows + kBwdRows - 1) / kBwdRows);
+  const bool split = 2 * slices <= multiprocessors() && max_routed_tokens(dm) > kBwdKeys * kBwdWarps;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((int64_t)dm.B * dm.Hkv * dm.NQB * ((dm.rows + kBwdRows - 1) / kBwdRows)));
+  cfg.gridDim = dim3((unsigned)(split ? 2 * slices : slices));
   cfg.blockDim = dim3(32 * kBwdWarps);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr;                 // may start under the zero fill; waits for it before its first add
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = zero ? 1 : 0;
+  cudaLaunchAttribute attrs[2];
+  cfg.attrs = attrs;
+  cfg.numAttrs = 0;
+  if (zero) {                               // may start under the zero fill; waits for it before its first add
+    attrs[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attrs[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (split) {
+    attrs[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    attrs[cfg.numAttrs].val.clusterDim.x = 2;
+    attrs[cfg.numAttrs].val.clusterDim.y = attrs[cfg.numAttrs].val.clusterDim.z = 1;
+    ++cfg.numAttrs;
+  }
   const cudaError_t e = cudaLaunchKernelEx(&cfg, k_attn_bwd_generic<D>, Q, K, V, O, LSE, dO, group_idx, n_groups, dm, dQ, dK, dV,
                                            status_word);
   count_launch(HGA_KERNELS_BWD_GENERIC);
