@@ -649,18 +649,26 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         } else if (warp_real) {
           const int first = kFT * j + 64 * c + 32 * hw, lo_c = limit - first, hi_c = 8 * n_loc_oct - first, end_c = 8 * n_oct - first;
           const uint32_t s_addr = lane_base + 64 * c + 32 * hw;
-          // (two copies of the code: a compare per element in the common one doubled its time)
-          auto exponentials = [&](auto masked) {
-            // weights of keys k and k + 1 of the 32
-            auto weights = [&](int k, uint32_t x0, uint32_t x1, float& p0, float& p1) {
+          // Logits of keys that the row does not see become -inf, in a pass of its own where there are any.  (A compare per element in
+          // the common code doubled its time; a masked copy of it is that much more for the roles to fetch.)
+          const bool masked = !__all_sync(0xffffffffu, (lo_c >= 32 || hi_c <= 0) && end_c >= 32);
+          uint32_t see = 0xffffffffu;                  // bit k: key k of the 32 is visible
+          if (masked) {
+            auto below = [](int n) { return n >= 32 ? 0xffffffffu : n <= 0 ? 0u : (1u << n) - 1u; };
+            see = (below(lo_c) | ~below(hi_c)) & below(end_c);
+          }
+          auto hide = [](uint32_t bits, auto& x) {
+#pragma unroll
+            for (int i = 0; i < (int)(sizeof(x) / 4); ++i)
+              if (!((bits >> i) & 1u)) x[i] = 0xff800000u;
+          };
+          {
+            // weights of two neighbouring keys
+            auto weights = [&](uint32_t x0, uint32_t x1, float& p0, float& p1) {
               float a0, a1;
               unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(x0), __uint_as_float(x1)), sl2_2, neg_m2), a0, a1);
               p0 = fast_exp2(a0);
               p1 = fast_exp2(a1);
-              if constexpr (decltype(masked)::value) {
-                if (!((k < lo_c || k >= hi_c) && k < end_c)) p0 = 0.f;
-                if (!((k + 1 < lo_c || k + 1 >= hi_c) && k + 1 < end_c)) p1 = 0.f;
-              }
             };
             auto sum_of = [](uint32_t pk) { return pack_f32x2(__uint_as_float(pk << 16), __uint_as_float(pk & 0xffff0000u)); };
             [[maybe_unused]] bool two = kTwoTerms;
@@ -669,10 +677,11 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               uint64_t sum = pack_f32x2(0.f, 0.f);
               tmem_ld32(s_addr, x);
               tmem_wait_ld();
+              if (masked) hide(see, x);
 #pragma unroll
               for (int i = 0; i < 16; ++i) {
                 float p0, p1;
-                weights(2 * i, x[2 * i], x[2 * i + 1], p0, p1);
+                weights(x[2 * i], x[2 * i + 1], p0, p1);
                 sum = add_f32x2(sum, pack_f32x2(p0, p1));
                 pk[i] = pack_bf16(p0, p1);
                 rsum = add_f32x2(rsum, sum_of(pk[i]));
@@ -690,12 +699,13 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               }
             }
             // 16 keys with two terms each (S is fetched again rather than kept)
-            auto two_terms_of = [&](int k0, const uint32_t (&x)[16]) {
+            auto two_terms_of = [&](int k0, uint32_t (&x)[16]) {
               uint32_t out[16];
+              if (masked) hide(see >> k0, x);
 #pragma unroll
               for (int i = 0; i < 8; ++i) {
                 float p0, p1;
-                weights(k0 + 2 * i, x[2 * i], x[2 * i + 1], p0, p1);
+                weights(x[2 * i], x[2 * i + 1], p0, p1);
                 out[i] = pack_bf16(p0, p1);
                 out[8 + i] = pack_bf16(p0 - __uint_as_float(out[i] << 16), p1 - __uint_as_float(out[i] & 0xffff0000u));
                 if constexpr (kTwoTerms) lsum = add_f32x2(lsum, pack_f32x2(p0, p1));
@@ -719,9 +729,7 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                 two_terms_of(k0, x);
               }
             }
-          };
-          if (__all_sync(0xffffffffu, (lo_c >= 32 || hi_c <= 0) && end_c >= 32)) exponentials(std::false_type{});
-          else exponentials(std::true_type{});
+          }
           tmem_wait_st();
         }
         tc_fence_before_sync();
