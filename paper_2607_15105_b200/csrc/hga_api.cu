@@ -74,6 +74,7 @@ static int resolve(const hga_params* p, Dims& dm) {
   dm.flags = p->flags;
   dm.scale = p->softmax_scale > 0.f ? p->softmax_scale : 1.0f / sqrtf((float)dm.d);
   if ((int64_t)dm.B * dm.Hkv * dm.NQB > 0x7fffffff) return HGA_ERR_SHAPE;
+  dm.set_divisors();
   struct { const int64_t* in; int64_t* out; int heads, tokens; } t[4] = {
       {p->q_stride, dm.qs, dm.Hq, dm.S}, {p->k_stride, dm.ks, dm.Hkv, dm.L},
       {p->v_stride, dm.vs, dm.Hkv, dm.L}, {p->o_stride, dm.os, dm.Hq, dm.S}};

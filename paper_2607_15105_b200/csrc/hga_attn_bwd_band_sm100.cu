@@ -103,16 +103,15 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
   int cta;
   const Segment sg = segment_of(dm, segs, blockIdx.x, cta);
   const int tiles_per_seq = (sg.S + kKeys - 1) / kKeys;
-  const int kt = cta % tiles_per_seq;
-  const int bh = cta / tiles_per_seq;
-  const int h = bh % dm.Hkv, b = bh / dm.Hkv;
+  const int bh = cta / tiles_per_seq, kt = cta - bh * tiles_per_seq;
+  const int b = dm.by_Hkv(bh), h = bh - b * dm.Hkv;
   const int k0 = sg.H + kt * kKeys;               // first key position of the tile
   const int k_end = min(k0 + kKeys, sg.H + sg.S);        // one past its last real key
   // query blocks whose band [ls, p0 + Bq) touches the tile: from the block that holds the tile's first
   // key, while the local window still starts before the tile's end
-  const int qb_first = (kt * kKeys) / dm.Bq;
+  const int qb_first = dm.by_Bq(kt * kKeys);
   int n_qb = 1;
-  while (qb_first + n_qb < sg.S / dm.Bq && window_at(dm, sg.H + (qb_first + n_qb) * dm.Bq).ls < k_end) ++n_qb;
+  while (qb_first + n_qb < dm.by_Bq(sg.S) && window_at(dm, sg.H + (qb_first + n_qb) * dm.Bq).ls < k_end) ++n_qb;
   const int n_hq = dm.rows / 64;                  // half-steps of a query block
   const int n_steps = (n_qb * n_hq + 1) / 2;
   const int qb_last = qb_first + n_qb - 1;

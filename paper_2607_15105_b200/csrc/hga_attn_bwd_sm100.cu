@@ -25,7 +25,7 @@
 // Code size: the roles run side by side, and what they execute per pair and unit has to stay in the instruction caches.  The same
 // kernel with everything in line (138 KB of code, now 62) was slower than one CTA per unit: 16K layer (whole step) 161 us with
 // one CTA per unit, 185 persistent with 138 KB, 155 with 79, 147 with 62; 3 KB of unrolling more cost 2.5 us.  Hence the waits
-// by call, one copy of the code for S and dP, rolled loops wherever a role has time, and the division out of line.
+// by call, one copy of the code for S and dP and rolled loops wherever a role has time.
 //
 // What bounds it: the row threads, ~2.7k cycles per pair (1.0k of exponentials; tensor-memory loads and barrier hand-offs), a unit's
 // first pair, which waits for dO (its buffer is free only behind the last pair's dP), and a pair with dK/dV, whose place costs the K
@@ -142,15 +142,11 @@ __device__ __forceinline__ void red_add(float* to, float x) {
   asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(__cvta_generic_to_global(to)), "f"(x) : "memory");
 }
 
-// A quotient where nothing waits for it (400 bytes of code; called from the set-up of the other kernels, whose CTAs do wait for
-// it, this made the forward 2 us slower)
-__device__ __noinline__ int quotient(int a, int b) { return a / b; }
-
 // The units of a segment in launch order.  The first blocks see no routed key of the active segment: they come first, for the
 // SMs that the band kernel leaves idle, where a dK/dV addition would wait for its end.  Then late blocks first: they have the
 // most such keys, so the cheapest units are the ones that fill the last round.
 __device__ __forceinline__ int block_in_order(const Dims& dm, int i, int n_qb) {
-  const int lead = quotient(dm.local + dm.c - 1, dm.Bq) + 1;
+  const int lead = dm.by_Bq(dm.local + dm.c - 1) + 1;
   return i < lead ? i : n_qb - 1 - (i - lead);
 }
 
@@ -233,9 +229,9 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       }
       int cta;
       const Segment sg = segment_of(dm, segs, id, cta);
-      const int n_mt = dm.rows / 128, n_bh = dm.B * dm.Hkv, n_qb = quotient(sg.S, dm.Bq);
-      const int unit = quotient(cta, n_mt), mt = cta - unit * n_mt, i = quotient(unit, n_bh), bh = unit - i * n_bh;
-      const int qb = block_in_order(dm, i, n_qb), b = quotient(bh, dm.Hkv), h = bh - b * dm.Hkv;
+      const int n_mt = dm.rows / 128, n_bh = dm.B * dm.Hkv, n_qb = dm.by_Bq(sg.S);
+      const int unit = dm.by_mt(cta), mt = cta - unit * n_mt, i = dm.by_bh(unit), bh = unit - i * n_bh;
+      const int qb = block_in_order(dm, i, n_qb), b = dm.by_Hkv(bh), h = bh - b * dm.Hkv;
       const int64_t item = item_base(dm, sg, b) + h * n_qb + qb;
       const Window w = window_at(dm, sg.H + qb * dm.Bq);
       FarList far(dm, w, group_idx + item * dm.width);
@@ -252,7 +248,7 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         // (Bq is a multiple of 64: 64 rows are of one head)
 #pragma unroll 1
         for (int half = 0; half < 2; ++half) {
-          const int r = mt * 128 + 64 * half, a = quotient(r, dm.Bq), t = r - a * dm.Bq;
+          const int r = mt * 128 + 64 * half, a = dm.by_Bq(r), t = r - a * dm.Bq;
           un.head[half] = h * dm.G + a;
           un.pos[half] = t;
           un.token[half] = sg.q0 + qb * dm.Bq + t;

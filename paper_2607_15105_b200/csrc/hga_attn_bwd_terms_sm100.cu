@@ -104,8 +104,8 @@ k_attn_bwd_terms_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_c
   // expensive dK/dV tiles), early ones none, so the cheapest CTAs are the ones that fill the last wave.
   int cta;
   const Segment sg = segment_of(dm, segs, blockIdx.x, cta);
-  const int n_qb = sg.S / dm.Bq, unit = cta / n_mt_item, n_bh = dm.B * dm.Hkv, mt = cta - unit * n_mt_item;
-  const int i_qb = unit / n_bh, bh = unit - i_qb * n_bh, qb = n_qb - 1 - i_qb, b = bh / dm.Hkv, h = bh - b * dm.Hkv;
+  const int n_qb = dm.by_Bq(sg.S), unit = dm.by_mt(cta), n_bh = dm.B * dm.Hkv, mt = cta - unit * n_mt_item;
+  const int i_qb = dm.by_bh(unit), bh = unit - i_qb * n_bh, qb = n_qb - 1 - i_qb, b = dm.by_Hkv(bh), h = bh - b * dm.Hkv;
   const int64_t item = item_base(dm, sg, b) + h * n_qb + qb;
   const bool twice = dm.rows - mt * 128 == 64;          // the M-tile's rows are there twice (Bq is a multiple of 64)
   const int qrow = sg.q0 + qb * dm.Bq;                  // the block's first row in Q, O, dO and dQ
@@ -120,7 +120,7 @@ k_attn_bwd_terms_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_c
   int row_pos = 0;                                      // position inside the query block
   uint4 o_row[D / 8];
   if (warp >= 2 && warp < 6) {
-    const int r = mt * 128 + (((warp & 3) * 32 + lane) & (twice ? 63 : 127)), a = r / dm.Bq;
+    const int r = mt * 128 + (((warp & 3) * 32 + lane) & (twice ? 63 : 127)), a = dm.by_Bq(r);
     row_pos = r - a * dm.Bq;
     const int hq = h * dm.G + a, srow = qrow + row_pos;
     row_lse = LSE[row_base(dm, sg, b) * dm.Hq + (int64_t)hq * sg.S + (srow - sg.q0)];
@@ -163,7 +163,7 @@ k_attn_bwd_terms_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_c
       if (lane < 4 * kPanels) {
         // boxes of 64 rows x one panel, Q first, then dO
         const int is_do = lane / (2 * kPanels), hf = lane & 1, panel = (lane >> 1) % kPanels;
-        const int r = mt * 128 + (twice ? 0 : 64 * hf), a = r / dm.Bq;
+        const int r = mt * 128 + (twice ? 0 : 64 * hf), a = dm.by_Bq(r);
         tma_load_5d((is_do ? sm.dO : sm.q) + panel * 16384 + hf * 8192, is_do ? &map_do : &map_q, &sm.q_full, 0,
                     qrow + r - a * dm.Bq, panel, h * dm.G + a, b);
       }
@@ -649,7 +649,7 @@ k_attn_bwd_terms_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_c
       fence_proxy_async_smem();
       mbar_arrive_warp(&sm.dq_staged);
       if (warp == 2 && ok && lane < 2 * kPanels && bwd_wait(&sm.dq_staged, 0, abort)) {      // all 128 rows are in shared memory
-        const int hf = lane & 1, panel = lane >> 1, r0 = mt * 128 + 64 * hf, a = r0 / dm.Bq;
+        const int hf = lane & 1, panel = lane >> 1, r0 = mt * 128 + 64 * hf, a = dm.by_Bq(r0);
         if (r0 < dm.rows) {
           tma_store_5d(&map_dq, sm.q + panel * 16384 + hf * 8192, 0, qrow + r0 - a * dm.Bq, panel, h * dm.G + a, b);
           tma_store_commit();

@@ -127,7 +127,7 @@ k_attn_decode(const uint16_t* __restrict__ Q, const uint16_t* __restrict__ K, co
   for (int n = 0; n < NT; ++n) {
     const int r = 8 * n + g;
     const bool real = r < dm.rows;
-    const int a = real ? r / dm.Bq : 0, t = real ? r % dm.Bq : 0;
+    const int a = real ? dm.by_Bq(r) : 0, t = real ? r - a * dm.Bq : 0;
     pos[n] = w.p0 + t;
     const uint16_t* qp = Q + b * dm.qs[0] + (h * dm.G + a) * dm.qs[1] + (int64_t)(qb * dm.Bq + t) * dm.qs[2] + 8 * q;
 #pragma unroll
@@ -294,7 +294,7 @@ k_attn_decode(const uint16_t* __restrict__ Q, const uint16_t* __restrict__ K, co
     Sum a{-INFINITY, 0.f, 0.f, 0.f, 0.f};
     for (int u = 0; u < n_split; ++u) add_part(a, cluster.map_shared_rank(cst, u), cluster.map_shared_rank(so, u), r, d);
     if (r < dm.rows) {
-      const int hq = h * dm.G + r / dm.Bq, sr = qb * dm.Bq + r % dm.Bq;
+      const int head = dm.by_Bq(r), hq = h * dm.G + head, sr = qb * dm.Bq + r - head * dm.Bq;
       const float inv = 1.f / a.l_mma;
       *reinterpret_cast<uint32_t*>(O + b * dm.os[0] + hq * dm.os[1] + (int64_t)sr * dm.os[2] + d) = pack2(a.x * inv, a.y * inv);
       if (d == 0) LSE[((int64_t)b * dm.Hq + hq) * dm.S + sr] = (a.m + log2f(a.l)) * 0.6931471805599453f;

@@ -99,15 +99,15 @@ struct Place {
     const int n_mt_item = (rows_padded(dm) + 127) / 128, n_bh = dm.B * dm.Hkv;
     int cta;
     sg = segment_of(dm, segs, cta_id, cta);
-    const int unit = cta / n_mt_item;
-    mt = cta % n_mt_item;
-    qb = sg.S / dm.Bq - 1 - unit / n_bh;
-    b = unit % n_bh / dm.Hkv;
-    h = unit % n_bh % dm.Hkv;
+    const int unit = dm.by_mt(cta), i = dm.by_bh(unit), bh = unit - i * n_bh;
+    mt = cta - unit * n_mt_item;
+    qb = dm.by_Bq(sg.S) - 1 - i;
+    b = dm.by_Hkv(bh);
+    h = bh - b * dm.Hkv;
     qrow = sg.q0 + qb * dm.Bq;
     w = window_at(dm, sg.H + qb * dm.Bq);
   }
-  __device__ int64_t item(const Dims& dm) const { return item_base(dm, sg, b) + h * (sg.S / dm.Bq) + qb; }
+  __device__ int64_t item(const Dims& dm) const { return item_base(dm, sg, b) + h * dm.by_Bq(sg.S) + qb; }
 };
 
 // Whether an M-tile's rows are there twice
@@ -124,8 +124,8 @@ struct Row {
     hw = (warp - 4) >> 2;
     row = (warp & 3) * 32 + (tid & 31);
     r = pl.mt * 128 + (twice ? row & 63 : row);
-    a = r / bq_padded(dm);
-    t = r % bq_padded(dm);
+    a = dm.by_Bq_pad(r);
+    t = r - a * bq_padded(dm);
     real = r < rows_padded(dm) && t < dm.Bq;
   }
 };
@@ -206,9 +206,9 @@ __device__ __forceinline__ void share_row(FwdSmem<D>& sm, const Row& rw, uint32_
 // The staged M-tile as boxes of 64 rows x one panel (the first lanes of one warp, after every row has been staged)
 template <int D>
 __device__ __forceinline__ void store_boxes(FwdSmem<D>& sm, const Dims& dm, const Place& pl, const CUtensorMap& map_o, int lane) {
-  const int hf = lane & 1, panel = lane >> 1, r0 = pl.mt * 128 + 64 * hf;
+  const int hf = lane & 1, panel = lane >> 1, r0 = pl.mt * 128 + 64 * hf, a = dm.by_Bq(r0);
   if (lane < 2 * (D / 64) && r0 < dm.rows) {
-    tma_store_5d(&map_o, sm.q + panel * 16384 + hf * 8192, 0, pl.qrow + r0 % dm.Bq, panel, pl.h * dm.G + r0 / dm.Bq, pl.b);
+    tma_store_5d(&map_o, sm.q + panel * 16384 + hf * 8192, 0, pl.qrow + r0 - a * dm.Bq, panel, pl.h * dm.G + a, pl.b);
     tma_store_commit();
     tma_store_wait_read();      // (the source has been read; the writes complete before the grid does)
   }
@@ -221,12 +221,12 @@ __device__ __forceinline__ void copy_q(FwdSmem<D>& sm, const Dims& dm, const Pla
   constexpr int kOct = 8 * D * 2, kPanels = D / 64;
   if (dm.Bq % 64 == 0) {
     if (lane < 2 * kPanels && (twice || 8 * (lane & 1) < q_oct)) {
-      const int hf = lane & 1, panel = lane >> 1, r = pl.mt * 128 + (twice ? 0 : 64 * hf), a = r / dm.Bq;
+      const int hf = lane & 1, panel = lane >> 1, r = pl.mt * 128 + (twice ? 0 : 64 * hf), a = dm.by_Bq(r);
       tma_load_5d(sm.q + panel * 16384 + hf * 8192, &map_q, bar, 0, pl.qrow + r - a * dm.Bq, panel, pl.h * dm.G + a, pl.b);
     }
   } else if (lane < (twice ? 2 : 1) * q_oct) {
     const int again = lane >= q_oct, oct = lane - again * q_oct;
-    const int bq_pad = bq_padded(dm), r = pl.mt * 128 + 8 * oct, a = r / bq_pad;
+    const int bq_pad = bq_padded(dm), r = pl.mt * 128 + 8 * oct, a = dm.by_Bq_pad(r);
     tma_load_5d(sm.q + (oct + 8 * again) * kOct, &map_q, bar, 0, pl.qrow + r - a * bq_pad, 0, pl.h * dm.G + a, pl.b);
   }
 }

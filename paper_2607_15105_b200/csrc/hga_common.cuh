@@ -20,6 +20,22 @@ __host__ __device__ inline int score_agg_of(int flags) {
 // kernels.
 constexpr int kFlagNoPdl = 1 << 30;
 
+// Division of 0 <= n < 2^31 by a number that the host knows: three instructions on the device.  (A division by a value that the
+// compiler does not know is 25 instructions and a chain of as many steps, and a CTA has half a dozen of them ahead of its
+// first copy: whole steps, 16K layer 143.7 -> 140.4 us, 2K layer 137.6 -> 134.7, 128K 87.9 -> 86.3, walk of 16K 1062 -> 1039.)
+struct Div {
+  uint32_t by, mul, shift;
+  __host__ __device__ Div() : by(1), mul(1), shift(0) {}
+  // 2^shift the smallest power of two >= by, mul = ceil(2^32 (2^shift - by) / by) up to the + 1 that makes it exact
+  explicit Div(int d) : by((uint32_t)d), mul(1), shift(0) {
+    while ((1u << shift) < by) ++shift;
+    mul = (uint32_t)((((uint64_t)1 << 32) * (((uint64_t)1 << shift) - by)) / by + 1);
+  }
+  __host__ __device__ int operator()(int n) const {
+    return (int)(((uint32_t)(((uint64_t)mul * (uint32_t)n) >> 32) + (uint32_t)n) >> shift);
+  }
+};
+
 // Resolved problem description handed to kernels by value.
 struct Dims {
   int B, Hq, Hkv, G, d;
@@ -35,6 +51,8 @@ struct Dims {
   int flags;
   float scale;          // softmax scale
   int64_t qs[3], ks[3], vs[3], os[3];  // element strides (batch, head, token)
+  Div by_Bq, by_Bq_pad, by_c, by_g, by_Hkv, by_bh, by_mt;      // query block (and padded to octets), chunk, group, kv heads, batch * kv heads, M-tiles of an item
+  inline void set_divisors();          // from the fields above
 };
 
 // Window geometry of a query block (local start, sink end), see hga.h.
@@ -47,7 +65,7 @@ __host__ __device__ inline Window window_at(const Dims& dm, int p0) {
   Window w;
   w.p0 = p0;
   int l = w.p0 - dm.local;
-  w.ls = l <= 0 ? 0 : (l / dm.c) * dm.c;
+  w.ls = l <= 0 ? 0 : dm.by_c(l) * dm.c;
   w.se = dm.sink < w.ls ? dm.sink : w.ls;
   return w;
 }
@@ -85,7 +103,7 @@ __device__ __forceinline__ Segment segment_of(const Dims&, const SegTable& t, in
 }
 // Where a segment's routing lists (in items) and per-row outputs (in rows of one head) start for batch entry b
 __device__ __forceinline__ int64_t item_base(const Dims& dm, const Segment& sg, int b) {
-  return ((int64_t)dm.B * (sg.q0 / dm.Bq) + (int64_t)b * (sg.S / dm.Bq)) * dm.Hkv;
+  return ((int64_t)dm.B * dm.by_Bq(sg.q0) + (int64_t)b * dm.by_Bq(sg.S)) * dm.Hkv;
 }
 __device__ __forceinline__ int64_t row_base(const Dims& dm, const Segment& sg, int b) {
   return (int64_t)dm.B * sg.q0 + (int64_t)b * sg.S;
@@ -111,6 +129,11 @@ __host__ __device__ inline void item_coords(const Dims& dm, int item, int& b, in
 // generation-shaped problems (HGA_FLAG_DECODE), where bq_pad = 8 or 16 for 1..16 new tokens.
 __host__ __device__ inline int bq_padded(const Dims& dm) { return (dm.Bq + 7) & ~7; }
 __host__ __device__ inline int rows_padded(const Dims& dm) { return dm.G * bq_padded(dm); }
+
+inline void Dims::set_divisors() {
+  by_Bq = Div(Bq); by_Bq_pad = Div(bq_padded(*this)); by_c = Div(c); by_g = Div(g); by_Hkv = Div(Hkv); by_bh = Div(B * Hkv);
+  by_mt = Div((rows_padded(*this) + 127) / 128);
+}
 
 // Upper bound of routed tokens per item (sink + groups + local window + the block itself).
 __host__ __device__ inline int max_routed_tokens(const Dims& dm) {

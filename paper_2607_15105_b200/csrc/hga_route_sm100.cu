@@ -166,12 +166,12 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
   // (late query blocks first: where the history is short they have the most candidates)
   int cta;
   const Segment sg = segment_of(dm, segs, blockIdx.x, cta);
-  const int n_bh = dm.B * dm.Hkv, n_qb = sg.S / dm.Bq, i_qb = cta / n_bh, bh = cta - i_qb * n_bh;
-  const int qb = n_qb - 1 - i_qb, b = bh / dm.Hkv, h = bh - b * dm.Hkv;
+  const int n_bh = dm.B * dm.Hkv, n_qb = dm.by_Bq(sg.S), i_qb = dm.by_bh(cta), bh = cta - i_qb * n_bh;
+  const int qb = n_qb - 1 - i_qb, b = dm.by_Hkv(bh), h = bh - b * dm.Hkv;
   const int64_t item = item_base(dm, sg, b) + h * n_qb + qb;
   const Window w = window_at(dm, sg.H + qb * dm.Bq);
-  const int j0 = w.se / dm.c, n_cand = (w.ls - w.se) / dm.c;
-  const int ct0 = sg.k0 / dm.c, gs0 = sg.k0 / dm.g;          // the segment's first rows in the summary tables
+  const int j0 = dm.by_c(w.se), n_cand = dm.by_c(w.ls - w.se);
+  const int ct0 = dm.by_c(sg.k0), gs0 = dm.by_g(sg.k0);          // the segment's first rows in the summary tables
   // query rows on N: every head's Bq rows padded to whole octets (padding columns hold whatever shared memory held and
   // are masked when the columns are reduced)
   const int bq_pad = bq_padded(dm), rows_pad = rows_padded(dm);
@@ -278,13 +278,13 @@ k_route_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
         if (boxes) {
 #pragma unroll 1
           for (int i = (warp - 2) + kRtCopyWarps * lane; i < rows_pad / 64 * kPanels; i += 32 * kRtCopyWarps) {
-            const int panel = i % kPanels, r = i / kPanels * 64, a = r / dm.Bq;
+            const int panel = i % kPanels, r = i / kPanels * 64, a = dm.by_Bq(r);
             tma_load_5d(q_smem + panel * q_panel + r * 128, &map_q, &sm.q_full, 0, sg.q0 + qb * dm.Bq + r - a * dm.Bq, panel, h * dm.G + a, b);
           }
         } else {
 #pragma unroll 1
           for (int o = (warp - 2) + kRtCopyWarps * lane; o < rows_pad / 8; o += 32 * kRtCopyWarps) {
-            const int r = 8 * o, a = r / bq_pad, t = r - a * bq_pad;    // rows past the segment arrive as zeros
+            const int r = 8 * o, a = dm.by_Bq_pad(r), t = r - a * bq_pad;    // rows past the segment arrive as zeros
             tma_load_5d(q_smem + o * kOctBytes, &map_q, &sm.q_full, 0, sg.q0 + qb * dm.Bq + t, 0, h * dm.G + a, b);
           }
         }

@@ -34,9 +34,9 @@ k_build_summaries(const uint16_t* __restrict__ K, const Dims dm, int chunk_begin
   extern __shared__ double part[];            // [warps][D]: per-warp sums of the groups it handled
   int i_chunk;                                // of the segment's active range (or of the range from chunk_begin on)
   const Segment sg = segment_of(dm, segs, blockIdx.x, i_chunk);
-  const int j = chunk_begin + (chunk_begin < 0 ? 1 + (sg.k0 + sg.H) / dm.c : 0) + i_chunk;      // row in the chunk table
+  const int j = chunk_begin + (chunk_begin < 0 ? 1 + dm.by_c(sg.k0 + sg.H) : 0) + i_chunk;      // row in the chunk table
   const int bh = blockIdx.y;
-  const int b = bh / dm.Hkv, h = bh % dm.Hkv;
+  const int b = dm.by_Hkv(bh), h = bh - b * dm.Hkv;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
   const int v = lane % VEC, sub = lane / VEC;
   const uint16_t* Kb = K + b * dm.ks[0] + h * dm.ks[1] + v * 8;

@@ -45,6 +45,7 @@ int main(int argc, char** argv) {
   dm.c = 64; dm.g = 8; dm.Bq = 64; dm.kc = 16; dm.kg = 4; dm.kge = 4; dm.per = 8; dm.sink = 64; dm.local = 128;
   dm.NQB = dm.S / dm.Bq; dm.Nc = dm.L / dm.c; dm.Ng = dm.L / dm.g; dm.NcS = dm.Nc; dm.NgS = dm.Ng; dm.width = 64; dm.rows = 256; dm.flags = 0; dm.rows_q = dm.S; dm.rows_k = dm.L;
   dm.scale = 1.f / sqrtf(128.f);
+  dm.set_divisors();
   auto dense = [&](int64_t* s, int heads, int toks) { s[2] = dm.d; s[1] = (int64_t)toks * dm.d; s[0] = (int64_t)heads * toks * dm.d; };
   dense(dm.qs, dm.Hq, dm.S); dense(dm.ks, dm.Hkv, dm.L); dense(dm.vs, dm.Hkv, dm.L); dense(dm.os, dm.Hq, dm.S);
   size_t nq = (size_t)dm.Hq * dm.S * dm.d, nk = (size_t)dm.Hkv * dm.L * dm.d;
