@@ -229,6 +229,17 @@ HGA_API int hga_step_host(const hga_params* p, const void* Q_host, const void* K
                   void* stream);
 HGA_API int hga_step_arena_bytes(const hga_params* p, size_t* bytes);
 
+/* The four calls of a step on resident device tensors, one behind the other: hga_build_summaries(tok_begin, tok_end) ->
+ * hga_route -> hga_attn_fwd -> hga_attn_bwd (left out with dO == NULL), with the arguments, results and status codes of
+ * those.  As one call the library knows which kernel precedes which, and starts the copies of Q, K, V and dO of the attention
+ * kernels before the kernel ahead of them has ended. */
+HGA_API int hga_layer_step(const hga_params* p, const void* Q, const void* K, const void* V, const void* dO,
+                           int32_t tok_begin, int32_t tok_end, void* chunk_sum, void* group_sum,
+                           int32_t* chunk_idx, int32_t* group_idx, int32_t* n_groups, float* chunk_scores,
+                           float* group_scores, void* O, float* LSE, void* dQ, void* dK, void* dV,
+                           void* route_workspace, size_t route_bytes, void* bwd_workspace, size_t bwd_bytes,
+                           int32_t* status_word, void* stream);
+
 /* Section 2.2 (training walks a long sequence in fixed-size segments; the K/V of earlier
  * segments are kept as detached history, gradients never cross a segment boundary): one layer's
  * forward and backward over a WHOLE sequence, segment by segment, on device buffers.

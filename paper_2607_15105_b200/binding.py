@@ -29,7 +29,7 @@ HGA_STATUS_WAIT_TIMEOUT = 2
 HGA_ROUTE_STATIC_SCRATCH_BYTES = 4 << 20
 
 EXPORTS = ("hga_build_summaries", "hga_route", "hga_route_static", "hga_attn_fwd", "hga_attn_bwd",
-           "hga_workspace_bytes", "hga_step_host", "hga_step_arena_bytes", "hga_tbptt_walk", "hga_varlen_step",
+           "hga_workspace_bytes", "hga_layer_step", "hga_step_host", "hga_step_arena_bytes", "hga_tbptt_walk", "hga_varlen_step",
            "hga_varlen_workspace_bytes", "hga_status_string",
            "hga_version", "hga_last_cuda_error", "hga_kernel_launch_count", "hga_kernel_launch_count_by_family",
            "hga_selftest_bounded_wait")
@@ -85,6 +85,7 @@ def lib():
         L.hga_workspace_bytes.argtypes = [pp, C.POINTER(sz), C.POINTER(sz)]
         L.hga_step_arena_bytes.argtypes = [pp, C.POINTER(sz)]
         L.hga_step_host.argtypes = [pp] + [vp] * 13 + [sz, vp, vp]
+        L.hga_layer_step.argtypes = [pp, vp, vp, vp, vp, i32, i32] + [vp] * 13 + [sz, vp, sz, vp, vp]
         L.hga_tbptt_walk.argtypes = [pp] + [vp] * 15 + [sz, vp, vp]
         L.hga_varlen_step.argtypes = [pp, C.c_int32] + [vp] * 17 + [sz, vp, vp]
         L.hga_varlen_workspace_bytes.argtypes = [pp, C.c_int32, vp, vp, C.POINTER(sz)]
@@ -217,6 +218,16 @@ def hga_attn_bwd(p, Q, K, V, O, LSE, dO, group_idx, n_groups, dQ, dK, dV, worksp
         _stream(stream)))
 
 
+def hga_layer_step(p, Q, K, V, dO, tok_begin, tok_end, chunk_sum, group_sum, chunk_idx, group_idx, n_groups,
+                   chunk_scores, group_scores, O, LSE, dQ, dK, dV, route_workspace, bwd_workspace, status_word=None, stream=None):
+    """The four calls of a step in one (dO None: without the backward; see hga.h)."""
+    _check("hga_layer_step", lib().hga_layer_step(
+        C.byref(p), _ptr(Q), _ptr(K), _ptr(V), _ptr(dO), tok_begin, tok_end, _ptr(chunk_sum), _ptr(group_sum), _ptr(chunk_idx),
+        _ptr(group_idx), _ptr(n_groups), _ptr(chunk_scores), _ptr(group_scores), _ptr(O), _ptr(LSE), _ptr(dQ), _ptr(dK), _ptr(dV),
+        _ptr(route_workspace), _nbytes(route_workspace), _ptr(bwd_workspace), _nbytes(bwd_workspace), _ptr(status_word),
+        _stream(stream)))
+
+
 def hga_step_host(p, Q_host, Kseg_host, Vseg_host, dO_host, K_dev, V_dev, chunk_sum, group_sum,
                   O_host, dQ_host, dK_host, dV_host, arena, status_word=None, stream=None):
     """Host tensors are CPU (ideally pinned) torch tensors; *_dev / summaries / arena are CUDA."""
@@ -320,8 +331,7 @@ class HgaLayerBuffers:
 
     def step(self, Q, K, V, dO=None, stream=None):
         """One pass of the whole hot path over resident device tensors."""
-        self.build_summaries(K, stream=stream)
-        self.route(Q, stream)
-        self.attn_fwd(Q, K, V, stream=stream)
-        if dO is not None:
-            self.attn_bwd(Q, K, V, dO, stream=stream)
+        bwd = (self.dQ, self.dK, self.dV, self.bwd_ws) if dO is not None else (None,) * 4
+        hga_layer_step(self.p, Q, K, V, dO, self.cfg.total_len - self.cfg.seg_len, self.cfg.total_len, self.chunk_sum, self.group_sum,
+                       self.chunk_idx, self.group_idx, self.n_groups, self.chunk_scores, self.group_scores, self.O, self.LSE,
+                       *bwd[:3], self.route_ws, bwd[3], self.status, stream)

@@ -56,7 +56,7 @@ static int resolve(const hga_params* p, Dims& dm) {
   if (p->chunk / p->group > 64) return HGA_ERR_UNSUPPORTED;
   if (p->topk_chunks > 1024) return HGA_ERR_UNSUPPORTED;
   if ((p->flags & HGA_FLAG_SCORE_MEAN) && (p->flags & HGA_FLAG_SCORE_LSE)) return HGA_ERR_UNSUPPORTED;
-  if (p->flags & ~0x7f & ~(t_internal_flags ? kFlagNoPdl : 0)) return HGA_ERR_UNSUPPORTED;   // unknown flag bits
+  if (p->flags & ~0x7f & ~(t_internal_flags ? kFlagNoPdl | kFlagChained : 0)) return HGA_ERR_UNSUPPORTED;   // unknown flag bits
   if ((p->flags & HGA_FLAG_GLOBAL_GROUP_BUDGET) && (int64_t)p->topk_chunks * (p->chunk / p->group) > 4096)
     return HGA_ERR_UNSUPPORTED;
   dm.B = p->batch; dm.Hq = p->n_q_heads; dm.Hkv = p->n_kv_heads; dm.G = dm.Hq / dm.Hkv;
@@ -132,11 +132,12 @@ static bool segments_supported(const Dims& dm, const std::vector<Segment>& segs,
 // backward was queued too (it is not where its kernels have no room for the widest item).  HGA_ERR_UNSUPPORTED: the routing or
 // the forward of these tensors is not for the tensor-core kernels after all (a stride that no tensor map takes), the same for
 // every group of segments; the caller goes on segment by segment, which repeats what has been queued.
-static int run_segments(const Dims& dm, std::vector<Segment> segs, bool summaries, const void* Q, const void* K, const void* V,
+static int run_segments(Dims dm, std::vector<Segment> segs, bool summaries, const void* Q, const void* K, const void* V,
                         const void* dO, void* chunk_sum, void* group_sum, int32_t* chunk_idx, int32_t* group_idx, int32_t* n_groups,
                         void* O, float* LSE, void* dQ, float* dK, float* dV, int32_t* status_word, cudaStream_t st, bool* bwd_done) {
   std::stable_sort(segs.begin(), segs.end(), [](const Segment& a, const Segment& b) { return a.H + a.S > b.H + b.S; });
   *bwd_done = dO != nullptr;
+  dm.flags |= kFlagChained;
   for (size_t i = 0; i < segs.size(); i += kMaxSegments) {
     SegTable t;
     t.n = (int)std::min<size_t>(kMaxSegments, segs.size() - i);
@@ -322,6 +323,24 @@ int hga_attn_bwd(const hga_params* p, const void* Q, const void* K, const void* 
     rc = launch_attn_bwd_generic(dm, Q, K, V, O, LSE, dO, group_idx, n_groups, dQ, dK, dV, status_word, st);
   if (rc || !bf16_grads) return rc;
   return launch_grads_to_bf16(dK, dK_out, dV_out, n_kv, tensor_path && !(dm.flags & kFlagNoPdl), st);
+}
+
+int hga_layer_step(const hga_params* p, const void* Q, const void* K, const void* V, const void* dO, int32_t tok_begin,
+                   int32_t tok_end, void* chunk_sum, void* group_sum, int32_t* chunk_idx, int32_t* group_idx, int32_t* n_groups,
+                   float* chunk_scores, float* group_scores, void* O, float* LSE, void* dQ, void* dK, void* dV,
+                   void* route_workspace, size_t route_bytes, void* bwd_workspace, size_t bwd_bytes, int32_t* status_word,
+                   void* stream) {
+  int rc = hga_build_summaries(p, K, tok_begin, tok_end, chunk_sum, group_sum, stream);
+  if (rc) return rc;
+  rc = hga_route(p, Q, chunk_sum, group_sum, chunk_idx, group_idx, n_groups, chunk_scores, group_scores, route_workspace, route_bytes, stream);
+  if (rc) return rc;
+  if (p->flags & ~0x7f) return HGA_ERR_UNSUPPORTED;
+  hga_params pc = *p;
+  pc.flags |= kFlagChained;
+  InternalFlagsScope internal;                       // lets the calls below accept that bit
+  rc = hga_attn_fwd(&pc, Q, K, V, group_idx, n_groups, O, LSE, status_word, stream);
+  if (rc || !dO) return rc;
+  return hga_attn_bwd(&pc, Q, K, V, O, LSE, dO, group_idx, n_groups, dQ, dK, dV, bwd_workspace, bwd_bytes, status_word, stream);
 }
 
 int hga_step_arena_bytes(const hga_params* p, size_t* bytes) {

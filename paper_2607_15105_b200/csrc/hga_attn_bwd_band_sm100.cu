@@ -142,7 +142,8 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
-  pdl_wait();
+  const bool chained = dm.flags & kFlagChained;      // (then only O and LSE come from the kernel before)
+  if (!chained || warp < 2) pdl_wait();
   // the sweep, next in the stream, may start on SMs this grid leaves idle (it waits for this grid only
   // before it adds to dK/dV; what it reads earlier was complete when this grid's wait returned)
   if (tid == 0) pdl_launch_dependents();
@@ -191,11 +192,15 @@ k_attn_bwd_band_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_co
       const int grp = i / n, k = i % n;
       if (grp < 2) copy_kv(grp == 0 ? sm.k : sm.v, grp == 0 ? &map_k : &map_v, k);
       else if (grp < 4) copy_qdo(grp == 2 ? first[0] : first[1], 0, grp - 2, k);
-      else if (grp == 4) copy_o(first[0], first[1], k);
+      else if (grp == 4) {
+        if (chained) pdl_wait();
+        copy_o(first[0], first[1], k);
+      }
       else copy_qdo(grp == 5 ? first[2] : first[3], 1, grp - 5, k);
     }
   }
   __syncwarp();
+  if (chained) pdl_wait();
 
   if (warp == 0) {
     // ------------------------------------------------------------------ producer (Q and dO from the third step on)

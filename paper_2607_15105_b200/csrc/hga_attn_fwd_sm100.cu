@@ -438,7 +438,8 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // Q and a first tile of local octets do not depend on the routing: their copies start before the CTA meets.  Barrier 2
     // makes the mbarrier initialisation above visible to the issuing warps.
     asm volatile("bar.sync 2, 96;" ::: "memory");
-    pdl_wait();
+    const bool chained = dm.flags & kFlagChained;
+    if (!chained) pdl_wait();
     if (warp == 3) {
       const int q_oct = min(16, rows_padded(dm) / 8 - 16 * pl.mt);   // octets of real rows in this M-tile
       if (lane == 0) mbar_arrive_expect_tx(&sm.q_full, (uint32_t)(twice ? 2 * q_oct : q_oct) * kOct);
@@ -450,6 +451,7 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       copy_tile(sm.v, &map_v, &sm.v_full, row, true);
     }
     __syncwarp();
+    if (chained) pdl_wait();                       // (the routing list)
   }
   if (warp == 1) {
     tmem_alloc(&sm.tmem_base, kTmemCols);
