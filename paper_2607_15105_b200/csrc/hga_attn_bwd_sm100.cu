@@ -740,8 +740,8 @@ bool attn_bwd_sm100_supported(const Dims& dm) {
   if (dm.flags & HGA_FLAG_GENERIC_KERNELS) return false;
   if (dm.g % 8 != 0 || !attn_bwd_band_sm100_supported(dm)) return false;
   // The smallest layers of head_dim 64 (fewer than eight M-tiles, few keys) keep the CUDA-core kernel, whose dV is 1.2e-7 closer
-  // to fp64, for some microseconds: 4 tiles of 320 keys 20.8 us, 14.6 here.  Its time grows with the keys faster than this
-  // path's: 704 keys 35 us, 24 here; 2240 keys 92, 63; 4288 keys 167, 116 (1 to 8 tiles alike on both sides).
+  // to fp64, for two microseconds: 4 tiles of 320 keys 16.4 us, 14.5 here.  Its time grows with the keys faster than this path's
+  // (one CTA per eight rows: 704 keys 35 us, 24 here; 2240 keys 92, 63; 4288 keys 167, 116; 1 to 8 tiles alike on both sides).
   if (dm.d == 64 && dm.B * dm.Hkv * dm.NQB * ((dm.rows + 127) / 128) < 8 && max_routed_tokens(dm) <= 512) return false;
   return true;
 }

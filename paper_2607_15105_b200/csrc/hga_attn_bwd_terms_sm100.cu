@@ -8,8 +8,8 @@
 // against fp64 (head_dim 64, 64 rows; relative, dQ / dK / dV): 1.68e-3 / 1.33e-4 / 5.0e-7, on CUDA cores 1.68e-3 / 1.33e-4 /
 // 3.8e-7 (the tensor pipe cuts S and its sums off at 2^-24), with one term 2.9e-3 / 2.1e-3 / 1.6e-3; at head_dim 128 dV
 // is off by 0.8e-6 to 1.8e-6 (see k_attn_bwd_band_sm100 for why not less).
-// hga_attn_bwd, 16 heads of 64 rows, 512 items of 768 keys: head_dim 64 98 us (one term 68, CUDA cores 918), head_dim 128
-// 160 us (99, 1970).  What bounds it: the row threads, with twice the instructions per weight, and the hand-offs.
+// hga_attn_bwd, 16 heads of 64 rows, 512 items of 768 keys: head_dim 64 71 us (CUDA cores 918), head_dim 128 128 us (1970).
+// What bounds it: the row threads, with twice the instructions per weight, and the hand-offs.
 //
 // Work unit (one CTA): one 128-row M-tile of one item (b, kv head, query block), swept over the item's routed
 // keys in 64-key tiles (eight octets of 8 consecutive tokens, one TMA box each).  At head_dim 64 a CTA takes less than

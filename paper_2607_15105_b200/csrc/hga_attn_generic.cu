@@ -408,10 +408,12 @@ k_attn_bwd_generic(const uint16_t* __restrict__ Q, const uint16_t* __restrict__ 
   if (n_split > 1) cluster_meet();               // (the other CTA may still be reading this one's shared memory)
 }
 
-// dK and dV to zero, one launch for both tensors (n elements each, a multiple of 8)
+// dK and dV to zero, one launch for both tensors (n elements each, a multiple of 8).  It waits for what is before it ahead of
+// releasing the backward, which reads the forward's results at once.
 __global__ void __launch_bounds__(256) k_zero_grads(float4* __restrict__ a, float4* __restrict__ b, size_t n4) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (i < n4) a[i] = b[i] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
@@ -496,7 +498,10 @@ static int bwd_generic(const Dims& dm, const uint16_t* Q, const uint16_t* K, con
   const bool zero = !(dm.flags & HGA_FLAG_BWD_ACCUMULATE);
   if (zero) {
     const size_t n4 = (size_t)dm.B * dm.Hkv * dm.S * D / 4;
-    k_zero_grads<<<(unsigned)((n4 + 255) / 256), 256, 0, st>>>((float4*)dK, (float4*)dV, n4);
+    // (set up under the forward's end, like the tensor-core kernels: tiny layer 35.0 -> 34.1 us a whole step)
+    PdlLaunch fill(dim3((unsigned)((n4 + 255) / 256)), 256, 0, st, dm.flags);
+    const cudaError_t e = cudaLaunchKernelEx(&fill.c, k_zero_grads, (float4*)dK, (float4*)dV, n4);
+    if (e != cudaSuccess) return record_cuda(e);
     count_launch(HGA_KERNELS_BWD_GENERIC);
   }
   // Two CTAs per eight rows where both fit the device at once and there is more than a round of keys for the second: tiny layer
