@@ -183,8 +183,11 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     }
     mbar_init(&sm.plan, 1); mbar_init(&sm.cancel_full, 1);
     mbar_init(&sm.q_full, 1); mbar_init(&sm.do_full, 1);
-    mbar_init(&sm.q_empty, 2);                    // S of the last pair, and the dK GEMMs
-    mbar_init(&sm.do_empty, 6);                   // dP of the last pair, the dV GEMMs, and the four statistics warps
+    // S (dP) of the last pair and the dK (dV) GEMMs; of dO also the four statistics warps.  Both issuing warps arrive by commits
+    // only, the second one for units without dK/dV too: a commit stands behind all GEMMs that its warp has issued, so it cannot
+    // be counted for the unit before while that unit's dK and dV still read Q and dO, as a plain arrival could.
+    mbar_init(&sm.q_empty, 2);
+    mbar_init(&sm.do_empty, 6);
     for (int s = 0; s < kKStages; ++s) { mbar_init(&sm.k_full[s], 2); mbar_init(&sm.k_empty[s], 1); }
     for (int s = 0; s < kVStages; ++s) { mbar_init(&sm.v_full[s], 2); mbar_init(&sm.v_empty[s], 1); }
     mbar_init(&sm.lse_full, 4); mbar_init(&sm.stat_full, 4); mbar_init(&sm.stat_empty, 8);
@@ -414,8 +417,7 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       if (n_pairs == 0) break;
       const Pairs pairs(un);
       done_with_info(n);
-      if (pairs.n_a == 0 && lane == 0) { mbar_arrive(&sm.q_empty); mbar_arrive(&sm.do_empty); }
-      __syncwarp();
+      if (pairs.n_a == 0) { mma_commit_w(lead, &sm.q_empty); mma_commit_w(lead, &sm.do_empty); }
       for (int u = 0; u < n_pairs; ++u, ++U) {
         if (!wait_by_call(&sm.ds_full[U & 1], U >> 1) || (u == 0 && n > 0 && !wait_by_call(&sm.dq_free, n - 1))) break;
         tc_fence_after_sync();
