@@ -232,7 +232,8 @@ HGA_API int hga_step_arena_bytes(const hga_params* p, size_t* bytes);
 /* The four calls of a step on resident device tensors, one behind the other: hga_build_summaries(tok_begin, tok_end) ->
  * hga_route -> hga_attn_fwd -> hga_attn_bwd (left out with dO == NULL), with the arguments, results and status codes of
  * those.  As one call the library knows which kernel precedes which, and starts the copies of Q, K, V and dO of the attention
- * kernels before the kernel ahead of them has ended. */
+ * kernels before the kernel ahead of them has ended.  dO may be O (the gradient of |O|^2 / 2), here and in hga_tbptt_walk and
+ * hga_varlen_step: those copies then wait for the forward's end. */
 HGA_API int hga_layer_step(const hga_params* p, const void* Q, const void* K, const void* V, const void* dO,
                            int32_t tok_begin, int32_t tok_end, void* chunk_sum, void* group_sum,
                            int32_t* chunk_idx, int32_t* group_idx, int32_t* n_groups, float* chunk_scores,

@@ -785,10 +785,22 @@ static int launch_sweep(const Dims& dm, SegTable* table, const Segs& segs, int64
   return record_cuda(e);
 }
 
-int launch_attn_bwd_sm100(const Dims& dm, SegTable* segs, const void* Q, const void* K, const void* V, const void* O,
+// Whether two bf16 tensors of query rows (strides as in Dims) may share bytes: the spans between their first and last elements meet
+static bool rows_meet(const Dims& dm, const void* a, const int64_t* sa, const void* b, const int64_t* sb) {
+  auto last = [&](const void* p, const int64_t* s) {
+    return (uintptr_t)p + 2 * (uintptr_t)((dm.B - 1) * s[0] + (dm.Hq - 1) * s[1] + (dm.rows_q - 1) * s[2] + dm.d - 1);
+  };
+  return (uintptr_t)a <= last(b, sb) && (uintptr_t)b <= last(a, sa);
+}
+
+int launch_attn_bwd_sm100(const Dims& given, SegTable* segs, const void* Q, const void* K, const void* V, const void* O,
                           const float* LSE, const void* dO, const int32_t* group_idx,
                           const int32_t* n_groups, void* dQ, float* dK, float* dV, int32_t* status_word,
                           cudaStream_t st) {
+  Dims dm = given;
+  // Inside a step the band kernel copies Q and dO while the forward still stores O: not where O is one of them (the gradient of
+  // |O|^2 / 2 is O).
+  if (rows_meet(dm, O, dm.os, dO, dm.os) || rows_meet(dm, O, dm.os, Q, dm.qs)) dm.flags &= ~kFlagChained;
   if (bwd_in_terms(dm))
     return launch_attn_bwd_terms_sm100(dm, segs, Q, K, V, O, LSE, dO, group_idx, n_groups, dQ, dK, dV, status_word, st);
   const int64_t units = (int64_t)dm.B * dm.Hkv * dm.NQB * (dm.rows / 128);

@@ -38,7 +38,8 @@ struct Div {
 
 // Internal flag: the kernel's predecessor in the stream is the one of this library that precedes it in a step.  That kernel has
 // waited for everything before it ahead of letting this one start, and writes neither Q, K, V nor dO: their copies need not wait
-// for its end.  (Behind a caller's kernel, which may let its successor start before it has written them, they do.)
+// for its end.  (Behind a caller's kernel, which may let its successor start before it has written them, they do.  The backward takes
+// the flag back where the caller has O, which the forward does write, share bytes with Q or dO.)
 constexpr int kFlagChained = 1 << 29;
 
 // Resolved problem description handed to kernels by value.

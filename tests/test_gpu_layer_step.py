@@ -71,3 +71,65 @@ def test_step_refuses_what_its_calls_refuse():
     buf.route_ws = buf.route_ws[:8]
     with pytest.raises(binding.HgaError):
         buf.step(x["Q"], x["K"], x["V"], x["dO"])
+
+
+HEADS = {"d128": dict(n_q_heads=32, n_kv_heads=8), "d64_rows64": dict(head_dim=64, n_q_heads=16, n_kv_heads=16)}
+
+
+def outputs(cfg):
+    """Tensors of a whole sequence of one row (walk, or step where it is one segment) or of packed documents."""
+    Hq, Hkv, d, n = cfg.n_q_heads, cfg.n_kv_heads, cfg.head_dim, cfg.total_len
+    z = lambda *s, dt=torch.bfloat16: torch.zeros(*s, dtype=dt, device="cuda")
+    items = Hkv * n // cfg.q_block
+    return dict(cs=z(Hkv, n // cfg.chunk, d), gs=z(Hkv, n // cfg.group, d), ci=z(items, cfg.topk_chunks, dt=torch.int32),
+                gi=z(items, cfg.topk_chunks * cfg.kg_eff, dt=torch.int32), ng=z(items, dt=torch.int32), O=z(Hq * n * d).fill_(3.0),
+                LSE=z(Hq * n, dt=torch.float32), dQ=z(Hq * n * d), dK=z(Hkv * n * d, dt=torch.float32), dV=z(Hkv * n * d, dt=torch.float32))
+
+
+def one_call(kind, cfg, x, o, dO, status, flags=0):
+    """The step, the walk in segments of a third, or three packed documents of a third each: no history, dO may be None."""
+    n, third = cfg.total_len, cfg.total_len // 3
+    args = [x["Q"], x["K"], x["V"], dO] + [o[k] for k in ("cs", "gs", "ci", "gi", "ng", "O", "LSE", "dQ", "dK", "dV")]
+    if kind == "step":
+        p = binding.make_params(cfg, flags=flags)
+        w1, w2 = (torch.empty(b, dtype=torch.uint8, device="cuda") for b in binding.hga_workspace_bytes(p))
+        binding.hga_layer_step(p, *args[:4], 0, n, *args[4:9], None, None, *args[9:], w1, w2, status)
+    elif kind == "walk":
+        p = binding.make_params(cfg.scaled(seg_len=third), flags=flags)
+        binding.hga_tbptt_walk(p, *args, torch.empty(sum(binding.hga_workspace_bytes(p)) + 512, dtype=torch.uint8, device="cuda"), status)
+    else:
+        cu = [0, third, 2 * third, n]
+        p = binding.make_params(cfg, flags=flags)
+        binding.hga_varlen_step(p, cu, cu, *args, torch.empty(binding.hga_varlen_workspace_bytes(p, cu, cu), dtype=torch.uint8, device="cuda"), status)
+
+
+def random_inputs(cfg, seed):
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    draw = lambda h: torch.randn(h * cfg.total_len * cfg.head_dim, generator=gen, device="cuda").to(torch.bfloat16)
+    return dict(Q=draw(cfg.n_q_heads), K=draw(cfg.n_kv_heads), V=draw(cfg.n_kv_heads), dO=draw(cfg.n_q_heads))
+
+
+def check_equal(a, b, keys):
+    for k in keys:
+        if k in ("dK", "dV"):                # up to the order of their fp32 adds
+            assert float((a[k] - b[k]).norm()) <= 1e-5 * float(b[k].norm()), k
+        else:
+            assert torch.equal(a[k], b[k]), k
+
+
+@pytest.mark.parametrize("heads", list(HEADS))
+@pytest.mark.parametrize("kind", ["step", "walk", "packed"])
+def test_the_gradient_may_be_the_output(kind, heads):
+    """dO is O (the gradient of |O|^2 / 2), against a call with a copy of that O as dO."""
+    cfg = cfg_of(total_len=3072, seg_len=3072, **HEADS[heads])
+    x, status = random_inputs(cfg, 5), torch.zeros(1, dtype=torch.int32, device="cuda")
+    ref, got = outputs(cfg), outputs(cfg)
+    one_call(kind, cfg, x, ref, None, status)
+    torch.cuda.synchronize()
+    one_call(kind, cfg, x, ref, ref["O"].clone(), status)
+    for _ in range(3):
+        got["O"].fill_(3.0)
+        one_call(kind, cfg, x, got, got["O"], status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        check_equal(got, ref, ("gi", "ng", "O", "LSE", "dQ", "dK", "dV"))
