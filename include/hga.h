@@ -194,7 +194,8 @@ HGA_API int hga_attn_fwd(const hga_params* p, const void* Q, const void* K, cons
  * (Section 2.2: history K/V is detached at the segment boundary, so no gradient reaches an
  * earlier segment): writes dQ for all S rows and dK/dV for the
  * S active rows only; history keys contribute to dQ but receive no gradient.
- * O and LSE are hga_attn_fwd's outputs, dO the upstream gradient (layout of O).
+ * O and LSE are hga_attn_fwd's outputs, dO the upstream gradient (layout of O).  dQ may take the place of Q, dO or O (same
+ * strides: a row is stored when it has been read for the last time).
  * dK/dV are fp32 [B,Hkv,S,d] (bf16 with HGA_FLAG_BWD_BF16_GRADS) and are overwritten unless
  * HGA_FLAG_BWD_ACCUMULATE is set.  The sum over query blocks
  * uses floating-point atomics: results may differ in the last bits from run to run.  At head_dim 128 and whole 128-row

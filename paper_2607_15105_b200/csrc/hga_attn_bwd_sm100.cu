@@ -801,6 +801,9 @@ int launch_attn_bwd_sm100(const Dims& given, SegTable* segs, const void* Q, cons
   // Inside a step the band kernel copies Q and dO while the forward still stores O: not where O is one of them (the gradient of
   // |O|^2 / 2 is O).
   if (rows_meet(dm, O, dm.os, dO, dm.os) || rows_meet(dm, O, dm.os, Q, dm.qs)) dm.flags &= ~kFlagChained;
+  // The sweep stores dQ while the band kernel may still read other key tiles' share of the same rows of Q, dO and O: where dQ is
+  // one of those, it starts behind the band kernel's end.
+  if (rows_meet(dm, dQ, dm.qs, Q, dm.qs) || rows_meet(dm, dQ, dm.qs, dO, dm.os) || rows_meet(dm, dQ, dm.qs, O, dm.os)) dm.flags |= kFlagNoPdl;
   if (bwd_in_terms(dm))
     return launch_attn_bwd_terms_sm100(dm, segs, Q, K, V, O, LSE, dO, group_idx, n_groups, dQ, dK, dV, status_word, st);
   const int64_t units = (int64_t)dm.B * dm.Hkv * dm.NQB * (dm.rows / 128);

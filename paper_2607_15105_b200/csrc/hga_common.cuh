@@ -17,7 +17,7 @@ __host__ __device__ inline int score_agg_of(int flags) {
 // Internal flag (a bit of Dims.flags that hga.h does not define and the exported calls reject): launch
 // the backward's kernels without programmatic serialization.  Set by hga_step_host, whose steps are bound
 // by the host link: there the early-started CTAs only get in the way of the next (batch, kv head) pair's
-// kernels.
+// kernels; and where dQ takes the place of Q, dO or O.
 constexpr int kFlagNoPdl = 1 << 30;
 
 // Division of 0 <= n < 2^31 by a number that the host knows: three instructions on the device.  (A division by a value that the

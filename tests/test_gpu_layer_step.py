@@ -133,3 +133,29 @@ def test_the_gradient_may_be_the_output(kind, heads):
         torch.cuda.synchronize()
         assert int(status.item()) == 0
         check_equal(got, ref, ("gi", "ng", "O", "LSE", "dQ", "dK", "dV"))
+
+
+@pytest.mark.parametrize("heads", list(HEADS))
+@pytest.mark.parametrize("over", ["Q", "dO", "O"])
+@pytest.mark.parametrize("kind", ["bwd", "step", "walk", "packed"])
+def test_dq_may_take_the_place_of_an_input(kind, over, heads):
+    """dQ in the buffer of Q, dO or O, by hga_attn_bwd itself and by the calls that make it, against buffers of its own."""
+    cfg = cfg_of(total_len=3072, seg_len=3072, **HEADS[heads])
+    x, status = random_inputs(cfg, 6), torch.zeros(1, dtype=torch.int32, device="cuda")
+    ref = outputs(cfg)
+    one_call("step" if kind == "bwd" else kind, cfg, x, ref, x["dO"], status)
+    torch.cuda.synchronize()
+    for _ in range(3):
+        got, y = outputs(cfg), {k: v.clone() for k, v in x.items()}
+        if kind == "bwd":
+            one_call("step", cfg, y, got, None, status)
+        got["dQ"] = got["O"] if over == "O" else y[over]
+        if kind == "bwd":
+            p = binding.make_params(cfg)
+            ws = torch.empty(binding.hga_workspace_bytes(p)[1], dtype=torch.uint8, device="cuda")
+            binding.hga_attn_bwd(p, y["Q"], y["K"], y["V"], got["O"], got["LSE"], y["dO"], got["gi"], got["ng"], got["dQ"], got["dK"], got["dV"], ws, status)
+        else:
+            one_call(kind, cfg, y, got, y["dO"], status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        check_equal(got, ref, ("gi", "ng", "LSE", "dQ", "dK", "dV"))
