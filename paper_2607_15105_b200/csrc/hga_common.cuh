@@ -26,8 +26,9 @@ constexpr int kFlagNoPdl = 1 << 30;
 struct Div {
   uint32_t by, mul, shift;
   __host__ __device__ Div() : by(1), mul(1), shift(0) {}
-  // 2^shift the smallest power of two >= by, mul = ceil(2^32 (2^shift - by) / by) up to the + 1 that makes it exact
-  explicit Div(int d) : by((uint32_t)d), mul(1), shift(0) {
+  // 2^shift the smallest power of two >= by, mul = ceil(2^32 (2^shift - by) / by) up to the + 1 that makes it exact.  (d < 1 comes
+  // from products that overflow, of sizes that no tensor can have but a size query may: any divisor does.)
+  explicit Div(int d) : by(d > 0 ? (uint32_t)d : 1), mul(1), shift(0) {
     while ((1u << shift) < by) ++shift;
     mul = (uint32_t)((((uint64_t)1 << 32) * (((uint64_t)1 << shift) - by)) / by + 1);
   }

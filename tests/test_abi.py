@@ -134,6 +134,15 @@ def test_workspace_sizes_follow_their_formulas(lib):
     assert rc == 0 and b2 == b + 2 * cfg.batch * cfg.n_kv_heads * cfg.seg_len * cfg.head_dim * 4
 
 
+@pytest.mark.parametrize("n_q,q_block,flags", [(65536, 65536, 0), (40000, 65536, 0), (2, 2 ** 31 - 64, 0), (1, 2 ** 31 - 1, binding.HGA_FLAG_DECODE)])
+def test_size_queries_beyond_any_tensor(lib, n_q, q_block, flags):
+    """Query rows per item (and query blocks padded to octets) past 2^31 wrap to zero or below; a size query answers all the same."""
+    cfg = CONFIGS[1].scaled(n_q_heads=n_q, n_kv_heads=1, q_block=q_block, seg_len=q_block, total_len=q_block, sink=0, local=0)
+    rc, r, b = _ws(lib, binding.make_params(cfg, flags=flags))
+    assert rc == 0 and r == q_block // cfg.chunk * 4 + 16
+    assert b == ((n_q * q_block * 4 + 255) & ~255) + 16
+
+
 def test_varlen_prefix_sums_are_validated_on_the_host(lib):
     cfg = CONFIGS[1]
     p = binding.make_params(cfg)
