@@ -20,9 +20,9 @@ __host__ __device__ inline int score_agg_of(int flags) {
 // kernels; and where dQ takes the place of Q, dO or O.
 constexpr int kFlagNoPdl = 1 << 30;
 
-// Division of 0 <= n < 2^31 by a number that the host knows: three instructions on the device.  (A division by a value that the
-// compiler does not know is 25 instructions and a chain of as many steps, and a CTA has half a dozen of them ahead of its
-// first copy: whole steps, 16K layer 143.7 -> 140.4 us, 2K layer 137.6 -> 134.7, 128K 87.9 -> 86.3, walk of 16K 1062 -> 1039.)
+// Division of 0 <= n < 2^31 by a number that the host knows, as a multiplication and a shift (T. Granlund, P. Montgomery:
+// Division by Invariant Integers using Multiplication, 1994).  A CTA has half a dozen such divisions ahead of its first copy, one
+// behind the other: 16K layer (whole step) 143.7 us with plain divisions, 140.4 so.
 struct Div {
   uint32_t by, mul, shift;
   __host__ __device__ Div() : by(1), mul(1), shift(0) {}
