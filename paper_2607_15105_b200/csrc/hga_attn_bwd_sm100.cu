@@ -753,7 +753,7 @@ static int launch_sweep(const Dims& dm, SegTable* table, const Segs& segs, int64
                         const void* O, const float* LSE, const void* dO, const int32_t* group_idx,
                         const int32_t* n_groups, void* dQ, float* dK, float* dV, int32_t* status_word, cudaStream_t st) {
   // (items wider than this have always had the CUDA-core kernel, whose probabilities are fp32)
-  if (max_routed_tokens(dm) > kMostRoutedTokens) return HGA_ERR_UNSUPPORTED;
+  if ((int64_t)dm.sink + (int64_t)dm.width * dm.g + dm.local + dm.Bq + dm.c > kMostRoutedTokens) return HGA_ERR_UNSUPPORTED;
   CUtensorMap mq, mdo, mk, mv;
   const uint32_t box[5] = {64, 8, 2, 1, 1};
   const uint32_t box_q[5] = {64, 64, 1, 1, 1};

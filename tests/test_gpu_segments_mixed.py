@@ -174,3 +174,24 @@ def test_the_widest_items_the_sweep_has_room_for(kc, tensor):
     torch.cuda.synchronize()
     for a, b in zip(*grads):          # bf16 P and dS against fp32 ones: 2^-9 per term
         assert float((a - b).norm()) <= 1e-2 * float(b.norm())
+
+
+def test_a_window_that_no_sequence_reaches_is_a_wide_item():
+    """A local window near 2^31 (every key is local): its sum with the other parts of an item does not fit 32 bits."""
+    cfg = cfg_of(1024, 256, chunk=64, group=8, q_block=64, topk_chunks=4, topk_groups=3, sink=64, local=2 ** 31 - 128)
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    Q, dO = (draw(gen, 1, cfg.n_q_heads, 256, 128) for _ in range(2))
+    K, V = (draw(gen, 1, cfg.n_kv_heads, 1024, 128) for _ in range(2))
+    grads = []
+    for c, flags in ((cfg, 0), (cfg.scaled(local=1024), binding.HGA_FLAG_GENERIC_KERNELS)):
+        buf = binding.HgaLayerBuffers(c, flags=flags)
+        buf.build_summaries(K, 0, 1024)
+        buf.route(Q)
+        buf.attn_fwd(Q, K, V)
+        before = binding.hga_kernel_launch_counts()
+        buf.attn_bwd(Q, K, V, dO)
+        n = ran(before)
+        assert n[binding.HGA_KERNELS_BWD_TENSOR] == 0 and n[binding.HGA_KERNELS_BWD_GENERIC] == 2 and int(buf.status.item()) == 0
+        grads.append((buf.dQ.float(), buf.dK, buf.dV))
+    for a, b in zip(*grads):          # (O, which delta is taken of, comes from two forward kernels: bf16 weights and fp32 ones)
+        assert float((a - b).norm()) <= 1e-2 * float(b.norm())
