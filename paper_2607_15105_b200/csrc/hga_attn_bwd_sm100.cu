@@ -210,14 +210,14 @@ k_attn_bwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 
   bool ok = true;
   // all lanes poll (one lane and a shuffle took longer)
-  auto wait = [&](uint64_t* bar, uint32_t parity) {
-    ok = __all_sync(0xffffffffu, bwd_wait(bar, parity & 1, abort));
+  auto wait = [&](uint64_t* bar, uint32_t parity, int line = __builtin_LINE()) {
+    ok = __all_sync(0xffffffffu, bwd_wait_(bar, parity & 1, abort, HGA_WAIT_CODE(line)));
     return ok;
   };
   // ... out of line, for the roles that can spare the call (the row threads cannot: 1 us of the 16K layer)
-  auto wait_by_call = [&](uint64_t* bar, uint32_t parity) { return ok = wait_out_of_line(bar, parity, abort); };
+  auto wait_by_call = [&](uint64_t* bar, uint32_t parity, int line = __builtin_LINE()) { return ok = wait_out_of_line(bar, parity, abort, line); };
   // Description of the CTA's n-th unit; done_with_info() once its fields have been read
-  auto unit_info = [&](int n) -> const Unit& { wait_by_call(&sm.info_full[n & 1], n >> 1); return sm.unit[n & 1]; };
+  auto unit_info = [&](int n, int line = __builtin_LINE()) -> const Unit& { wait_by_call(&sm.info_full[n & 1], n >> 1, line); return sm.unit[n & 1]; };
   auto done_with_info = [&](int n) { mbar_arrive_warp(&sm.info_empty[n & 1]); };
 
   if (warp == 18) {

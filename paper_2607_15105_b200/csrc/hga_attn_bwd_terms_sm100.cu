@@ -212,7 +212,7 @@ k_attn_bwd_terms_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_c
       const int o = 8 * (j - n_lt) + 4 * half + (lane & 3);
       return o < far.n_far ? sg.k0 + far.row(o) : dm.rows_k;
     };
-    auto wait_for = [&](uint64_t* bar, uint32_t parity) { return ok = wait_out_of_line(bar, parity, abort); };
+    auto wait_for = [&](uint64_t* bar, uint32_t parity, int line = __builtin_LINE()) { return ok = wait_out_of_line(bar, parity, abort, line); };
     auto copy_k = [&](int j, int row) {
       note_rows(j, row);
       __syncwarp();                            // (all of them, before the arrival that publishes them)
@@ -245,7 +245,7 @@ k_attn_bwd_terms_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_c
     // ------------------------------------------------------------------ MMA issuer
     // The whole warp runs this branch converged (waits included) and one elected lane issues: see mma_ss_w.
     const uint32_t lead = elect_one();
-    auto mma_wait = [&](uint64_t* bar, uint32_t parity) { return wait_out_of_line(bar, parity, abort); };
+    auto mma_wait = [&](uint64_t* bar, uint32_t parity, int line = __builtin_LINE()) { return wait_out_of_line(bar, parity, abort, line); };
     constexpr uint32_t idesc_sdp = idesc_bf16_f32(128, kKT, 0, 0);       // rows x 64 keys, both K-major
     constexpr uint32_t idesc_dq = idesc_bf16_f32(128, D, 0, 1);          // dS K-major, K tile MN-major
     constexpr uint32_t idesc_dkv = idesc_bf16_f32(128, kKT, 1, 1);       // both MN-major

@@ -470,7 +470,7 @@ k_attn_fwd_sm100(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // ------------------------------------------------------------------ producers
     bool ok = true, known = false;
     int n_oct = 16 * n_pre + 1;                    // (enough until the list is known)
-    auto wait_for = [&](uint64_t* bar, uint32_t parity) { return ok = wait_out_of_line(bar, parity, abort); };
+    auto wait_for = [&](uint64_t* bar, uint32_t parity, int line = __builtin_LINE()) { return ok = wait_out_of_line(bar, parity, abort, line); };
     auto learn = [&]() {
       known = true;
       if (!wait_for(&sm.info_full, 0)) return false;

@@ -31,17 +31,27 @@ __device__ __forceinline__ bool bwd_wait_(uint64_t* bar, uint32_t parity, volati
   return fine;
 }
 #ifdef HGA_DEBUG_WAIT
-#define bwd_wait(bar, parity, abort) bwd_wait_((bar), (parity), (abort), __LINE__)
+#define HGA_WAIT_CODE(line) (line)
 #define HGA_ABORT_CODE(kernel, flag) (HGA_STATUS_WAIT_TIMEOUT | ((flag) << 8) | ((kernel) << 28))
 #else
-#define bwd_wait(bar, parity, abort) bwd_wait_((bar), (parity), (abort), 1)
+#define HGA_WAIT_CODE(line) 1
 #define HGA_ABORT_CODE(kernel, flag) HGA_STATUS_WAIT_TIMEOUT
 #endif
 
-// The same for a whole warp, all of whose lanes poll, and out of line: for roles that can spare the call
-static __device__ __noinline__ bool wait_out_of_line(uint64_t* bar, uint32_t parity, volatile int* abort) {
+#define bwd_wait(bar, parity, abort) bwd_wait_((bar), (parity), (abort), HGA_WAIT_CODE(__LINE__))
+
+// The same for a whole warp, all of whose lanes poll, and out of line: for roles that can spare the call.  (What a role wraps it
+// in hands the line of its own call on; only the diagnostic build has the argument.)
+#ifdef HGA_DEBUG_WAIT
+static __device__ __noinline__ bool wait_out_of_line(uint64_t* bar, uint32_t parity, volatile int* abort, int line = __builtin_LINE()) {
+  return __all_sync(0xffffffffu, bwd_wait_(bar, parity & 1, abort, line));
+}
+#else
+static __device__ __noinline__ bool poll_by_warp(uint64_t* bar, uint32_t parity, volatile int* abort) {
   return __all_sync(0xffffffffu, bwd_wait(bar, parity & 1, abort));
 }
+__device__ __forceinline__ bool wait_out_of_line(uint64_t* bar, uint32_t parity, volatile int* abort, int = 0) { return poll_by_warp(bar, parity, abort); }
+#endif
 
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
