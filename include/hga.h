@@ -200,7 +200,7 @@ HGA_API int hga_attn_fwd(const hga_params* p, const void* Q, const void* K, cons
  * HGA_FLAG_BWD_ACCUMULATE is set.  The sum over query blocks
  * uses floating-point atomics: results may differ in the last bits from run to run.  At head_dim 128 and whole 128-row
  * tiles per item (G*Bq a multiple of 128) the tensor-core kernels take items of up to 3327 routed keys (sink + k_c*kg_eff*g +
- * local + Bq + c); wider ones have the CUDA-core kernel.
+ * local + Bq + c), with bf16 P and dS; wider ones have the CUDA-core kernel, with fp32 ones.
  * workspace: device scratch of at least hga_workspace_bytes().bwd bytes. */
 HGA_API int hga_attn_bwd(const hga_params* p, const void* Q, const void* K, const void* V, const void* O,
                  const float* LSE, const void* dO, const int32_t* group_idx,

@@ -129,7 +129,7 @@ static bool segments_supported(const Dims& dm, const std::vector<Segment>& segs,
 }
 
 // Routing, forward and (dO given) backward of all segments, up to kMaxSegments per launch, longest first.  *bwd_done: the
-// backward was queued too (it is not where its kernels have no room for the widest item).  HGA_ERR_UNSUPPORTED: the routing or
+// backward was queued too (it is not where the items are so wide that they have the CUDA-core kernel).  HGA_ERR_UNSUPPORTED: the routing or
 // the forward of these tensors is not for the tensor-core kernels after all (a stride that no tensor map takes), the same for
 // every group of segments; the caller goes on segment by segment, which repeats what has been queued.
 static int run_segments(Dims dm, std::vector<Segment> segs, bool summaries, const void* Q, const void* K, const void* V,

@@ -61,7 +61,7 @@ constexpr int kOct = 8 * kBwdD * 2;             // bytes of one octet of K/V row
 constexpr int kStage = 16 * kOct;               // bytes of one stage: the octets of a pair
 constexpr int kKStages = 3, kVStages = 2;
 constexpr int kInfoReaders = 19;                // warps that read a unit's description (all but the planner)
-constexpr int kMostRoutedTokens = 3327;         // wider items have the CUDA-core kernel (see launch_sweep)
+constexpr int kMostRoutedTokens = 3327;         // wider items keep the CUDA-core kernel's precision (see launch_sweep)
 
 struct Unit {
   int n_pairs;                                  // none: there is no further unit
@@ -752,7 +752,11 @@ template <class Segs>
 static int launch_sweep(const Dims& dm, SegTable* table, const Segs& segs, int64_t units, const void* Q, const void* K, const void* V,
                         const void* O, const float* LSE, const void* dO, const int32_t* group_idx,
                         const int32_t* n_groups, void* dQ, float* dK, float* dV, int32_t* status_word, cudaStream_t st) {
-  // (items wider than this have always had the CUDA-core kernel, whose probabilities are fp32)
+  // Nothing here depends on the width; the line is one of precision.  The CUDA-core kernel, which the wider items were given by an
+  // earlier sweep that had no room for their table, holds P and dS in fp32, and their callers have had its errors since.  Against fp64
+  // (dQ / dK / dV), 16 items of 256 rows and 4.5K keys: CUDA cores 1.67e-3 / 5.9e-5 / 5.6e-7 in 1359 us, this kernel 2.86e-3 / 2.00e-3 /
+  // 1.65e-3 in 76 us, k_attn_bwd_terms_sm100 1.67e-3 / 5.9e-5 / 1.30e-6 in 164 us.  Narrower items have this kernel's errors:
+  // 3.2K keys 2.86e-3 / 2.02e-3 / 1.67e-3, 56 us.
   if ((int64_t)dm.sink + (int64_t)dm.width * dm.g + dm.local + dm.Bq + dm.c > kMostRoutedTokens) return HGA_ERR_UNSUPPORTED;
   CUtensorMap mq, mdo, mk, mv;
   const uint32_t box[5] = {64, 8, 2, 1, 1};

@@ -1,6 +1,6 @@
 """hga_varlen_step and hga_tbptt_walk where one launch for all segments does not take every step, against the four calls
-made segment by segment: items too wide for the sweep's table of routed octets (the forward of all segments in one
-launch per 64, the backward segment by segment on the CUDA cores, on library streams), with gradients that are
+made segment by segment: items so wide that they keep the CUDA-core backward's fp32 probabilities (the forward of all segments in one
+launch per 64, the backward segment by segment, on library streams), with gradients that are
 overwritten or added to; and strides that no tensor map takes (everything segment by segment, as the calls by themselves)."""
 import numpy as np
 import pytest
@@ -155,7 +155,7 @@ def test_walk_with_bf16_gradients():
 
 @pytest.mark.parametrize("kc,tensor", [(383, True), (384, False)])
 def test_the_widest_items_the_sweep_has_room_for(kc, tensor):
-    """Room for 3327 routed keys per item (sink, groups, window, block and a chunk) beside the tiles; from there on the CUDA cores."""
+    """Up to 3327 routed keys per item (sink, groups, window, block and a chunk) the sweep; from there on the CUDA cores, with fp32 P and dS."""
     cfg = cfg_of(1024, 256, chunk=64, group=8, q_block=64, topk_chunks=kc, topk_groups=1, sink=64, local=64)
     gen = torch.Generator(device="cuda").manual_seed(kc)
     Q, dO = (draw(gen, 1, cfg.n_q_heads, 256, 128) for _ in range(2))
