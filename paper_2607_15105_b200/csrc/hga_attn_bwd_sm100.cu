@@ -30,7 +30,7 @@
 // What bounds it: the row threads, ~2.7k cycles per pair (1.0k of exponentials; tensor-memory loads and barrier hand-offs), a unit's
 // first pair, which waits for dO (its buffer is free only behind the last pair's dP), and a pair with dK/dV, whose place costs the K
 // ring its third stage.  Whole steps, one CTA per unit -> persistent: 16K layer 161 -> 147 us, walk of 16K 1147 -> 1076; 2K layer,
-// nearly all of whose pairs have dK/dV, 149 -> 139; twelve packed sequences 369 -> 334.  The 2K layer's additions (168 MB of
+// nearly all of whose pairs have dK/dV, 149 -> 139; twelve packed sequences 369 -> 334.  The 2K layer's additions (133 MB of
 // fp32) are what it waits for.
 //
 // Warp roles (640 threads, 96 registers):
